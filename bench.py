@@ -121,6 +121,28 @@ def phase_bytes(H, W, L, DK, DB, refine=1):
     }
 
 
+def tap_flops_per_ccd(H, W, L, DK):
+    """Multiply-adds x 2 of the image-space sums over the pixels (L >= 7): L^2
+    and (L - 1)^2 taps of the two corner products with 2 D_K + 1 powers of x,
+    and L^2 taps of the right-hand side with D_K + 1."""
+    return 2 * H * W * ((L * L + (L - 1) ** 2) * (2 * DK + 1) + L * L * (DK + 1))
+
+
+def direct_phase_bytes(H, W, L, DK, DB, refine=1):
+    """phase_bytes of the image-space assembly: no spectra, so the sums read
+    R_m, S (or the residual) and M_fit and write partial sums that are small
+    against the images."""
+    px = H * W
+    return {
+        # sky sums (R, S, bad), masks and R_m (R, S, bad in; good, R_m out), two
+        # erosion passes (1 B in, 1 B out each), edge lists (M_fit twice)
+        "prep": px * (9 + 14 + 4 + 2),
+        "contract_kk": px * 9,
+        "contract_rk": px * 8 * refine,
+        "apply": px * (13 * refine + 12),
+    }
+
+
 def half_plane_differences(L):
     return L + (L - 1) * (2 * L - 1)
 
@@ -467,7 +489,7 @@ def time_exposure(dev, stream, pairs, args, dist, steps=3, warmup=2):
            "warmup": warmup, "ms_per_step": 1e3 * sec / steps, "ms_per_ccd": 1e3 * sec / steps / B,
            "tiles": {"d_batch": plan.tiles[0], "rows_per_cta": plan.tiles[1], "lag_parts": plan.tiles[2],
                      "ccd_group": plan.ccd_group},
-           "kk_engine": plan.engine, "clocks": clk.summary(),
+           "kk_engine": "image_space", "clocks": clk.summary(),
            "status": [int(v) for v in out["info"].cpu()],
            "masked_fraction": [float(p["masked_fraction"]) for p in pairs],
            "workload": (f"{B} CCD pairs of one DECam exposure (2048x4096 FP32 each, seeds 100+, independent PSF "
@@ -524,11 +546,15 @@ def run_gpu(args):
                     fma_contract=args.fma_contract, mma_sync_contract=args.mma_sync_contract,
                     pair_lane_contract=args.pair_lane_contract)
         tiles = plan.tiles
-        engine = plan.engine
+        # an engine flag or a tile field selects the spectral assembly
+        spectral = bool(args.d_batch or args.lag_parts or (args.prec == "mixed" and (
+            args.fma_contract or args.mma_sync_contract or args.pair_lane_contract)))
+        engine = plan.engine if spectral else "image_space"
         if batched:
             # per-phase times and launch counts from an eager profiled pass of the same plan
             eager = Plan(Hs, W, L, DK, DB, batch=B, prec=args.prec, stream=stream, device=dev,
-                         d_batch=tiles[0], rows_per_cta=tiles[1], lag_parts=tiles[2], fma_contract=args.fma_contract,
+                         **(dict(d_batch=tiles[0], rows_per_cta=tiles[1], lag_parts=tiles[2]) if spectral else {}),
+                         fma_contract=args.fma_contract,
                          mma_sync_contract=args.mma_sync_contract, pair_lane_contract=args.pair_lane_contract)
             eo = eager.subtract(R, S, bad, None, refine=REFINE)
             eager.profile(True)
@@ -604,7 +630,7 @@ def run_gpu(args):
             stream.synchronize()
         s64 = _max_over_ranks(dist, dev, e0.elapsed_time(e1) / 1e3)
         fp64 = {"value": world * n64 / s64, "unit": UNIT, "ms_per_ccd": 1e3 * s64 / n64, "ccds_timed": n64,
-                "note": "plain FP64 GPU path (FP64 FFTs, products and contraction), sequential single-CCD calls"}
+                "note": "plain FP64 GPU path (every sum, the solve and the convolutions in FP64), sequential single-CCD calls"}
         del p64, o64
 
     # the KK contraction on the FP32 FMA pipes (tensor cores left to the stamp classifier), same pair
@@ -630,7 +656,19 @@ def run_gpu(args):
     kk_ms, kk_n = prof["contract_kk"]
     roof = None
     clocks = clk.summary()
-    if kk_n:
+    if kk_n and engine == "image_space":
+        avg_ms = kk_ms / args.steps
+        fp64_run = args.prec == "fp64"
+        flop = B * tap_flops_per_ccd(Hs, W, L, DK)
+        peak = alu_peaks["fp64_tflops"] if fp64_run else alu_peaks["fp32_tflops"]
+        achieved = flop / (avg_ms * 1e-3) / 1e12
+        roof = {"bound": "alu", "kernel": "k_tap_sums (image-space sums of the normal equations, with their reduction)",
+                "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": args.traffic,
+                "peak_note": f"{'FP64' if fp64_run else 'FP32'} FMA peak of measured (sfft_probe_fma_peak, this run)",
+                "algorithmic_flop_per_launch": flop, "avg_launch_ms": avg_ms, "launches_per_step": 1}
+        if batched:
+            roof["timing_note"] = "kernel durations from an eager profiled pass of the same plan (timed steps replay a CUDA graph)"
+    elif kk_n:
         on_tc = args.prec == "mixed" and not args.fma_contract
         # the contract_kk phase holds one contraction launch per batch of offset
         # differences on the tensor-core engines (their lag DFT and exact
@@ -686,7 +724,7 @@ def run_gpu(args):
         hbm = {"peak_gbs": pk, "peak_note": f"STREAM-style copy of {psrc} (MEASURED_PEAKS.json)",
                "note": "per CCD: algorithmic bytes (each kernel's inputs read once, outputs written once) / phase "
                        "time (CUDA events around the phase's kernels)"}
-        for k, nbytes in phase_bytes(Hs, W, L, DK, DB, REFINE).items():
+        for k, nbytes in (direct_phase_bytes if engine == "image_space" else phase_bytes)(Hs, W, L, DK, DB, REFINE).items():
             ms = prof[k][0] / args.steps
             if ms > 0:
                 gbs = nbytes / (ms * 1e-3) / 1e9

@@ -99,6 +99,7 @@ typedef struct {
   int32_t batch;             /* CCD pairs per call */
   int32_t prec;              /* sfft_prec_t */
   int32_t autotune;          /* 1: time contraction tile shapes at plan time and keep the fastest */
+  /* tile shape of the spectral assembly; a non-zero value also selects that assembly */
   int32_t d_batch;           /* kernel-offset differences per product/FFT pass (0 = auto) */
   int32_t rows_per_cta;      /* rows of one contraction partial sum (0 = auto) */
   int32_t lag_parts;         /* threads sharing the lags of one contraction k-slot: 2 or 3 (0 = auto;
@@ -119,7 +120,8 @@ void          sfft_plan_destroy(sfft_plan_t plan);
 sfft_status_t sfft_plan_set_stream(sfft_plan_t plan, void* cuda_stream);
 int64_t       sfft_num_unknowns(sfft_plan_t plan);          /* N */
 size_t        sfft_workspace_bytes(sfft_plan_t plan);       /* bytes for `ws` */
-/* KK-contraction engine the plan runs: 0 FP64 FMA (FP64 path), 1 FP32 FMA,
+/* KK-contraction engine of the plan's spectral assembly (see
+ * sfft_build_normal for when a plan takes it): 0 FP64 FMA (FP64 path), 1 FP32 FMA,
  * 2 tensor cores through mma.sync, 3 tcgen05 with one tensor-memory lane per
  * (difference, u_y) pair, 4 tcgen05 with one lane per difference; -1 for a
  * null plan. */
@@ -175,7 +177,14 @@ int64_t       sfft_debug_live_allocations(void);
 
 /* Normal-matrix assembly (the method's Fourier-domain normal equations):
  *   A = sum_x M_fit Phi Phi^T,  b = sum_x M_fit Phi S'   (FP64 outputs)
- * KK block: for every kernel-offset difference d = u - u' and weight monomial
+ * By default the sums are formed in image space: for every kernel-offset
+ * difference d = u - u' one weighted sum over the pixels, the other offsets u
+ * from it by sums over the edges of M_fit (L >= 7; for L <= 5 every offset pair
+ * is summed over the pixels), and b_K and the moments in the same pass.
+ * Plans that choose a spectral engine (an engine flag on the mixed path) or set
+ * one of the spectral stage's tile fields (d_batch, rows_per_cta, lag_parts,
+ * ccd_group), and images of 2^31 pixels or more, are assembled from row
+ * spectra: the KK block is then, for every d and weight monomial
  * xt^a yt^b, the row-FFT cross-correlation of the masked product
  * R_m(z) R_m(z + d) with M_fit xt^a yt^b, sampled at the lags u; KB block and
  * b_K: the same with R_m against M_fit phi_p psi_q and M_fit phi_p S'; BB and
@@ -185,7 +194,7 @@ int64_t       sfft_debug_live_allocations(void);
  *          mean of the good pixels (any constant gives the same kernel and D
  *          away from non-finite pixels and the w-pixel border);
  *   A    : double [batch][N][N] (written fully, symmetric);  b : double [batch][N];
- *   ws   : workspace; keeps the masks, spectra and sky for sfft_solve/apply. */
+ *   ws   : workspace; keeps the masks, R_m and sky for sfft_solve/apply. */
 sfft_status_t sfft_build_normal(sfft_plan_t plan, const float* R, const float* S,
                                 const uint8_t* bad, const double* sky,
                                 double* A, double* b, void* ws);
@@ -264,13 +273,15 @@ enum {
   SFFT_PROF_PREP = 0,        /* sky, masks, erosion, moments */
   SFFT_PROF_FFT_WEIGHTS = 1, /* row FFTs of weight maps, R_m and residual maps */
   SFFT_PROF_FFT_PROD = 2,    /* row FFTs of the products R_m(z) R_m(z + d) */
-  SFFT_PROF_CONTRACT_KK = 3, /* lag contraction of the product spectra (KK block) */
-  SFFT_PROF_CONTRACT_RK = 4, /* lag contraction against R_m spectra (KB, b_K, refinement) */
+  SFFT_PROF_CONTRACT_KK = 3, /* image-space tap sums of the fit, or the lag contraction of the product
+                                spectra (KK block) */
+  SFFT_PROF_CONTRACT_RK = 4, /* tap sums of the refinement residual, or the lag contraction against
+                                R_m spectra (KB, b_K, refinement) */
   SFFT_PROF_SCATTER = 5,     /* assembly of A and b from the accumulators */
   SFFT_PROF_SOLVE = 6,       /* Cholesky, triangular solves (and, mixed with no refinement steps,
                                 one FP64 residual step) */
   SFFT_PROF_APPLY = 7,       /* convolve-and-subtract and refinement residual */
-  SFFT_PROF_LAG_DFT = 8,     /* tensor-core KK paths: lags u_x over the k-slot products and the
+  SFFT_PROF_LAG_DFT = 8,     /* image space: mask-edge sums and their chains; tensor-core KK paths: lags u_x over the k-slot products and the
                                 exact slot-0 sums */
   SFFT_PROF_N = 9
 };

@@ -184,6 +184,9 @@ class Plan:
     mma.sync instead of tcgen05 (SFFT_FLAG_MMA_SYNC_CONTRACT);
     pair_lane_contract=True runs the tcgen05 contraction with one tensor-memory
     lane per (difference, u_y) pair (SFFT_FLAG_PAIR_LANE_CONTRACT).
+    The flags above, and a non-zero d_batch, rows_per_cta, lag_parts or
+    ccd_group, select the spectral assembly of A and b instead of the
+    image-space sums; `engine` names the contraction of that assembly.
     ccd_group: CCDs whose product spectra are held at once (0: the plan's choice)."""
 
     def __init__(self, H, W, L, DK, DB, batch=1, prec="mixed", d_batch=0, rows_per_cta=0, autotune=0,

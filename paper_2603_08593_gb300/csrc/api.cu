@@ -124,10 +124,18 @@ static void build_layout(sfft_plan_s* p) {
   add_region(p->rowflag, cur, sizeof(int) * (size_t)p->rf_stride * B);
   add_region(p->rm, cur, npx * e * B);
   add_region(p->eimg, cur, npx * e * B);
-  add_region(p->wspec, cur, slab * p->n_wa * B);
-  add_region(p->uspec, cur, slab * (p->d.DK + 1) * B);
-  add_region(p->rhat, cur, slab * B);
-  add_region(p->phat, cur, slab * p->d_batch * p->ccd_group);
+  const size_t spectra = p->direct ? 0 : 1;
+  add_region(p->wspec, cur, spectra * slab * p->n_wa * B);
+  add_region(p->uspec, cur, spectra * slab * (p->d.DK + 1) * B);
+  add_region(p->rhat, cur, spectra * slab * B);
+  add_region(p->phat, cur, spectra * slab * p->d_batch * p->ccd_group);
+  size_t part = 0, hp = 0, hs = 0, list = 0, cnt = 0;
+  if (p->direct) tap_region_bytes(p, &part, &hp, &hs, &list, &cnt);
+  add_region(p->tappart, cur, part);
+  add_region(p->hpart, cur, hp);
+  add_region(p->hsum, cur, hs);
+  add_region(p->elist, cur, list);
+  add_region(p->ecnt, cur, cnt);
   add_region(p->gkk, cur, sizeof(double) * p->n_hd * LL * n_mono(p->DM_KK) * B);
   add_region(p->gkb, cur, sizeof(double) * LL * n_mono(p->DM_KB) * B);
   add_region(p->gbk, cur, sizeof(double) * LL * n_mono(p->DM_bK) * B);
@@ -141,7 +149,7 @@ static void build_layout(sfft_plan_s* p) {
   add_region(p->swave, cur, sizeof(double) * 2 * p->N * B);
   add_region(p->vec, cur, sizeof(double) * 4 * p->N * B);
   // lane-per-difference contraction: k-slot products C[k][d_local][u_y][32] per CCD of a group
-  add_region(p->cbuf, cur, p->dl ? sizeof(float) * (size_t)p->M * p->d_batch * p->d.L * 32 * p->ccd_group : 0);
+  add_region(p->cbuf, cur, p->dl && !p->direct ? sizeof(float) * (size_t)p->M * p->d_batch * p->d.L * 32 * p->ccd_group : 0);
   add_region(p->theta_off, cur, sizeof(double) * p->N * B);
   p->ws_bytes = cur;
 }
@@ -370,6 +378,10 @@ void sfft::plan_free(void* ptr) {
 extern "C" int64_t sfft_debug_live_allocations(void) { return (int64_t)g_live_allocs.load(); }
 
 static void free_plan_device(sfft_plan_s* p) {
+  plan_free(p->tap.d_tasks);
+  plan_free(p->tap.d_dst);
+  plan_free(p->tap.d_pairs);
+  p->tap.d_tasks = nullptr; p->tap.d_dst = nullptr; p->tap.d_pairs = nullptr;
   plan_free(p->d_dljobs);
   plan_free(p->d_dlpairs);
   plan_free(p->d_tcjobs);
@@ -494,22 +506,43 @@ static sfft_status_t plan_impl(const sfft_desc_t* desc, void* cuda_stream, sfft_
   p->dl = p->umma && !(d.flags & SFFT_FLAG_PAIR_LANE_CONTRACT) && p->M % 16 == 0 && d.H >= 32 &&
           p->d_batch >= std::min(p->n_hd, 96);
   p->tc_rows = d.H;
+  // Image-space sums, unless the caller chooses a spectral engine or its tile
+  // shape: 1468 multiply-adds per pixel at L = 11, D_K = 2 in place of 221 row
+  // FFTs and a contraction of 6.4e11 flop per 2048 x 4096 CCD, 8.51 against
+  // 2.28 ms for its whole subtraction.  The line would lie at masks: their
+  // edges cost 7 ns each (y, L = 11, D_K = 2), so at 2 % to 30 % masked sky
+  // frames (10^4 - 10^5 edges) the assembly takes 0.9 ms against 6.9, and with
+  // 0.3 % isolated bad pixels 3.7; only a grid of bad pixels every 12 px
+  // (10.6 ms) passes the spectra.  The size is not known to the host, and a
+  // caller with such masks sets a tile field.  An edge's list entry holds its
+  // pixel in 31 bits.
+  const bool spectral = d.d_batch > 0 || d.rows_per_cta > 0 || d.lag_parts > 0 || d.ccd_group > 0 ||
+                        (!p->fp64 && (d.flags & (SFFT_FLAG_FMA_CONTRACT | SFFT_FLAG_MMA_SYNC_CONTRACT |
+                                                 SFFT_FLAG_PAIR_LANE_CONTRACT)));
+  p->direct = !spectral && (int64_t)d.H * d.W < (int64_t(1) << 31);
+  if (p->direct) build_tap_plan(p);
   build_layout(p);
-  build_jobs(p);
-  if (p->dl) build_dl_jobs(p);
-  if (p->umma) build_tc_jobs(p, kUmmaPairs, 1, 1 << 30, kUmmaMaxDiffs);
-  else if (p->tc) build_tc_jobs(p, 8 * kTcNT, kTcChunk, kTcRowCap, 1 << 30);
+  if (!p->direct) {
+    build_jobs(p);
+    if (p->dl) build_dl_jobs(p);
+    if (p->umma) build_tc_jobs(p, kUmmaPairs, 1, 1 << 30, kUmmaMaxDiffs);
+    else if (p->tc) build_tc_jobs(p, 8 * kTcNT, kTcChunk, kTcRowCap, 1 << 30);
+  }
 
   // yt(y)^b for b = 0..4 per row, FP64 on the host, stored in the path's precision
-  std::vector<double> ypow((size_t)d.H * 8, 0.0);
-  for (int y = 0; y < d.H; ++y) {
+  std::vector<double> ypow((size_t)(p->direct ? 0 : d.H) * 8, 0.0);
+  for (int y = 0; y < d.H && !p->direct; ++y) {
     const double yt = 2.0 * y / (double)(d.H > 1 ? d.H - 1 : 1) - 1.0;
     double pw = 1.0;
     for (int b = 0; b < 5; ++b) { ypow[(size_t)y * 8 + b] = pw; pw *= yt; }
   }
 
   sfft_status_t st = SFFT_OK;
-  if (p->fp64) {
+  if (p->direct) {
+    st = upload((void**)&p->tap.d_tasks, p->tap.tasks);
+    if (st == SFFT_OK) st = upload((void**)&p->tap.d_dst, p->tap.dst);
+    if (st == SFFT_OK) st = upload((void**)&p->tap.d_pairs, p->tap.pairs);
+  } else if (p->fp64) {
     std::vector<double2> a, b, c;
     fill_twiddles<double2, double>(p, a, b, c);
     if (st == SFFT_OK) st = upload(&p->twM, a);
@@ -531,12 +564,14 @@ static sfft_status_t plan_impl(const sfft_desc_t* desc, void* cuda_stream, sfft_
   }
   if (st == SFFT_OK) st = upload((void**)&p->d_dlist, p->dlist);
   if (st == SFFT_OK) st = upload((void**)&p->d_hdidx, hdidx);
-  if (st == SFFT_OK) st = upload((void**)&p->d_jobs, p->h_jobs);
-  if (st == SFFT_OK && p->tc) st = upload((void**)&p->d_tcjobs, p->h_tcjobs);
-  if (st == SFFT_OK && p->tc) st = upload((void**)&p->d_tcpairs, p->h_tcpairs);
-  if (st == SFFT_OK && p->tc) st = upload((void**)&p->d_tcdj, p->h_tcdj);
-  if (st == SFFT_OK && p->dl) st = upload((void**)&p->d_dljobs, p->h_dljobs);
-  if (st == SFFT_OK && p->dl) st = upload((void**)&p->d_dlpairs, p->h_dlpairs);
+  if (!p->direct) {
+    if (st == SFFT_OK) st = upload((void**)&p->d_jobs, p->h_jobs);
+    if (st == SFFT_OK && p->tc) st = upload((void**)&p->d_tcjobs, p->h_tcjobs);
+    if (st == SFFT_OK && p->tc) st = upload((void**)&p->d_tcpairs, p->h_tcpairs);
+    if (st == SFFT_OK && p->tc) st = upload((void**)&p->d_tcdj, p->h_tcdj);
+    if (st == SFFT_OK && p->dl) st = upload((void**)&p->d_dljobs, p->h_dljobs);
+    if (st == SFFT_OK && p->dl) st = upload((void**)&p->d_dlpairs, p->h_dlpairs);
+  }
   if (st != SFFT_OK) {
     free_plan_device(p);
     delete p;
@@ -583,8 +618,34 @@ extern "C" sfft_status_t sfft_plan_tiles(sfft_plan_t p, int32_t* o) {
 
 static bool aligned(const void* ptr, size_t a) { return ((uintptr_t)ptr % a) == 0; }
 
+// A and b from image-space sums (kernels_tap.cu)
+static sfft_status_t build_normal_direct(sfft_plan_t p, const float* R, const float* S, const uint8_t* bad,
+                                         const double* sky, double* A, double* b, void* ws) {
+  {
+    Phase ph(p, SFFT_PROF_PREP);
+    CK(cudaMemsetAsync(ws_at<char>(ws, p->status), 0, p->status.bytes, p->stream));
+    CK(launch_sky(p, R, S, bad, sky, ws));
+    CK(launch_prep(p, R, S, bad, ws));
+    CK(launch_edge_lists(p, ws));
+  }
+  {
+    Phase ph(p, SFFT_PROF_CONTRACT_KK);
+    CK(launch_tap_fit(p, S, ws));
+  }
+  {
+    Phase ph(p, SFFT_PROF_LAG_DFT);
+    CK(launch_edge_sums(p, ws));
+  }
+  {
+    Phase ph(p, SFFT_PROF_SCATTER);
+    CK(launch_scatter(p, A, b, ws, false, nullptr));
+  }
+  return SFFT_OK;
+}
+
 static sfft_status_t build_normal_impl(sfft_plan_t p, const float* R, const float* S, const uint8_t* bad,
                                        const double* sky, double* A, double* b, void* ws) {
+  if (p->direct) return build_normal_direct(p, R, S, bad, sky, A, b, ws);
   cudaStream_t st = p->stream;
   {
     Phase ph(p, SFFT_PROF_PREP);
@@ -685,6 +746,10 @@ static sfft_status_t solve_impl(sfft_plan_t p, const double* A, const double* b,
       Phase ph(p, SFFT_PROF_APPLY);
       CK(launch_apply(p, R, S, toff, nullptr, nullptr, e, true, ws));
     }
+    if (p->direct) {
+      Phase ph(p, SFFT_PROF_CONTRACT_RK);
+      CK(launch_tap_rhs(p, e, ws));
+    } else {
     {
       Phase ph(p, SFFT_PROF_FFT_WEIGHTS);
       CK(launch_rfft_weights(p, nullptr, e, 0, p->d.DK + 1, ws_at<char>(ws, p->uspec), p->d.DK + 1, ws));
@@ -697,6 +762,7 @@ static sfft_status_t solve_impl(sfft_plan_t p, const double* A, const double* b,
     {
       Phase ph(p, SFFT_PROF_PREP);
       CK(launch_moments(p, nullptr, e, true, ws));
+    }
     }
     {
       Phase ph(p, SFFT_PROF_SCATTER);

@@ -1,0 +1,1000 @@
+// Normal-matrix sums in image space: tap sums, mask-edge sums and the chains
+// that join them.
+//
+// Every entry of the kernel-kernel block is
+//   F_m(u, u') = sum_x M(x) m(x) R(x - u) R(x - u'),   m = xt^a yt^b,
+// with M the 0/1 fit mask and R the masked, sky-subtracted reference.  Moving
+// both offsets by one pixel e only moves the mask against the images:
+//   F(u + e, u' + e) = shift_e( F(u, u') + H(u, u') ),
+//   H_m(u, u') = sum_x [M(x + e) - M(x)] m(x) R(x - u) R(x - u'),
+// where shift_e substitutes xt + 2 e_x / (W - 1), yt + 2 e_y / (H - 1) in the
+// monomials.  M(x + e) - M(x) is non-zero only on the mask's edges, so for
+// each difference d = u - u' one sum over the image is enough (a corner of
+// the offset box) and the edges give the other offsets:
+//   * tap sums (k_tap_sums): per tile of 32 rows, sum_x c(x) xt^a R(x - u')
+//     for the L^2 offsets u', with c = M R(. - u0) for the two upper corners
+//     u0 = (+-w, w) (between them every half-plane d), and c = M S' (the
+//     right-hand side) or the refinement residual; yt^b at the tile's end.
+//   * edge sums (k_edge_gram): H for every pair, over the lists of mask edges
+//     in x (offsets with u_y = w) and in y (all offsets below w).
+//   * chains (k_edge_chain): along x at u_y = w, then down in y, in FP64.
+// At 2048 x 4096, L = 11, D_K = 2 a CCD takes 221 sums over the image in place
+// of 7381, and its mask has 10^4 - 10^5 edges against 8.4e6 pixels.  L <= 5
+// sums every pair over the image (15 distinct u_y rows of 5 taps at L = 5):
+// fewer launches, and no edges to list.
+#include <algorithm>
+#include <vector>
+
+#include "common.cuh"
+#include "plan.h"
+
+namespace sfft {
+
+// ------------------------------------------------------------------ packed pairs
+template <typename T> struct v2 { T x, y; };
+template <> struct v2<float> { float2 p; };
+
+__device__ __forceinline__ void v2_zero(v2<float>& a) { a.p = make_float2(0.f, 0.f); }
+__device__ __forceinline__ void v2_zero(v2<double>& a) { a.x = 0.0; a.y = 0.0; }
+// acc += (q0, q1) r
+__device__ __forceinline__ void v2_fma(v2<float>& a, float q0, float q1, float r) {
+  a.p = __ffma2_rn(make_float2(q0, q1), make_float2(r, r), a.p);
+}
+__device__ __forceinline__ void v2_fma(v2<double>& a, double q0, double q1, double r) {
+  a.x = fma(q0, r, a.x);
+  a.y = fma(q1, r, a.y);
+}
+__device__ __forceinline__ float v2_get(const v2<float>& a, int i) { return i ? a.p.y : a.p.x; }
+__device__ __forceinline__ double v2_get(const v2<double>& a, int i) { return i ? a.y : a.x; }
+
+__device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
+__device__ __forceinline__ void ld4(const double* p, double (&v)[4]) {
+  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, bool valid) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(BYTES), "r"(valid ? BYTES : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// ------------------------------------------------------------------ tap sums
+// A task is one row u'_y of taps against one centre image c: a warp's lanes
+// are the tile's 32 rows, each lane walks its row with the NT taps in a
+// sliding register window and keeps (rows of powers) x (taps) sums in
+// registers, so a shared-memory value read once feeds 2 x NT multiply-adds
+// per row of powers.  What bounds it is the FP32 FMA pipe (44 packed FMAs per
+// pixel, centre and tap row at D_K = 2); lanes as rows need no reduction
+// until the row's end, and the odd pitch keeps their reads free of bank
+// conflicts.
+enum { TAP_CS = 0, TAP_C = 1, TAP_S = 2, TAP_M = 3, TAP_MOM = 4 };
+enum { TAP_FIT_EDGE = 0, TAP_FIT_ALL = 1, TAP_RHS = 2 };
+
+constexpr int kTapRows = 32;
+constexpr int kTapWarps = 4;
+constexpr int kTapU = 8;          // pixels per unrolled step
+constexpr int kTapScr = 16;       // staged rows of the y fold per warp
+constexpr int kTapScrPitch = 36;
+constexpr int kTapMaxOut = 40;
+
+template <typename T>
+struct TapTile {
+  const T* r;              // [32 + 2 wt][pitch]: R, column 0 = x0 - wt, row 0 = y0 - wt
+  const T* s;              // [32][spitch]: M S' or the residual
+  const unsigned* m;       // [32][nw] mask bits
+  const T* xp;             // [tw][4] xt .. xt^4
+  const T* yp;             // [5][kTapScrPitch] yt^b of the tile's rows
+  T* scr;                  // this warp's [kTapScr][kTapScrPitch]
+  const unsigned char (*ot)[2];   // this type's outputs: (row of powers, b)
+  int pitch, spitch, nw, n;       // n: columns to walk (a multiple of kTapU)
+};
+
+// sum over the 32 staged values of row `row` times yt^b
+template <typename T>
+__device__ __forceinline__ T fold_row(const TapTile<T>& t, int row, int b) {
+  const T* v = t.scr + row * kTapScrPitch;
+  const T* y = t.yp + b * kTapScrPitch;
+  T s[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int i = 0; i < 32; i += 4) {
+    T a[4], c[4];
+    ld4(v + i, a);
+    ld4(y + i, c);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] += a[k] * c[k];
+  }
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
+// RC rows of powers of the centre c (MB: the mask itself), RS rows of s, against
+// the first K of the NT taps.  Rows go in packed pairs (two cycles of the FMA
+// pipe), an odd last row alone (one cycle).
+template <typename T, int NT, int K, int RC, int RS, bool MB>
+__device__ __forceinline__ void tap_task(const TapTile<T>& t, int u0x, int u0y, int uy, int nout, T* __restrict__ out) {
+  constexpr int NR = RC + RS, NP = NR / 2, ODD = NR & 1, wt = (NT - 1) / 2;
+  const int lane = threadIdx.x & 31;
+  const T* rr = t.r + (lane + wt - uy) * t.pitch;
+  const T* cr = t.r + (lane + wt - u0y) * t.pitch + (wt - u0x);
+  const T* sr = t.s + lane * t.spitch;
+  const unsigned* mr = t.m + lane * t.nw;
+  v2<T> acc[K][NP > 0 ? NP : 1];
+  T last[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    last[k] = 0;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) v2_zero(acc[k][p]);
+  }
+  T win[K - 1 + kTapU];
+#pragma unroll
+  for (int k = 0; k < K - 1; ++k) win[k] = rr[k];
+  for (int xb = 0; xb < t.n; xb += kTapU) {
+#pragma unroll
+    for (int i = 0; i < kTapU; ++i) win[K - 1 + i] = rr[xb + K - 1 + i];
+    const unsigned bits = RC > 0 ? mr[xb >> 5] >> (xb & 31) : 0u;
+#pragma unroll
+    for (int i = 0; i < kTapU; ++i) {
+      T q[NR];
+      T xp[4];
+      if (RC > 1 || RS > 1) ld4(t.xp + 4 * (xb + i), xp);
+      if constexpr (RC > 0) {
+        const bool on = (bits >> i) & 1u;
+        const T c = MB ? (on ? (T)1 : (T)0) : (on ? cr[xb + i] : (T)0);
+        q[0] = c;
+#pragma unroll
+        for (int a = 1; a < RC; ++a) q[a] = c * xp[a - 1];
+      }
+      if constexpr (RS > 0) {
+        const T s = sr[xb + i];
+        q[RC] = s;
+#pragma unroll
+        for (int a = 1; a < RS; ++a) q[RC + a] = s * xp[a - 1];
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) v2_fma(acc[k][p], q[2 * p], q[2 * p + 1], win[i + k]);
+        if (ODD) last[k] = fma(q[NR - 1], win[i + k], last[k]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < K - 1; ++k) win[k] = win[k + kTapU];
+  }
+  // yt^b over the tile's rows, KT taps at a time
+  constexpr int KT = kTapScr / NR;
+#pragma unroll
+  for (int k0 = 0; k0 < K; k0 += KT) {
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < KT; ++k)
+#pragma unroll
+      for (int a = 0; a < NR; ++a)
+        if (k0 + k < K) {
+          const int kk = k0 + k < K ? k0 + k : 0;
+          t.scr[(k * NR + a) * kTapScrPitch + lane] = a < 2 * NP ? v2_get(acc[kk][a < 2 * NP ? a / 2 : 0], a & 1) : last[kk];
+        }
+    __syncwarp();
+    const int nk = K - k0 < KT ? K - k0 : KT;
+    for (int o = lane; o < nk * nout; o += 32) {
+      const int k = o / nout, j = o % nout;
+      out[(k0 + k) * nout + j] = fold_row(t, k * NR + t.ot[j][0], t.ot[j][1]);
+    }
+  }
+}
+
+// Moments without taps: M xt^a (a <= 4), s xt^a (a <= 2), c xt^a (a <= 4), c = M R(. - (w, w))
+template <typename T>
+__device__ __forceinline__ void tap_moments(const TapTile<T>& t, int wt, int w, int nout, T* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const T* cr = t.r + (lane + wt - w) * t.pitch + (wt - w);
+  const T* sr = t.s + lane * t.spitch;
+  const unsigned* mr = t.m + lane * t.nw;
+  T acc[13];
+#pragma unroll
+  for (int a = 0; a < 13; ++a) acc[a] = 0;
+  for (int x = 0; x < t.n; ++x) {
+    const bool on = (mr[x >> 5] >> (x & 31)) & 1u;
+    const T m = on ? (T)1 : (T)0, c = on ? cr[x] : (T)0, s = sr[x];
+    const T* xp = t.xp + 4 * x;
+    acc[0] += m;
+    acc[5] += s;
+    acc[8] += c;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      acc[1 + a] += m * xp[a];
+      if (a < 2) acc[6 + a] += s * xp[a];
+      acc[9 + a] += c * xp[a];
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int a = 0; a < 13; ++a) t.scr[a * kTapScrPitch + lane] = acc[a];
+  __syncwarp();
+  for (int o = lane; o < nout; o += 32) out[o] = fold_row(t, t.ot[o][0], t.ot[o][1]);
+}
+
+template <typename T>
+__host__ __device__ constexpr size_t tap_smem(int wt, int tw) {
+  const int pitch = (tw + 2 * wt) | 1, spitch = tw | 1;
+  return sizeof(T) * ((size_t)5 * kTapScrPitch + (size_t)kTapWarps * kTapScr * kTapScrPitch + 4 * (size_t)tw +
+                      (size_t)(kTapRows + 2 * wt) * pitch + (size_t)kTapRows * spitch) +
+         4 * (size_t)kTapRows * (tw / 32);
+}
+
+// One CTA: a tile of 32 rows x tw columns and every nsplit-th task of the
+// table, taken in order by its warps.  Partial sums go to
+// part[ccd][tile][nout_tot]; k_tap_reduce adds the tiles in FP64.
+template <typename T, int NT, int DK, int MODE>
+__global__ void __launch_bounds__(kTapWarps * 32, sizeof(T) == 4 ? 3 : 2)
+k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const T* __restrict__ E,
+           const uint8_t* __restrict__ mfit, const double* __restrict__ sky, const int4* __restrict__ tasks, int ntask,
+           T* __restrict__ part, int nout_tot, int H, int W, int w, int tw) {
+  constexpr int wt = (NT - 1) / 2, RC = 2 * DK + 1, RS = DK + 1, RM = DK + 3;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ unsigned char ot[5][kTapMaxOut][2];
+  __shared__ int next;
+  const int pitch = (tw + 2 * wt) | 1, spitch = tw | 1, nw = tw / 32;
+  T* yp = reinterpret_cast<T*>(smraw);
+  T* scr = yp + 5 * kTapScrPitch;
+  T* xp = scr + kTapWarps * kTapScr * kTapScrPitch;
+  T* rt = xp + 4 * tw;
+  T* st = rt + (kTapRows + 2 * wt) * pitch;
+  unsigned* mw = reinterpret_cast<unsigned*>(st + kTapRows * spitch);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nth = kTapWarps * 32;
+  const int ntx = (W + tw - 1) / tw;
+  const int tile = blockIdx.x, ccd = blockIdx.z;
+  const int x0 = (tile % ntx) * tw, y0 = (tile / ntx) * kTapRows;
+  const int64_t img = (int64_t)ccd * H * W;
+  if (tid == 0) next = 0;
+  // outputs of each type: (row of powers, power of yt), in monomial order
+  if (tid < 5) {
+    int n = 0;
+    auto put = [&](int deg, int row0) {
+      for (int g = 0; g <= deg; ++g)
+        for (int b = 0; b <= g; ++b, ++n) { ot[tid][n][0] = (unsigned char)(row0 + g - b); ot[tid][n][1] = (unsigned char)b; }
+    };
+    if (tid == TAP_CS) { put(2 * DK, 0); put(DK, RC); }
+    if (tid == TAP_C) put(2 * DK, 0);
+    if (tid == TAP_S) put(DK, 0);
+    if (tid == TAP_M) put(DK + 2, 0);
+    if (tid == TAP_MOM) { put(4, 0); put(2, 5); put(4, 8); }
+  }
+  const double xs = 2.0 / (double)(W > 1 ? W - 1 : 1), ys = 2.0 / (double)(H > 1 ? H - 1 : 1);
+  for (int i = tid; i < tw; i += nth) {
+    const double x = (x0 + i) * xs - 1.0;
+    xp[4 * i] = (T)x; xp[4 * i + 1] = (T)(x * x); xp[4 * i + 2] = (T)(x * x * x); xp[4 * i + 3] = (T)(x * x * x * x);
+  }
+  if (tid < kTapRows) {
+    const double y = (y0 + tid) * ys - 1.0;
+    double v = 1.0;
+    for (int b = 0; b < 5; ++b) { yp[b * kTapScrPitch + tid] = (T)v; v *= y; }
+  }
+  // R with its halo, zero outside the image: copied asynchronously, every
+  // element in flight at once (plain loads kept 29 % of the warps' time
+  // waiting), a warp per row
+  for (int row = warp; row < kTapRows + 2 * wt; row += kTapWarps) {
+    const int gy = y0 - wt + row;
+    const bool in = gy >= 0 && gy < H;
+    const T* src = Rm + img + (int64_t)(in ? gy : 0) * W;
+    for (int c = lane; c < tw + 2 * wt; c += 32) {
+      const int gx = x0 - wt + c;
+      const bool ok = in && gx >= 0 && gx < W;
+      cp_async<sizeof(T)>(rt + row * pitch + c, src + (ok ? gx : 0), ok);
+    }
+  }
+  const T sS = MODE == TAP_RHS ? (T)0 : (T)sky[2 * ccd + 1];
+  for (int row = warp; row < kTapRows; row += kTapWarps) {
+    const int gy = y0 + row;
+    const int64_t o = img + (int64_t)gy * W;
+    if constexpr (MODE == TAP_RHS) {
+      for (int c = lane; c < tw; c += 32) {
+        const bool ok = gy < H && x0 + c < W;
+        cp_async<sizeof(T)>(st + row * spitch + c, E + (ok ? o + x0 + c : 0), ok);
+      }
+    } else {
+      // four columns at a time (tw is a multiple of 32)
+      for (int c0 = 0; c0 < tw; c0 += 128) {
+        float v[4];
+        bool on[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int gx = x0 + c0 + 32 * k + lane;
+          const bool ok = c0 + 32 * k < tw && gy < H && gx < W;
+          on[k] = ok && mfit[o + gx] != 0;
+          v[k] = ok ? S[o + gx] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int c = c0 + 32 * k;
+          if (c >= tw) break;
+          st[row * spitch + c + lane] = on[k] ? (T)v[k] - sS : (T)0;
+          const unsigned word = __ballot_sync(0xffffffffu, on[k]);
+          if (lane == 0) mw[row * nw + (c >> 5)] = word;
+        }
+      }
+    }
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  TapTile<T> t;
+  t.r = rt; t.s = st; t.m = mw; t.xp = xp; t.yp = yp;
+  t.scr = scr + warp * kTapScr * kTapScrPitch;
+  t.pitch = pitch; t.spitch = spitch; t.nw = nw;
+  t.n = min(tw, (W - x0 + kTapU - 1) / kTapU * kTapU);
+  T* po = part + ((int64_t)ccd * gridDim.x + tile) * nout_tot;
+  for (;;) {
+    int k = 0;
+    if (lane == 0) k = atomicAdd(&next, 1);
+    k = __shfl_sync(0xffffffffu, k, 0) * gridDim.y + blockIdx.y;
+    if (k >= ntask) break;
+    const int4 q = tasks[k];   // type | nout << 8, u0 (x, y biased by 64), u'_y, first output
+    const int type = q.x & 255, nout = q.x >> 8;
+    const int u0x = (q.y & 255) - 64, u0y = (q.y >> 8) - 64;
+    t.ot = ot[type];
+    T* out = po + q.w;
+    if constexpr (MODE != TAP_RHS) {
+      constexpr int KC = MODE == TAP_FIT_EDGE ? NT - 1 : NT;   // the corner (-w, w) has no d_x = 0
+      if (type == TAP_CS) tap_task<T, NT, NT, RC, RS, false>(t, u0x, u0y, q.z, nout, out);
+      else if (type == TAP_C) tap_task<T, NT, KC, RC, 0, false>(t, u0x, u0y, q.z, nout, out);
+      else if (MODE == TAP_FIT_ALL && type == TAP_M) tap_task<T, NT, NT, RM, 0, true>(t, 0, 0, q.z, nout, out);
+      else tap_moments<T>(t, wt, w, nout, out);
+    } else {
+      if (type == TAP_S) tap_task<T, NT, NT, 0, RS, false>(t, 0, 0, q.z, nout, out);
+      else tap_moments<T>(t, wt, w, nout, out);
+    }
+  }
+}
+
+// Sums of the tiles' partial sums, FP32 in fours and FP64 over them (FP64
+// throughout on the FP64 path), to the G and moment arrays: dst = region << 28
+// | offset, -1 = not needed.
+struct TapDst {
+  double* base[5];
+  int64_t stride[5];   // per CCD
+};
+
+template <typename T>
+__global__ void __launch_bounds__(512)
+k_tap_reduce(const T* __restrict__ part, const int* __restrict__ dst, TapDst d, int ntile, int nout) {
+  __shared__ double red[16][33];
+  const int ccd = blockIdx.y, lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int o = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (o < nout) {
+    const T* p = part + (int64_t)ccd * ntile * nout + o;
+    int t = g * 4;
+#pragma unroll 2
+    for (; t + 3 < ntile; t += 64) {
+      const T a = p[(int64_t)t * nout], b = p[(int64_t)(t + 1) * nout], c = p[(int64_t)(t + 2) * nout],
+              e = p[(int64_t)(t + 3) * nout];
+      s += (double)((a + b) + (c + e));
+    }
+    for (int k = t; k < min(t + 4, ntile); ++k) s += (double)p[(int64_t)k * nout];
+  }
+  red[g][lane] = s;
+  __syncthreads();
+  if (g == 0 && o < nout) {
+#pragma unroll
+    for (int k = 1; k < 16; ++k) s += red[k][lane];
+    const int q = dst[o];
+    if (q >= 0) {
+      const int r = q >> 28;
+      d.base[r][ccd * d.stride[r] + (q & 0xfffffff)] = s;
+    }
+  }
+}
+
+// ------------------------------------------------------------------ mask edges
+// Per row the numbers of x edges (M(x + 1, y) != M(x, y)) and y edges
+// (M(x, y + 1) != M(x, y)); then the lists, in row order, entry
+// (y W + x) << 1 | (M falls).  A warp per row.
+template <bool WRITE>
+__global__ void __launch_bounds__(256)
+k_edge_rows(const uint8_t* __restrict__ mfit, int H, int W, int* __restrict__ cnt, int64_t cnt_stride,
+            unsigned* __restrict__ lx, unsigned* __restrict__ ly, int64_t lstride) {
+  const int y = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, ccd = blockIdx.y;
+  if (y >= H) return;
+  const uint8_t* m = mfit + ((int64_t)ccd * H + y) * W;
+  const uint8_t* m1 = y + 1 < H ? m + W : m;
+  int* c = cnt + ccd * cnt_stride;
+  int nx = 0, ny = 0;
+  if (WRITE) { nx = c[y]; ny = c[H + 1 + y]; }
+  unsigned* ox = lx + ccd * lstride;
+  unsigned* oy = ly + ccd * lstride;
+  for (int x0 = 0; x0 < W; x0 += 32) {
+    const int x = x0 + lane;
+    int a = 0, b = 0, d = 0;
+    if (x < W) { a = m[x] != 0; b = x + 1 < W ? m[x + 1] != 0 : a; d = m1[x] != 0; }
+    const unsigned ex = __ballot_sync(0xffffffffu, a != b), ey = __ballot_sync(0xffffffffu, a != d);
+    if (WRITE) {
+      const unsigned below = (1u << lane) - 1u;
+      const unsigned v = ((unsigned)y * (unsigned)W + (unsigned)x) << 1 | (unsigned)a;
+      if (a != b) ox[nx + __popc(ex & below)] = v;
+      if (a != d) oy[ny + __popc(ey & below)] = v;
+    }
+    nx += __popc(ex);
+    ny += __popc(ey);
+  }
+  if (!WRITE && lane == 0) { c[y] = nx; c[H + 1 + y] = ny; }
+}
+
+// exclusive scan of the row counts; entry H is the total
+__global__ void __launch_bounds__(1024)
+k_edge_scan(int* __restrict__ cnt, int64_t cnt_stride, int H) {
+  __shared__ int wsum[32];
+  __shared__ int carry;
+  int* c = cnt + blockIdx.x * cnt_stride + blockIdx.y * (H + 1);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) carry = 0;
+  __syncthreads();
+  for (int base = 0; base < H; base += 1024) {
+    const int i = base + tid;
+    const int v = i < H ? c[i] : 0;
+    int s = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += t;
+    }
+    if (lane == 31) wsum[warp] = s;
+    __syncthreads();
+    int off = carry;
+    for (int k = 0; k < warp; ++k) off += wsum[k];
+    if (i < H) c[i] = off + s - v;
+    __syncthreads();
+    if (tid == 1023) carry = off + s;
+    __syncthreads();
+  }
+  if (tid == 0) c[H] = carry;
+}
+
+// ------------------------------------------------------------------ edge sums
+// H_m(u, u') over one list: a CTA stages 32 edge points at a time (the L^2
+// reference values around each, and the signed monomials) and each thread
+// keeps kGramP pairs x all monomials in registers.  The points of the next
+// batch are copied (cp.async) while this one is summed, and the list is read
+// two batches ahead; without it the gathers' latency took 60 % of the warps'
+// time.  Slot g of U takes batches g, g + U, ..., at least kGramMin<T> points, and
+// writes hp[ccd][slot][pair][MP]; a short list uses few slots.  Blocks y < nby
+// are y-edge pairs, the others x-edge pairs.
+constexpr int kGramP = 5;
+constexpr int kGramPts = 32;
+constexpr int kGramThreads = 256;
+constexpr int kGramPatch = 125;   // L^2 <= 121 values, then 1 (single offsets) and padding to an odd pitch
+// least points of a slot: FP64 multiply-adds are 64 times slower than FP32
+// ones, so there a short list spreads over more slots (one 512 x 512 pair,
+// L = 7, D_K = 1: 1.6 ms with 256 points, 1.1 ms with 32)
+template <typename T> constexpr int kGramMin = sizeof(T) == 4 ? 256 : kGramPts;
+
+struct GramArgs {
+  const int* pairs;        // i | j << 8: y pairs, then x pairs
+  int npy, npx, nby;       // pairs and y blocks
+  int gy, gx;              // most slots per list
+  int64_t hp_stride;       // per CCD
+  int64_t hx_off;          // x partials after the y ones
+};
+
+template <typename T>
+__device__ __forceinline__ int gram_slots(int n, int g) { return max(1, min(g, (n + kGramMin<T> - 1) / kGramMin<T>)); }
+
+template <typename T, int DE>
+__host__ __device__ constexpr size_t gram_smem() {
+  constexpr int MP = (n_mono(DE) + 3) / 4 * 4;
+  return 2 * sizeof(T) * kGramPts * (MP + kGramPatch) + 2 * kGramPts * sizeof(unsigned);
+}
+
+template <typename T, int DE>
+__global__ void __launch_bounds__(kGramThreads, sizeof(T) == 4 ? 2 : 1)
+k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const unsigned* __restrict__ ly, int64_t lstride,
+            const int* __restrict__ cnt, int64_t cnt_stride, GramArgs a, T* __restrict__ hp, int H, int W, int L) {
+  constexpr int NM = n_mono(DE), MP = (NM + 3) / 4 * 4;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  T(*mono)[kGramPts][MP] = reinterpret_cast<T(*)[kGramPts][MP]>(smraw);
+  T(*patch)[kGramPts][kGramPatch] =
+      reinterpret_cast<T(*)[kGramPts][kGramPatch]>(smraw + 2 * sizeof(T) * kGramPts * MP);
+  unsigned(*ent)[kGramPts] =
+      reinterpret_cast<unsigned(*)[kGramPts]>(smraw + 2 * sizeof(T) * kGramPts * (MP + kGramPatch));
+  const int ccd = blockIdx.z, tid = threadIdx.x, w = (L - 1) / 2, lane = tid & 31, warp = tid >> 5;
+  const bool isx = (int)blockIdx.y >= a.nby;
+  const int n = cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H];
+  const int U = gram_slots<T>(n, isx ? a.gx : a.gy), g = blockIdx.x;
+  if (g >= U) return;
+  const int blk = isx ? blockIdx.y - a.nby : blockIdx.y;
+  const int np = isx ? a.npx : a.npy;
+  const int* ptab = a.pairs + (isx ? a.npy : 0);
+  const unsigned* list = (isx ? lx : ly) + ccd * lstride;
+  int pi[kGramP], pj[kGramP];
+#pragma unroll
+  for (int p = 0; p < kGramP; ++p) {
+    const int id = (blk * kGramP + p) * kGramThreads + tid;
+    const int v = id < np ? ptab[id] : 0;
+    pi[p] = v & 255;
+    pj[p] = v >> 8;
+  }
+  // this lane's offsets j = lane + 32 k: u_y, u_x
+  int oy[4], ox[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int j = lane + 32 * k;
+    oy[k] = j / L - w;
+    ox[k] = j % L - w;
+  }
+  v2<T> acc[kGramP][MP / 2];
+#pragma unroll
+  for (int p = 0; p < kGramP; ++p)
+#pragma unroll
+    for (int m = 0; m < MP / 2; ++m) v2_zero(acc[p][m]);
+  const double xs = 2.0 / (double)(W > 1 ? W - 1 : 1), ys = 2.0 / (double)(H > 1 ? H - 1 : 1);
+  const T* img = Rm + (int64_t)ccd * H * W;
+  if (tid < 2 * kGramPts) patch[tid / kGramPts][tid % kGramPts][L * L] = (T)1;
+  const int nb = (n + kGramPts - 1) / kGramPts;
+  // the points of batch b into buffer s
+  auto stage = [&](int b, int s) {
+    const int m = min(kGramPts, n - b * kGramPts);
+    for (int pt = warp; pt < m; pt += kGramThreads / 32) {
+      const unsigned e = ent[s][pt] >> 1;
+      const int y = (int)(e / (unsigned)W), x = (int)(e % (unsigned)W);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int j = lane + 32 * k;
+        const int yy = y - oy[k], xx = x - ox[k];
+        const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
+        if (j < L * L) cp_async<sizeof(T)>(&patch[s][pt][j], img + (in ? (int64_t)yy * W + xx : 0), in);
+      }
+    }
+    if (warp == kGramThreads / 32 - 1) {
+      const unsigned e = ent[s][lane];
+      const T sg = lane >= m ? (T)0 : ((e & 1u) ? (T)-1 : (T)1);
+      const T xt = (T)((double)((e >> 1) % (unsigned)W) * xs - 1.0), yt = (T)((double)((e >> 1) / (unsigned)W) * ys - 1.0);
+      T px[DE + 1], py[DE + 1];
+      px[0] = sg;
+      py[0] = 1;
+#pragma unroll
+      for (int k = 1; k <= DE; ++k) { px[k] = px[k - 1] * xt; py[k] = py[k - 1] * yt; }
+#pragma unroll
+      for (int q = 0; q <= DE; ++q)
+#pragma unroll
+        for (int k = 0; k <= q; ++k) mono[s][lane][mono_index(q - k, k)] = px[q - k] * py[k];
+#pragma unroll
+      for (int k = NM; k < MP; ++k) mono[s][lane][k] = 0;
+    }
+  };
+  auto entry = [&](int b) { return b < nb && b * kGramPts + lane < n ? list[(int64_t)b * kGramPts + lane] : 0u; };
+  if (warp == 0) {
+    ent[0][lane] = entry(g);
+    ent[1][lane] = entry(g + U);
+  }
+  __syncthreads();
+  if (g < nb) stage(g, 0);
+  int s = 0;
+  for (int b = g; b < nb; b += U, s ^= 1) {
+    cp_async_wait_all();
+    __syncthreads();
+    unsigned e2 = 0;
+    if (warp == 0) e2 = entry(b + 2 * U);
+    if (b + U < nb) stage(b + U, s ^ 1);
+    const int m = min(kGramPts, n - b * kGramPts);
+    for (int pt = 0; pt < m; ++pt) {
+      T mv[MP];
+#pragma unroll
+      for (int k = 0; k < MP; k += 4) {
+        T q[4];
+        ld4(&mono[s][pt][k], q);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) mv[k + i] = q[i];
+      }
+#pragma unroll
+      for (int p = 0; p < kGramP; ++p) {
+        const T r = patch[s][pt][pi[p]] * patch[s][pt][pj[p]];
+#pragma unroll
+        for (int k = 0; k < MP / 2; ++k) v2_fma(acc[p][k], mv[2 * k], mv[2 * k + 1], r);
+      }
+    }
+    if (warp == 0) ent[s][lane] = e2;
+  }
+  T* out = hp + ccd * a.hp_stride + (isx ? a.hx_off : 0) + (int64_t)g * np * MP;
+#pragma unroll
+  for (int p = 0; p < kGramP; ++p) {
+    const int id = (blk * kGramP + p) * kGramThreads + tid;
+    if (id < np)
+#pragma unroll
+      for (int k = 0; k < MP; ++k) out[(int64_t)id * MP + k] = v2_get(acc[p][k / 2], k & 1);
+  }
+}
+
+// the slots' partial sums, FP64 (FP32 in fours first on the mixed path)
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_edge_reduce(const T* __restrict__ hp, GramArgs a, const int* __restrict__ cnt, int64_t cnt_stride, int H, int MP,
+              double* __restrict__ hs) {
+  const int ccd = blockIdx.y, ny = a.npy * MP, nx = a.npx * MP;
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= ny + nx) return;
+  const bool isx = i >= ny;
+  const int U = gram_slots<T>(cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H], isx ? a.gx : a.gy);
+  const int64_t st = isx ? nx : ny;
+  const T* p = hp + ccd * a.hp_stride + (isx ? a.hx_off + i - ny : i);
+  double s = 0.0;
+  int g = 0;
+#pragma unroll 2
+  for (; g + 3 < U; g += 4) {
+    const T v0 = p[g * st], v1 = p[(g + 1) * st], v2_ = p[(g + 2) * st], v3 = p[(g + 3) * st];
+    s += (double)((v0 + v1) + (v2_ + v3));
+  }
+  for (; g < U; ++g) s += (double)p[g * st];
+  hs[(int64_t)ccd * (ny + nx) + i] = s;
+}
+
+// Pair numbering shared by the table (host) and the chains.  y pairs: offsets
+// i, j < L (L - 1) in row-major order, j <= i; then the single offsets i.
+// x pairs: i in the row u_y = w with u_x < w, j <= i with u_x < w; then the
+// single offsets.
+__host__ __device__ inline int ypair_id(int i, int j) { return i * (i + 1) / 2 + j; }
+__host__ __device__ inline int ypair_single(int L, int i) { const int n = L * (L - 1); return n * (n + 1) / 2 + i; }
+__host__ __device__ inline int xpair_id(int L, int ix, int jy, int jx) {   // biased indices 0 .. L-1
+  const int q = (L - 1) * (L - 1);
+  return ix * q + ix * (ix + 1) / 2 + (jy < L - 1 ? jy * (L - 1) + jx : q + jx);
+}
+__host__ __device__ inline int xpair_single(int L, int ix) {
+  const int q = (L - 1) * (L - 1), n = L - 1;
+  return n * q + n * (n + 1) / 2 + ix;
+}
+
+// ------------------------------------------------------------------ chains
+// One CTA per (half-plane difference, CCD), and one for the kernel-background
+// block (block n_hd: single offsets).  The CTA fetches the edge sums of its pairs
+// into shared memory; a thread per power of yt then walks the x
+// chain at u_y = w, and a thread per (u_x, power of xt) the y chains, in FP64.
+// shift(h) acts within one power: new_k = sum_i binom(k, i) h^(k - i) old_i.
+template <int DEG>
+__device__ __forceinline__ void shift_poly(double (&f)[DEG + 1], int deg, double h) {
+  // repeated synthetic division: f(x) coefficients' dual, highest first
+#pragma unroll
+  for (int s = 0; s < DEG; ++s)
+#pragma unroll
+    for (int k = DEG; k > s; --k)
+      if (k <= deg) f[k] += h * f[k - 1];
+}
+
+__global__ void __launch_bounds__(128)
+k_edge_chain(const double* __restrict__ hs, int npy, int npx, int MP, int L, int DKK, int DKB, const int2* __restrict__ dlist,
+             int n_hd, double* __restrict__ gkk, int64_t kk_stride, double* __restrict__ gkb, int64_t kb_stride,
+             double hx, double hy) {
+  extern __shared__ double sm[];
+  const int ccd = blockIdx.y, id = blockIdx.x, w = (L - 1) / 2, tid = threadIdx.x;
+  const bool kb = id == n_hd;
+  const int DEG = kb ? DKB : DKK, NM = n_mono(DEG);
+  const int dy = kb ? 0 : dlist[id].x, dx = kb ? 0 : dlist[id].y;
+  // biased ranges of u (0 .. 2w)
+  const int uy_lo = kb ? 0 : max(0, dy), ux_lo = max(0, dx), ux_hi = min(L - 1, L - 1 + dx);
+  const int nx = ux_hi - ux_lo + 1, ny = L - 1 - uy_lo;   // u_x count; y steps
+  double* G = kb ? gkb + ccd * kb_stride : gkk + ccd * kk_stride + (int64_t)id * L * L * NM;
+  double* sx = sm;                       // [nx - 1][NM]
+  double* sy = sm + (L - 1) * NM;        // [ny][nx][NM]
+  const double* hc = hs + (int64_t)ccd * (npy + npx) * MP;
+  const int tot_x = (nx - 1) * NM, tot = tot_x + ny * nx * NM;
+  for (int e = tid; e < tot; e += blockDim.x) {
+    const bool isx = e < tot_x;
+    const int q = isx ? e : e - tot_x;
+    const int m = q % NM, k = q / NM;
+    int pid;
+    if (isx) {
+      const int ix = ux_lo + k;
+      pid = kb ? xpair_single(L, ix) : xpair_id(L, ix, L - 1 - dy, ix - dx);
+    } else {
+      const int iy = uy_lo + k / nx, ix = ux_lo + k % nx;
+      pid = kb ? ypair_single(L, iy * L + ix) : ypair_id(iy * L + ix, (iy - dy) * L + (ix - dx));
+    }
+    (isx ? sx : sy)[q] = hc[(int64_t)(isx ? npy + pid : pid) * MP + m];
+  }
+  __syncthreads();
+  // x chain at u_y = w from the corner u_x = w (d_x >= 0) or -w (d_x < 0)
+  if (tid <= DEG) {
+    const int b = tid, n = DEG - b;
+    double f[kMaxWeightDeg + 1];
+    const bool up = dx < 0;
+    int ux = up ? 0 : L - 1;
+    if (!up) ux = ux_hi;
+#pragma unroll
+    for (int k = 0; k <= kMaxWeightDeg; ++k) f[k] = k <= n ? G[((int64_t)(L - 1) * L + ux) * NM + mono_index(k, b)] : 0.0;
+    for (int s = 0; s < nx - 1; ++s) {
+      if (up) {
+        const double* h = sx + (ux - ux_lo) * NM;
+#pragma unroll
+        for (int k = 0; k <= kMaxWeightDeg; ++k)
+          if (k <= n) f[k] += h[mono_index(k, b)];
+        shift_poly<kMaxWeightDeg>(f, n, hx);
+        ++ux;
+      } else {
+        shift_poly<kMaxWeightDeg>(f, n, -hx);
+        --ux;
+        const double* h = sx + (ux - ux_lo) * NM;
+#pragma unroll
+        for (int k = 0; k <= kMaxWeightDeg; ++k)
+          if (k <= n) f[k] -= h[mono_index(k, b)];
+      }
+#pragma unroll
+      for (int k = 0; k <= kMaxWeightDeg; ++k)
+        if (k <= n) G[((int64_t)(L - 1) * L + ux) * NM + mono_index(k, b)] = f[k];
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < nx * (DEG + 1); e += blockDim.x) {
+    const int ux = ux_lo + e / (DEG + 1), av = e % (DEG + 1), n = DEG - av;
+    double f[kMaxWeightDeg + 1];
+#pragma unroll
+    for (int k = 0; k <= kMaxWeightDeg; ++k) f[k] = k <= n ? G[((int64_t)(L - 1) * L + ux) * NM + mono_index(av, k)] : 0.0;
+    for (int uy = L - 2; uy >= uy_lo; --uy) {
+      shift_poly<kMaxWeightDeg>(f, n, -hy);
+      const double* h = sy + ((uy - uy_lo) * nx + (ux - ux_lo)) * NM;
+#pragma unroll
+      for (int k = 0; k <= kMaxWeightDeg; ++k)
+        if (k <= n) {
+          f[k] -= h[mono_index(av, k)];
+          G[((int64_t)uy * L + ux) * NM + mono_index(av, k)] = f[k];
+        }
+    }
+  }
+}
+
+// ------------------------------------------------------------------ host: tables
+// Tasks and destinations of the fit and of the right-hand side, the pair
+// table of the edge sums, and the tile and slot counts.
+void build_tap_plan(sfft_plan_s* p) {
+  const int L = p->d.L, w = p->w, DK = p->d.DK, DB = p->d.DB, B = p->d.batch;
+  const int dKK = 2 * DK, dKB = DK + DB;
+  const int nkk = n_mono(dKK), nkb = n_mono(dKB), nbk = n_mono(DK);
+  TapPlan& t = p->tap;
+  t.nt = std::max(L, 3);
+  t.mode = L <= 5 ? TAP_FIT_ALL : TAP_FIT_EDGE;
+  const int wt = (t.nt - 1) / 2;
+  auto half_id = [&](int dy, int dx) {
+    for (int i = 0; i < p->n_hd; ++i)
+      if (p->dlist[i].x == dy && p->dlist[i].y == dx) return i;
+    return -1;
+  };
+  auto q = [](int region, int64_t off) { return (int)((region << 28) | off); };
+  auto add = [&](std::vector<int4>& tasks, std::vector<int>& dst, int type, int u0x, int u0y, int uy) {
+    const int nc = type == TAP_CS || type == TAP_C ? n_mono(2 * DK) : (type == TAP_M ? n_mono(DK + 2) : 0);
+    const int ns = type == TAP_CS || type == TAP_S ? nbk : 0;
+    const int nout = nc + ns;
+    tasks.push_back(int4{type | nout << 8, (u0x + 64) | (u0y + 64) << 8, uy, (int)dst.size()});
+    const int taps = t.mode == TAP_FIT_EDGE && type == TAP_C ? t.nt - 1 : t.nt;
+    for (int k = 0; k < taps; ++k) {
+      const int ux = wt - k;
+      const bool in = ux >= -w && ux <= w;
+      const int j = (uy + w) * L + (ux + w);
+      for (int m = 0; m < nc; ++m) {
+        int v = -1;
+        if (in && type == TAP_M) {
+          if (m < nkb) v = q(1, (int64_t)j * nkb + m);
+        } else if (in) {
+          const int dy = u0y - uy, dx = u0x - ux;
+          // the lower corner's own column repeats the upper corner's d_x = 0 entries elsewhere: not needed
+          const bool want = (dy > 0 || dx >= 0) && (t.mode == TAP_FIT_ALL || u0x == w || dx < 0);
+          const int id = want ? half_id(dy, dx) : -1;
+          if (id >= 0) v = q(0, (((int64_t)id * L + (u0y + w)) * L + (u0x + w)) * nkk + m);
+        }
+        dst.push_back(v);
+      }
+      for (int m = 0; m < ns; ++m) dst.push_back(in ? q(2, (int64_t)j * nbk + m) : -1);
+    }
+  };
+  auto moments = [&](std::vector<int4>& tasks, std::vector<int>& dst, bool fit) {
+    tasks.push_back(int4{TAP_MOM | 36 << 8, 0, 0, (int)dst.size()});
+    const int64_t corner = (int64_t)(L * L - 1) * nkb;   // the single offset (w, w)
+    for (int m = 0; m < 15; ++m) dst.push_back(fit && m < n_mono(2 * DB) ? q(3, m) : -1);
+    for (int m = 0; m < 6; ++m) dst.push_back(m < n_mono(DB) ? q(4, m) : -1);
+    for (int m = 0; m < 15; ++m) dst.push_back(fit && t.mode == TAP_FIT_EDGE && m < nkb ? q(1, corner + m) : -1);
+  };
+  t.tasks.clear();
+  t.dst.clear();
+  std::vector<int4> rhs_tasks;
+  std::vector<int> rhs_dst;
+  for (int uy = -w; uy <= w; ++uy) add(t.tasks, t.dst, TAP_CS, w, w, uy);
+  if (t.mode == TAP_FIT_ALL) {
+    for (int uy = -w; uy <= w; ++uy) add(t.tasks, t.dst, TAP_M, 0, 0, uy);
+    for (int u0y = -w; u0y <= w; ++u0y)
+      for (int u0x = -w; u0x <= w; ++u0x)
+        if (u0x != w || u0y != w)
+          for (int uy = -w; uy <= u0y; ++uy) add(t.tasks, t.dst, TAP_C, u0x, u0y, uy);
+  } else {
+    for (int uy = -w; uy < w; ++uy) add(t.tasks, t.dst, TAP_C, -w, w, uy);
+  }
+  moments(t.tasks, t.dst, true);
+  for (int uy = -w; uy <= w; ++uy) add(rhs_tasks, rhs_dst, TAP_S, 0, 0, uy);
+  moments(rhs_tasks, rhs_dst, false);
+  t.ntask = (int)t.tasks.size();
+  t.nout = (int)t.dst.size();
+  t.ntask_rhs = (int)rhs_tasks.size();
+  t.nout_rhs = (int)rhs_dst.size();
+  t.tasks.insert(t.tasks.end(), rhs_tasks.begin(), rhs_tasks.end());
+  t.dst.insert(t.dst.end(), rhs_dst.begin(), rhs_dst.end());
+  // wide tiles amortise the halo and the fold of yt^b; a small image takes
+  // narrow ones, and then splits a tile's tasks over CTAs, to reach two CTAs
+  // per SM
+  const int want = 2 * 152;
+  auto tiles = [&](int tw) { return ((p->d.W + tw - 1) / tw) * ((p->d.H + kTapRows - 1) / kTapRows); };
+  t.tw = 128;
+  while (t.tw > 32 && (int64_t)tiles(t.tw) * B < want) t.tw /= 2;
+  t.ntile = tiles(t.tw);
+  auto split = [&](int ntask) {
+    const int64_t n = (int64_t)t.ntile * B;
+    return (int)std::max<int64_t>(1, std::min<int64_t>((want + n - 1) / n, (ntask + kTapWarps - 1) / kTapWarps));
+  };
+  t.nsplit = split(t.ntask);
+  t.nsplit_rhs = split(t.ntask_rhs);
+  // edge sums
+  t.pairs.clear();
+  t.npy = t.npx = 0;
+  if (t.mode == TAP_FIT_EDGE) {
+    const int one = L * L, n = L * (L - 1);
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j <= i; ++j) t.pairs.push_back(i | j << 8);
+    for (int i = 0; i < n; ++i) t.pairs.push_back(i | one << 8);
+    t.npy = (int)t.pairs.size();
+    for (int ix = 0; ix < L - 1; ++ix) {
+      const int i = (L - 1) * L + ix;
+      for (int jy = 0; jy < L - 1; ++jy)
+        for (int jx = 0; jx < L - 1; ++jx) t.pairs.push_back(i | (jy * L + jx) << 8);
+      for (int jx = 0; jx <= ix; ++jx) t.pairs.push_back(i | ((L - 1) * L + jx) << 8);
+    }
+    for (int ix = 0; ix < L - 1; ++ix) t.pairs.push_back(((L - 1) * L + ix) | one << 8);
+    t.npx = (int)t.pairs.size() - t.npy;
+    // two CTAs per SM when both lists fill their slots: the x pairs take one
+    // block at L = 11, the y pairs five
+    t.gx = std::max(32, 304 / B);
+    t.gy = std::max(8, 64 / B);
+    const int per = kGramP * kGramThreads;
+    t.nby = (t.npy + per - 1) / per;
+    t.nbx = (t.npx + per - 1) / per;
+  }
+  t.DE = std::max(dKK, dKB);
+  t.MP = (n_mono(t.DE) + 3) / 4 * 4;
+  // M is an erosion by L x L: its zero runs are at least L wide between the borders
+  t.row_cap = L == 1 ? p->d.W : std::min(p->d.W, 2 * (p->d.W / (L + 1) + 2));
+  t.col_cap = L == 1 ? p->d.H : std::min(p->d.H, 2 * (p->d.H / (L + 1) + 2));
+}
+
+// ------------------------------------------------------------------ launchers
+static int64_t edge_cap(const sfft_plan_s* p) {
+  return std::max((int64_t)p->d.H * p->tap.row_cap, (int64_t)p->d.W * p->tap.col_cap);
+}
+
+void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs, size_t* list, size_t* cnt) {
+  const TapPlan& t = p->tap;
+  const size_t B = p->d.batch;
+  *part = p->elem * B * (size_t)t.ntile * std::max(t.nout, t.nout_rhs);
+  const bool edge = t.mode == TAP_FIT_EDGE;
+  *hp = edge ? p->elem * B * ((size_t)t.gy * t.npy + (size_t)t.gx * t.npx) * t.MP : 0;
+  *hs = edge ? sizeof(double) * B * (size_t)(t.npy + t.npx) * t.MP : 0;
+  *list = edge ? 2 * sizeof(unsigned) * B * (size_t)edge_cap(p) : 0;
+  *cnt = edge ? 2 * sizeof(int) * B * (size_t)(p->d.H + 1) : 0;
+}
+
+template <typename T, int NT, int DK, int MODE>
+static cudaError_t tap_sums(const sfft_plan_s* p, const float* S, const void* E, void* ws) {
+  const TapPlan& t = p->tap;
+  const bool rhs = MODE == TAP_RHS;
+  auto kern = k_tap_sums<T, NT, DK, MODE>;
+  const size_t smem = tap_smem<T>((NT - 1) / 2, t.tw);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  dim3 grid(t.ntile, rhs ? t.nsplit_rhs : t.nsplit, p->d.batch);
+  kern<<<grid, kTapWarps * 32, smem, p->stream>>>(
+      ws_at<T>(ws, p->rm), S, (const T*)E, ws_at<uint8_t>(ws, p->mfit), ws_at<double>(ws, p->sky),
+      t.d_tasks + (rhs ? t.ntask : 0), rhs ? t.ntask_rhs : t.ntask, ws_at<T>(ws, p->tappart),
+      rhs ? t.nout_rhs : t.nout, p->d.H, p->d.W, p->w, t.tw);
+  p->nlaunch += 1;
+  return cudaGetLastError();
+}
+
+template <typename T, int NT, int MODE>
+static cudaError_t tap_sums_dk(const sfft_plan_s* p, const float* S, const void* E, void* ws) {
+  switch (p->d.DK) {
+    case 0: return tap_sums<T, NT, 0, MODE>(p, S, E, ws);
+    case 1: return tap_sums<T, NT, 1, MODE>(p, S, E, ws);
+    default: return tap_sums<T, NT, 2, MODE>(p, S, E, ws);
+  }
+}
+
+template <typename T>
+static cudaError_t tap_launch(const sfft_plan_s* p, const float* S, const void* E, bool rhs, void* ws) {
+  const TapPlan& t = p->tap;
+  cudaError_t e = cudaErrorInvalidValue;
+  switch (t.nt) {
+    case 3: e = rhs ? tap_sums_dk<T, 3, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 3, TAP_FIT_ALL>(p, S, E, ws); break;
+    case 5: e = rhs ? tap_sums_dk<T, 5, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 5, TAP_FIT_ALL>(p, S, E, ws); break;
+    case 7: e = rhs ? tap_sums_dk<T, 7, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 7, TAP_FIT_EDGE>(p, S, E, ws); break;
+    case 9: e = rhs ? tap_sums_dk<T, 9, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 9, TAP_FIT_EDGE>(p, S, E, ws); break;
+    case 11: e = rhs ? tap_sums_dk<T, 11, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 11, TAP_FIT_EDGE>(p, S, E, ws); break;
+  }
+  if (e != cudaSuccess) return e;
+  const int LL = p->d.L * p->d.L, nout = rhs ? t.nout_rhs : t.nout;
+  TapDst d;
+  const Region* reg[5] = {&p->gkk, &p->gkb, &p->gbk, &p->mom_bb, &p->mom_b};
+  const int64_t stride[5] = {(int64_t)p->n_hd * LL * n_mono(p->DM_KK), (int64_t)LL * n_mono(p->DM_KB),
+                             (int64_t)LL * n_mono(p->DM_bK), n_mono(p->DM_BB), n_mono(p->d.DB)};
+  for (int i = 0; i < 5; ++i) { d.base[i] = ws_at<double>(ws, *reg[i]); d.stride[i] = stride[i]; }
+  k_tap_reduce<T><<<dim3((nout + 31) / 32, p->d.batch), 512, 0, p->stream>>>(
+      ws_at<T>(ws, p->tappart), t.d_dst + (rhs ? t.nout : 0), d, t.ntile, nout);
+  p->nlaunch += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tap_fit(const sfft_plan_s* p, const float* S, void* ws) {
+  return p->fp64 ? tap_launch<double>(p, S, nullptr, false, ws) : tap_launch<float>(p, S, nullptr, false, ws);
+}
+
+cudaError_t launch_tap_rhs(const sfft_plan_s* p, const void* eimg, void* ws) {
+  return p->fp64 ? tap_launch<double>(p, nullptr, eimg, true, ws) : tap_launch<float>(p, nullptr, eimg, true, ws);
+}
+
+cudaError_t launch_edge_lists(const sfft_plan_s* p, void* ws) {
+  if (p->tap.mode != TAP_FIT_EDGE) return cudaSuccess;
+  const int H = p->d.H, W = p->d.W, B = p->d.batch;
+  const uint8_t* m = ws_at<uint8_t>(ws, p->mfit);
+  int* cnt = ws_at<int>(ws, p->ecnt);
+  unsigned* lx = ws_at<unsigned>(ws, p->elist);
+  const int64_t cap = edge_cap(p), cs = 2 * (int64_t)(H + 1);
+  dim3 g((H + 7) / 8, B);
+  k_edge_rows<false><<<g, 256, 0, p->stream>>>(m, H, W, cnt, cs, nullptr, nullptr, 0);
+  k_edge_scan<<<dim3(B, 2), 1024, 0, p->stream>>>(cnt, cs, H);
+  k_edge_rows<true><<<g, 256, 0, p->stream>>>(m, H, W, cnt, cs, lx, lx + cap, 2 * cap);
+  p->nlaunch += 3;
+  return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t edge_sums_T(const sfft_plan_s* p, void* ws) {
+  const TapPlan& t = p->tap;
+  const int H = p->d.H, W = p->d.W, L = p->d.L, B = p->d.batch;
+  GramArgs a;
+  a.pairs = t.d_pairs;
+  a.npy = t.npy; a.npx = t.npx; a.nby = t.nby;
+  a.gy = t.gy; a.gx = t.gx;
+  a.hx_off = (int64_t)t.gy * t.npy * t.MP;
+  a.hp_stride = a.hx_off + (int64_t)t.gx * t.npx * t.MP;
+  const unsigned* lx = ws_at<unsigned>(ws, p->elist);
+  const int* cnt = ws_at<int>(ws, p->ecnt);
+  const int64_t cap = edge_cap(p), cs = 2 * (int64_t)(H + 1);
+  const T* rm = ws_at<T>(ws, p->rm);
+  T* hp = ws_at<T>(ws, p->hpart);
+  dim3 grid(std::max(t.gx, t.gy), t.nby + t.nbx, B);
+  cudaError_t e = cudaSuccess;
+#define SFFT_GRAM(D)                                                                                                  \
+  case D:                                                                                                             \
+    e = cudaFuncSetAttribute(k_edge_gram<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem<T, D>()); \
+    if (e != cudaSuccess) return e;                                                                                   \
+    k_edge_gram<T, D><<<grid, kGramThreads, gram_smem<T, D>(), p->stream>>>(rm, lx, lx + cap, 2 * cap, cnt, cs, a, hp, \
+                                                                            H, W, L);                                 \
+    break
+  switch (t.DE) {
+    SFFT_GRAM(0); SFFT_GRAM(1); SFFT_GRAM(2); SFFT_GRAM(3); SFFT_GRAM(4);
+    default: return cudaErrorInvalidValue;
+  }
+#undef SFFT_GRAM
+  const int LL = L * L;
+  const size_t smem = sizeof(double) * (size_t)(L - 1) * (L + 1) * n_mono(t.DE);
+  double* hs = ws_at<double>(ws, p->hsum);
+  k_edge_reduce<T><<<dim3(((t.npy + t.npx) * t.MP + 255) / 256, B), 256, 0, p->stream>>>(hp, a, cnt, cs, H, t.MP, hs);
+  k_edge_chain<<<dim3(p->n_hd + 1, B), 128, smem, p->stream>>>(
+      hs, t.npy, t.npx, t.MP, L, p->DM_KK, p->DM_KB, p->d_dlist, p->n_hd, ws_at<double>(ws, p->gkk),
+      (int64_t)p->n_hd * LL * n_mono(p->DM_KK), ws_at<double>(ws, p->gkb), (int64_t)LL * n_mono(p->DM_KB),
+      2.0 / (double)(W > 1 ? W - 1 : 1), 2.0 / (double)(H > 1 ? H - 1 : 1));
+  p->nlaunch += 3;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_edge_sums(const sfft_plan_s* p, void* ws) {
+  if (p->tap.mode != TAP_FIT_EDGE) return cudaSuccess;
+  return p->fp64 ? edge_sums_T<double>(p, ws) : edge_sums_T<float>(p, ws);
+}
+
+}  // namespace sfft

@@ -56,6 +56,22 @@ struct DlJob {
 constexpr int kDlChunk = 16;
 constexpr int kDlMaxU = 6;
 
+// Image-space assembly (kernels_tap.cu): tap-sum tasks (the fit's, then the
+// right-hand side's), the destinations of their outputs, the pair table of the
+// mask-edge sums, and the tile and slot counts.
+struct TapPlan {
+  int mode = 0, nt = 0, tw = 0, ntile = 0;
+  int ntask = 0, nout = 0, nsplit = 1, ntask_rhs = 0, nout_rhs = 0, nsplit_rhs = 1;
+  int npy = 0, npx = 0, nby = 0, nbx = 0, gy = 0, gx = 0;
+  int DE = 0, MP = 0;           // degree and padded monomial count of the edge sums
+  int row_cap = 0, col_cap = 0; // most x edges of a row, y edges of a column
+  std::vector<int4> tasks;
+  std::vector<int> dst, pairs;
+  int4* d_tasks = nullptr;
+  int* d_dst = nullptr;
+  int* d_pairs = nullptr;
+};
+
 }  // namespace sfft
 
 struct sfft_plan_s {
@@ -76,6 +92,8 @@ struct sfft_plan_s {
   bool tc = false;                    // KK contraction on the tensor cores (FP32 path)
   bool umma = false;                  // ... with tcgen05 (else mma.sync)
   bool dl = false;                    // ... with one tensor-memory lane per difference (else per (d, u_y) pair)
+  bool direct = false;                // A and b from image-space sums (kernels_tap.cu), no spectra
+  sfft::TapPlan tap;
   int tc_rows = 0;                    // weight rows per CTA of the tensor-core contraction
   double tuned_ms = 0.0;              // autotuned build_normal time per CCD (0: not tuned)
   int bar_spin_limit = 1 << 24;       // tries of the factorisation's grid-barrier wait (about a second)
@@ -109,7 +127,8 @@ struct sfft_plan_s {
   int4* d_dlpairs = nullptr;
   // workspace regions (per-CCD strides where noted)
   sfft::Region sky, skyacc, good, gh, mfit, rowflag, rm, wspec, uspec, rhat, phat, gkk, gkb, gbk,
-      mom_bb, mom_b, eimg, lfac, scale, dinv, gbar, swave, vec, theta_off, status, cbuf;
+      mom_bb, mom_b, eimg, lfac, scale, dinv, gbar, swave, vec, theta_off, status, cbuf,
+      tappart, hpart, hsum, elist, ecnt;
   size_t ws_bytes = 0;
   // graph cache for sfft_subtract
   std::map<std::vector<uintptr_t>, cudaGraphExec_t> graphs;
@@ -144,6 +163,13 @@ cudaError_t launch_contract_umma(const sfft_plan_s* p, int batch_index, int c0, 
 cudaError_t launch_contract_dlane(const sfft_plan_s* p, int batch_index, int c0, int nc, void* ws);
 cudaError_t launch_lag_dft(const sfft_plan_s* p, int batch_index, int c0, int nc, void* ws);
 cudaError_t launch_contract_slot0(const sfft_plan_s* p, int DM, int job0, int njobs, void* ws);
+// image-space assembly
+void build_tap_plan(sfft_plan_s* p);
+void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs, size_t* list, size_t* cnt);
+cudaError_t launch_tap_fit(const sfft_plan_s* p, const float* S, void* ws);
+cudaError_t launch_tap_rhs(const sfft_plan_s* p, const void* eimg, void* ws);
+cudaError_t launch_edge_lists(const sfft_plan_s* p, void* ws);
+cudaError_t launch_edge_sums(const sfft_plan_s* p, void* ws);
 cudaError_t launch_scatter(const sfft_plan_s* p, double* A, double* b, void* ws, bool rhs_only, double* rhs_out);
 cudaError_t launch_cholesky(const sfft_plan_s* p, const double* A, void* ws);
 cudaError_t launch_chol_solve(const sfft_plan_s* p, const double* rhs, double* x, void* ws);
