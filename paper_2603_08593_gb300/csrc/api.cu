@@ -123,8 +123,8 @@ static void build_layout(sfft_plan_s* p) {
   add_region(p->mfit, cur, npx * B);
   add_region(p->rowflag, cur, sizeof(int) * (size_t)p->rf_stride * B);
   add_region(p->rm, cur, npx * e * B);
-  add_region(p->eimg, cur, npx * e * B);
   const size_t spectra = p->direct ? 0 : 1;
+  add_region(p->eimg, cur, spectra * npx * e * B);
   add_region(p->wspec, cur, spectra * slab * p->n_wa * B);
   add_region(p->uspec, cur, spectra * slab * (p->d.DK + 1) * B);
   add_region(p->rhat, cur, spectra * slab * B);
@@ -741,28 +741,29 @@ static sfft_status_t solve_impl(sfft_plan_t p, const double* A, const double* b,
     }
   }
   for (int r = 0; r < refine; ++r) {
-    void* e = ws_at<char>(ws, p->eimg);
-    {
-      Phase ph(p, SFFT_PROF_APPLY);
-      CK(launch_apply(p, R, S, toff, nullptr, nullptr, e, true, ws));
-    }
     if (p->direct) {
       Phase ph(p, SFFT_PROF_CONTRACT_RK);
-      CK(launch_tap_rhs(p, e, ws));
+      CK(launch_residual_sums(p, S, toff, ws));
+      CK(launch_tap_rhs_reduce(p, ws));
     } else {
-    {
-      Phase ph(p, SFFT_PROF_FFT_WEIGHTS);
-      CK(launch_rfft_weights(p, nullptr, e, 0, p->d.DK + 1, ws_at<char>(ws, p->uspec), p->d.DK + 1, ws));
-    }
-    {
-      Phase ph(p, SFFT_PROF_CONTRACT_RK);
-      CK(cudaMemsetAsync(ws_at<char>(ws, p->gbk), 0, p->gbk.bytes, p->stream));
-      CK(launch_contract(p, p->DM_bK, p->bk_first, p->bk_count, p->rows_per_cta, p->csplit, ws));
-    }
-    {
-      Phase ph(p, SFFT_PROF_PREP);
-      CK(launch_moments(p, nullptr, e, true, ws));
-    }
+      void* e = ws_at<char>(ws, p->eimg);
+      {
+        Phase ph(p, SFFT_PROF_APPLY);
+        CK(launch_residual_image(p, R, S, toff, e, ws));
+      }
+      {
+        Phase ph(p, SFFT_PROF_FFT_WEIGHTS);
+        CK(launch_rfft_weights(p, nullptr, e, 0, p->d.DK + 1, ws_at<char>(ws, p->uspec), p->d.DK + 1, ws));
+      }
+      {
+        Phase ph(p, SFFT_PROF_CONTRACT_RK);
+        CK(cudaMemsetAsync(ws_at<char>(ws, p->gbk), 0, p->gbk.bytes, p->stream));
+        CK(launch_contract(p, p->DM_bK, p->bk_first, p->bk_count, p->rows_per_cta, p->csplit, ws));
+      }
+      {
+        Phase ph(p, SFFT_PROF_PREP);
+        CK(launch_moments(p, nullptr, e, true, ws));
+      }
     }
     {
       Phase ph(p, SFFT_PROF_SCATTER);
@@ -787,7 +788,7 @@ static sfft_status_t apply_impl(sfft_plan_t p, const float* R, const float* S, c
   double* toff = ws_at<double>(ws, p->theta_off);
   Phase ph(p, SFFT_PROF_APPLY);
   CK(launch_theta_to_off(p, theta, sky, toff, ws));
-  CK(launch_apply(p, R, S, toff, sky, D, nullptr, false, ws));
+  CK(launch_apply(p, R, S, toff, sky, D, ws));
   return SFFT_OK;
 }
 

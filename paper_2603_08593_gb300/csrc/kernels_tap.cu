@@ -27,197 +27,9 @@
 
 #include "common.cuh"
 #include "plan.h"
+#include "tap.cuh"
 
 namespace sfft {
-
-// ------------------------------------------------------------------ packed pairs
-template <typename T> struct v2 { T x, y; };
-template <> struct v2<float> { float2 p; };
-
-__device__ __forceinline__ void v2_zero(v2<float>& a) { a.p = make_float2(0.f, 0.f); }
-__device__ __forceinline__ void v2_zero(v2<double>& a) { a.x = 0.0; a.y = 0.0; }
-// acc += (q0, q1) r
-__device__ __forceinline__ void v2_fma(v2<float>& a, float q0, float q1, float r) {
-  a.p = __ffma2_rn(make_float2(q0, q1), make_float2(r, r), a.p);
-}
-__device__ __forceinline__ void v2_fma(v2<double>& a, double q0, double q1, double r) {
-  a.x = fma(q0, r, a.x);
-  a.y = fma(q1, r, a.y);
-}
-__device__ __forceinline__ float v2_get(const v2<float>& a, int i) { return i ? a.p.y : a.p.x; }
-__device__ __forceinline__ double v2_get(const v2<double>& a, int i) { return i ? a.y : a.x; }
-
-__device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
-  const float4 q = *reinterpret_cast<const float4*>(p);
-  v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-}
-__device__ __forceinline__ void ld4(const double* p, double (&v)[4]) {
-  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
-  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-}
-
-template <int BYTES>
-__device__ __forceinline__ void cp_async(void* dst, const void* src, bool valid) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(BYTES), "r"(valid ? BYTES : 0)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// ------------------------------------------------------------------ tap sums
-// A task is one row u'_y of taps against one centre image c: a warp's lanes
-// are the tile's 32 rows, each lane walks its row with the NT taps in a
-// sliding register window and keeps (rows of powers) x (taps) sums in
-// registers, so a shared-memory value read once feeds 2 x NT multiply-adds
-// per row of powers.  What bounds it is the FP32 FMA pipe (44 packed FMAs per
-// pixel, centre and tap row at D_K = 2); lanes as rows need no reduction
-// until the row's end, and the odd pitch keeps their reads free of bank
-// conflicts.
-enum { TAP_CS = 0, TAP_C = 1, TAP_S = 2, TAP_M = 3, TAP_MOM = 4 };
-enum { TAP_FIT_EDGE = 0, TAP_FIT_ALL = 1, TAP_RHS = 2 };
-
-constexpr int kTapRows = 32;
-constexpr int kTapWarps = 4;
-constexpr int kTapU = 8;          // pixels per unrolled step
-constexpr int kTapScr = 16;       // staged rows of the y fold per warp
-constexpr int kTapScrPitch = 36;
-constexpr int kTapMaxOut = 40;
-
-template <typename T>
-struct TapTile {
-  const T* r;              // [32 + 2 wt][pitch]: R, column 0 = x0 - wt, row 0 = y0 - wt
-  const T* s;              // [32][spitch]: M S' or the residual
-  const unsigned* m;       // [32][nw] mask bits
-  const T* xp;             // [tw][4] xt .. xt^4
-  const T* yp;             // [5][kTapScrPitch] yt^b of the tile's rows
-  T* scr;                  // this warp's [kTapScr][kTapScrPitch]
-  const unsigned char (*ot)[2];   // this type's outputs: (row of powers, b)
-  int pitch, spitch, nw, n;       // n: columns to walk (a multiple of kTapU)
-};
-
-// sum over the 32 staged values of row `row` times yt^b
-template <typename T>
-__device__ __forceinline__ T fold_row(const TapTile<T>& t, int row, int b) {
-  const T* v = t.scr + row * kTapScrPitch;
-  const T* y = t.yp + b * kTapScrPitch;
-  T s[4] = {0, 0, 0, 0};
-#pragma unroll
-  for (int i = 0; i < 32; i += 4) {
-    T a[4], c[4];
-    ld4(v + i, a);
-    ld4(y + i, c);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) s[k] += a[k] * c[k];
-  }
-  return (s[0] + s[1]) + (s[2] + s[3]);
-}
-
-// RC rows of powers of the centre c (MB: the mask itself), RS rows of s, against
-// the first K of the NT taps.  Rows go in packed pairs (two cycles of the FMA
-// pipe), an odd last row alone (one cycle).
-template <typename T, int NT, int K, int RC, int RS, bool MB>
-__device__ __forceinline__ void tap_task(const TapTile<T>& t, int u0x, int u0y, int uy, int nout, T* __restrict__ out) {
-  constexpr int NR = RC + RS, NP = NR / 2, ODD = NR & 1, wt = (NT - 1) / 2;
-  const int lane = threadIdx.x & 31;
-  const T* rr = t.r + (lane + wt - uy) * t.pitch;
-  const T* cr = t.r + (lane + wt - u0y) * t.pitch + (wt - u0x);
-  const T* sr = t.s + lane * t.spitch;
-  const unsigned* mr = t.m + lane * t.nw;
-  v2<T> acc[K][NP > 0 ? NP : 1];
-  T last[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    last[k] = 0;
-#pragma unroll
-    for (int p = 0; p < NP; ++p) v2_zero(acc[k][p]);
-  }
-  T win[K - 1 + kTapU];
-#pragma unroll
-  for (int k = 0; k < K - 1; ++k) win[k] = rr[k];
-  for (int xb = 0; xb < t.n; xb += kTapU) {
-#pragma unroll
-    for (int i = 0; i < kTapU; ++i) win[K - 1 + i] = rr[xb + K - 1 + i];
-    const unsigned bits = RC > 0 ? mr[xb >> 5] >> (xb & 31) : 0u;
-#pragma unroll
-    for (int i = 0; i < kTapU; ++i) {
-      T q[NR];
-      T xp[4];
-      if (RC > 1 || RS > 1) ld4(t.xp + 4 * (xb + i), xp);
-      if constexpr (RC > 0) {
-        const bool on = (bits >> i) & 1u;
-        const T c = MB ? (on ? (T)1 : (T)0) : (on ? cr[xb + i] : (T)0);
-        q[0] = c;
-#pragma unroll
-        for (int a = 1; a < RC; ++a) q[a] = c * xp[a - 1];
-      }
-      if constexpr (RS > 0) {
-        const T s = sr[xb + i];
-        q[RC] = s;
-#pragma unroll
-        for (int a = 1; a < RS; ++a) q[RC + a] = s * xp[a - 1];
-      }
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-#pragma unroll
-        for (int p = 0; p < NP; ++p) v2_fma(acc[k][p], q[2 * p], q[2 * p + 1], win[i + k]);
-        if (ODD) last[k] = fma(q[NR - 1], win[i + k], last[k]);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < K - 1; ++k) win[k] = win[k + kTapU];
-  }
-  // yt^b over the tile's rows, KT taps at a time
-  constexpr int KT = kTapScr / NR;
-#pragma unroll
-  for (int k0 = 0; k0 < K; k0 += KT) {
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < KT; ++k)
-#pragma unroll
-      for (int a = 0; a < NR; ++a)
-        if (k0 + k < K) {
-          const int kk = k0 + k < K ? k0 + k : 0;
-          t.scr[(k * NR + a) * kTapScrPitch + lane] = a < 2 * NP ? v2_get(acc[kk][a < 2 * NP ? a / 2 : 0], a & 1) : last[kk];
-        }
-    __syncwarp();
-    const int nk = K - k0 < KT ? K - k0 : KT;
-    for (int o = lane; o < nk * nout; o += 32) {
-      const int k = o / nout, j = o % nout;
-      out[(k0 + k) * nout + j] = fold_row(t, k * NR + t.ot[j][0], t.ot[j][1]);
-    }
-  }
-}
-
-// Moments without taps: M xt^a (a <= 4), s xt^a (a <= 2), c xt^a (a <= 4), c = M R(. - (w, w))
-template <typename T>
-__device__ __forceinline__ void tap_moments(const TapTile<T>& t, int wt, int w, int nout, T* __restrict__ out) {
-  const int lane = threadIdx.x & 31;
-  const T* cr = t.r + (lane + wt - w) * t.pitch + (wt - w);
-  const T* sr = t.s + lane * t.spitch;
-  const unsigned* mr = t.m + lane * t.nw;
-  T acc[13];
-#pragma unroll
-  for (int a = 0; a < 13; ++a) acc[a] = 0;
-  for (int x = 0; x < t.n; ++x) {
-    const bool on = (mr[x >> 5] >> (x & 31)) & 1u;
-    const T m = on ? (T)1 : (T)0, c = on ? cr[x] : (T)0, s = sr[x];
-    const T* xp = t.xp + 4 * x;
-    acc[0] += m;
-    acc[5] += s;
-    acc[8] += c;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      acc[1 + a] += m * xp[a];
-      if (a < 2) acc[6 + a] += s * xp[a];
-      acc[9 + a] += c * xp[a];
-    }
-  }
-  __syncwarp();
-#pragma unroll
-  for (int a = 0; a < 13; ++a) t.scr[a * kTapScrPitch + lane] = acc[a];
-  __syncwarp();
-  for (int o = lane; o < nout; o += 32) out[o] = fold_row(t, t.ot[o][0], t.ot[o][1]);
-}
 
 template <typename T>
 __host__ __device__ constexpr size_t tap_smem(int wt, int tw) {
@@ -232,9 +44,9 @@ __host__ __device__ constexpr size_t tap_smem(int wt, int tw) {
 // part[ccd][tile][nout_tot]; k_tap_reduce adds the tiles in FP64.
 template <typename T, int NT, int DK, int MODE>
 __global__ void __launch_bounds__(kTapWarps * 32, sizeof(T) == 4 ? 3 : 2)
-k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const T* __restrict__ E,
-           const uint8_t* __restrict__ mfit, const double* __restrict__ sky, const int4* __restrict__ tasks, int ntask,
-           T* __restrict__ part, int nout_tot, int H, int W, int w, int tw) {
+k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const uint8_t* __restrict__ mfit,
+           const double* __restrict__ sky, const int4* __restrict__ tasks, int ntask,
+           T* __restrict__ part, int nout_tot, int H, int W, int w, int tw, double xs, double ys) {
   constexpr int wt = (NT - 1) / 2, RC = 2 * DK + 1, RS = DK + 1, RM = DK + 3;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned char ot[5][kTapMaxOut][2];
@@ -252,20 +64,7 @@ k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const T* __res
   const int x0 = (tile % ntx) * tw, y0 = (tile / ntx) * kTapRows;
   const int64_t img = (int64_t)ccd * H * W;
   if (tid == 0) next = 0;
-  // outputs of each type: (row of powers, power of yt), in monomial order
-  if (tid < 5) {
-    int n = 0;
-    auto put = [&](int deg, int row0) {
-      for (int g = 0; g <= deg; ++g)
-        for (int b = 0; b <= g; ++b, ++n) { ot[tid][n][0] = (unsigned char)(row0 + g - b); ot[tid][n][1] = (unsigned char)b; }
-    };
-    if (tid == TAP_CS) { put(2 * DK, 0); put(DK, RC); }
-    if (tid == TAP_C) put(2 * DK, 0);
-    if (tid == TAP_S) put(DK, 0);
-    if (tid == TAP_M) put(DK + 2, 0);
-    if (tid == TAP_MOM) { put(4, 0); put(2, 5); put(4, 8); }
-  }
-  const double xs = 2.0 / (double)(W > 1 ? W - 1 : 1), ys = 2.0 / (double)(H > 1 ? H - 1 : 1);
+  if (tid < 5) tap_outputs(tid, DK, ot[tid]);
   for (int i = tid; i < tw; i += nth) {
     const double x = (x0 + i) * xs - 1.0;
     xp[4 * i] = (T)x; xp[4 * i + 1] = (T)(x * x); xp[4 * i + 2] = (T)(x * x * x); xp[4 * i + 3] = (T)(x * x * x * x);
@@ -288,44 +87,37 @@ k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const T* __res
       cp_async<sizeof(T)>(rt + row * pitch + c, src + (ok ? gx : 0), ok);
     }
   }
-  const T sS = MODE == TAP_RHS ? (T)0 : (T)sky[2 * ccd + 1];
+  const T sS = (T)sky[2 * ccd + 1];
   for (int row = warp; row < kTapRows; row += kTapWarps) {
     const int gy = y0 + row;
     const int64_t o = img + (int64_t)gy * W;
-    if constexpr (MODE == TAP_RHS) {
-      for (int c = lane; c < tw; c += 32) {
-        const bool ok = gy < H && x0 + c < W;
-        cp_async<sizeof(T)>(st + row * spitch + c, E + (ok ? o + x0 + c : 0), ok);
+    // four columns at a time (tw is a multiple of 32)
+    for (int c0 = 0; c0 < tw; c0 += 128) {
+      float v[4];
+      bool on[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int gx = x0 + c0 + 32 * k + lane;
+        const bool ok = c0 + 32 * k < tw && gy < H && gx < W;
+        on[k] = ok && mfit[o + gx] != 0;
+        v[k] = ok ? S[o + gx] : 0.f;
       }
-    } else {
-      // four columns at a time (tw is a multiple of 32)
-      for (int c0 = 0; c0 < tw; c0 += 128) {
-        float v[4];
-        bool on[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int gx = x0 + c0 + 32 * k + lane;
-          const bool ok = c0 + 32 * k < tw && gy < H && gx < W;
-          on[k] = ok && mfit[o + gx] != 0;
-          v[k] = ok ? S[o + gx] : 0.f;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int c = c0 + 32 * k;
-          if (c >= tw) break;
-          st[row * spitch + c + lane] = on[k] ? (T)v[k] - sS : (T)0;
-          const unsigned word = __ballot_sync(0xffffffffu, on[k]);
-          if (lane == 0) mw[row * nw + (c >> 5)] = word;
-        }
+      for (int k = 0; k < 4; ++k) {
+        const int c = c0 + 32 * k;
+        if (c >= tw) break;
+        st[row * spitch + c + lane] = on[k] ? (T)v[k] - sS : (T)0;
+        const unsigned word = __ballot_sync(0xffffffffu, on[k]);
+        if (lane == 0) mw[row * nw + (c >> 5)] = word;
       }
     }
   }
   cp_async_wait_all();
   __syncthreads();
   TapTile<T> t;
-  t.r = rt; t.s = st; t.m = mw; t.xp = xp; t.yp = yp;
+  t.r = rt + lane * pitch; t.s = st + lane * spitch; t.m = mw + lane * nw; t.xp = xp; t.yp = yp;
   t.scr = scr + warp * kTapScr * kTapScrPitch;
-  t.pitch = pitch; t.spitch = spitch; t.nw = nw;
+  t.pitch = pitch;
   t.n = min(tw, (W - x0 + kTapU - 1) / kTapU * kTapU);
   T* po = part + ((int64_t)ccd * gridDim.x + tile) * nout_tot;
   for (;;) {
@@ -338,16 +130,11 @@ k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const T* __res
     const int u0x = (q.y & 255) - 64, u0y = (q.y >> 8) - 64;
     t.ot = ot[type];
     T* out = po + q.w;
-    if constexpr (MODE != TAP_RHS) {
-      constexpr int KC = MODE == TAP_FIT_EDGE ? NT - 1 : NT;   // the corner (-w, w) has no d_x = 0
-      if (type == TAP_CS) tap_task<T, NT, NT, RC, RS, false>(t, u0x, u0y, q.z, nout, out);
-      else if (type == TAP_C) tap_task<T, NT, KC, RC, 0, false>(t, u0x, u0y, q.z, nout, out);
-      else if (MODE == TAP_FIT_ALL && type == TAP_M) tap_task<T, NT, NT, RM, 0, true>(t, 0, 0, q.z, nout, out);
-      else tap_moments<T>(t, wt, w, nout, out);
-    } else {
-      if (type == TAP_S) tap_task<T, NT, NT, 0, RS, false>(t, 0, 0, q.z, nout, out);
-      else tap_moments<T>(t, wt, w, nout, out);
-    }
+    constexpr int KC = MODE == TAP_FIT_EDGE ? NT - 1 : NT;   // the corner (-w, w) has no d_x = 0
+    if (type == TAP_CS) tap_task<T, NT, NT, RC, RS, false, 1>(t, u0x, u0y, q.z, nout, out);
+    else if (type == TAP_C) tap_task<T, NT, KC, RC, 0, false, 1>(t, u0x, u0y, q.z, nout, out);
+    else if (MODE == TAP_FIT_ALL && type == TAP_M) tap_task<T, NT, NT, RM, 0, true, 1>(t, 0, 0, q.z, nout, out);
+    else tap_moments<T, true>(t, wt, w, nout, out);
   }
 }
 
@@ -478,6 +265,7 @@ struct GramArgs {
   int gy, gx;              // most slots per list
   int64_t hp_stride;       // per CCD
   int64_t hx_off;          // x partials after the y ones
+  double xs, ys;           // 2 / (W - 1), 2 / (H - 1)
 };
 
 template <typename T>
@@ -530,7 +318,7 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
   for (int p = 0; p < kGramP; ++p)
 #pragma unroll
     for (int m = 0; m < MP / 2; ++m) v2_zero(acc[p][m]);
-  const double xs = 2.0 / (double)(W > 1 ? W - 1 : 1), ys = 2.0 / (double)(H > 1 ? H - 1 : 1);
+  const double xs = a.xs, ys = a.ys;
   const T* img = Rm + (int64_t)ccd * H * W;
   if (tid < 2 * kGramPts) patch[tid / kGramPts][tid % kGramPts][L * L] = (T)1;
   const int nb = (n + kGramPts - 1) / kGramPts;
@@ -829,7 +617,8 @@ void build_tap_plan(sfft_plan_s* p) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((want + n - 1) / n, (ntask + kTapWarps - 1) / kTapWarps));
   };
   t.nsplit = split(t.ntask);
-  t.nsplit_rhs = split(t.ntask_rhs);
+  // the refinement's half tiles (kernels_apply.cu)
+  t.ntile_rhs = 2 * conv_tiles(p->d.H, p->d.W, conv_half_width(p->d.H, p->d.W, B));
   // edge sums
   t.pairs.clear();
   t.npy = t.npx = 0;
@@ -870,7 +659,7 @@ static int64_t edge_cap(const sfft_plan_s* p) {
 void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs, size_t* list, size_t* cnt) {
   const TapPlan& t = p->tap;
   const size_t B = p->d.batch;
-  *part = p->elem * B * (size_t)t.ntile * std::max(t.nout, t.nout_rhs);
+  *part = p->elem * B * std::max((size_t)t.ntile * t.nout, (size_t)t.ntile_rhs * t.nout_rhs);
   const bool edge = t.mode == TAP_FIT_EDGE;
   *hp = edge ? p->elem * B * ((size_t)t.gy * t.npy + (size_t)t.gx * t.npx) * t.MP : 0;
   *hs = edge ? sizeof(double) * B * (size_t)(t.npy + t.npx) * t.MP : 0;
@@ -878,44 +667,37 @@ void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs
   *cnt = edge ? 2 * sizeof(int) * B * (size_t)(p->d.H + 1) : 0;
 }
 
+// one pixel in xt or yt
+static double step_of(int n) { return 2.0 / (double)(n > 1 ? n - 1 : 1); }
+
 template <typename T, int NT, int DK, int MODE>
-static cudaError_t tap_sums(const sfft_plan_s* p, const float* S, const void* E, void* ws) {
+static cudaError_t tap_sums(const sfft_plan_s* p, const float* S, void* ws) {
   const TapPlan& t = p->tap;
-  const bool rhs = MODE == TAP_RHS;
   auto kern = k_tap_sums<T, NT, DK, MODE>;
   const size_t smem = tap_smem<T>((NT - 1) / 2, t.tw);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid(t.ntile, rhs ? t.nsplit_rhs : t.nsplit, p->d.batch);
-  kern<<<grid, kTapWarps * 32, smem, p->stream>>>(
-      ws_at<T>(ws, p->rm), S, (const T*)E, ws_at<uint8_t>(ws, p->mfit), ws_at<double>(ws, p->sky),
-      t.d_tasks + (rhs ? t.ntask : 0), rhs ? t.ntask_rhs : t.ntask, ws_at<T>(ws, p->tappart),
-      rhs ? t.nout_rhs : t.nout, p->d.H, p->d.W, p->w, t.tw);
+  dim3 grid(t.ntile, t.nsplit, p->d.batch);
+  kern<<<grid, kTapWarps * 32, smem, p->stream>>>(ws_at<T>(ws, p->rm), S, ws_at<uint8_t>(ws, p->mfit),
+                                                  ws_at<double>(ws, p->sky), t.d_tasks, t.ntask,
+                                                  ws_at<T>(ws, p->tappart), t.nout, p->d.H, p->d.W, p->w, t.tw,
+                                                  step_of(p->d.W), step_of(p->d.H));
   p->nlaunch += 1;
   return cudaGetLastError();
 }
 
 template <typename T, int NT, int MODE>
-static cudaError_t tap_sums_dk(const sfft_plan_s* p, const float* S, const void* E, void* ws) {
+static cudaError_t tap_sums_dk(const sfft_plan_s* p, const float* S, void* ws) {
   switch (p->d.DK) {
-    case 0: return tap_sums<T, NT, 0, MODE>(p, S, E, ws);
-    case 1: return tap_sums<T, NT, 1, MODE>(p, S, E, ws);
-    default: return tap_sums<T, NT, 2, MODE>(p, S, E, ws);
+    case 0: return tap_sums<T, NT, 0, MODE>(p, S, ws);
+    case 1: return tap_sums<T, NT, 1, MODE>(p, S, ws);
+    default: return tap_sums<T, NT, 2, MODE>(p, S, ws);
   }
 }
 
 template <typename T>
-static cudaError_t tap_launch(const sfft_plan_s* p, const float* S, const void* E, bool rhs, void* ws) {
+static cudaError_t tap_reduce(const sfft_plan_s* p, bool rhs, void* ws) {
   const TapPlan& t = p->tap;
-  cudaError_t e = cudaErrorInvalidValue;
-  switch (t.nt) {
-    case 3: e = rhs ? tap_sums_dk<T, 3, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 3, TAP_FIT_ALL>(p, S, E, ws); break;
-    case 5: e = rhs ? tap_sums_dk<T, 5, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 5, TAP_FIT_ALL>(p, S, E, ws); break;
-    case 7: e = rhs ? tap_sums_dk<T, 7, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 7, TAP_FIT_EDGE>(p, S, E, ws); break;
-    case 9: e = rhs ? tap_sums_dk<T, 9, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 9, TAP_FIT_EDGE>(p, S, E, ws); break;
-    case 11: e = rhs ? tap_sums_dk<T, 11, TAP_RHS>(p, S, E, ws) : tap_sums_dk<T, 11, TAP_FIT_EDGE>(p, S, E, ws); break;
-  }
-  if (e != cudaSuccess) return e;
   const int LL = p->d.L * p->d.L, nout = rhs ? t.nout_rhs : t.nout;
   TapDst d;
   const Region* reg[5] = {&p->gkk, &p->gkb, &p->gbk, &p->mom_bb, &p->mom_b};
@@ -923,17 +705,30 @@ static cudaError_t tap_launch(const sfft_plan_s* p, const float* S, const void* 
                              (int64_t)LL * n_mono(p->DM_bK), n_mono(p->DM_BB), n_mono(p->d.DB)};
   for (int i = 0; i < 5; ++i) { d.base[i] = ws_at<double>(ws, *reg[i]); d.stride[i] = stride[i]; }
   k_tap_reduce<T><<<dim3((nout + 31) / 32, p->d.batch), 512, 0, p->stream>>>(
-      ws_at<T>(ws, p->tappart), t.d_dst + (rhs ? t.nout : 0), d, t.ntile, nout);
+      ws_at<T>(ws, p->tappart), t.d_dst + (rhs ? t.nout : 0), d, rhs ? t.ntile_rhs : t.ntile, nout);
   p->nlaunch += 1;
   return cudaGetLastError();
 }
 
-cudaError_t launch_tap_fit(const sfft_plan_s* p, const float* S, void* ws) {
-  return p->fp64 ? tap_launch<double>(p, S, nullptr, false, ws) : tap_launch<float>(p, S, nullptr, false, ws);
+template <typename T>
+static cudaError_t tap_fit_T(const sfft_plan_s* p, const float* S, void* ws) {
+  cudaError_t e = cudaErrorInvalidValue;
+  switch (p->tap.nt) {
+    case 3: e = tap_sums_dk<T, 3, TAP_FIT_ALL>(p, S, ws); break;
+    case 5: e = tap_sums_dk<T, 5, TAP_FIT_ALL>(p, S, ws); break;
+    case 7: e = tap_sums_dk<T, 7, TAP_FIT_EDGE>(p, S, ws); break;
+    case 9: e = tap_sums_dk<T, 9, TAP_FIT_EDGE>(p, S, ws); break;
+    case 11: e = tap_sums_dk<T, 11, TAP_FIT_EDGE>(p, S, ws); break;
+  }
+  return e != cudaSuccess ? e : tap_reduce<T>(p, false, ws);
 }
 
-cudaError_t launch_tap_rhs(const sfft_plan_s* p, const void* eimg, void* ws) {
-  return p->fp64 ? tap_launch<double>(p, nullptr, eimg, true, ws) : tap_launch<float>(p, nullptr, eimg, true, ws);
+cudaError_t launch_tap_fit(const sfft_plan_s* p, const float* S, void* ws) {
+  return p->fp64 ? tap_fit_T<double>(p, S, ws) : tap_fit_T<float>(p, S, ws);
+}
+
+cudaError_t launch_tap_rhs_reduce(const sfft_plan_s* p, void* ws) {
+  return p->fp64 ? tap_reduce<double>(p, true, ws) : tap_reduce<float>(p, true, ws);
 }
 
 cudaError_t launch_edge_lists(const sfft_plan_s* p, void* ws) {
@@ -959,6 +754,7 @@ static cudaError_t edge_sums_T(const sfft_plan_s* p, void* ws) {
   a.pairs = t.d_pairs;
   a.npy = t.npy; a.npx = t.npx; a.nby = t.nby;
   a.gy = t.gy; a.gx = t.gx;
+  a.xs = step_of(W); a.ys = step_of(H);
   a.hx_off = (int64_t)t.gy * t.npy * t.MP;
   a.hp_stride = a.hx_off + (int64_t)t.gx * t.npx * t.MP;
   const unsigned* lx = ws_at<unsigned>(ws, p->elist);
@@ -987,7 +783,7 @@ static cudaError_t edge_sums_T(const sfft_plan_s* p, void* ws) {
   k_edge_chain<<<dim3(p->n_hd + 1, B), 128, smem, p->stream>>>(
       hs, t.npy, t.npx, t.MP, L, p->DM_KK, p->DM_KB, p->d_dlist, p->n_hd, ws_at<double>(ws, p->gkk),
       (int64_t)p->n_hd * LL * n_mono(p->DM_KK), ws_at<double>(ws, p->gkb), (int64_t)LL * n_mono(p->DM_KB),
-      2.0 / (double)(W > 1 ? W - 1 : 1), 2.0 / (double)(H > 1 ? H - 1 : 1));
+      a.xs, a.ys);
   p->nlaunch += 3;
   return cudaGetLastError();
 }

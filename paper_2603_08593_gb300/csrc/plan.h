@@ -61,7 +61,7 @@ constexpr int kDlMaxU = 6;
 // mask-edge sums, and the tile and slot counts.
 struct TapPlan {
   int mode = 0, nt = 0, tw = 0, ntile = 0;
-  int ntask = 0, nout = 0, nsplit = 1, ntask_rhs = 0, nout_rhs = 0, nsplit_rhs = 1;
+  int ntask = 0, nout = 0, nsplit = 1, ntask_rhs = 0, nout_rhs = 0, ntile_rhs = 0;
   int npy = 0, npx = 0, nby = 0, nbx = 0, gy = 0, gx = 0;
   int DE = 0, MP = 0;           // degree and padded monomial count of the edge sums
   int row_cap = 0, col_cap = 0; // most x edges of a row, y edges of a column
@@ -167,7 +167,9 @@ cudaError_t launch_contract_slot0(const sfft_plan_s* p, int DM, int job0, int nj
 void build_tap_plan(sfft_plan_s* p);
 void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs, size_t* list, size_t* cnt);
 cudaError_t launch_tap_fit(const sfft_plan_s* p, const float* S, void* ws);
-cudaError_t launch_tap_rhs(const sfft_plan_s* p, const void* eimg, void* ws);
+cudaError_t launch_tap_rhs_reduce(const sfft_plan_s* p, void* ws);
+int conv_half_width(int H, int W, int batch);
+int conv_tiles(int H, int W, int hw);
 cudaError_t launch_edge_lists(const sfft_plan_s* p, void* ws);
 cudaError_t launch_edge_sums(const sfft_plan_s* p, void* ws);
 cudaError_t launch_scatter(const sfft_plan_s* p, double* A, double* b, void* ws, bool rhs_only, double* rhs_out);
@@ -181,7 +183,11 @@ cudaError_t launch_cpr_expand(const sfft_plan_s* p, const double* x, double* the
 cudaError_t launch_theta_to_orig(const sfft_plan_s* p, const double* theta_off, double* theta, void* ws);
 cudaError_t launch_theta_to_off(const sfft_plan_s* p, const double* theta, const double* sky, double* theta_off, void* ws);
 cudaError_t launch_apply(const sfft_plan_s* p, const float* R, const float* S, const double* theta_off,
-                         const double* sky, float* D, void* eimg, bool resid, void* ws);
+                         const double* sky, float* D, void* ws);
+// residual image e (spectral assembly), or its tap sums without the image (image-space assembly)
+cudaError_t launch_residual_image(const sfft_plan_s* p, const float* R, const float* S, const double* theta_off,
+                                  void* eimg, void* ws);
+cudaError_t launch_residual_sums(const sfft_plan_s* p, const float* S, const double* theta_off, void* ws);
 cudaError_t launch_info(const sfft_plan_s* p, int32_t* info, void* ws);
 cudaError_t launch_kernel_at(const sfft_plan_s* p, const double* theta, double x, double y, double* K);
 
