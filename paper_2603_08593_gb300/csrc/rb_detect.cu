@@ -1,12 +1,14 @@
 // Candidate detection on difference images and the plain SNR/shape cuts.
 //
-// Per CCD: four passes of FP64 clipped statistics over the interior (pass 0
-// unclipped, passes 1-3 clipped at 3 RMS about the previous pass's mean), a
-// separable FP32 Gaussian matched filter (rows, then columns with the
-// 1 / (sigma_D ||G||) scale folded in), a 5 x 5 local-maximum test counted per
-// row, an exclusive scan over rows and an ordered compaction that writes the
-// candidates in row-major order, then a stamp gather.  Block partials of the
-// statistics are reduced in a fixed order, so results are deterministic.
+// Per CCD: four passes of clipped statistics over the interior (pass 0
+// unclipped, passes 1-3 clipped at 3 RMS about the previous pass's mean), then
+// one tile kernel for the separable FP32 Gaussian matched filter (rows, then
+// columns with the 1 / (sigma_D ||G||) scale folded in) and the 5 x 5
+// local-maximum test, whose result is one bit per pixel and a count per row;
+// an exclusive scan over rows, an ordered compaction that writes the candidates
+// in row-major order, and a stamp gather.  Masks travel as bits.  Block
+// partials of the statistics are reduced in a fixed order, so results are
+// deterministic.
 #include <math.h>
 #include <stdint.h>
 
@@ -20,7 +22,7 @@
 namespace {
 
 constexpr int kMargin = 15, kHalf = 15, kNms = 2, kMaxR = 15;
-constexpr int kStatBlocks = 128, kStatPasses = 4;
+constexpr int kStatBlocks = 608, kStatPasses = 4;   // four CTAs per SM
 constexpr double kClipNsig = 3.0, kClipVarShare = 0.97334;
 
 struct Taps {
@@ -30,213 +32,293 @@ struct Taps {
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// What one statistics pass hands to the next, and the last one to the filter
+struct PassStats {
+  float shift, lo, hi;   // the next pass sums about shift the pixels in [lo, hi]
+  float scale;           // 1 / (sigma_D ||G||)
+};
+
 struct DetectLayout {
-  size_t snr, tmp, guard, part, rowcnt, rowoff, total;
+  size_t snr, good, bad, guard, cand, part, stats, zero, rowcnt, rowoff, total;
+  size_t zero_bytes;
+  int words;   // mask words per row
   DetectLayout(int H, int W, int B) {
-    const size_t img = (size_t)B * H * W * sizeof(float);
-    snr = 0;
-    tmp = snr + align256(img);
-    guard = tmp + align256(img);
-    part = guard + align256((size_t)B * H * W);
-    rowcnt = part + align256((size_t)B * kStatPasses * (kStatBlocks * 3 + 1) * sizeof(double));
-    rowoff = rowcnt + align256((size_t)B * H * sizeof(int));
+    words = (W + 31) / 32;
+    const size_t bits = align256((size_t)B * H * words * sizeof(unsigned));
+    snr = 0;   // first: callers view the SNR map here
+    good = snr + align256((size_t)B * H * W * sizeof(float));
+    bad = good + bits;
+    guard = bad + bits;
+    cand = guard + bits;
+    part = cand + bits;
+    stats = part + align256((size_t)B * kStatBlocks * 3 * sizeof(double));
+    zero = stats + align256((size_t)B * sizeof(PassStats));   // counters and row counts, cleared together
+    rowcnt = zero + (size_t)B * kStatPasses * sizeof(int);
+    zero_bytes = (size_t)B * (kStatPasses + H) * sizeof(int);
+    rowoff = zero + align256(zero_bytes);
     total = rowoff + align256((size_t)B * H * sizeof(int));
   }
 };
 
-__device__ __forceinline__ bool good_px(const uint8_t* bad, int64_t i) { return bad == nullptr || bad[i] == 0; }
-
-// Per CCD and pass: kStatBlocks block partials (n, sum(x - shift),
-// sum((x - shift)^2)) followed by the shift the pass accumulated about.
-constexpr int kPassStride = kStatBlocks * 3 + 1;
-
-// Mean and variance of one pass from its partials, summed in a fixed order.
-__device__ void pass_moments(const double* pp, double& mean, double& var) {
-  __shared__ double red[3][kStatBlocks / 32];
-  const int t = threadIdx.x;
-  double v[3] = {0.0, 0.0, 0.0};
-  if (t < kStatBlocks)
-    for (int q = 0; q < 3; ++q) v[q] = pp[t * 3 + q];
-  for (int q = 0; q < 3; ++q) v[q] = sfft::warp_sum(v[q]);
-  if (t < kStatBlocks && (t & 31) == 0)
-    for (int q = 0; q < 3; ++q) red[q][t >> 5] = v[q];
-  __syncthreads();
-  double acc[3];
-  for (int q = 0; q < 3; ++q) {
-    double s = 0.0;
-    for (int w = 0; w < kStatBlocks / 32; ++w) s += red[q][w];
-    acc[q] = s;
-  }
-  __syncthreads();
-  const double m1 = acc[1] / acc[0];
-  mean = pp[kStatBlocks * 3] + m1;
-  var = acc[2] / acc[0] - m1 * m1;
+// x + y = s + e exactly (Knuth's two-sum; no contraction)
+__device__ __forceinline__ float two_sum(float x, float y, float& e) {
+  const float s = __fadd_rn(x, y), t = __fsub_rn(s, x);
+  e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, t)), __fsub_rn(y, t));
+  return s;
 }
 
-// One statistics pass.  Pass p > 0 keeps |x - mean_{p-1}| <= 3 sqrt(var_{p-1})
-// and accumulates about mean_{p-1}; pass 0 keeps every pixel, about 0.
+// the clipping rule of a pass
+__device__ __forceinline__ bool kept(float x, double mean, double thr) { return fabs((double)x - mean) <= thr; }
+
+// One statistics pass over the rows blockIdx.x, blockIdx.x + gridDim.x, ...
+// Sums n, sum d, sum d^2 of d = x - shift in pairs of floats (two-sums and an
+// exact product, about 2^-46 relative: FP64 additions run at 1/64 of the FP32
+// rate and took 70 us per pass of 2048 x 4096), FP64 from the thread's end on.
+// The last CTA to finish adds the partials in index order and prepares the next
+// pass: its clipping rule |x - mean| <= 3 sqrt(var), evaluated in FP64, becomes
+// the float interval of the pixels that satisfy it (the rule is monotone on
+// either side of the mean).  Pass 0 keeps every good pixel, about 0, and packs
+// the masks of all rows.
+template <bool FIRST>
 __global__ void __launch_bounds__(256)
-k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict__ bad, double* __restrict__ part,
-            int pass) {
-  const int b = blockIdx.y;
-  const int64_t img = (int64_t)H * W;
-  const float* Db = D + b * img;
-  const uint8_t* bb = bad ? bad + b * img : nullptr;
-  double* pb = part + (int64_t)b * kStatPasses * kPassStride;
-  double shift = 0.0, thr = INFINITY;
-  if (pass > 0) {
-    double mean, var;
-    pass_moments(pb + (pass - 1) * kPassStride, mean, var);
-    shift = mean;
-    thr = kClipNsig * sqrt(var);
-  }
-  const int iw = W - 2 * kMargin, ih = H - 2 * kMargin;
-  const int64_t n_in = (int64_t)iw * ih;
-  double c = 0.0, s1 = 0.0, s2 = 0.0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n_in; k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = (int64_t)(kMargin + k / iw) * W + kMargin + k % iw;
-    const float x = Db[i];
-    if (!isfinite(x) || !good_px(bb, i)) continue;
-    const double d = (double)x - shift;
-    if (!(fabs(d) <= thr)) continue;
-    c += 1.0;
-    s1 += d;
-    s2 += d * d;
+k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict__ bad, unsigned* __restrict__ goodw,
+            unsigned* __restrict__ badw, double* __restrict__ part, PassStats* __restrict__ stats,
+            int* __restrict__ counter, int pass, Taps taps) {
+  const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (W + 31) / 32;
+  const float* Db = D + (int64_t)b * H * W;
+  const uint8_t* bb = bad ? bad + (int64_t)b * H * W : nullptr;
+  unsigned* gw = goodw + (int64_t)b * H * nw;
+  unsigned* bw = badw + (int64_t)b * H * nw;
+  double* pb = part + (int64_t)b * kStatBlocks * 3;
+  float shift = 0.f, lo = 0.f, hi = 0.f;
+  if (!FIRST) { shift = stats[b].shift; lo = stats[b].lo; hi = stats[b].hi; }
+  int n = 0;
+  float s1 = 0.f, e1 = 0.f, s2 = 0.f, e2 = 0.f;
+  double b1 = 0.0, b2 = 0.0;
+  constexpr int U = 4;
+  for (int y = blockIdx.x; y < H; y += gridDim.x) {
+    const bool row_in = y >= kMargin && y < H - kMargin;
+    if (!FIRST && !row_in) continue;
+    for (int w0 = warp * U; w0 < nw; w0 += 8 * U) {
+      float v[U];
+      unsigned m[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        const int x = (w0 + k) * 32 + lane;
+        const bool in = x < W;
+        v[k] = in ? Db[(int64_t)y * W + x] : 0.f;
+        if (FIRST) m[k] = in && bb ? bb[(int64_t)y * W + x] : 0u;
+        else m[k] = w0 + k < nw ? gw[(int64_t)y * nw + w0 + k] : 0u;
+      }
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        const int x = (w0 + k) * 32 + lane;
+        bool ok;
+        if (FIRST) {
+          const bool isbad = m[k] != 0u;
+          ok = x < W && !isbad && isfinite(v[k]);
+          const unsigned g = __ballot_sync(0xffffffffu, ok), q = __ballot_sync(0xffffffffu, isbad);
+          if (lane == 0 && w0 + k < nw) {
+            gw[(int64_t)y * nw + w0 + k] = g;
+            if (bb) bw[(int64_t)y * nw + w0 + k] = q;
+          }
+        } else {
+          ok = ((m[k] >> lane) & 1u) && v[k] >= lo && v[k] <= hi;
+        }
+        if (!(ok && row_in && x >= kMargin && x < W - kMargin)) continue;
+        ++n;
+        float dl = 0.f, t;
+        const float d = FIRST ? v[k] : two_sum(v[k], -shift, dl);
+        const float ad = fabsf(d);
+        if (ad > 1e18f || (ad < 1e-12f && ad > 0.f)) {   // the square or its error leaves the range of a float
+          const double dd = (double)d + (double)dl;
+          b1 += dd;
+          b2 += dd * dd;
+          continue;
+        }
+        s1 = two_sum(s1, d, t);
+        e1 += t + dl;
+        const float p = __fmul_rn(d, d), pe = __fmaf_rn(2.f * d, dl, __fmaf_rn(d, d, -p));
+        s2 = two_sum(s2, p, t);
+        e2 += t + pe;
+      }
+    }
   }
   __shared__ double red[3][8];
-  double v[3] = {c, s1, s2};
-  for (int q = 0; q < 3; ++q) v[q] = sfft::warp_sum(v[q]);
-  if ((threadIdx.x & 31) == 0)
-    for (int q = 0; q < 3; ++q) red[q][threadIdx.x >> 5] = v[q];
+  __shared__ bool last;
+  double v[3] = {(double)__reduce_add_sync(0xffffffffu, n), (double)s1 + (double)e1 + b1, (double)s2 + (double)e2 + b2};
+  for (int q = 1; q < 3; ++q) v[q] = sfft::warp_sum(v[q]);
+  if (lane == 0)
+    for (int q = 0; q < 3; ++q) red[q][warp] = v[q];
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int q = 0; q < 3; ++q) {
       double s = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[q][w];
-      pb[pass * kPassStride + blockIdx.x * 3 + q] = s;
+      for (int w = 0; w < 8; ++w) s += red[q][w];
+      pb[blockIdx.x * 3 + q] = s;
     }
-    if (blockIdx.x == 0) pb[pass * kPassStride + kStatBlocks * 3] = shift;
-  }
-}
-
-__global__ void __launch_bounds__(256)
-k_filter_rows(int H, int W, const float* __restrict__ D, const uint8_t* __restrict__ bad, Taps taps,
-              float* __restrict__ T) {
-  extern __shared__ float row[];
-  __shared__ float g[2 * kMaxR + 1];
-  const int b = blockIdx.y, r = taps.r;
-  if (threadIdx.x <= 2 * r) g[threadIdx.x] = taps.g[threadIdx.x];
-  const int64_t img = (int64_t)H * W;
-  for (int y = blockIdx.x; y < H; y += gridDim.x) {
-    const int64_t base = b * img + (int64_t)y * W;
-    for (int i = threadIdx.x; i < W + 2 * r; i += blockDim.x) {
-      const int x = i - r;
-      float v = 0.f;
-      if (x >= 0 && x < W) {
-        const float d = D[base + x];
-        if (isfinite(d) && (bad == nullptr || bad[base + x] == 0)) v = d;
-      }
-      row[i] = v;
-    }
-    __syncthreads();
-    for (int x = threadIdx.x; x < W; x += blockDim.x) {
-      float s = 0.f;
-      for (int k = 0; k <= 2 * r; ++k) s = fmaf(g[k], row[x + k], s);
-      T[base + x] = s;
-    }
-    __syncthreads();
-  }
-}
-
-constexpr int kColTile = 64;   // output rows per block in the column pass
-
-__global__ void __launch_bounds__(256)
-k_filter_cols(int H, int W, const float* __restrict__ T, Taps taps, const double* __restrict__ part,
-              float* __restrict__ snr) {
-  __shared__ float tile[kColTile + 2 * kMaxR][32];
-  __shared__ float g[2 * kMaxR + 1];
-  const int b = blockIdx.z, r = taps.r;
-  if (threadIdx.x <= 2 * r) g[threadIdx.x] = taps.g[threadIdx.x];
-  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * kColTile;
-  double mean, var;
-  pass_moments(part + ((int64_t)b * kStatPasses + kStatPasses - 1) * kPassStride, mean, var);
-  float norm = 0.f;
-  for (int k = 0; k <= 2 * r; ++k) norm += g[k] * g[k];
-  const double sigma = sqrt(var / kClipVarShare);
-  const float scale = (float)(1.0 / (sigma * (double)norm));
-  const int64_t img = (int64_t)H * W;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int j = ty; j < kColTile + 2 * r; j += 8) {
-    const int y = y0 + j - r, x = x0 + tx;
-    tile[j][tx] = (y >= 0 && y < H && x < W) ? T[b * img + (int64_t)y * W + x] : 0.f;
+    __threadfence();
+    last = atomicAdd(&counter[b * kStatPasses + pass], 1) == (int)gridDim.x - 1;
   }
   __syncthreads();
-  const int x = x0 + tx;
-  if (x >= W) return;
-  for (int j = ty; j < kColTile; j += 8) {
-    const int y = y0 + j;
-    if (y >= H) break;
-    float s = 0.f;
-    for (int k = 0; k <= 2 * r; ++k) s = fmaf(g[k], tile[j + k][tx], s);
-    snr[b * img + (int64_t)y * W + x] = s * scale;
+  if (!last) return;
+  __threadfence();
+  double t[3] = {0.0, 0.0, 0.0};
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x)
+    for (int q = 0; q < 3; ++q) t[q] += __ldcg(pb + i * 3 + q);
+  for (int q = 0; q < 3; ++q) t[q] = sfft::warp_sum(t[q]);
+  if (lane == 0)
+    for (int q = 0; q < 3; ++q) red[q][warp] = t[q];
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int q = 0; q < 3; ++q) {
+    t[q] = 0.0;
+    for (int w = 0; w < 8; ++w) t[q] += red[q][w];
   }
+  const double m1 = t[1] / t[0];
+  const double mean = (double)shift + m1, var = t[2] / t[0] - m1 * m1;
+  PassStats o;
+  o.shift = (float)mean;
+  const double thr = kClipNsig * sqrt(var);
+  // the outermost floats that the rule keeps (none: an empty interval)
+  float a = (float)(mean - thr), c = (float)(mean + thr);
+  for (int k = 0; k < 4 && !kept(a, mean, thr); ++k) a = nextafterf(a, INFINITY);
+  for (int k = 0; k < 4 && kept(nextafterf(a, -INFINITY), mean, thr); ++k) a = nextafterf(a, -INFINITY);
+  for (int k = 0; k < 4 && !kept(c, mean, thr); ++k) c = nextafterf(c, -INFINITY);
+  for (int k = 0; k < 4 && kept(nextafterf(c, INFINITY), mean, thr); ++k) c = nextafterf(c, INFINITY);
+  const bool any = kept(a, mean, thr) && kept(c, mean, thr);
+  o.lo = any ? a : INFINITY;
+  o.hi = any ? c : -INFINITY;
+  float norm = 0.f;
+  for (int k = 0; k <= 2 * taps.r; ++k) norm += taps.g[k] * taps.g[k];
+  const double sigma = sqrt(var / kClipVarShare);
+  o.scale = (float)(1.0 / (sigma * (double)norm));
+  stats[b] = o;
 }
 
-// bad-pixel guard band, separable: rows then columns (Chebyshev distance <= g)
+// bad pixels within Chebyshev distance g, a thread per 32-pixel word
 __global__ void __launch_bounds__(256)
-k_dilate_rows(int H, int W, const uint8_t* __restrict__ bad, int g, uint8_t* __restrict__ out) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)H * W; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t base = (int64_t)blockIdx.y * H * W;
-    const int x = (int)(e % W);
-    const int64_t row = base + e - x;
-    uint8_t v = 0;
-    for (int dx = max(0, x - g); dx <= min(W - 1, x + g); ++dx) v |= bad[row + dx];
-    out[base + e] = v ? 1 : 0;
-  }
-}
-
-__global__ void __launch_bounds__(256)
-k_dilate_cols(int H, int W, const uint8_t* __restrict__ in, int g, uint8_t* __restrict__ out) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)H * W; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t base = (int64_t)blockIdx.y * H * W;
-    const int x = (int)(e % W), y = (int)(e / W);
-    uint8_t v = 0;
-    for (int dy = max(0, y - g); dy <= min(H - 1, y + g); ++dy) v |= in[base + (int64_t)dy * W + x];
+k_guard(int H, int nw, const unsigned* __restrict__ badw, int g, unsigned* __restrict__ out) {
+  const int64_t base = (int64_t)blockIdx.y * H * nw;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)H * nw; e += (int64_t)gridDim.x * blockDim.x) {
+    const int wi = (int)(e % nw), y = (int)(e / nw);
+    unsigned l = 0, c = 0, r = 0;
+    for (int yy = max(0, y - g); yy <= min(H - 1, y + g); ++yy) {
+      const unsigned* p = badw + base + (int64_t)yy * nw + wi;
+      if (wi > 0) l |= p[-1];
+      c |= p[0];
+      if (wi + 1 < nw) r |= p[1];
+    }
+    unsigned v = c;
+    for (int k = 1; k <= g; ++k) v |= __funnelshift_l(l, c, k) | __funnelshift_r(c, r, k);
     out[base + e] = v;
   }
 }
 
-// candidate predicate; (y, x) inside the margin
-__device__ __forceinline__ bool is_candidate(const float* sb, const uint8_t* bb, int W, int y, int x, float thresh) {
-  const int64_t i = (int64_t)y * W + x;
-  if (bb && bb[i]) return false;
-  const float v = sb[i];
-  if (!isfinite(v) || !(v >= thresh)) return false;
-  for (int dy = -kNms; dy <= kNms; ++dy)
-    for (int dx = -kNms; dx <= kNms; ++dx) {
-      const float n = sb[i + (int64_t)dy * W + dx];
-      if (isfinite(n) && n > v) return false;
+// Matched filter and candidate test of one 64 x 32 tile.  The tile of D^ (zero
+// at bad and non-finite pixels and outside the image) carries a halo of R + 2;
+// the row sums, the column sums (taps ascending in both) and the SNR of the
+// 68 x 36 pixels that the 5 x 5 test reads stay in shared memory.  Four outputs
+// per thread slide over a register window, so a staged value is read (2 R + 4) /
+// 4 times per pass instead of 2 R + 1; only the SNR map and one bit per pixel
+// are written.
+constexpr int kMtX = 64, kMtY = 32;
+
+template <int R>
+__global__ void __launch_bounds__(256)
+k_match(int H, int W, const float* __restrict__ D, const unsigned* __restrict__ goodw,
+        const unsigned* __restrict__ guardw, Taps taps, const PassStats* __restrict__ stats, float thresh,
+        float* __restrict__ snr, unsigned* __restrict__ cand, int* __restrict__ rowcnt) {
+  constexpr int OX = kMtX + 2 * kNms, OY = kMtY + 2 * kNms;       // SNR pixels of the tile
+  constexpr int NV = (4 + 2 * R + 3) / 4, PD = OX - 4 + 4 * NV;   // staged columns, read in groups of four
+  constexpr int RY = OY + 2 * R, PS = OX + 1;
+  __shared__ __align__(16) float dt[RY * PD > OY * PS ? RY * PD : OY * PS];
+  __shared__ __align__(16) float tt[RY * OX];
+  const int b = blockIdx.y, nw = (W + 31) / 32, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ntx = (W + kMtX - 1) / kMtX, x0 = (int)(blockIdx.x % ntx) * kMtX, y0 = (int)(blockIdx.x / ntx) * kMtY;
+  const float* Db = D + (int64_t)b * H * W;
+  const unsigned* gw = goodw + (int64_t)b * H * nw;
+  const float scale = stats[b].scale;
+  for (int j = warp; j < RY; j += 8) {
+    const int y = y0 - kNms - R + j;
+    const bool iny = y >= 0 && y < H;
+#pragma unroll
+    for (int i0 = 0; i0 < PD; i0 += 32) {
+      const int i = i0 + lane, x = x0 - kNms - R + i;
+      float v = 0.f;
+      if (iny && x >= 0 && x < W && i < PD) {
+        const float d = Db[(int64_t)y * W + x];
+        v = (gw[(int64_t)y * nw + (x >> 5)] >> (x & 31)) & 1u ? d : 0.f;
+      }
+      if (i < PD) dt[j * PD + i] = v;
     }
-  return true;
+  }
+  __syncthreads();
+  for (int e = tid; e < RY * (OX / 4); e += 256) {
+    const int j = e / (OX / 4), i = 4 * (e % (OX / 4));
+    float w[4 * NV], s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const float4 q = *reinterpret_cast<const float4*>(&dt[j * PD + i + 4 * k]);
+      w[4 * k] = q.x; w[4 * k + 1] = q.y; w[4 * k + 2] = q.z; w[4 * k + 3] = q.w;
+    }
+#pragma unroll
+    for (int k = 0; k <= 2 * R; ++k)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) s[o] = fmaf(taps.g[k], w[k + o], s[o]);
+    *reinterpret_cast<float4*>(&tt[j * OX + i]) = make_float4(s[0], s[1], s[2], s[3]);
+  }
+  __syncthreads();
+  float* sn = dt;
+  for (int e = tid; e < (OY / 4) * OX; e += 256) {
+    const int i = e % OX, j = 4 * (e / OX);
+    float w[4 + 2 * R], s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 4 + 2 * R; ++k) w[k] = tt[(j + k) * OX + i];
+#pragma unroll
+    for (int k = 0; k <= 2 * R; ++k)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) s[o] = fmaf(taps.g[k], w[k + o], s[o]);
+#pragma unroll
+    for (int o = 0; o < 4; ++o) sn[(j + o) * PS + i] = s[o] * scale;
+  }
+  __syncthreads();
+  for (int j = warp; j < kMtY; j += 8) {
+    const int y = y0 + j;
+    if (y >= H) break;
+    int c = 0;
+#pragma unroll
+    for (int h = 0; h < kMtX / 32; ++h) {
+      const int x = x0 + 32 * h + lane, wi = x0 / 32 + h;
+      if (wi >= nw) break;
+      const float* p = sn + (j + kNms) * PS + 32 * h + lane + kNms;
+      const float v = *p;
+      if (x < W) snr[((int64_t)b * H + y) * W + x] = v;
+      bool ok = y >= kMargin && y < H - kMargin && x >= kMargin && x < W - kMargin && isfinite(v) && v >= thresh;
+      if (ok && guardw) ok = !((guardw[((int64_t)b * H + y) * nw + wi] >> lane) & 1u);
+      if (ok)
+        for (int dy = -kNms; dy <= kNms; ++dy)
+          for (int dx = -kNms; dx <= kNms; ++dx) {
+            const float q = p[dy * PS + dx];
+            if (isfinite(q) && q > v) ok = false;
+          }
+      const unsigned word = __ballot_sync(0xffffffffu, ok);
+      if (lane == 0) cand[((int64_t)b * H + y) * nw + wi] = word;
+      c += __popc(word);
+    }
+    if (lane == 0 && c) atomicAdd(&rowcnt[(int64_t)b * H + y], c);
+  }
 }
 
-__global__ void __launch_bounds__(256)
-k_cand_count(int H, int W, const float* __restrict__ snr, const uint8_t* __restrict__ bad, float thresh,
-             int* __restrict__ rowcnt) {
-  const int b = blockIdx.y, y = blockIdx.x;
-  const int64_t img = (int64_t)H * W;
-  int c = 0;
-  if (y >= kMargin && y < H - kMargin)
-    for (int x = kMargin + threadIdx.x; x < W - kMargin; x += blockDim.x)
-      c += is_candidate(snr + b * img, bad ? bad + b * img : nullptr, W, y, x, thresh);
-  c = __reduce_add_sync(0xffffffffu, c);
-  __shared__ int red[8];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int s = 0;
-    for (int w = 0; w < 8; ++w) s += red[w];
-    rowcnt[(int64_t)b * H + y] = s;
+template <int R>
+void run_match(int r, dim3 grid, cudaStream_t s, int H, int W, const float* D, const unsigned* goodw,
+               const unsigned* guardw, const Taps& taps, const PassStats* stats, float thresh, float* snr,
+               unsigned* cand, int* rowcnt) {
+  if constexpr (R <= kMaxR) {
+    if (r == R)
+      k_match<R><<<grid, 256, 0, s>>>(H, W, D, goodw, guardw, taps, stats, thresh, snr, cand, rowcnt);
+    else
+      run_match<R + 1>(r, grid, s, H, W, D, goodw, guardw, taps, stats, thresh, snr, cand, rowcnt);
   }
 }
 
@@ -267,39 +349,36 @@ k_cand_scan(int H, const int* __restrict__ rowcnt, int* __restrict__ rowoff, int
   if (t == 1023) count[b] = part[1023];
 }
 
+// candidates of a row from its bits, in order: a warp per row, a lane per word
 __global__ void __launch_bounds__(256)
-k_cand_write(int H, int W, const float* __restrict__ snr, const uint8_t* __restrict__ bad, float thresh,
+k_cand_write(int H, int W, const float* __restrict__ snr, const unsigned* __restrict__ cand,
              const int* __restrict__ rowcnt, const int* __restrict__ rowoff, int max_cand, int32_t* __restrict__ xy,
              float* __restrict__ osnr) {
-  const int b = blockIdx.y, y = blockIdx.x;
-  if (rowcnt[(int64_t)b * H + y] == 0) return;
-  const int64_t img = (int64_t)H * W;
-  const float* sb = snr + b * img;
-  const uint8_t* bb = bad ? bad + b * img : nullptr;
-  __shared__ int wtot[8];
+  const int b = blockIdx.y, y = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, nw = (W + 31) / 32;
+  if (y >= H || rowcnt[(int64_t)b * H + y] == 0) return;
+  const unsigned* cw = cand + ((int64_t)b * H + y) * nw;
+  const float* sr = snr + ((int64_t)b * H + y) * W;
   int base = rowoff[(int64_t)b * H + y];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int x0 = kMargin; x0 < W - kMargin; x0 += blockDim.x) {
-    const int x = x0 + threadIdx.x;
-    const bool c = x < W - kMargin && is_candidate(sb, bb, W, y, x, thresh);
-    const unsigned m = __ballot_sync(0xffffffffu, c);
-    if (lane == 0) wtot[warp] = __popc(m);
-    __syncthreads();
-    int before = 0, total = 0;
-    for (int w = 0; w < 8; ++w) {
-      before += w < warp ? wtot[w] : 0;
-      total += wtot[w];
+  for (int w0 = 0; w0 < nw; w0 += 32) {
+    unsigned m = w0 + lane < nw ? cw[w0 + lane] : 0u;
+    int off = __popc(m);
+    const int mine = off;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, off, o);
+      if (lane >= o) off += t;
     }
-    if (c) {
-      const int idx = base + before + __popc(m & ((1u << lane) - 1u));
+    const int total = __shfl_sync(0xffffffffu, off, 31);
+    int idx = base + off - mine;
+    for (; m; m &= m - 1u, ++idx) {
+      const int x = (w0 + lane) * 32 + __ffs(m) - 1;
       if (idx < max_cand) {
         xy[((int64_t)b * max_cand + idx) * 2 + 0] = x;
         xy[((int64_t)b * max_cand + idx) * 2 + 1] = y;
-        osnr[(int64_t)b * max_cand + idx] = sb[(int64_t)y * W + x];
+        osnr[(int64_t)b * max_cand + idx] = sr[x];
       }
     }
     base += total;
-    __syncthreads();
   }
 }
 
@@ -465,8 +544,12 @@ extern "C" sfft_status_t rb_detect(int32_t H, int32_t W, int32_t batch, const fl
   const DetectLayout L(H, W, batch);
   char* base = static_cast<char*>(ws);
   float* snr_map = reinterpret_cast<float*>(base + L.snr);
-  float* tmp = reinterpret_cast<float*>(base + L.tmp);
+  unsigned* goodw = reinterpret_cast<unsigned*>(base + L.good);
+  unsigned* badw = reinterpret_cast<unsigned*>(base + L.bad);
+  unsigned* cand = reinterpret_cast<unsigned*>(base + L.cand);
   double* part = reinterpret_cast<double*>(base + L.part);
+  PassStats* stats = reinterpret_cast<PassStats*>(base + L.stats);
+  int* counter = reinterpret_cast<int*>(base + L.zero);
   int* rowcnt = reinterpret_cast<int*>(base + L.rowcnt);
   int* rowoff = reinterpret_cast<int*>(base + L.rowoff);
 
@@ -476,24 +559,24 @@ extern "C" sfft_status_t rb_detect(int32_t H, int32_t W, int32_t batch, const fl
     const double t = k - taps.r;
     taps.g[k] = (float)exp(-t * t / (2.0 * (double)psf_sigma * (double)psf_sigma));
   }
-  for (int p = 0; p < kStatPasses; ++p) k_clip_pass<<<dim3(kStatBlocks, batch), 256, 0, s>>>(H, W, D, bad, part, p);
-  const size_t row_smem = sizeof(float) * (W + 2 * taps.r);
-  k_filter_rows<<<dim3(std::min(H, 1024), batch), 256, row_smem, s>>>(H, W, D, bad, taps, tmp);
-  k_filter_cols<<<dim3((W + 31) / 32, (H + kColTile - 1) / kColTile, batch), 256, 0, s>>>(H, W, tmp, taps, part,
-                                                                                             snr_map);
-  const uint8_t* cbad = bad;   // the mask the candidate test reads
+  cudaError_t z = cudaMemsetAsync(counter, 0, L.zero_bytes, s);
+  if (z != cudaSuccess) return fail(z, "rb_detect");
+  const dim3 gs(std::min(kStatBlocks, H), batch);
+  k_clip_pass<true><<<gs, 256, 0, s>>>(H, W, D, bad, goodw, badw, part, stats, counter, 0, taps);
+  for (int p = 1; p < kStatPasses; ++p)
+    k_clip_pass<false><<<gs, 256, 0, s>>>(H, W, D, bad, goodw, badw, part, stats, counter, p, taps);
+  const unsigned* guardw = bad ? badw : nullptr;   // the mask the candidate test reads
   if (bad && guard > 0) {
-    uint8_t* rows = reinterpret_cast<uint8_t*>(base + L.tmp);    // the row-filtered image is consumed by now
-    uint8_t* gm = reinterpret_cast<uint8_t*>(base + L.guard);
-    const int gx = (int)std::min<int64_t>(((int64_t)H * W + 255) / 256, 2048);
-    k_dilate_rows<<<dim3(gx, batch), 256, 0, s>>>(H, W, bad, guard, rows);
-    k_dilate_cols<<<dim3(gx, batch), 256, 0, s>>>(H, W, rows, guard, gm);
-    cbad = gm;
+    unsigned* gm = reinterpret_cast<unsigned*>(base + L.guard);
+    const int gx = (int)std::min<int64_t>(((int64_t)H * L.words + 255) / 256, 2048);
+    k_guard<<<dim3(gx, batch), 256, 0, s>>>(H, L.words, badw, guard, gm);
+    guardw = gm;
   }
-  k_cand_count<<<dim3(H, batch), 256, 0, s>>>(H, W, snr_map, cbad, thresh, rowcnt);
+  run_match<1>(taps.r, dim3((unsigned)(((W + kMtX - 1) / kMtX) * ((H + kMtY - 1) / kMtY)), batch), s, H, W, D, goodw, guardw, taps,
+               stats, thresh, snr_map, cand, rowcnt);
   k_cand_scan<<<batch, 1024, 0, s>>>(H, rowcnt, rowoff, count);
   if (max_cand > 0) {
-    k_cand_write<<<dim3(H, batch), 256, 0, s>>>(H, W, snr_map, cbad, thresh, rowcnt, rowoff, max_cand, xy, snr);
+    k_cand_write<<<dim3((H + 7) / 8, batch), 256, 0, s>>>(H, W, snr_map, cand, rowcnt, rowoff, max_cand, xy, snr);
     k_stamps<<<dim3(max_cand, batch), 256, 0, s>>>(H, W, S, R, D, count, xy, max_cand, stamps);
   }
   const cudaError_t e = cudaGetLastError();
