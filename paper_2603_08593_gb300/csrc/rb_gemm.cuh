@@ -26,48 +26,115 @@ constexpr int SO_A = BM + 8, SO_B = BN + 8;              // padded rows of outer
 __device__ __forceinline__ uint4 zero4() { return make_uint4(0u, 0u, 0u, 0u); }
 
 // ---------------------------------------------------------------- loaders
+// A thread keeps either one row (Row: the pixel's coordinates, split once; k
+// moves on) or one column (Col: the tap, split once; the row moves on by BK per
+// step, with carries in place of divisions).  With both split for every vector
+// the convolutions spent most of their instructions on divisions (32 -> 32
+// channels, 900,000 pixels: 208 us).
 struct Dense {
   const bf16* p;
   int rows, cols, ld;   // the matrix is [rows][cols] with row stride ld (a multiple of 8)
-  // 8 values along the contiguous dimension: (r, c .. c + 7)
-  __device__ __forceinline__ uint4 row8(int r, int c) const {
-    if (r >= rows || c >= cols) return zero4();
-    return *reinterpret_cast<const uint4*>(p + (int64_t)r * ld + c);
+  struct Row { const bf16* q; };
+  struct Col { const bf16* q; int r; };
+  __device__ __forceinline__ Row row(int r) const { return Row{r < rows ? p + (int64_t)r * ld : nullptr}; }
+  __device__ __forceinline__ uint4 at(const Row& s, int c) const {
+    if (s.q == nullptr || c >= cols) return zero4();
+    return *reinterpret_cast<const uint4*>(s.q + c);
+  }
+  __device__ __forceinline__ Col col(int r, int c) const { return Col{c < cols ? p + (int64_t)r * ld + c : nullptr, r}; }
+  __device__ __forceinline__ uint4 at(const Col& s) const {
+    return s.q != nullptr && s.r < rows ? *reinterpret_cast<const uint4*>(s.q) : zero4();
+  }
+  __device__ __forceinline__ void next(Col& s) const {
+    s.r += BK;
+    if (s.q != nullptr) s.q += (int64_t)BK * ld;
   }
 };
 
-struct ConvRows {   // c % 8 == 0
+// (x, y) of a pixel that moves on by BK in an h x w image (BK / w < h)
+struct PixelPos {
+  int x, y;
+  int pix;
+  __device__ __forceinline__ void set(int p, int h, int w) { pix = p; x = p % w; y = p / w % h; }
+  __device__ __forceinline__ void next(int h, int w) {
+    pix += BK;
+    x += BK % w;
+    y += BK / w;
+    if (x >= w) { x -= w; ++y; }
+    while (y >= h) y -= h;
+  }
+};
+
+struct ConvRows {   // c = 32 or 64
   const bf16* x;
   int n, h, w, c, dir;
-  __device__ __forceinline__ uint4 row8(int pix, int k) const {
-    if (pix >= n * h * w || k >= 9 * c) return zero4();
-    const int tap = k / c, ci = k - tap * c;
-    const int xx = pix % w, t = pix / w, yy = t % h, nn = t / h;
-    const int sy = yy + dir * (tap / 3 - 1), sx = xx + dir * (tap % 3 - 1);
-    if (sy < 0 || sy >= h || sx < 0 || sx >= w) return zero4();
-    return *reinterpret_cast<const uint4*>(x + (((int64_t)nn * h + sy) * w + sx) * c + ci);
+  struct Row { const bf16* q; int x, y; };
+  struct Col { PixelPos p; int dy, dx, off; };
+  __device__ __forceinline__ int lc() const { return c == 64 ? 6 : 5; }
+  __device__ __forceinline__ Row row(int pix) const {
+    Row s;
+    s.q = pix < n * h * w ? x + (int64_t)pix * c : nullptr;
+    s.x = pix % w;
+    s.y = pix / w % h;
+    return s;
   }
+  __device__ __forceinline__ uint4 at(const Row& s, int k) const {
+    const int tap = k >> lc(), ci = k & (c - 1);
+    const int ty = (tap * 11) >> 5;                       // tap / 3 for tap < 9
+    const int dy = dir * (ty - 1), dx = dir * (tap - 3 * ty - 1);
+    const bool in = s.q != nullptr && (unsigned)(s.y + dy) < (unsigned)h && (unsigned)(s.x + dx) < (unsigned)w;
+    return in && k < 9 * c ? *reinterpret_cast<const uint4*>(s.q + (dy * w + dx) * c + ci) : zero4();
+  }
+  __device__ __forceinline__ Col col(int pix, int k) const {
+    Col s;
+    s.p.set(pix, h, w);
+    const int tap = k >> lc(), ci = k & (c - 1), ty = (tap * 11) >> 5;
+    s.dy = k < 9 * c ? dir * (ty - 1) : h;                // past the last tap: outside every image
+    s.dx = dir * (tap - 3 * ty - 1);
+    s.off = (dir * (ty - 1) * w + s.dx) * c + ci;
+    return s;
+  }
+  __device__ __forceinline__ uint4 at(const Col& s) const {
+    const bool in = s.p.pix < n * h * w && (unsigned)(s.p.y + s.dy) < (unsigned)h &&
+                    (unsigned)(s.p.x + s.dx) < (unsigned)w;
+    return in ? *reinterpret_cast<const uint4*>(x + (int64_t)s.p.pix * c + s.off) : zero4();
+  }
+  __device__ __forceinline__ void next(Col& s) const { s.p.next(h, w); }
 };
 
 struct Conv1Rows {   // c = 3, k = (ky * 3 + kx) * 3 + ci < 27, padded to 32
   const bf16* x;       // NHWC stamps, sstride values apart
   int n, h, w, sstride;
-  __device__ __forceinline__ uint4 row8(int pix, int k) const {
+  struct Row { PixelPos p; const bf16* q; };
+  struct Col { Row r; int k, nn; };
+  __device__ __forceinline__ Row row(int pix) const {
+    Row s;
+    s.p.set(pix, h, w);
+    s.q = pix < n * h * w ? x + (int64_t)(pix / (h * w)) * sstride + (s.p.y * w + s.p.x) * 3 : nullptr;
+    return s;
+  }
+  __device__ __forceinline__ uint4 at(const Row& s, int k) const {
     __align__(16) bf16 v[8];
-    const bool okp = pix < n * h * w;
-    const int xx = okp ? pix % w : 0, t = okp ? pix / w : 0, yy = t % h, nn = t / h;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int kk = k + j;
       bf16 e = __float2bfloat16(0.f);
-      if (okp && kk < 27) {
+      if (s.q != nullptr && kk < 27) {
         const int tap = kk / 3, ci = kk - tap * 3;
-        const int sy = yy + tap / 3 - 1, sx = xx + tap % 3 - 1;
-        if (sy >= 0 && sy < h && sx >= 0 && sx < w) e = x[(int64_t)nn * sstride + (sy * w + sx) * 3 + ci];
+        const int dy = tap / 3 - 1, dx = tap % 3 - 1;
+        if ((unsigned)(s.p.y + dy) < (unsigned)h && (unsigned)(s.p.x + dx) < (unsigned)w) e = s.q[(dy * w + dx) * 3 + ci];
       }
       v[j] = e;
     }
     return *reinterpret_cast<const uint4*>(v);
+  }
+  __device__ __forceinline__ Col col(int pix, int k) const { return Col{row(pix), k, pix / (h * w)}; }
+  __device__ __forceinline__ uint4 at(const Col& s) const { return at(s.r, s.k); }
+  __device__ __forceinline__ void next(Col& s) const {
+    const int y = s.r.p.y;
+    s.r.p.next(h, w);
+    if (s.r.p.y < y) ++s.nn;                              // BK / w < h: at most one image on
+    s.r.q = s.r.p.pix < n * h * w ? x + (int64_t)s.nn * sstride + (s.r.p.y * w + s.r.p.x) * 3 : nullptr;
   }
 };
 
@@ -112,24 +179,37 @@ k_igemm(int M, int N, int K, int kchunk, LA la, LB lb, float* __restrict__ C, in
   C += (int64_t)blockIdx.z * cz;
 
   // per-thread load slots: A 128 x 32 = 512 vectors (2 per thread), B 64 x 32 = 256 (1 per thread)
+  typename LA::Row arow[2];
+  typename LA::Col acol[2];
+  typename LB::Row brow;
+  typename LB::Col bcol;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int v = tid + 256 * j;
+    if constexpr (A_KM) arow[j] = la.row(m0 + (v >> 2));                     // v -> (m = v / 4, k = (v % 4) * 8)
+    else acol[j] = la.col(kbeg + (v >> 4), m0 + (v & 15) * 8);     // v -> (k = v / 16, m = (v % 16) * 8)
+  }
+  if constexpr (B_KM) brow = lb.row(n0 + (tid >> 2));                        // tid -> (n = tid / 4, k = (tid % 4) * 8)
+  else bcol = lb.col(kbeg + (tid >> 3), n0 + (tid & 7) * 8);       // tid -> (k = tid / 8, n = (tid % 8) * 8)
+  // the tile at k0; called for k0 = kbeg, kbeg + BK, ... in turn
   auto load_tile = [&](int k0, uint4 (&ra)[2], uint4& rb) {
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int v = tid + 256 * j;
-      if (A_KM) {   // v -> (m = v / 4, k = (v % 4) * 8)
-        const int m = v >> 2, k = k0 + (v & 3) * 8;
-        ra[j] = (k < kend) ? la.row8(m0 + m, k) : zero4();
-      } else {      // v -> (k = v / 16, m = (v % 16) * 8)
-        const int k = k0 + (v >> 4), m = (v & 15) * 8;
-        ra[j] = (k < kend) ? la.row8(k, m0 + m) : zero4();
+      if constexpr (A_KM) {
+        const int k = k0 + (v & 3) * 8;
+        ra[j] = k < kend ? la.at(arow[j], k) : zero4();
+      } else {
+        ra[j] = k0 + (v >> 4) < kend ? la.at(acol[j]) : zero4();
+        la.next(acol[j]);
       }
     }
-    if (B_KM) {     // tid -> (n = tid / 4, k = (tid % 4) * 8)
-      const int n = tid >> 2, k = k0 + (tid & 3) * 8;
-      rb = (k < kend) ? lb.row8(n0 + n, k) : zero4();
-    } else {        // tid -> (k = tid / 8, n = (tid % 8) * 8)
-      const int k = k0 + (tid >> 3), n = (tid & 7) * 8;
-      rb = (k < kend) ? lb.row8(k, n0 + n) : zero4();
+    if constexpr (B_KM) {
+      const int k = k0 + (tid & 3) * 8;
+      rb = k < kend ? lb.at(brow, k) : zero4();
+    } else {
+      rb = k0 + (tid >> 3) < kend ? lb.at(bcol) : zero4();
+      lb.next(bcol);
     }
   };
   auto store_tile = [&](int buf, const uint4 (&ra)[2], const uint4& rb) {

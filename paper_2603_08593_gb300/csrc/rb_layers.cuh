@@ -78,11 +78,14 @@ cudaError_t igemm_wgrad(cudaStream_t s, int M, int N, int K, const LA& la, const
 // B operand of the input gradient: row = ci, k = (tap, co) -> W[(tap * cin + ci)][co .. co + 7]
 struct ConvW {
   const bf16* w;
-  int cin, cout;
-  __device__ __forceinline__ uint4 row8(int ci, int k) const {
-    if (ci >= cin || k >= 9 * cout) return rbg::zero4();
-    const int tap = k / cout, co = k - tap * cout;
-    return *reinterpret_cast<const uint4*>(w + ((int64_t)tap * cin + ci) * cout + co);
+  int cin, cout;        // cout = 32 or 64
+  struct Row { const bf16* q; };
+  struct Col {};        // only read along k
+  __device__ __forceinline__ Row row(int ci) const { return Row{ci < cin ? w + (int64_t)ci * cout : nullptr}; }
+  __device__ __forceinline__ uint4 at(const Row& s, int k) const {
+    if (s.q == nullptr || k >= 9 * cout) return rbg::zero4();
+    const int lc = cout == 64 ? 6 : 5, tap = k >> lc, co = k & (cout - 1);
+    return *reinterpret_cast<const uint4*>(s.q + tap * cin * cout + co);
   }
 };
 
