@@ -95,7 +95,7 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
   int n = 0;
   float s1 = 0.f, e1 = 0.f, s2 = 0.f, e2 = 0.f;
   double b1 = 0.0, b2 = 0.0;
-  constexpr int U = 4;
+  constexpr int U = 8;   // words in flight per warp
   for (int y = blockIdx.x; y < H; y += gridDim.x) {
     const bool row_in = y >= kMargin && y < H - kMargin;
     if (!FIRST && !row_in) continue;
