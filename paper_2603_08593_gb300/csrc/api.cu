@@ -118,12 +118,14 @@ static void build_layout(sfft_plan_s* p) {
   add_region(p->status, cur, sizeof(int) * B);
   add_region(p->sky, cur, sizeof(double) * 2 * B);
   add_region(p->skyacc, cur, sizeof(double) * 4 * B);
-  add_region(p->good, cur, npx * B);
-  add_region(p->gh, cur, npx * B);
-  add_region(p->mfit, cur, npx * B);
-  add_region(p->rowflag, cur, sizeof(int) * (size_t)p->rf_stride * B);
+  const size_t spectra = p->direct ? 0 : 1, bits = p->direct ? sizeof(unsigned) * B * H * ((W + 31) / 32) : 0;
+  add_region(p->good, cur, spectra * npx * B);
+  add_region(p->gh, cur, spectra * npx * B);
+  add_region(p->mfit, cur, spectra * npx * B);
+  add_region(p->goodw, cur, bits);
+  add_region(p->mfitw, cur, bits);
+  add_region(p->rowflag, cur, spectra * sizeof(int) * (size_t)p->rf_stride * B);
   add_region(p->rm, cur, npx * e * B);
-  const size_t spectra = p->direct ? 0 : 1;
   add_region(p->eimg, cur, spectra * npx * e * B);
   add_region(p->wspec, cur, spectra * slab * p->n_wa * B);
   add_region(p->uspec, cur, spectra * slab * (p->d.DK + 1) * B);
@@ -625,8 +627,7 @@ static sfft_status_t build_normal_direct(sfft_plan_t p, const float* R, const fl
     Phase ph(p, SFFT_PROF_PREP);
     CK(cudaMemsetAsync(ws_at<char>(ws, p->status), 0, p->status.bytes, p->stream));
     CK(launch_sky(p, R, S, bad, sky, ws));
-    CK(launch_prep(p, R, S, bad, ws));
-    CK(launch_edge_lists(p, ws));
+    CK(launch_prep_bits(p, R, S, bad, p->tap.npy > 0, ws));
   }
   {
     Phase ph(p, SFFT_PROF_CONTRACT_KK);

@@ -68,7 +68,8 @@ struct ConvArgs {
   const float *R, *S;
   const T* Rm;
   const double *theta, *sky;
-  const uint8_t* mfit;
+  const uint8_t* mfit;      // CV_E: M_fit as bytes
+  const unsigned* mfitw;    // CV_SUMS: M_fit as bits
   float* D;
   T* E;
   const int4* tasks;
@@ -121,20 +122,21 @@ k_conv(const ConvArgs<T> a) {
     if (tid < NB) tht[NT * NT * NK + tid] = (T)th[L * L * NK + tid];
     for (int i = tid; i < 2 * hw; i += kCvWarps * 32) xt1[i] = (T)((x0 + i) * xsc - 1.0);
   }
-  // masks: a warp per row of a half tile
-  if constexpr (MODE != CV_D) {
+  // the mask's words (hw < 32: the low bits of one)
+  if constexpr (MODE == CV_SUMS) {
+    const int wpr = (W + 31) / 32;
+    for (int i = tid; i < 2 * kCvRows * nw; i += kCvWarps * 32) {
+      const int r = i / nw, gy = y0 + r % kCvRows, gx = x0 + r / kCvRows * hw + 32 * (i % nw);
+      mw[i] = gy < H && gx < W ? a.mfitw[((int64_t)ccd * H + gy) * wpr + (gx >> 5)] >> (gx & 31) : 0u;
+    }
+  } else if constexpr (MODE == CV_E) {
     for (int r = warp; r < 2 * kCvRows; r += kCvWarps) {
       const int gy = y0 + r % kCvRows, gx0 = x0 + r / kCvRows * hw;
-      bool on[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int c = 32 * k + lane;
-        on[k] = c < hw && gy < H && gx0 + c < W && a.mfit[img + (int64_t)gy * W + gx0 + c] != 0;
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const unsigned word = __ballot_sync(0xffffffffu, on[k]);
-        if (lane == 0 && k < nw) mw[r * nw + k] = word;
+      for (int k = 0; k < nw; ++k) {
+        const int cc = 32 * k + lane;
+        const bool on = cc < hw && gy < H && gx0 + cc < W && a.mfit[img + (int64_t)gy * W + gx0 + cc] != 0;
+        const unsigned word = __ballot_sync(0xffffffffu, on);
+        if (lane == 0) mw[r * nw + k] = word;
       }
     }
   }
@@ -451,7 +453,7 @@ template <typename T>
 static cudaError_t residual_sums_T(const sfft_plan_s* p, const float* S, const double* theta_off, void* ws) {
   ConvArgs<T> a = conv_args<T>(nullptr, S, theta_off, ws_at<double>(ws, p->sky), p->d.H, p->d.W, p->d.L, p->d.DB);
   a.Rm = ws_at<T>(ws, p->rm);
-  a.mfit = ws_at<uint8_t>(ws, p->mfit);
+  a.mfitw = ws_at<unsigned>(ws, p->mfitw);
   a.tasks = p->tap.d_tasks + p->tap.ntask;
   a.ntask = p->tap.ntask_rhs;
   a.nout_tot = p->tap.nout_rhs;

@@ -44,7 +44,7 @@ __host__ __device__ constexpr size_t tap_smem(int wt, int tw) {
 // part[ccd][tile][nout_tot]; k_tap_reduce adds the tiles in FP64.
 template <typename T, int NT, int DK, int MODE>
 __global__ void __launch_bounds__(kTapWarps * 32, sizeof(T) == 4 ? 3 : 2)
-k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const uint8_t* __restrict__ mfit,
+k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const unsigned* __restrict__ mfitw,
            const double* __restrict__ sky, const int4* __restrict__ tasks, int ntask,
            T* __restrict__ part, int nout_tot, int H, int W, int w, int tw, double xs, double ys) {
   constexpr int wt = (NT - 1) / 2, RC = 2 * DK + 1, RS = DK + 1, RM = DK + 3;
@@ -87,32 +87,32 @@ k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const uint8_t*
       cp_async<sizeof(T)>(rt + row * pitch + c, src + (ok ? gx : 0), ok);
     }
   }
-  const T sS = (T)sky[2 * ccd + 1];
+  // the mask's words and S, then M (S - s_S) in place
+  {
+    const int wpr = (W + 31) / 32;   // words per image row
+    for (int i = tid; i < kTapRows * nw; i += nth) {
+      const int gy = y0 + i / nw, wi = x0 / 32 + i % nw;
+      mw[i] = gy < H && wi < wpr ? mfitw[((int64_t)ccd * H + gy) * wpr + wi] : 0u;
+    }
+  }
   for (int row = warp; row < kTapRows; row += kTapWarps) {
     const int gy = y0 + row;
     const int64_t o = img + (int64_t)gy * W;
-    // four columns at a time (tw is a multiple of 32)
-    for (int c0 = 0; c0 < tw; c0 += 128) {
-      float v[4];
-      bool on[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int gx = x0 + c0 + 32 * k + lane;
-        const bool ok = c0 + 32 * k < tw && gy < H && gx < W;
-        on[k] = ok && mfit[o + gx] != 0;
-        v[k] = ok ? S[o + gx] : 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int c = c0 + 32 * k;
-        if (c >= tw) break;
-        st[row * spitch + c + lane] = on[k] ? (T)v[k] - sS : (T)0;
-        const unsigned word = __ballot_sync(0xffffffffu, on[k]);
-        if (lane == 0) mw[row * nw + (c >> 5)] = word;
-      }
+#pragma unroll 4
+    for (int c = lane; c < tw; c += 32) {
+      const bool ok = gy < H && x0 + c < W;
+      if constexpr (sizeof(T) == 4) cp_async<4>(st + row * spitch + c, S + (ok ? o + x0 + c : 0), ok);
+      else st[row * spitch + c] = (T)(ok ? S[o + x0 + c] : 0.f);
     }
   }
   cp_async_wait_all();
+  __syncthreads();
+  const T sS = (T)sky[2 * ccd + 1];
+  for (int row = warp; row < kTapRows; row += kTapWarps)
+    for (int c = lane; c < tw; c += 32) {
+      T* p = st + row * spitch + c;
+      *p = (mw[row * nw + (c >> 5)] >> lane) & 1u ? *p - sS : (T)0;
+    }
   __syncthreads();
   TapTile<T> t;
   t.r = rt + lane * pitch; t.s = st + lane * spitch; t.m = mw + lane * nw; t.xp = xp; t.yp = yp;
@@ -146,18 +146,23 @@ struct TapDst {
   int64_t stride[5];   // per CCD
 };
 
+// Eight outputs (a 32-byte sector of a tile's partials) x 64 groups of tiles per
+// CTA: the reads wait for memory, so more CTAs and eight reads in flight per
+// thread (32 outputs x 16 groups: 15 us for the 747 outputs of the refinement).
+constexpr int kRedOut = 8, kRedGroups = 64;
+
 template <typename T>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(kRedOut * kRedGroups)
 k_tap_reduce(const T* __restrict__ part, const int* __restrict__ dst, TapDst d, int ntile, int nout) {
-  __shared__ double red[16][33];
-  const int ccd = blockIdx.y, lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-  const int o = blockIdx.x * 32 + lane;
+  __shared__ double red[kRedGroups][kRedOut + 1];
+  const int ccd = blockIdx.y, lane = threadIdx.x % kRedOut, g = threadIdx.x / kRedOut;
+  const int o = blockIdx.x * kRedOut + lane;
   double s = 0.0;
   if (o < nout) {
     const T* p = part + (int64_t)ccd * ntile * nout + o;
     int t = g * 4;
 #pragma unroll 2
-    for (; t + 3 < ntile; t += 64) {
+    for (; t + 3 < ntile; t += 4 * kRedGroups) {
       const T a = p[(int64_t)t * nout], b = p[(int64_t)(t + 1) * nout], c = p[(int64_t)(t + 2) * nout],
               e = p[(int64_t)(t + 3) * nout];
       s += (double)((a + b) + (c + e));
@@ -166,79 +171,18 @@ k_tap_reduce(const T* __restrict__ part, const int* __restrict__ dst, TapDst d, 
   }
   red[g][lane] = s;
   __syncthreads();
-  if (g == 0 && o < nout) {
 #pragma unroll
-    for (int k = 1; k < 16; ++k) s += red[k][lane];
+  for (int k = kRedGroups / 2; k > 0; k >>= 1) {
+    if (g < k) red[g][lane] += red[g + k][lane];
+    __syncthreads();
+  }
+  if (g == 0 && o < nout) {
     const int q = dst[o];
     if (q >= 0) {
       const int r = q >> 28;
-      d.base[r][ccd * d.stride[r] + (q & 0xfffffff)] = s;
+      d.base[r][ccd * d.stride[r] + (q & 0xfffffff)] = red[0][lane];
     }
   }
-}
-
-// ------------------------------------------------------------------ mask edges
-// Per row the numbers of x edges (M(x + 1, y) != M(x, y)) and y edges
-// (M(x, y + 1) != M(x, y)); then the lists, in row order, entry
-// (y W + x) << 1 | (M falls).  A warp per row.
-template <bool WRITE>
-__global__ void __launch_bounds__(256)
-k_edge_rows(const uint8_t* __restrict__ mfit, int H, int W, int* __restrict__ cnt, int64_t cnt_stride,
-            unsigned* __restrict__ lx, unsigned* __restrict__ ly, int64_t lstride) {
-  const int y = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, ccd = blockIdx.y;
-  if (y >= H) return;
-  const uint8_t* m = mfit + ((int64_t)ccd * H + y) * W;
-  const uint8_t* m1 = y + 1 < H ? m + W : m;
-  int* c = cnt + ccd * cnt_stride;
-  int nx = 0, ny = 0;
-  if (WRITE) { nx = c[y]; ny = c[H + 1 + y]; }
-  unsigned* ox = lx + ccd * lstride;
-  unsigned* oy = ly + ccd * lstride;
-  for (int x0 = 0; x0 < W; x0 += 32) {
-    const int x = x0 + lane;
-    int a = 0, b = 0, d = 0;
-    if (x < W) { a = m[x] != 0; b = x + 1 < W ? m[x + 1] != 0 : a; d = m1[x] != 0; }
-    const unsigned ex = __ballot_sync(0xffffffffu, a != b), ey = __ballot_sync(0xffffffffu, a != d);
-    if (WRITE) {
-      const unsigned below = (1u << lane) - 1u;
-      const unsigned v = ((unsigned)y * (unsigned)W + (unsigned)x) << 1 | (unsigned)a;
-      if (a != b) ox[nx + __popc(ex & below)] = v;
-      if (a != d) oy[ny + __popc(ey & below)] = v;
-    }
-    nx += __popc(ex);
-    ny += __popc(ey);
-  }
-  if (!WRITE && lane == 0) { c[y] = nx; c[H + 1 + y] = ny; }
-}
-
-// exclusive scan of the row counts; entry H is the total
-__global__ void __launch_bounds__(1024)
-k_edge_scan(int* __restrict__ cnt, int64_t cnt_stride, int H) {
-  __shared__ int wsum[32];
-  __shared__ int carry;
-  int* c = cnt + blockIdx.x * cnt_stride + blockIdx.y * (H + 1);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < H; base += 1024) {
-    const int i = base + tid;
-    const int v = i < H ? c[i] : 0;
-    int s = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += t;
-    }
-    if (lane == 31) wsum[warp] = s;
-    __syncthreads();
-    int off = carry;
-    for (int k = 0; k < warp; ++k) off += wsum[k];
-    if (i < H) c[i] = off + s - v;
-    __syncthreads();
-    if (tid == 1023) carry = off + s;
-    __syncthreads();
-  }
-  if (tid == 0) c[H] = carry;
 }
 
 // ------------------------------------------------------------------ edge sums
@@ -248,8 +192,8 @@ k_edge_scan(int* __restrict__ cnt, int64_t cnt_stride, int H) {
 // batch are copied (cp.async) while this one is summed, and the list is read
 // two batches ahead; without it the gathers' latency took 60 % of the warps'
 // time.  Slot g of U takes batches g, g + U, ..., at least kGramMin<T> points, and
-// writes hp[ccd][slot][pair][MP]; a short list uses few slots.  Blocks y < nby
-// are y-edge pairs, the others x-edge pairs.
+// writes hp[ccd][slot][pair][MP]; a short list uses few slots.  The x-edge
+// blocks, whose lists are the longer, come first.
 constexpr int kGramP = 5;
 constexpr int kGramPts = 32;
 constexpr int kGramThreads = 256;
@@ -261,7 +205,7 @@ template <typename T> constexpr int kGramMin = sizeof(T) == 4 ? 256 : kGramPts;
 
 struct GramArgs {
   const int* pairs;        // i | j << 8: y pairs, then x pairs
-  int npy, npx, nby;       // pairs and y blocks
+  int npy, npx, nbx;       // pairs and x blocks
   int gy, gx;              // most slots per list
   int64_t hp_stride;       // per CCD
   int64_t hx_off;          // x partials after the y ones
@@ -289,11 +233,11 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
   unsigned(*ent)[kGramPts] =
       reinterpret_cast<unsigned(*)[kGramPts]>(smraw + 2 * sizeof(T) * kGramPts * (MP + kGramPatch));
   const int ccd = blockIdx.z, tid = threadIdx.x, w = (L - 1) / 2, lane = tid & 31, warp = tid >> 5;
-  const bool isx = (int)blockIdx.y >= a.nby;
+  const bool isx = (int)blockIdx.y < a.nbx;
   const int n = cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H];
   const int U = gram_slots<T>(n, isx ? a.gx : a.gy), g = blockIdx.x;
   if (g >= U) return;
-  const int blk = isx ? blockIdx.y - a.nby : blockIdx.y;
+  const int blk = isx ? blockIdx.y : blockIdx.y - a.nbx;
   const int np = isx ? a.npx : a.npy;
   const int* ptab = a.pairs + (isx ? a.npy : 0);
   const unsigned* list = (isx ? lx : ly) + ccd * lstride;
@@ -638,8 +582,8 @@ void build_tap_plan(sfft_plan_s* p) {
     t.npx = (int)t.pairs.size() - t.npy;
     // two CTAs per SM when both lists fill their slots: the x pairs take one
     // block at L = 11, the y pairs five
-    t.gx = std::max(32, 304 / B);
-    t.gy = std::max(8, 64 / B);
+    t.gx = std::max(64, 304 / B);
+    t.gy = std::max(16, 64 / B);
     const int per = kGramP * kGramThreads;
     t.nby = (t.npy + per - 1) / per;
     t.nbx = (t.npx + per - 1) / per;
@@ -652,10 +596,6 @@ void build_tap_plan(sfft_plan_s* p) {
 }
 
 // ------------------------------------------------------------------ launchers
-static int64_t edge_cap(const sfft_plan_s* p) {
-  return std::max((int64_t)p->d.H * p->tap.row_cap, (int64_t)p->d.W * p->tap.col_cap);
-}
-
 void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs, size_t* list, size_t* cnt) {
   const TapPlan& t = p->tap;
   const size_t B = p->d.batch;
@@ -678,7 +618,7 @@ static cudaError_t tap_sums(const sfft_plan_s* p, const float* S, void* ws) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid(t.ntile, t.nsplit, p->d.batch);
-  kern<<<grid, kTapWarps * 32, smem, p->stream>>>(ws_at<T>(ws, p->rm), S, ws_at<uint8_t>(ws, p->mfit),
+  kern<<<grid, kTapWarps * 32, smem, p->stream>>>(ws_at<T>(ws, p->rm), S, ws_at<unsigned>(ws, p->mfitw),
                                                   ws_at<double>(ws, p->sky), t.d_tasks, t.ntask,
                                                   ws_at<T>(ws, p->tappart), t.nout, p->d.H, p->d.W, p->w, t.tw,
                                                   step_of(p->d.W), step_of(p->d.H));
@@ -704,7 +644,7 @@ static cudaError_t tap_reduce(const sfft_plan_s* p, bool rhs, void* ws) {
   const int64_t stride[5] = {(int64_t)p->n_hd * LL * n_mono(p->DM_KK), (int64_t)LL * n_mono(p->DM_KB),
                              (int64_t)LL * n_mono(p->DM_bK), n_mono(p->DM_BB), n_mono(p->d.DB)};
   for (int i = 0; i < 5; ++i) { d.base[i] = ws_at<double>(ws, *reg[i]); d.stride[i] = stride[i]; }
-  k_tap_reduce<T><<<dim3((nout + 31) / 32, p->d.batch), 512, 0, p->stream>>>(
+  k_tap_reduce<T><<<dim3((nout + kRedOut - 1) / kRedOut, p->d.batch), kRedOut * kRedGroups, 0, p->stream>>>(
       ws_at<T>(ws, p->tappart), t.d_dst + (rhs ? t.nout : 0), d, rhs ? t.ntile_rhs : t.ntile, nout);
   p->nlaunch += 1;
   return cudaGetLastError();
@@ -731,28 +671,13 @@ cudaError_t launch_tap_rhs_reduce(const sfft_plan_s* p, void* ws) {
   return p->fp64 ? tap_reduce<double>(p, true, ws) : tap_reduce<float>(p, true, ws);
 }
 
-cudaError_t launch_edge_lists(const sfft_plan_s* p, void* ws) {
-  if (p->tap.mode != TAP_FIT_EDGE) return cudaSuccess;
-  const int H = p->d.H, W = p->d.W, B = p->d.batch;
-  const uint8_t* m = ws_at<uint8_t>(ws, p->mfit);
-  int* cnt = ws_at<int>(ws, p->ecnt);
-  unsigned* lx = ws_at<unsigned>(ws, p->elist);
-  const int64_t cap = edge_cap(p), cs = 2 * (int64_t)(H + 1);
-  dim3 g((H + 7) / 8, B);
-  k_edge_rows<false><<<g, 256, 0, p->stream>>>(m, H, W, cnt, cs, nullptr, nullptr, 0);
-  k_edge_scan<<<dim3(B, 2), 1024, 0, p->stream>>>(cnt, cs, H);
-  k_edge_rows<true><<<g, 256, 0, p->stream>>>(m, H, W, cnt, cs, lx, lx + cap, 2 * cap);
-  p->nlaunch += 3;
-  return cudaGetLastError();
-}
-
 template <typename T>
 static cudaError_t edge_sums_T(const sfft_plan_s* p, void* ws) {
   const TapPlan& t = p->tap;
   const int H = p->d.H, W = p->d.W, L = p->d.L, B = p->d.batch;
   GramArgs a;
   a.pairs = t.d_pairs;
-  a.npy = t.npy; a.npx = t.npx; a.nby = t.nby;
+  a.npy = t.npy; a.npx = t.npx; a.nbx = t.nbx;
   a.gy = t.gy; a.gx = t.gx;
   a.xs = step_of(W); a.ys = step_of(H);
   a.hx_off = (int64_t)t.gy * t.npy * t.MP;

@@ -128,7 +128,7 @@ struct sfft_plan_s {
   // workspace regions (per-CCD strides where noted)
   sfft::Region sky, skyacc, good, gh, mfit, rowflag, rm, wspec, uspec, rhat, phat, gkk, gkb, gbk,
       mom_bb, mom_b, eimg, lfac, scale, dinv, gbar, swave, vec, theta_off, status, cbuf,
-      tappart, hpart, hsum, elist, ecnt;
+      tappart, hpart, hsum, elist, ecnt, goodw, mfitw;
   size_t ws_bytes = 0;
   // graph cache for sfft_subtract
   std::map<std::vector<uintptr_t>, cudaGraphExec_t> graphs;
@@ -170,7 +170,9 @@ cudaError_t launch_tap_fit(const sfft_plan_s* p, const float* S, void* ws);
 cudaError_t launch_tap_rhs_reduce(const sfft_plan_s* p, void* ws);
 int conv_half_width(int H, int W, int batch);
 int conv_tiles(int H, int W, int hw);
-cudaError_t launch_edge_lists(const sfft_plan_s* p, void* ws);
+cudaError_t launch_prep_bits(const sfft_plan_s* p, const float* R, const float* S, const uint8_t* bad, bool edges,
+                             void* ws);
+int64_t edge_cap(const sfft_plan_s* p);   // most entries of an edge list
 cudaError_t launch_edge_sums(const sfft_plan_s* p, void* ws);
 cudaError_t launch_scatter(const sfft_plan_s* p, double* A, double* b, void* ws, bool rhs_only, double* rhs_out);
 cudaError_t launch_cholesky(const sfft_plan_s* p, const double* A, void* ws);
