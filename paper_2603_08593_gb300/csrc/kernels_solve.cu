@@ -227,7 +227,12 @@ k_chol_init(const double* __restrict__ A, T* __restrict__ Lf, const double* __re
 struct GridBar { unsigned count, gen, abort, pad; };
 
 constexpr int kBarSpin = 1 << 24;   // x >= 64 ns per try: about a second (the default wait limit)
-constexpr int PRW = 8;              // rows per piece of the panel and trailing updates
+constexpr int PRW = 8;              // rows per piece of the panel updates
+// rows per piece of the trailing updates: FP64 pieces are small to spread a
+// step's multiply-adds over every SM's FP64 pipe; an FP32 step waits for its
+// loads, so a CTA takes a whole 32 x 32 tile with all of them in flight (one
+// round of 253 tiles at N = 732 against 2.2 rounds of 8 x 32 pieces)
+template <typename T> constexpr int TRW = sizeof(T) == 4 ? NBK : 8;
 constexpr int NTRI = NBK * (NBK + 1) / 2;
 
 __device__ bool grid_sync_bounded(GridBar* bar, int* flag_sh, int spin_limit) {
@@ -244,10 +249,9 @@ __device__ bool grid_sync_bounded(GridBar* bar, int* flag_sh, int spin_limit) {
       __threadfence();
       atomicAdd(&bar->gen, 1u);
     } else {
-      for (int it = 0; *vgen == g; ++it) {
+      // a poll is a round trip to L2, well above 64 ns: no sleep between polls
+      for (int it = 0; *vgen == g; ++it)
         if (*vab != 0u || it >= spin_limit) { ok = false; break; }
-        __nanosleep(64);
-      }
     }
     if (!ok) atomicExch(&bar->abort, 1u);
     __threadfence();
@@ -286,9 +290,40 @@ __device__ __forceinline__ void set_pivot(CholSmem<T>& S, int c, T d0, int* st) 
 // looking on the unscaled Schur complement, a_ij -= a_ic a_jc / d_c for
 // c < j <= i, one barrier per column (the thread that updates the next
 // diagonal element forms its pivot at once), then l_ij = a_ij / sqrt(d_j).
+//
+// FP32: one warp, a row per lane in registers, columns handed around by
+// shuffles; no barriers (the column loop below takes 31).
+__device__ __forceinline__ void factor_block_warp(CholSmem<float>& S, int* st) {
+  const int lane = threadIdx.x;
+  float a[NBK];
+#pragma unroll
+  for (int j = 0; j < NBK; ++j) a[j] = S.blk[lane][j];
+  int flags = 0;
+#pragma unroll
+  for (int c = 0; c < NBK; ++c) {
+    const float d0 = __shfl_sync(0xffffffffu, a[c], c);
+    const bool bad = !(d0 > 0.f) || !isfinite(d0);
+    if (bad) flags |= isfinite(d0) ? 1 : 2;
+    const float d = bad ? 1.f : d0, r = rsq(d);
+    const float l = lane == c ? d * r : a[c] * r;
+    a[c] = l;
+#pragma unroll
+    for (int j = c + 1; j < NBK; ++j) a[j] -= l * __shfl_sync(0xffffffffu, l, j);
+  }
+  if (lane == 0 && flags) atomicOr(st, flags);
+#pragma unroll
+  for (int j = 0; j < NBK; ++j)
+    if (j <= lane) S.blk[lane][j] = a[j];
+}
+
 template <typename T>
 __device__ void factor_block(CholSmem<T>& S, int* st) {
   const int tid = threadIdx.x;
+  if constexpr (sizeof(T) == 4) {
+    if (tid < 32) factor_block_warp(S, st);
+    __syncthreads();
+    return;
+  }
   if (tid == 0) set_pivot(S, 0, S.blk[0][0], st);
   __syncthreads();
   for (int c = 0; c < NBK - 1; ++c) {
@@ -408,30 +443,38 @@ k_chol_coop(T* __restrict__ Lf, T* __restrict__ dinv, int* __restrict__ status, 
     // (C) the next diagonal block of every CCD (one CTA each: update and
     // factor), then 8 x 32 pieces of the other trailing tiles
     const int ntile = TB * (TB + 1) / 2;
-    const int npiece = (ntile - 1) * (NBK / PRW);
+    const int npiece = (ntile - 1) * (NBK / TRW<T>);
     for (int item = blockIdx.x; item < B + B * npiece; item += G) {
       __syncthreads();
       if (item < B) {
         const int ccd = item, nb2 = min(NBK, rem);
         T* l = Lf + ccd * NN;
+        constexpr int NE = (NTRI + 255) / 256;
+        T old[NE];   // in flight with the panel rows
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+          const int e = tid + 256 * q;
+          const int i = e < NTRI ? S.ti[e] : 0, j = e < NTRI ? S.tj[e] : 0;
+          old[q] = e < NTRI && i < nb2 ? __ldcg(l + (int64_t)(r0 + i) * N + r0 + j) : (i == j ? T(1) : T(0));
+        }
         for (int e = tid; e < NBK * NBK; e += blockDim.x) {
           const int i = e / NBK, c = e % NBK;
           S.aux[i][c] = (i < nb2 && c < nb) ? __ldcg(l + (int64_t)(r0 + i) * N + kb + c) : T(0);
         }
         __syncthreads();
-        for (int e = tid; e < NTRI; e += blockDim.x) {
-          const int i = S.ti[e], j = S.tj[e];
-          T v = i == j ? T(1) : T(0);
-          if (i < nb2) {
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+          const int e = tid + 256 * q;
+          if (e < NTRI) {
+            const int i = S.ti[e], j = S.tj[e];
             T s0 = T(0), s1 = T(0);
 #pragma unroll 8
             for (int c = 0; c < NBK; c += 2) {
               s0 += S.aux[i][c] * S.aux[j][c];
               s1 += S.aux[i][c + 1] * S.aux[j][c + 1];
             }
-            v = __ldcg(l + (int64_t)(r0 + i) * N + r0 + j) - (s0 + s1);
+            S.blk[i][j] = old[q] - (s0 + s1);   // rows past nb2 are zero in aux: identity
           }
-          S.blk[i][j] = v;
         }
         __syncthreads();
         factor_block(S, status + ccd);
@@ -439,30 +482,46 @@ k_chol_coop(T* __restrict__ Lf, T* __restrict__ dinv, int* __restrict__ status, 
         continue;
       }
       const int q = item - B, ccd = q / npiece, pc = q % npiece;
-      int t = 1 + pc / (NBK / PRW), bi = 0;
+      int t = 1 + pc / (NBK / TRW<T>), bi = 0;
       while (t > bi) { t -= bi + 1; ++bi; }
       const int bj = t;
-      const int i0 = r0 + bi * NBK + (pc % (NBK / PRW)) * PRW, j0 = r0 + bj * NBK;
+      const int i0 = r0 + bi * NBK + (pc % (NBK / TRW<T>)) * TRW<T>, j0 = r0 + bj * NBK;
       T* l = Lf + ccd * NN;
-      for (int e = tid; e < NBK * NBK; e += blockDim.x) {
-        const int j = e / NBK, c = e % NBK;
-        S.aux[j][c] = (j0 + j < N && c < nb) ? __ldcg(l + (int64_t)(j0 + j) * N + kb + c) : T(0);
+      constexpr int NQ = TRW<T> * NBK / 256;
+      T old[NQ], pi[NQ], pj[4];   // every load of the piece in flight at once
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const int i = tid / NBK + 8 * q, j = tid % NBK;
+        old[q] = i0 + i < N && j0 + j <= i0 + i ? __ldcg(l + (int64_t)(i0 + i) * N + j0 + j) : T(0);
+        pi[q] = i0 + i < N && j < nb ? __ldcg(l + (int64_t)(i0 + i) * N + kb + j) : T(0);
       }
-      for (int e = tid; e < PRW * NBK; e += blockDim.x) {
-        const int i = e / NBK, c = e % NBK;
-        S.blk[i][c] = (i0 + i < N && c < nb) ? __ldcg(l + (int64_t)(i0 + i) * N + kb + c) : T(0);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int j = tid / NBK + 8 * q, c = tid % NBK;
+        pj[q] = j0 + j < N && c < nb ? __ldcg(l + (int64_t)(j0 + j) * N + kb + c) : T(0);
       }
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) S.blk[tid / NBK + 8 * q][tid % NBK] = pi[q];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) S.aux[tid / NBK + 8 * q][tid % NBK] = pj[q];
       __syncthreads();
-      const int i = tid / NBK, j = tid % NBK;
-      const int gi = i0 + i, gj = j0 + j;
-      if (i < PRW && gi < N && gj < N && gj <= gi) {
-        T s0 = T(0), s1 = T(0);
+      const int j = tid % NBK, gj = j0 + j;
+      T s0[NQ], s1[NQ];
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) { s0[q] = T(0); s1[q] = T(0); }
 #pragma unroll 8
-        for (int c = 0; c < NBK; c += 2) {
-          s0 += S.blk[i][c] * S.aux[j][c];
-          s1 += S.blk[i][c + 1] * S.aux[j][c + 1];
+      for (int c = 0; c < NBK; c += 2) {
+        const T a0 = S.aux[j][c], a1 = S.aux[j][c + 1];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          s0[q] += S.blk[tid / NBK + 8 * q][c] * a0;
+          s1[q] += S.blk[tid / NBK + 8 * q][c + 1] * a1;
         }
-        l[(int64_t)gi * N + gj] = __ldcg(l + (int64_t)gi * N + gj) - (s0 + s1);
+      }
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const int gi = i0 + tid / NBK + 8 * q;
+        if (gi < N && gj < N && gj <= gi) l[(int64_t)gi * N + gj] = old[q] - (s0[q] + s1[q]);
       }
     }
     ok = grid_sync_bounded(bar, &S.flag, spin_limit);
@@ -772,7 +831,7 @@ static cudaError_t cholesky_T(const sfft_plan_s* p, const double* A, void* ws) {
   if (e != cudaSuccess) return e;
   // every CTA of the cooperative grid must be resident at once
   const int T0 = (N - NBK + NBK - 1) / NBK;
-  const int want = std::max(B, B + B * std::max(T0 * (T0 + 1) / 2 - 1, 1) * (NBK / PRW));
+  const int want = std::max(B, B + B * std::max(T0 * (T0 + 1) / 2 - 1, 1) * (NBK / TRW<T>));
   // FP32: three CTAs per SM shorten each block step's pieces (solve phase
   // 0.622 ms, against 0.637 with two and 0.69 with one); one per SM stays
   // better for the FP64 pipe

@@ -230,14 +230,17 @@ __device__ __forceinline__ void tap_moments(const TapTile<T>& t, int wt, int w, 
     const bool on = FIT && ((mr[x >> 5] >> (x & 31)) & 1u);
     const T m = on ? (T)1 : (T)0, c = on ? cr[x] : (T)0, s = sr[x];
     const T* xp = t.xp + 4 * x;
-    acc[0] += m;
     acc[5] += s;
-    acc[8] += c;
+    acc[6] += s * xp[0];
+    acc[7] += s * xp[1];
+    if (FIT) {
+      acc[0] += m;
+      acc[8] += c;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      acc[1 + a] += m * xp[a];
-      if (a < 2) acc[6 + a] += s * xp[a];
-      acc[9 + a] += c * xp[a];
+      for (int a = 0; a < 4; ++a) {
+        acc[1 + a] += m * xp[a];
+        acc[9 + a] += c * xp[a];
+      }
     }
   }
   __syncwarp();
