@@ -625,7 +625,6 @@ static sfft_status_t build_normal_direct(sfft_plan_t p, const float* R, const fl
                                          const double* sky, double* A, double* b, void* ws) {
   {
     Phase ph(p, SFFT_PROF_PREP);
-    CK(cudaMemsetAsync(ws_at<char>(ws, p->status), 0, p->status.bytes, p->stream));
     CK(launch_sky(p, R, S, bad, sky, ws));
     CK(launch_prep_bits(p, R, S, bad, p->tap.npy > 0, ws));
   }
@@ -639,7 +638,7 @@ static sfft_status_t build_normal_direct(sfft_plan_t p, const float* R, const fl
   }
   {
     Phase ph(p, SFFT_PROF_SCATTER);
-    CK(launch_scatter(p, A, b, ws, false, nullptr));
+    CK(launch_scatter(p, A, b, ws));
   }
   return SFFT_OK;
 }
@@ -650,7 +649,6 @@ static sfft_status_t build_normal_impl(sfft_plan_t p, const float* R, const floa
   cudaStream_t st = p->stream;
   {
     Phase ph(p, SFFT_PROF_PREP);
-    CK(cudaMemsetAsync(ws_at<char>(ws, p->status), 0, p->status.bytes, st));
     CK(launch_sky(p, R, S, bad, sky, ws));
     CK(launch_prep(p, R, S, bad, ws));
     CK(launch_moments(p, S, nullptr, false, ws));
@@ -701,7 +699,7 @@ static sfft_status_t build_normal_impl(sfft_plan_t p, const float* R, const floa
   }
   {
     Phase ph(p, SFFT_PROF_SCATTER);
-    CK(launch_scatter(p, A, b, ws, false, nullptr));
+    CK(launch_scatter(p, A, b, ws));
   }
   return SFFT_OK;
 }
@@ -711,33 +709,42 @@ static sfft_status_t solve_impl(sfft_plan_t p, const double* A, const double* b,
   double* vec = ws_at<double>(ws, p->vec);
   const size_t NBt = (size_t)p->N * p->d.batch;
   double* rhs = vec;
-  double* x = vec + NBt;
   double* toff = ws_at<double>(ws, p->theta_off);
   // constant-ratio fit: right-hand sides projected to, and solutions expanded
   // from, the constrained basis (vec's third and fourth quarters)
   double* rhs_c = vec + 2 * NBt;
   double* x_c = vec + 3 * NBt;
-  auto solve_rhs = [&](const double* r, bool add) -> sfft_status_t {
-    if (p->cpr) {
+  const bool small = small_system(p);
+  // the constant-ratio solution stays in FP64: rounded coefficients would not
+  // keep the kernel sum constant
+  const bool rounds = !p->fp64 && !p->cpr;
+  auto solve_rhs = [&](const RhsSrc& r, int add) -> sfft_status_t {
+    if (small) {
+      CK(launch_small(p, A, r, false, add, ws));
+    } else if (p->cpr) {
       CK(launch_cpr_rhs(p, r, rhs_c));
-      CK(launch_chol_solve(p, rhs_c, x_c, ws));
-      CK(launch_cpr_expand(p, x_c, toff, add));
+      CK(launch_chol_solve(p, RhsSrc{rhs_c, rhs_c, p->Nsol, p->Nsol, p->Nsol}, x_c, 0, ws));
+      CK(launch_cpr_expand(p, x_c, toff, add & 1));
     } else {
-      CK(launch_chol_solve(p, r, x, ws));
-      CK(launch_theta_finish(p, x, toff, add));
+      CK(launch_chol_solve(p, r, toff, add, ws));
     }
     return SFFT_OK;
   };
   {
     Phase ph(p, SFFT_PROF_SOLVE);
-    CK(launch_cholesky(p, A, ws));
-    const sfft_status_t s0 = solve_rhs(b, false);
-    if (s0 != SFFT_OK) return s0;
+    const int first = rounds && refine > 0 ? 2 : 0;   // bit 1: FP32 values
+    if (small) {
+      CK(launch_small(p, A, rhs_of_vector(p, b), true, first, ws));
+    } else {
+      CK(launch_cholesky(p, A, ws));
+      const sfft_status_t s0 = solve_rhs(rhs_of_vector(p, b), first);
+      if (s0 != SFFT_OK) return s0;
+    }
     if (!p->fp64 && refine == 0) {
       // the FP32 factor's solution, refined once against the FP64 system
       // (the image-space steps below refine it otherwise)
       CK(launch_residual(p, A, b, toff, rhs));
-      const sfft_status_t s1 = solve_rhs(rhs, true);
+      const sfft_status_t s1 = solve_rhs(rhs_of_vector(p, rhs), 1);
       if (s1 != SFFT_OK) return s1;
     }
   }
@@ -767,19 +774,14 @@ static sfft_status_t solve_impl(sfft_plan_t p, const double* A, const double* b,
       }
     }
     {
-      Phase ph(p, SFFT_PROF_SCATTER);
-      CK(launch_scatter(p, nullptr, nullptr, ws, true, rhs));
-    }
-    {
       Phase ph(p, SFFT_PROF_SOLVE);
-      const sfft_status_t s1 = solve_rhs(rhs, true);
+      const sfft_status_t s1 = solve_rhs(rhs_of_sums(p, ws), 1 | (rounds && r + 1 < refine ? 2 : 0));
       if (s1 != SFFT_OK) return s1;
     }
   }
   {
     Phase ph(p, SFFT_PROF_SOLVE);
-    CK(launch_theta_to_orig(p, toff, theta, ws));
-    if (info) CK(launch_info(p, info, ws));
+    CK(launch_theta_to_orig(p, toff, theta, info, ws));
   }
   return SFFT_OK;
 }
@@ -832,7 +834,10 @@ static sfft_status_t subtract_enqueue(sfft_plan_t p, const float* R, const float
   if (s != SFFT_OK) return s;
   s = solve_impl(p, A, b, theta, refine, R, S, info, ws);
   if (s != SFFT_OK) return s;
-  return apply_impl(p, R, S, theta, nullptr, D, ws);
+  // the workspace still holds theta in offset units
+  Phase ph(p, SFFT_PROF_APPLY);
+  CK(launch_apply(p, R, S, ws_at<double>(ws, p->theta_off), nullptr, D, ws));
+  return SFFT_OK;
 }
 
 extern "C" sfft_status_t sfft_subtract(sfft_plan_t p, const float* R, const float* S, const uint8_t* bad,

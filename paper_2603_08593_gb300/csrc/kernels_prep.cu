@@ -24,7 +24,7 @@ namespace sfft {
 // sums.
 __global__ void __launch_bounds__(256)
 k_sky_sum(const float* __restrict__ R, const float* __restrict__ S, const uint8_t* __restrict__ bad, int64_t npx,
-          double* __restrict__ acc) {
+          double* __restrict__ acc, double* __restrict__ sky) {
   __shared__ double red[2][8];
   __shared__ int redn[8];
   const int ccd = blockIdx.y;
@@ -74,15 +74,18 @@ k_sky_sum(const float* __restrict__ R, const float* __restrict__ S, const uint8_
     double t = 0.0;
     for (int k = 0; k < 8; ++k) t += threadIdx.x < 2 ? red[threadIdx.x][k] : (double)redn[k];
     atomicAdd(&acc[4 * ccd + threadIdx.x], t);
+    __threadfence();
   }
-}
-
-__global__ void k_sky_final(const double* __restrict__ acc, double* __restrict__ sky, int batch) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= batch) return;
-  const double n = acc[4 * c + 2];
-  sky[2 * c + 0] = n > 0 ? rint(acc[4 * c + 0] / n) : 0.0;
-  sky[2 * c + 1] = n > 0 ? rint(acc[4 * c + 1] / n) : 0.0;
+  __syncthreads();
+  // the CCD's last CTA (the count is the fourth, cleared word of its sums)
+  if (threadIdx.x == 0) {
+    unsigned* done = reinterpret_cast<unsigned*>(&acc[4 * ccd + 3]);
+    if (atomicAdd(done, 1u) == gridDim.x - 1) {
+      __threadfence();
+      const double m = __ldcg(&acc[4 * ccd + 2]);
+      for (int k = 0; k < 2; ++k) sky[2 * ccd + k] = m > 0 ? rint(__ldcg(&acc[4 * ccd + k]) / m) : 0.0;
+    }
+  }
 }
 
 template <typename T>
@@ -446,11 +449,14 @@ cudaError_t launch_sky(const sfft_plan_s* p, const float* R, const float* S, con
                        const double* sky_in, void* ws) {
   double* sky = ws_at<double>(ws, p->sky);
   const int B = p->d.batch;
+  // the status words, the sky constants and their sums follow each other
+  const size_t clear = sky_in ? p->status.bytes : p->skyacc.off + p->skyacc.bytes - p->status.off;
+  cudaError_t e = cudaMemsetAsync(ws_at<char>(ws, p->status), 0, clear, p->stream);
+  if (e != cudaSuccess) return e;
   if (sky_in) {
     return cudaMemcpyAsync(sky, sky_in, sizeof(double) * 2 * B, cudaMemcpyDeviceToDevice, p->stream);
   }
   double* acc = ws_at<double>(ws, p->skyacc);
-  cudaMemsetAsync(acc, 0, sizeof(double) * 4 * B, p->stream);
   const int64_t npx = (int64_t)p->d.H * p->d.W;
   // at least four CTAs per SM, and at most 64 groups of four pixels per thread
   int dev = 0, sms = 0;
@@ -459,9 +465,8 @@ cudaError_t launch_sky(const sfft_plan_s* p, const float* R, const float* S, con
   const int64_t per_cta = 256 * 64 * 4;
   const int gx = (int)std::min<int64_t>(std::max<int64_t>(4 * (int64_t)std::max(sms, 1), (npx + per_cta - 1) / per_cta),
                                         1 << 20);
-  k_sky_sum<<<dim3(gx, B), 256, 0, p->stream>>>(R, S, bad, npx, acc);
-  k_sky_final<<<(B + 127) / 128, 128, 0, p->stream>>>(acc, sky, B);
-  p->nlaunch += 2;
+  k_sky_sum<<<dim3(gx, B), 256, 0, p->stream>>>(R, S, bad, npx, acc, sky);
+  p->nlaunch += 1;
   return cudaGetLastError();
 }
 

@@ -37,7 +37,7 @@ struct ScatterArgs {
 __global__ void __launch_bounds__(256)
 k_scatter(ScatterArgs a, const double* __restrict__ gkk, const double* __restrict__ gkb,
           const double* __restrict__ gbk, const double* __restrict__ mbb, const double* __restrict__ mb,
-          const int* __restrict__ hdidx, double* __restrict__ A, double* __restrict__ b, int rhs_only) {
+          const int* __restrict__ hdidx, double* __restrict__ A, double* __restrict__ b) {
   const int ccd = blockIdx.y;
   const int64_t NN = (int64_t)a.N * a.N;
   const int L = a.L, w = a.w, NK = a.NK;
@@ -46,10 +46,10 @@ k_scatter(ScatterArgs a, const double* __restrict__ gkk, const double* __restric
   const double* Gbk = gbk + ccd * a.s_gbk;
   const double* Mbb = mbb + ccd * a.s_mbb;
   const double* Mb = mb + ccd * a.s_mb;
-  const int64_t total = rhs_only ? a.N : NN + a.N;
+  const int64_t total = NN + a.N;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    if (rhs_only || t >= NN) {
-      const int r = (int)(rhs_only ? t : t - NN);
+    if (t >= NN) {
+      const int r = (int)(t - NN);
       double v;
       if (r < a.NKK) {
         const int j = r / NK, p = r % NK;
@@ -135,17 +135,27 @@ __device__ __forceinline__ double cpr_entry(const double* a, int64_t N, const Cp
   return v;
 }
 
-// out = T b (per CCD: b stride N, out stride Ns)
-__global__ void k_cpr_rhs(const double* __restrict__ b, double* __restrict__ out, int N, int Ns, CprMap m) {
+// out = T b (per CCD: out stride Ns)
+__global__ void k_cpr_rhs(RhsSrc b, double* __restrict__ out, int Ns, CprMap m) {
   const int ccd = blockIdx.y;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < Ns; r += gridDim.x * blockDim.x) {
     int idx[2];
     double sg[2];
     const int n = cpr_row(m, r, idx, sg);
     double v = 0.0;
-    for (int x = 0; x < n; ++x) v += sg[x] * b[(int64_t)ccd * N + idx[x]];
+    for (int x = 0; x < n; ++x) v += sg[x] * b.at(ccd, idx[x]);
     out[(int64_t)ccd * Ns + r] = v;
   }
+}
+
+// (T^T x)[i]
+__device__ __forceinline__ double cpr_coef(const CprMap& m, const double* xc, int i) {
+  if (i >= m.nkc + m.NK) return xc[i - m.NK + 1];   // background
+  const int j = i / m.NK, p = i % m.NK;
+  if (j != m.jc) return xc[(j < m.jc ? j : j - 1) * m.NK + p];
+  double v = p == 0 ? xc[m.nkc] : 0.0;
+  for (int jj = 0; jj < m.nkc / m.NK; ++jj) v -= xc[jj * m.NK + p];
+  return v;
 }
 
 // theta_off (=|+=) T^T x (per CCD: x stride Ns, theta_off stride N)
@@ -154,22 +164,18 @@ __global__ void k_cpr_expand(const double* __restrict__ x, double* __restrict__ 
   const int ccd = blockIdx.y;
   const double* xc = x + (int64_t)ccd * Ns;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-    double v;
-    if (i >= m.nkc + m.NK) {
-      v = xc[i - m.NK + 1];                      // background
-    } else {
-      const int j = i / m.NK, p = i % m.NK;
-      if (j != m.jc) {
-        v = xc[(j < m.jc ? j : j - 1) * m.NK + p];
-      } else {
-        v = p == 0 ? xc[m.nkc] : 0.0;
-        for (int jj = 0; jj < m.nkc / m.NK; ++jj) v -= xc[jj * m.NK + p];
-      }
-    }
+    const double v = cpr_coef(m, xc, i);
     double* o = theta_off + (int64_t)ccd * N + i;
     *o = add ? *o + v : v;
   }
 }
+
+// A solution that a refinement step starts from on the mixed path is kept in
+// FP32 values: the step's residual is formed with FP32 coefficients, and its
+// correction belongs to those.  Keeping the FP64 solution beside them left the
+// rounding in the result (a kernel sum off by 3e-8 is a background off by
+// 3e-5 ADU at a sky of 1000).
+__device__ __forceinline__ double stored_theta(double v, int to_float) { return to_float ? (double)(float)v : v; }
 
 // scale = diag(A_s)^-1/2 and the diagonal's status flags, a thread per row.
 // A_s is the solved system: A itself (row stride N = Ns) or T A T^T (size Ns).
@@ -586,8 +592,8 @@ __device__ __forceinline__ bool wait_value(const T* p, T& v) {
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_chol_solve(const T* __restrict__ Lf, const T* __restrict__ dinv, const double* __restrict__ scale,
-             const double* __restrict__ rhs, double* __restrict__ x, int N, int B, T* __restrict__ ybuf,
-             T* __restrict__ xbuf, int* __restrict__ status) {
+             RhsSrc rhs, double* __restrict__ x, int N, int B, T* __restrict__ ybuf, T* __restrict__ xbuf,
+             int* __restrict__ status, int add) {
   __shared__ SolveSmem<T> S;
   const int nblk = (N + NBK - 1) / NBK;
   const int nitem = nblk * B, G = gridDim.x;
@@ -622,7 +628,7 @@ k_chol_solve(const T* __restrict__ Lf, const T* __restrict__ dinv, const double*
       T s = T(0);
 #pragma unroll
       for (int p = 0; p < 8; ++p) s += S.part[tid][p];
-      S.v[tid] = tid < nb ? (T)(rhs[(int64_t)ccd * N + jb + tid] * scale[(int64_t)ccd * N + jb + tid]) - s : T(0);
+      S.v[tid] = tid < nb ? (T)(rhs.at(ccd, jb + tid) * scale[(int64_t)ccd * N + jb + tid]) - s : T(0);
     }
     __syncthreads();
     if (tid < nb) {
@@ -686,7 +692,8 @@ k_chol_solve(const T* __restrict__ Lf, const T* __restrict__ dinv, const double*
       xbuf[(int64_t)ccd * N + jb + tid] = publishable(z);
       const double v = (double)z * scale[(int64_t)ccd * N + jb + tid];
       if (!isfinite(v)) atomicOr(&status[ccd], 2);
-      x[(int64_t)ccd * N + jb + tid] = v;
+      double* o = x + (int64_t)ccd * N + jb + tid;
+      *o = stored_theta(add & 1 ? *o + v : v, add & 2);
     }
     __syncthreads();
   }
@@ -694,42 +701,35 @@ k_chol_solve(const T* __restrict__ Lf, const T* __restrict__ dinv, const double*
     for (int c = 0; c < B; ++c) atomicOr(&status[c], 4);
 }
 
-__global__ void k_theta_finish(const double* __restrict__ x, double* __restrict__ theta_off, int N, int batch, int add) {
-  const int64_t n = (int64_t)N * batch;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-    theta_off[t] = add ? theta_off[t] + x[t] : x[t];
+// the status word's code: a wait that gave up leaves the normal matrix or the
+// factor partly unwritten, which then also looks singular or non-finite: the
+// time-out is the cause and is reported first
+__device__ __forceinline__ int32_t info_code(int s) {
+  return (s & 4) ? SFFT_ERR_TIMEOUT : ((s & 2) ? SFFT_ERR_NONFINITE : ((s & 1) ? SFFT_ERR_SINGULAR : SFFT_OK));
 }
 
-// background between offset and original units: B = B' + s_S - s_R sum_j K_j (q < N_K share phi_q)
-__global__ void k_theta_units(const double* __restrict__ src, double* __restrict__ dst, const double* __restrict__ sky,
-                              int L, int NK, int NB, int to_orig) {
-  const int ccd = blockIdx.x;
+// background between offset and original units: B = B' + s_S - s_R sum_j K_j
+// (q < N_K share phi_q), a warp per background term; info, if given, takes the
+// CCD's status
+__global__ void __launch_bounds__(256)
+k_theta_units(const double* __restrict__ src, double* __restrict__ dst, const double* __restrict__ sky, int L, int NK,
+              int NB, int to_orig, const int* __restrict__ status, int32_t* __restrict__ info) {
+  const int ccd = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N = L * L * NK + NB, NKK = L * L * NK;
   const double* s = src + (int64_t)ccd * N;
   double* d = dst + (int64_t)ccd * N;
   const double sR = sky[2 * ccd], sS = sky[2 * ccd + 1];
   const double sg = to_orig ? 1.0 : -1.0;
   for (int i = threadIdx.x; i < NKK; i += blockDim.x) d[i] = s[i];
-  for (int q = threadIdx.x; q < NB; q += blockDim.x) {
-    double v = s[NKK + q];
-    if (q == 0) v += sg * sS;
+  for (int q = warp; q < NB; q += 8) {
+    double ks = 0.0;
     if (q < NK) {
-      double ks = 0.0;
-      for (int j = 0; j < L * L; ++j) ks += s[j * NK + q];
-      v -= sg * sR * ks;
+      for (int j = lane; j < L * L; j += 32) ks += s[j * NK + q];
+      ks = warp_sum(ks);
     }
-    d[NKK + q] = v;
+    if (lane == 0) d[NKK + q] = s[NKK + q] + (q == 0 ? sg * sS : 0.0) - sg * sR * ks;
   }
-}
-
-__global__ void k_info(const int* __restrict__ status, int32_t* __restrict__ info, int batch) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= batch) return;
-  const int s = status[c];
-  // a wait that gave up leaves the normal matrix or the factor partly
-  // unwritten, which then also looks singular or non-finite: the time-out is
-  // the cause and is reported first
-  info[c] = (s & 4) ? SFFT_ERR_TIMEOUT : ((s & 2) ? SFFT_ERR_NONFINITE : ((s & 1) ? SFFT_ERR_SINGULAR : SFFT_OK));
+  if (info && threadIdx.x == 0) info[ccd] = info_code(status[ccd]);
 }
 
 __global__ void k_kernel_at(const double* __restrict__ theta, double* __restrict__ K, int L, int DK, int NK, int NB,
@@ -750,8 +750,189 @@ __global__ void k_kernel_at(const double* __restrict__ theta, double* __restrict
   }
 }
 
+// ---------------------------------------------------------------- small systems
+// FP32 systems of up to kSmallN unknowns (L <= 3, L = 5, and larger kernels of
+// low degree): one CTA per CCD holds the scaled matrix in shared memory, scales
+// and factors it (FACTOR) or fetches its factor, substitutes, and adds to or
+// sets theta_off.  The cooperative kernels hand every 32-block through L2 and
+// take two more launches per step (cutout of 160 x 192, N = 78: 51 + 19 us in
+// seven launches, 45 + 15 us in two, and the call 188 -> 138 us).  Above the limit one SM's multiply-adds and the FP64 scaling
+// of N^2 / 2 entries cost more than the hand-overs.
+constexpr int kSmallN = 160, kSmallThreads = 512, kSmallRows = kSmallN / 32;
+
+struct SmallArgs {
+  const double* A;
+  RhsSrc rhs;
+  float* Lf;
+  double *scale, *theta_off;
+  int* status;
+  int N, Ns, add;
+  CprMap m;
+};
+
+__host__ __device__ constexpr size_t small_smem(int Ns) {
+  return sizeof(double) * 2 * (size_t)kSmallN + sizeof(float) * ((size_t)Ns * (Ns | 1) + 4 * kSmallN);
+}
+
+// Factor of the lower triangle in l (Ns <= NMAX): right-looking on the unscaled
+// Schur complement, a_ij -= a_ic a_jc / d_c, with the triangle in registers (rows
+// warp + 16 q, columns lane + 32 r) and one barrier per column, through a column
+// buffer that its owners write as soon as it is up to date.
+template <int NMAX>
+__device__ __forceinline__ void small_factor(float* l, int P, int Ns, float* rd, float* colb, int* bad) {
+  constexpr int NW = kSmallThreads / 32, NQ = (NMAX + NW - 1) / NW, NR = (NMAX + 31) / 32;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float acc[NQ][NR];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q)
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int i = warp + NW * q, j = lane + 32 * r;
+      acc[q][r] = i < Ns && j <= i ? l[i * P + j] : 0.f;
+    }
+  if (tid < Ns) colb[tid] = l[tid * P];
+  __syncthreads();
+  for (int c = 0; c < Ns; ++c) {
+    const float* col = colb + (c & 1) * kSmallN;
+    float* nxt = colb + ((c + 1) & 1) * kSmallN;
+    const float d0 = col[c];
+    const bool wrong = !(d0 > 0.f) || !isfinite(d0);
+    const float rs = rsqrtf(wrong ? 1.f : d0), p = rs * rs;
+    if (tid >= c && tid < Ns) l[tid * P + c] = tid == c ? (wrong ? 1.f : d0) * rs : col[tid] * rs;
+    if (tid == c) {
+      rd[c] = rs;
+      if (wrong) atomicOr(bad, isfinite(d0) ? 1 : 2);
+    }
+    float f[NQ], g[NR];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int i = warp + NW * q;
+      f[q] = i > c && i < Ns ? col[i] * p : 0.f;
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int j = lane + 32 * r;
+      g[r] = j > c && j < Ns ? col[j] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) acc[q][r] -= f[q] * g[r];
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+      if (lane + 32 * r == c + 1) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+          if (warp + NW * q > c && warp + NW * q < Ns) nxt[warp + NW * q] = acc[q][r];
+      }
+    __syncthreads();
+  }
+}
+
+template <bool FACTOR>
+__global__ void __launch_bounds__(kSmallThreads)
+k_small(const SmallArgs a) {
+  extern __shared__ double smd[];
+  __shared__ int bad;
+  constexpr int NW = kSmallThreads / 32;
+  const int ccd = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, Ns = a.Ns, P = Ns | 1;
+  double* sc = smd;                       // [kSmallN] scale
+  double* xd = sc + kSmallN;              // [kSmallN] solution
+  float* l = reinterpret_cast<float*>(xd + kSmallN);
+  float* v = l + (size_t)Ns * P;          // [kSmallN] right-hand side
+  float* rd = v + kSmallN;                // [kSmallN] reciprocal pivots 1 / l_cc
+  float* colb = rd + kSmallN;             // [2][kSmallN] the factor's current column
+  const double* A = a.A + (int64_t)ccd * a.N * a.N;
+  float* Lg = a.Lf + (int64_t)ccd * Ns * Ns;
+  if (tid == 0) bad = 0;
+  if (FACTOR) {
+    __syncthreads();
+    for (int i = tid; i < Ns; i += kSmallThreads) {
+      const double d = cpr_entry(A, a.N, a.m, i, i);
+      if (!isfinite(d)) atomicOr(&bad, 2);
+      else if (!(d > 0.0)) atomicOr(&bad, 1);
+      sc[i] = d > 0.0 ? rsqrt(d) : 0.0;
+      a.scale[(int64_t)ccd * Ns + i] = sc[i];
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int i = warp; i < Ns; i += NW)
+      for (int j = lane; j <= i; j += 32) {
+        const double e = a.m.on ? cpr_entry(A, a.N, a.m, i, j) : A[(int64_t)i * a.N + j];
+        if (!isfinite(e)) atomicOr(&bad, 2);
+        l[i * P + j] = (float)(e * sc[i] * sc[j]);
+      }
+    __syncthreads();
+    if (Ns <= kSmallN / 2) small_factor<kSmallN / 2>(l, P, Ns, rd, colb, &bad);
+    else small_factor<kSmallN>(l, P, Ns, rd, colb, &bad);
+    for (int i = warp; i < Ns; i += NW)
+      for (int j = lane; j <= i; j += 32) Lg[(int64_t)i * Ns + j] = l[i * P + j];
+  } else {
+    for (int i = tid; i < Ns; i += kSmallThreads) {
+      sc[i] = a.scale[(int64_t)ccd * Ns + i];
+      rd[i] = 1.f / Lg[(int64_t)i * Ns + i];
+    }
+#pragma unroll 4
+    for (int i = warp; i < Ns; i += NW)
+      for (int j = lane; j <= i; j += 32) l[i * P + j] = Lg[(int64_t)i * Ns + j];
+    __syncthreads();
+  }
+  for (int i = tid; i < Ns; i += kSmallThreads) {
+    int idx[2];
+    double sg[2], r = 0.0;
+    const int n = cpr_row(a.m, i, idx, sg);
+    for (int k = 0; k < n; ++k) r += sg[k] * a.rhs.at(ccd, idx[k]);
+    v[i] = (float)(r * sc[i]);
+  }
+  __syncthreads();
+  // L y = v and L^T x = y in one warp, rows lane + 32 q in its registers
+  if (warp == 0) {
+    float x[kSmallRows];
+#pragma unroll
+    for (int q = 0; q < kSmallRows; ++q) x[q] = lane + 32 * q < Ns ? v[lane + 32 * q] : 0.f;
+#pragma unroll
+    for (int b = 0; b < kSmallRows; ++b)
+      for (int t = 0; t < min(32, Ns - 32 * b); ++t) {
+        const int c = 32 * b + t;
+        const float xc = __shfl_sync(0xffffffffu, x[b], t) * rd[c];
+        if (lane == t) x[b] = xc;
+#pragma unroll
+        for (int q = b; q < kSmallRows; ++q) {
+          const int i = lane + 32 * q;
+          if (i > c && i < Ns) x[q] -= l[i * P + c] * xc;
+        }
+      }
+#pragma unroll
+    for (int b = kSmallRows - 1; b >= 0; --b)
+      for (int t = min(32, Ns - 32 * b) - 1; t >= 0; --t) {
+        const int c = 32 * b + t;
+        const float xc = __shfl_sync(0xffffffffu, x[b], t) * rd[c];
+        if (lane == t) x[b] = xc;
+#pragma unroll
+        for (int q = 0; q <= b; ++q)
+          if (lane + 32 * q < c) x[q] -= l[c * P + lane + 32 * q] * xc;
+      }
+#pragma unroll
+    for (int q = 0; q < kSmallRows; ++q)
+      if (lane + 32 * q < Ns) v[lane + 32 * q] = x[q];
+  }
+  __syncthreads();
+  for (int i = tid; i < Ns; i += kSmallThreads) {
+    const double x = (double)v[i] * sc[i];
+    if (!isfinite(x)) atomicOr(&bad, 2);
+    xd[i] = x;
+  }
+  __syncthreads();
+  for (int i = tid; i < a.N; i += kSmallThreads) {
+    const double x = a.m.on ? cpr_coef(a.m, xd, i) : xd[i];
+    double* o = a.theta_off + (int64_t)ccd * a.N + i;
+    *o = stored_theta(a.add & 1 ? *o + x : x, a.add & 2);
+  }
+  if (tid == 0 && bad) atomicOr(&a.status[ccd], bad);
+}
+
 // ------------------------------------------------------------------ launchers
-cudaError_t launch_scatter(const sfft_plan_s* p, double* A, double* b, void* ws, bool rhs_only, double* rhs_out) {
+cudaError_t launch_scatter(const sfft_plan_s* p, double* A, double* b, void* ws) {
   ScatterArgs a;
   a.L = p->d.L; a.w = p->w; a.NK = p->NK; a.NB = p->NB; a.NKK = p->NKK; a.N = p->N;
   a.nm_kk = n_mono(p->DM_KK); a.nm_kb = n_mono(p->DM_KB); a.nm_bk = n_mono(p->DM_bK); a.nm_bb = n_mono(p->DM_BB);
@@ -761,14 +942,13 @@ cudaError_t launch_scatter(const sfft_plan_s* p, double* A, double* b, void* ws,
   a.s_gbk = (int64_t)LL * a.nm_bk;
   a.s_mbb = a.nm_bb;
   a.s_mb = n_mono(p->d.DB);
-  const int64_t total = rhs_only ? p->N : (int64_t)p->N * p->N + p->N;
+  const int64_t total = (int64_t)p->N * p->N + p->N;
   int gx = (int)((total + 255) / 256);
   if (gx > 2048) gx = 2048;
   dim3 grid(gx, p->d.batch);
   k_scatter<<<grid, 256, 0, p->stream>>>(a, ws_at<double>(ws, p->gkk), ws_at<double>(ws, p->gkb),
                                          ws_at<double>(ws, p->gbk), ws_at<double>(ws, p->mom_bb),
-                                         ws_at<double>(ws, p->mom_b), p->d_hdidx, A, rhs_only ? rhs_out : b,
-                                         rhs_only ? 1 : 0);
+                                         ws_at<double>(ws, p->mom_b), p->d_hdidx, A, b);
   p->nlaunch += 1;
   return cudaGetLastError();
 }
@@ -849,7 +1029,8 @@ cudaError_t launch_cholesky(const sfft_plan_s* p, const double* A, void* ws) {
 }
 
 template <typename T>
-static cudaError_t chol_solve_T(const sfft_plan_s* p, const double* rhs, double* x, void* ws) {
+static cudaError_t chol_solve_T(const sfft_plan_s* p, const RhsSrc& rhs_in, double* x, int add, void* ws) {
+  RhsSrc rhs = rhs_in;
   int N = p->Nsol, B = p->d.batch;
   const int nitem = ((N + NBK - 1) / NBK) * B;
   T* Lf = ws_at<T>(ws, p->lfac);
@@ -862,16 +1043,42 @@ static cudaError_t chol_solve_T(const sfft_plan_s* p, const double* rhs, double*
   cudaError_t e = cudaMemsetAsync(ybuf, 0xFF, sizeof(T) * 2 * (size_t)p->N * B, p->stream);
   if (e != cudaSuccess) return e;
   const int grid = coop_grid((const void*)k_chol_solve<T>, nitem, B);
-  void* args[] = {&Lf, &dinv, &scale, &rhs, &x, &N, &B, &ybuf, &xbuf, &status};
+  void* args[] = {&Lf, &dinv, &scale, &rhs, &x, &N, &B, &ybuf, &xbuf, &status, &add};
   e = launch_coop((const void*)k_chol_solve<T>, grid, p->stream, args);
   p->nlaunch += 1;
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
-cudaError_t launch_chol_solve(const sfft_plan_s* p, const double* rhs, double* x, void* ws) {
-  return p->fp64 ? chol_solve_T<double>(p, rhs, x, ws) : chol_solve_T<float>(p, rhs, x, ws);
+cudaError_t launch_chol_solve(const sfft_plan_s* p, const RhsSrc& rhs, double* x, int add, void* ws) {
+  return p->fp64 ? chol_solve_T<double>(p, rhs, x, add, ws) : chol_solve_T<float>(p, rhs, x, add, ws);
 }
+
+bool small_system(const sfft_plan_s* p) { return !p->fp64 && p->Nsol <= kSmallN; }
+
+cudaError_t launch_small(const sfft_plan_s* p, const double* A, const RhsSrc& rhs, bool factor, int add, void* ws) {
+  SmallArgs a;
+  a.A = A; a.rhs = rhs;
+  a.Lf = ws_at<float>(ws, p->lfac);
+  a.scale = ws_at<double>(ws, p->scale);
+  a.theta_off = ws_at<double>(ws, p->theta_off);
+  a.status = ws_at<int>(ws, p->status);
+  a.N = p->N; a.Ns = p->Nsol; a.add = add;
+  a.m = cpr_map(p);
+  const size_t smem = small_smem(p->Nsol);
+  auto kern = factor ? k_small<true> : k_small<false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem(kSmallN));
+  if (e != cudaSuccess) return e;
+  kern<<<p->d.batch, kSmallThreads, smem, p->stream>>>(a);
+  p->nlaunch += 1;
+  return cudaGetLastError();
+}
+
+// the image-space assembly's right-hand side, where the sums leave it
+RhsSrc rhs_of_sums(const sfft_plan_s* p, void* ws) {
+  return RhsSrc{ws_at<double>(ws, p->gbk), ws_at<double>(ws, p->mom_b), p->NKK, n_mono(p->d.DB), p->NKK};
+}
+RhsSrc rhs_of_vector(const sfft_plan_s* p, const double* b) { return RhsSrc{b, b, p->N, p->N, p->N}; }
 
 // r = b - A theta for every CCD (FP64; A full, N x N row-major): a warp per row
 __global__ void __launch_bounds__(256)
@@ -901,16 +1108,9 @@ cudaError_t launch_residual(const sfft_plan_s* p, const double* A, const double*
   return cudaGetLastError();
 }
 
-cudaError_t launch_theta_finish(const sfft_plan_s* p, const double* x, double* theta_off, bool add) {
-  const int64_t n = (int64_t)p->N * p->d.batch;
-  k_theta_finish<<<(int)((n + 255) / 256), 256, 0, p->stream>>>(x, theta_off, p->N, p->d.batch, add ? 1 : 0);
-  p->nlaunch += 1;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cpr_rhs(const sfft_plan_s* p, const double* b, double* out) {
+cudaError_t launch_cpr_rhs(const sfft_plan_s* p, const RhsSrc& b, double* out) {
   dim3 grid((p->Nsol + 255) / 256, p->d.batch);
-  k_cpr_rhs<<<grid, 256, 0, p->stream>>>(b, out, p->N, p->Nsol, cpr_map(p));
+  k_cpr_rhs<<<grid, 256, 0, p->stream>>>(b, out, p->Nsol, cpr_map(p));
   p->nlaunch += 1;
   return cudaGetLastError();
 }
@@ -922,29 +1122,25 @@ cudaError_t launch_cpr_expand(const sfft_plan_s* p, const double* x, double* the
   return cudaGetLastError();
 }
 
-cudaError_t launch_theta_to_orig(const sfft_plan_s* p, const double* theta_off, double* theta, void* ws) {
-  k_theta_units<<<p->d.batch, 128, 0, p->stream>>>(theta_off, theta, ws_at<double>(ws, p->sky), p->d.L, p->NK, p->NB, 1);
+cudaError_t launch_theta_to_orig(const sfft_plan_s* p, const double* theta_off, double* theta, int32_t* info,
+                                 void* ws) {
+  k_theta_units<<<p->d.batch, 256, 0, p->stream>>>(theta_off, theta, ws_at<double>(ws, p->sky), p->d.L, p->NK, p->NB, 1,
+                                                   ws_at<int>(ws, p->status), info);
   p->nlaunch += 1;
   return cudaGetLastError();
 }
 
 cudaError_t launch_theta_to_off(const sfft_plan_s* p, const double* theta, const double* sky, double* theta_off,
                                 void* ws) {
-  k_theta_units<<<p->d.batch, 128, 0, p->stream>>>(theta, theta_off, sky ? sky : ws_at<double>(ws, p->sky), p->d.L,
-                                                   p->NK, p->NB, 0);
+  k_theta_units<<<p->d.batch, 256, 0, p->stream>>>(theta, theta_off, sky ? sky : ws_at<double>(ws, p->sky), p->d.L,
+                                                   p->NK, p->NB, 0, nullptr, nullptr);
   p->nlaunch += 1;
   return cudaGetLastError();
 }
 
 cudaError_t launch_theta_units_raw(cudaStream_t s, const double* src, double* dst, const double* sky, int L, int NK,
                                    int NB, int batch, int to_orig) {
-  k_theta_units<<<batch, 128, 0, s>>>(src, dst, sky, L, NK, NB, to_orig);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_info(const sfft_plan_s* p, int32_t* info, void* ws) {
-  k_info<<<(p->d.batch + 127) / 128, 128, 0, p->stream>>>(ws_at<int>(ws, p->status), info, p->d.batch);
-  p->nlaunch += 1;
+  k_theta_units<<<batch, 256, 0, s>>>(src, dst, sky, L, NK, NB, to_orig, nullptr, nullptr);
   return cudaGetLastError();
 }
 

@@ -145,6 +145,7 @@ struct sfft_plan_s {
 namespace sfft {
 
 // kernels_*.cu launchers; all enqueue on p->stream and return cudaGetLastError()
+// also clears the status words
 cudaError_t launch_sky(const sfft_plan_s* p, const float* R, const float* S, const uint8_t* bad,
                        const double* sky_in, void* ws);
 cudaError_t launch_prep(const sfft_plan_s* p, const float* R, const float* S, const uint8_t* bad, void* ws);
@@ -174,15 +175,30 @@ cudaError_t launch_prep_bits(const sfft_plan_s* p, const float* R, const float* 
                              void* ws);
 int64_t edge_cap(const sfft_plan_s* p);   // most entries of an edge list
 cudaError_t launch_edge_sums(const sfft_plan_s* p, void* ws);
-cudaError_t launch_scatter(const sfft_plan_s* p, double* A, double* b, void* ws, bool rhs_only, double* rhs_out);
+cudaError_t launch_scatter(const sfft_plan_s* p, double* A, double* b, void* ws);
 cudaError_t launch_cholesky(const sfft_plan_s* p, const double* A, void* ws);
-cudaError_t launch_chol_solve(const sfft_plan_s* p, const double* rhs, double* x, void* ws);
+// A right-hand side, per CCD: the first `split` entries from a, the rest from b
+struct RhsSrc {
+  const double *a, *b;
+  int64_t sa, sb;      // per CCD
+  int split;
+  __host__ __device__ double at(int ccd, int i) const {
+    return i < split ? a[(int64_t)ccd * sa + i] : b[(int64_t)ccd * sb + i - split];
+  }
+};
+RhsSrc rhs_of_sums(const sfft_plan_s* p, void* ws);
+RhsSrc rhs_of_vector(const sfft_plan_s* p, const double* b);
+// add: bit 0 adds to x (else sets it), bit 1 keeps the result in FP32 values
+cudaError_t launch_chol_solve(const sfft_plan_s* p, const RhsSrc& rhs, double* x, int add, void* ws);
+// small FP32 systems: scale, factor (or use the factor), solve, theta_off (=|+=), one CTA per CCD
+bool small_system(const sfft_plan_s* p);
+cudaError_t launch_small(const sfft_plan_s* p, const double* A, const RhsSrc& rhs, bool factor, int add, void* ws);
 cudaError_t launch_residual(const sfft_plan_s* p, const double* A, const double* b, const double* theta_off,
                             double* r);
-cudaError_t launch_theta_finish(const sfft_plan_s* p, const double* x, double* theta_off, bool add);
-cudaError_t launch_cpr_rhs(const sfft_plan_s* p, const double* b, double* out);
+cudaError_t launch_cpr_rhs(const sfft_plan_s* p, const RhsSrc& b, double* out);
 cudaError_t launch_cpr_expand(const sfft_plan_s* p, const double* x, double* theta_off, bool add);
-cudaError_t launch_theta_to_orig(const sfft_plan_s* p, const double* theta_off, double* theta, void* ws);
+cudaError_t launch_theta_to_orig(const sfft_plan_s* p, const double* theta_off, double* theta, int32_t* info,
+                                 void* ws);
 cudaError_t launch_theta_to_off(const sfft_plan_s* p, const double* theta, const double* sky, double* theta_off, void* ws);
 cudaError_t launch_apply(const sfft_plan_s* p, const float* R, const float* S, const double* theta_off,
                          const double* sky, float* D, void* ws);
@@ -190,7 +206,6 @@ cudaError_t launch_apply(const sfft_plan_s* p, const float* R, const float* S, c
 cudaError_t launch_residual_image(const sfft_plan_s* p, const float* R, const float* S, const double* theta_off,
                                   void* eimg, void* ws);
 cudaError_t launch_residual_sums(const sfft_plan_s* p, const float* S, const double* theta_off, void* ws);
-cudaError_t launch_info(const sfft_plan_s* p, int32_t* info, void* ws);
 cudaError_t launch_kernel_at(const sfft_plan_s* p, const double* theta, double x, double y, double* K);
 
 // Plan-free launchers (explicit shapes and stream) used by the allocation-free entry point.
