@@ -30,8 +30,9 @@
 
 namespace {
 
-constexpr int NROT = 4;
+constexpr int NROT = 4, NROT_RI = NROT;
 constexpr int KA = 9 * C1, KC = 9 * C2;   // GEMM K of the residual convolutions (32 -> 32, 64 -> 64)
+constexpr int KA_RI = KA;
 
 // master parameter offsets (GEMM layout, floats)
 constexpr int QW1 = 0, QB1 = QW1 + K1 * C1, QWA = QB1 + C1, QBA = QWA + KA * C1, QWB = QBA + C1,
@@ -43,6 +44,12 @@ constexpr int QW1 = 0, QB1 = QW1 + K1 * C1, QWA = QB1 + C1, QBA = QWA + KA * C1,
 struct ConvSpec { int cin, cout, ow, ob; };
 constexpr ConvSpec kConv[6] = {{3, C1, QW1, QB1},  {C1, C1, QWA, QBA}, {C1, C1, QWB, QBB},
                                {C1, C2, QW2, QB2}, {C2, C2, QWC, QBC}, {C2, C2, QWD, QBD}};
+
+}  // namespace
+
+#include "rb_ri_stack.cuh"
+
+namespace {
 
 // xr[r n + i] = the r-th counterclockwise quarter turn of xn[i]:
 // r = 1: out(y, x) = in(x, 30 - y); r = 2: in(30 - y, 30 - x); r = 3: in(30 - x, y)
@@ -185,7 +192,22 @@ bool alloc(T** p, size_t n) {
   return cudaMalloc((void**)p, sizeof(T) * (n > 0 ? n : 1)) == cudaSuccess;
 }
 
-// forward for n normalised stamps in m->xn; logits to m->logit
+// The convolutional stack for inference: a3 from xn in two launches
+cudaError_t stack_inference(rbri_model_s* m, int n, cudaStream_t s) {
+  const bf16* W = m->wbf;
+  const float* P = m->params;
+  const int n4 = NROT * n;
+  cudaError_t e = cudaFuncSetAttribute(k_ri_front, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRiFrontSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ri_back, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRiBackSmem);
+  if (e != cudaSuccess) return e;
+  k_ri_front<<<std::min(n4, 152), 256, kRiFrontSmem, s>>>(m->xn, n, W + QW1, W + QWA, W + QWB, W + QW2, P + QB1, P + QBA,
+                                                          P + QBB, P + QB2, m->a2);
+  k_ri_back<<<std::min((n4 + 1) / 2, 152), 256, kRiBackSmem, s>>>(m->a2, n4, W + QWC, W + QWD, P + QBC, P + QBD, m->a3);
+  return cudaGetLastError();
+}
+
+// forward for n normalised stamps in m->xn; logits to m->logit.  keep_idx: for
+// a backward pass, every layer's pre-activations and pool positions are kept
 cudaError_t forward(rbri_model_s* m, int n, cudaStream_t s, bool keep_idx) {
   using rbg::ConvRows;
   using rbg::Conv1Rows;
@@ -194,12 +216,15 @@ cudaError_t forward(rbri_model_s* m, int n, cudaStream_t s, bool keep_idx) {
   const float* P = m->params;
   const int n4 = NROT * n;
   cudaError_t e;
+  if (!keep_idx) {
+    if ((e = stack_inference(m, n, s))) return e;
+  } else {
   k_rotate<<<grid1((int64_t)n4 * PIX1 * 3), 256, 0, s>>>(m->xn, n, m->xr);
   // conv1 + ReLU + pool
   if ((e = igemm<Conv1Rows, Dense, false>(s, n4 * PIX1, C1, K1, Conv1Rows{m->xr, n4, S31, S31, 3 * PIX1},
                                           Dense{W + QW1, K1, C1, C1}, m->z1, C1, P + QB1)))
     return e;
-  k_relu_pool<<<grid1((int64_t)n4 * PIX2 * C1), 256, 0, s>>>(m->z1, n4, S31, S31, C1, m->a1, keep_idx ? m->i1 : nullptr);
+  k_relu_pool<<<grid1((int64_t)n4 * PIX2 * C1), 256, 0, s>>>(m->z1, n4, S31, S31, C1, m->a1, m->i1);
   // res1
   const int64_t m1 = (int64_t)n4 * PIX2 * C1;
   if ((e = igemm<ConvRows, Dense, false>(s, n4 * PIX2, C1, KA, ConvRows{m->a1, n4, 15, 15, C1, 1},
@@ -215,7 +240,7 @@ cudaError_t forward(rbri_model_s* m, int n, cudaStream_t s, bool keep_idx) {
   if ((e = igemm<ConvRows, Dense, false>(s, n4 * PIX2, C2, K2, ConvRows{m->r1, n4, 15, 15, C1, 1},
                                          Dense{W + QW2, K2, C2, C2}, m->z2, C2, P + QB2)))
     return e;
-  k_relu_pool<<<grid1((int64_t)n4 * PIX3 * C2), 256, 0, s>>>(m->z2, n4, 15, 15, C2, m->a2, keep_idx ? m->i2 : nullptr);
+  k_relu_pool<<<grid1((int64_t)n4 * PIX3 * C2), 256, 0, s>>>(m->z2, n4, 15, 15, C2, m->a2, m->i2);
   // res2 + pool
   const int64_t m2 = (int64_t)n4 * PIX3 * C2;
   if ((e = igemm<ConvRows, Dense, false>(s, n4 * PIX3, C2, KC, ConvRows{m->a2, n4, 7, 7, C2, 1},
@@ -226,7 +251,8 @@ cudaError_t forward(rbri_model_s* m, int n, cudaStream_t s, bool keep_idx) {
                                          Dense{W + QWD, KC, C2, C2}, m->zd, C2, P + QBD)))
     return e;
   k_add_skip<<<grid1(m2), 256, 0, s>>>(m->zd, m->a2, m2);
-  k_relu_pool<<<grid1((int64_t)n4 * PIX4 * C2), 256, 0, s>>>(m->zd, n4, 7, 7, C2, m->a3, keep_idx ? m->i3 : nullptr);
+  k_relu_pool<<<grid1((int64_t)n4 * PIX4 * C2), 256, 0, s>>>(m->zd, n4, 7, 7, C2, m->a3, m->i3);
+  }
   // rotation average, dense head
   k_rot_mean<<<grid1((int64_t)n * K4), 256, 0, s>>>(m->a3, n, m->f, m->fb);
   if ((e = igemm<Dense, Dense, false>(s, n, F4, K4, Dense{m->fb, n, K4, K4}, Dense{W + QW4, K4, F4, F4}, m->z4, F4,
