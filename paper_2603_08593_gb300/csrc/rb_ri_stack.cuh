@@ -43,8 +43,8 @@ __device__ __forceinline__ void ri_conv(float (&acc)[2][4][4], const bf16* const
     for (int j = 0; j < 4; ++j)
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
-#pragma unroll 1
-  for (int tap = 0; tap < 9; ++tap) {
+#pragma unroll 3
+  for (int tap = 0; tap < 9; ++tap) {   // three taps of fragments ahead of their products
     const int off = (tap / 3 * RW + tap % 3) * AP;
 #pragma unroll
     for (int h = 0; h < C / 16; ++h) {
@@ -112,18 +112,30 @@ k_ri_front(const bf16* __restrict__ xn, int n, const bf16* __restrict__ W1, cons
     pa[i] = (p / 15 * 17 + p % 15) * RiP1 + lk;
   }
   float acc[2][4][4];
+  constexpr int NS = (3 * PIX1 + 255) / 256;
+  bf16 next[NS];   // the next image's values, fetched while this one is convolved
+  auto fetch = [&](int img) {
+    const bf16* src = xn + (int64_t)(img % n) * 3 * PIX1;
+#pragma unroll
+    for (int k = 0; k < NS; ++k)
+      if (tid + 256 * k < 3 * PIX1) next[k] = src[tid + 256 * k];
+  };
+  fetch(blockIdx.x);
   for (int img = blockIdx.x; img < NROT_RI * n; img += gridDim.x) {
     const int rot = img / n;
-    const bf16* src = xn + (int64_t)(img - rot * n) * 3 * PIX1;
-    for (int e = tid; e < 3 * PIX1; e += 256) {
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      const int e = tid + 256 * k;
+      if (e >= 3 * PIX1) break;
       const int p = e / 3, sy = p / S31, sxx = p - sy * S31;
       int y = sy, x = sxx;
       if (rot == 1) { y = S31 - 1 - sxx; x = sy; }
       else if (rot == 2) { y = S31 - 1 - sy; x = S31 - 1 - sxx; }
       else if (rot == 3) { y = sxx; x = S31 - 1 - sy; }
-      sx[((y + 1) * 33 + x + 1) * 3 + e - 3 * p] = src[e];
+      sx[((y + 1) * 33 + x + 1) * 3 + e - 3 * p] = next[k];
     }
     __syncthreads();
+    if (img + gridDim.x < NROT_RI * n) fetch(img + gridDim.x);
     for (int m = tid; m < 900; m += 256) {
       const int win = m >> 2, y = 2 * (win / 15) + ((m >> 1) & 1), x = 2 * (win % 15) + (m & 1);
       const unsigned short* s = reinterpret_cast<const unsigned short*>(sx) + (y * 33 + x) * 3;
