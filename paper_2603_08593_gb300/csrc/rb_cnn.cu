@@ -75,36 +75,15 @@ void abi_to_master(const float* a, std::vector<float>& m) {
   m[OB5] = b5[0];
 }
 
-void master_to_abi(const float* m, float* a) {
-  float* w1 = a;
-  float* b1 = w1 + 32 * 27;
-  float* w2 = b1 + 32;
-  float* b2 = w2 + 64 * 288;
-  float* w3 = b2 + 64;
-  float* b3 = w3 + 64 * 576;
-  float* w4 = b3 + 64;
-  float* b4 = w4 + 128 * 576;
-  float* w5 = b4 + 128;
-  float* b5 = w5 + 128;
-  auto conv = [&](float* w, int cin, int cout, int off) {
-    for (int o = 0; o < cout; ++o)
-      for (int ci = 0; ci < cin; ++ci)
-        for (int ky = 0; ky < 3; ++ky)
-          for (int kx = 0; kx < 3; ++kx)
-            w[((o * cin + ci) * 3 + ky) * 3 + kx] = m[off + ((ky * 3 + kx) * cin + ci) * cout + o];
-  };
-  conv(w1, 3, C1, OW1);
-  conv(w2, C1, C2, OW2);
-  conv(w3, C2, C3, OW3);
-  for (int i = 0; i < C1; ++i) b1[i] = m[OB1 + i];
-  for (int i = 0; i < C2; ++i) b2[i] = m[OB2 + i];
-  for (int i = 0; i < C3; ++i) b3[i] = m[OB3 + i];
-  for (int o = 0; o < F4; ++o)
-    for (int c = 0; c < C3; ++c)
-      for (int p = 0; p < PIX4; ++p) w4[o * K4 + c * PIX4 + p] = m[OW4 + (p * C3 + c) * F4 + o];
-  for (int i = 0; i < F4; ++i) b4[i] = m[OB4 + i];
-  for (int i = 0; i < F4; ++i) w5[i] = m[OW5 + i];
-  b5[0] = m[OB5];
+// the inverse of abi_to_master as an index map
+std::vector<int> abi_map() {
+  std::vector<float> a(RB_NPARAM), m;
+  for (int i = 0; i < RB_NPARAM; ++i) a[i] = (float)(i + 1);   // exact; 0 marks padding
+  abi_to_master(a.data(), m);
+  std::vector<int> map(RB_NPARAM);
+  for (size_t i = 0; i < m.size(); ++i)
+    if (m[i] > 0.f) map[(size_t)m[i] - 1] = (int)i;
+  return map;
 }
 
 
@@ -114,6 +93,8 @@ struct rb_model_s {
   int max_batch = 0;
   int64_t step = 0;
   float *params = nullptr, *grads = nullptr, *adam_m = nullptr, *adam_v = nullptr;
+  int* map = nullptr;                          // C-ABI index -> master index
+  float* abi = nullptr;                        // a vector in C-ABI order
   bf16* wbf = nullptr;                         // bf16 copy of the master vector
   // activations / scratch for max_batch stamps
   bf16 *xn = nullptr, *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *dzb = nullptr, *dz4 = nullptr;
@@ -130,7 +111,7 @@ struct rb_model_s {
 namespace {
 
 void free_model(rb_model_s* m) {
-  void* ptrs[] = {m->params, m->grads, m->adam_m, m->adam_v, m->wbf, m->xn,  m->a1,   m->a2,   m->a3,
+  void* ptrs[] = {m->map, m->abi, m->params, m->grads, m->adam_m, m->adam_v, m->wbf, m->xn,  m->a1,   m->a2,   m->a3,
                   m->dzb,    m->dz4,   m->z1,     m->z2,     m->z3,  m->z4, m->logit, m->dz5,  m->da,
                   m->part,   m->i1,    m->i2,     m->i3,  m->img1, m->img2, m->img3, m->p2,   m->p3,
                   m->err};
@@ -256,7 +237,7 @@ extern "C" sfft_status_t rb_create(const int32_t* desc, rb_model_t* out) {
   if (!m) return SFFT_ERR_NOMEM;
   const int B = desc[0];
   m->max_batch = B;
-  bool ok = alloc(&m->params, NMASTER) && alloc(&m->grads, NMASTER) && alloc(&m->adam_m, NMASTER) &&
+  bool ok = alloc(&m->map, RB_NPARAM) && alloc(&m->abi, RB_NPARAM) && alloc(&m->params, NMASTER) && alloc(&m->grads, NMASTER) && alloc(&m->adam_m, NMASTER) &&
             alloc(&m->adam_v, NMASTER) && alloc(&m->wbf, NMASTER) && alloc(&m->xn, (size_t)B * rbtc::kXnStride) &&
             alloc(&m->a1, (size_t)B * PIX2 * C1) && alloc(&m->a2, (size_t)B * PIX3 * C2) &&
             alloc(&m->a3, (size_t)B * PIX4 * C3) &&
@@ -287,7 +268,9 @@ extern "C" sfft_status_t rb_create(const int32_t* desc, rb_model_t* out) {
   }
   std::vector<float> master;
   abi_to_master(abi.data(), master);
+  const std::vector<int> map = abi_map();
   cudaError_t e = cudaMemcpy(m->params, master.data(), sizeof(float) * NMASTER, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(m->map, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(m->adam_m, 0, sizeof(float) * NMASTER);
   if (e == cudaSuccess) e = cudaMemset(m->adam_v, 0, sizeof(float) * NMASTER);
   if (e == cudaSuccess) e = cudaMemset(m->grads, 0, sizeof(float) * NMASTER);
@@ -326,29 +309,30 @@ extern "C" sfft_status_t rb_set_weights(rb_model_t m, const void* host_buf, size
   return e == cudaSuccess ? SFFT_OK : fail(e, "rb_set_weights");
 }
 
-static sfft_status_t get_vec(const float* dev, void* host_buf, size_t bytes, const char* where) {
+static sfft_status_t get_vec(rb_model_s* m, const float* dev, void* host_buf, size_t bytes, const char* where) {
   if (!dev || !host_buf || bytes != sizeof(float) * RB_NPARAM) return SFFT_ERR_ARG;
-  std::vector<float> master(NMASTER);
   cudaError_t e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) e = cudaMemcpy(master.data(), dev, sizeof(float) * NMASTER, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return fail(e, where);
-  master_to_abi(master.data(), static_cast<float*>(host_buf));
-  return SFFT_OK;
+  if (e == cudaSuccess) {
+    k_gather<<<grid1(RB_NPARAM), 256>>>(dev, m->map, RB_NPARAM, m->abi);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(host_buf, m->abi, sizeof(float) * RB_NPARAM, cudaMemcpyDeviceToHost);
+  return e == cudaSuccess ? SFFT_OK : fail(e, where);
 }
 
 extern "C" sfft_status_t rb_get_weights(rb_model_t m, void* host_buf, size_t bytes) {
-  return m ? get_vec(m->params, host_buf, bytes, "rb_get_weights") : SFFT_ERR_ARG;
+  return m ? get_vec(m, m->params, host_buf, bytes, "rb_get_weights") : SFFT_ERR_ARG;
 }
 extern "C" sfft_status_t rb_get_grads(rb_model_t m, void* host_buf, size_t bytes) {
-  return m ? get_vec(m->grads, host_buf, bytes, "rb_get_grads") : SFFT_ERR_ARG;
+  return m ? get_vec(m, m->grads, host_buf, bytes, "rb_get_grads") : SFFT_ERR_ARG;
 }
 
 extern "C" sfft_status_t rb_get_state(rb_model_t m, void* host_buf, size_t bytes, int64_t* step) {
   if (!m || !host_buf || bytes != 3 * sizeof(float) * RB_NPARAM) return SFFT_ERR_ARG;
   float* h = static_cast<float*>(host_buf);
-  sfft_status_t st = get_vec(m->params, h, sizeof(float) * RB_NPARAM, "rb_get_state");
-  if (st == SFFT_OK) st = get_vec(m->adam_m, h + RB_NPARAM, sizeof(float) * RB_NPARAM, "rb_get_state");
-  if (st == SFFT_OK) st = get_vec(m->adam_v, h + 2 * RB_NPARAM, sizeof(float) * RB_NPARAM, "rb_get_state");
+  sfft_status_t st = get_vec(m, m->params, h, sizeof(float) * RB_NPARAM, "rb_get_state");
+  if (st == SFFT_OK) st = get_vec(m, m->adam_m, h + RB_NPARAM, sizeof(float) * RB_NPARAM, "rb_get_state");
+  if (st == SFFT_OK) st = get_vec(m, m->adam_v, h + 2 * RB_NPARAM, sizeof(float) * RB_NPARAM, "rb_get_state");
   if (st == SFFT_OK && step) *step = m->step;
   return st;
 }

@@ -373,6 +373,13 @@ __global__ void k_to_bf16(const float* __restrict__ x, int64_t n, bf16* __restri
     y[e] = __float2bfloat16(x[e]);
 }
 
+// A parameter vector in the C ABI's order, gathered on the device: converting
+// it on the host walked half a megabyte with strides after the copy (a
+// 256-stamp backward pass with its gradients: 556 us, 280 of them on the host)
+__global__ void k_gather(const float* __restrict__ x, const int* __restrict__ map, int n, float* __restrict__ y) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) y[e] = x[map[e]];
+}
+
 int grid1(int64_t n) {
   int64_t g = (n + 255) / 256;
   return (int)(g > 4096 ? 4096 : (g < 1 ? 1 : g));
