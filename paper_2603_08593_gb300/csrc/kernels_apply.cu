@@ -85,8 +85,10 @@ struct ConvArgs {
   unsigned magic;          // ceil(2^20 / groups per staged row)
 };
 
+// Two CTAs per SM; FP64 only where window and sums fit 128 registers without
+// spills (L = 7, D_K = 1, one 512 x 512 pair: 64.8 us, 121.5 us at one CTA)
 template <typename T, int NT, int DK, int MODE>
-__global__ void __launch_bounds__(kCvWarps * 32, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(kCvWarps * 32, sizeof(T) == 4 || NT * (DK + 1) <= 14 ? 2 : 1)
 k_conv(const ConvArgs<T> a) {
   constexpr int wt = (NT - 1) / 2, NA = DK + 1, NK = n_mono(DK);
   extern __shared__ __align__(16) unsigned char smraw[];
