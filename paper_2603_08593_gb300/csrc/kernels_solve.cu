@@ -220,7 +220,10 @@ k_chol_init(const double* __restrict__ A, T* __restrict__ Lf, const double* __re
 // (a warp per row, a lane per column); (C) they take 8 x 32 pieces of the
 // trailing lower triangles and subtract P_i P_j^T, while one CTA per CCD
 // updates the next diagonal block in shared memory and factors it
-// (look-ahead).  GB300 retires about two FP64 FMAs per SM per clock, so the
+// (look-ahead).  FP32 steps whose trailing tiles all fit the grid at once take (B)
+// and (C) in one phase (whole_step): at N = 732 300 us, 13 us per block step,
+// against 365 us in two phases (437 us with the diagonal block by columns across
+// the CTA and 8-row pieces as well).  GB300 retires about two FP64 FMAs per SM per clock, so the
 // pieces are small enough to spread each step over every SM, and the chain
 // from one diagonal block to the next is kept short: the block factor takes
 // one barrier per column and maps the threads onto the elements each column
@@ -271,6 +274,7 @@ template <typename T>
 struct CholSmem {
   T blk[NBK][NBK + 1];   // diagonal block, or the rows of a piece
   T aux[NBK][NBK + 1];   // a diagonal factor, panel rows, or an inverse
+  T lkk[sizeof(T) == 4 ? NBK : 1][NBK + 1];   // the step's diagonal factor (whole steps)
   T pinv[NBK], prs[NBK], dgl[NBK];   // per pivot d: 1 / d, 1 / sqrt(d), sqrt(d)
   unsigned char ti[NTRI], tj[NTRI];       // e -> (i, j), j <= i, e = i (i + 1) / 2 + j
   int flag;
@@ -391,6 +395,127 @@ __device__ void store_block(const CholSmem<T>& S, T* __restrict__ l, int N, int 
   }
 }
 
+// a L^T = x by substitution, in place, for NR rows per warp (a lane per column)
+template <int NR>
+__device__ __forceinline__ void solve_rows(const float (*l)[NBK + 1], float (&a)[NR]) {
+  const int lane = threadIdx.x & 31;
+  const float rd = 1.f / l[lane][lane];
+  float x[NR];
+#pragma unroll
+  for (int q = 0; q < NR; ++q) x[q] = 0.f;
+#pragma unroll 4
+  for (int t = 0; t < NBK; ++t) {
+    const float lt = l[lane][t];
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+      if (lane == t) x[q] = a[q] * rd;
+      const float xt = __shfl_sync(0xffffffffu, x[q], t);
+      if (lane > t) a[q] -= xt * lt;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NR; ++q) a[q] = x[q];
+}
+
+// Step k in one phase (FP32): a trailing tile's CTA solves the panel rows of
+// both of its block rows itself, in registers, so that no CTA waits for another's
+// panel within the step.  The columns of block k stay as they are until every
+// CTA has read them: the tile of the first trailing column keeps its solved rows
+// transposed in the unused upper triangle, and copy_panels moves them at the end.
+__device__ __forceinline__ void whole_step(CholSmem<float>& S, float* __restrict__ Lf, int* __restrict__ status,
+                                           int N, int B, int kb) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int r0 = kb + NBK, rem = N - r0, TB = (rem + NBK - 1) / NBK, nother = TB * (TB + 1) / 2 - 1;
+  for (int item = blockIdx.x; item < B + B * nother; item += gridDim.x) {
+    __syncthreads();
+    const bool ahead = item < B;   // the next diagonal block
+    const int ccd = ahead ? item : (item - B) / nother;
+    int t = ahead ? 0 : 1 + (item - B) % nother, bi = 0;
+    while (t > bi) { t -= bi + 1; ++bi; }
+    const int i0 = r0 + bi * NBK, j0 = r0 + t * NBK;
+    float* l = Lf + (int64_t)ccd * N * N;
+    float old[4], p[8], d[4];   // every load of the tile in flight at once
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = warp + 8 * q, gi = i0 + i, gj = j0 + i;
+      p[q] = gi < N ? __ldcg(l + (int64_t)gi * N + kb + lane) : 0.f;
+      p[4 + q] = gj < N ? __ldcg(l + (int64_t)gj * N + kb + lane) : 0.f;
+      old[q] = gi < N && j0 + lane <= gi ? __ldcg(l + (int64_t)gi * N + j0 + lane) : (gi == j0 + lane ? 1.f : 0.f);
+      d[q] = lane <= i ? __ldcg(l + (int64_t)(kb + i) * N + kb + lane) : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) S.lkk[warp + 8 * q][lane] = d[q];
+    __syncthreads();
+    if (ahead) {
+      float x[4] = {p[0], p[1], p[2], p[3]};
+      solve_rows(S.lkk, x);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) p[q] = p[4 + q] = x[q];
+    } else {
+      solve_rows(S.lkk, p);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      S.blk[warp + 8 * q][lane] = p[q];
+      S.aux[warp + 8 * q][lane] = p[4 + q];
+    }
+    __syncthreads();
+    if (t == 0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (i0 + lane < N) l[(int64_t)(kb + warp + 8 * q) * N + i0 + lane] = S.blk[lane][warp + 8 * q];
+    }
+    float s0[4] = {}, s1[4] = {};
+#pragma unroll 8
+    for (int c = 0; c < NBK; c += 2) {
+      const float a0 = S.aux[lane][c], a1 = S.aux[lane][c + 1];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        s0[q] += S.blk[warp + 8 * q][c] * a0;
+        s1[q] += S.blk[warp + 8 * q][c + 1] * a1;
+      }
+    }
+    if (ahead) {
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < 4; ++q) S.blk[warp + 8 * q][lane] = old[q] - (s0[q] + s1[q]);   // identity past N
+      __syncthreads();
+      factor_block(S, status + ccd);
+      store_block(S, l, N, r0, min(NBK, rem));
+      continue;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int gi = i0 + warp + 8 * q, gj = j0 + lane;
+      if (gi < N && gj <= gi) l[(int64_t)gi * N + gj] = old[q] - (s0[q] + s1[q]);
+    }
+  }
+}
+
+// The solved panels of the whole steps (blocks k >= k0), from the upper triangle
+// to the lower one.
+__device__ __forceinline__ void copy_panels(CholSmem<float>& S, float* __restrict__ Lf, int N, int B, int nblk, int k0) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m = nblk - 1 - k0, per = m * (m + 1) / 2;
+  for (int item = blockIdx.x; item < B * per; item += gridDim.x) {
+    int t = item % per, j = 1;   // j block rows below block nblk - 1 - j
+    while (t >= j) t -= j++;
+    const int kb = (nblk - 1 - j) * NBK, p0 = kb + (t + 1) * NBK;
+    float* l = Lf + (int64_t)(item / per) * N * N;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = warp + 8 * q;
+      S.blk[c][lane] = p0 + lane < N ? __ldcg(l + (int64_t)(kb + c) * N + p0 + lane) : 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = warp + 8 * q;
+      if (p0 + i < N) l[(int64_t)(p0 + i) * N + kb + lane] = S.blk[lane][i];
+    }
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_chol_coop(T* __restrict__ Lf, T* __restrict__ dinv, int* __restrict__ status, int N, int B,
@@ -416,11 +541,22 @@ k_chol_coop(T* __restrict__ Lf, T* __restrict__ dinv, int* __restrict__ status, 
     store_block(S, Lf + ccd * NN, N, 0, min(NBK, N));
   }
   bool ok = grid_sync_bounded(bar, &S.flag, spin_limit);
+  int k0 = nblk;   // first of the whole steps (the trailing tiles only get fewer)
   for (int k = 0; ok && k < nblk; ++k) {
     const int kb = k * NBK, nb = min(NBK, N - kb), rem = N - kb - nb;
     if (rem <= 0) break;   // uniform: the last block has no panel
     const int TB = (rem + NBK - 1) / NBK;   // block rows below the diagonal block
     const int r0 = kb + nb;
+    if constexpr (sizeof(T) == 4) {
+      // a tile for every CTA at most: one phase and one barrier for the step (with
+      // more tiles each further round would solve its panel rows again)
+      if (B * (TB * (TB + 1) / 2) <= G) {
+        k0 = min(k0, k);
+        whole_step(S, Lf, status, N, B, kb);
+        ok = grid_sync_bounded(bar, &S.flag, spin_limit);
+        continue;
+      }
+    }
     // (B) panel pieces: X L_kk^T = A, warp = row of the piece, lane = column
     for (int item = blockIdx.x; item < B * TB * (NBK / PRW); item += G) {
       const int ccd = item / (TB * (NBK / PRW)), pc = item % (TB * (NBK / PRW));
@@ -531,6 +667,9 @@ k_chol_coop(T* __restrict__ Lf, T* __restrict__ dinv, int* __restrict__ status, 
       }
     }
     ok = grid_sync_bounded(bar, &S.flag, spin_limit);
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (ok && k0 < nblk) copy_panels(S, Lf, N, B, nblk, k0);
   }
   // inverses of the diagonal factors for the substitutions, all at once
   for (int item = blockIdx.x; ok && item < B * nblk; item += G) {
@@ -756,8 +895,9 @@ __global__ void k_kernel_at(const double* __restrict__ theta, double* __restrict
 // and factors it (FACTOR) or fetches its factor, substitutes, and adds to or
 // sets theta_off.  The cooperative kernels hand every 32-block through L2 and
 // take two more launches per step (cutout of 160 x 192, N = 78: 51 + 19 us in
-// seven launches, 45 + 15 us in two, and the call 188 -> 138 us).  Above the limit one SM's multiply-adds and the FP64 scaling
-// of N^2 / 2 entries cost more than the hand-overs.
+// seven launches, 45 + 15 us in two, and the call 188 -> 138 us).  Above the
+// limit one SM's multiply-adds and the FP64 scaling of N^2 / 2 entries cost more
+// than the hand-overs.
 constexpr int kSmallN = 160, kSmallThreads = 512, kSmallRows = kSmallN / 32;
 
 struct SmallArgs {
