@@ -134,12 +134,13 @@ def direct_phase_bytes(H, W, L, DK, DB, refine=1):
     against the images."""
     px = H * W
     return {
-        # sky sums (R, S, bad), masks and R_m (R, S, bad in; good, R_m out), two
-        # erosion passes (1 B in, 1 B out each), edge lists (M_fit twice)
-        "prep": px * (9 + 14 + 4 + 2),
-        "contract_kk": px * 9,
-        "contract_rk": px * 8 * refine,
-        "apply": px * (13 * refine + 12),
+        # sky sums (R, S, bad), R_m and the masks (R, S, bad in; R_m and good bits
+        # out), erosion (bits in and out) and edge lists (bits twice)
+        "prep": int(px * (9 + 13 + 5 / 8)),
+        "contract_kk": int(px * (8 + 1 / 8)),
+        # residual and its sums in one kernel: R, S and the fit bits
+        "contract_rk": int(px * (8 + 1 / 8)) * refine,
+        "apply": px * 12,
     }
 
 

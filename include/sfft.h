@@ -281,8 +281,9 @@ enum {
   SFFT_PROF_SOLVE = 6,       /* Cholesky, triangular solves (and, mixed with no refinement steps,
                                 one FP64 residual step) */
   SFFT_PROF_APPLY = 7,       /* convolve-and-subtract and refinement residual */
-  SFFT_PROF_LAG_DFT = 8,     /* image space: mask-edge sums and their chains; tensor-core KK paths: lags u_x over the k-slot products and the
-                                exact slot-0 sums */
+  SFFT_PROF_LAG_DFT = 8,     /* image space: mask-edge sums and their chains; tensor-core KK
+                                paths: lags u_x over the k-slot products and the exact
+                                slot-0 sums */
   SFFT_PROF_N = 9
 };
 sfft_status_t sfft_profile_enable(sfft_plan_t plan, int32_t enable);

@@ -511,7 +511,7 @@ static sfft_status_t plan_impl(const sfft_desc_t* desc, void* cuda_stream, sfft_
   // Image-space sums, unless the caller chooses a spectral engine or its tile
   // shape: 1468 multiply-adds per pixel at L = 11, D_K = 2 in place of 221 row
   // FFTs and a contraction of 6.4e11 flop per 2048 x 4096 CCD, 8.51 against
-  // 2.28 ms for its whole subtraction.  The line would lie at masks: their
+  // 1.79 ms for its whole subtraction.  The line would lie at masks: their
   // edges cost 7 ns each (y, L = 11, D_K = 2), so at 2 % to 30 % masked sky
   // frames (10^4 - 10^5 edges) the assembly takes 0.9 ms against 6.9, and with
   // 0.3 % isolated bad pixels 3.7; only a grid of bad pixels every 12 px

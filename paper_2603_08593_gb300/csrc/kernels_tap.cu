@@ -42,6 +42,10 @@ __host__ __device__ constexpr size_t tap_smem(int wt, int tw) {
 // One CTA: a tile of 32 rows x tw columns and every nsplit-th task of the
 // table, taken in order by its warps.  Partial sums go to
 // part[ccd][tile][nout_tot]; k_tap_reduce adds the tiles in FP64.
+// One 4096 x 2048 CCD, L = 11, D_K = 2: 497 us = 50 TFLOP/s, 0.65 of the FP32
+// FMA peak (the row FFTs of the 221 products and their contraction took 6.0 ms);
+// copies of the tile through registers took 638 us, R stored as
+// operand pairs (two CTAs of six warps instead of three of four) 572 us.
 template <typename T, int NT, int DK, int MODE>
 __global__ void __launch_bounds__(kTapWarps * 32, sizeof(T) == 4 ? 3 : 2)
 k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const unsigned* __restrict__ mfitw,
@@ -191,8 +195,10 @@ k_tap_reduce(const T* __restrict__ part, const int* __restrict__ dst, TapDst d, 
 // keeps kGramP pairs x all monomials in registers.  The points of the next
 // batch are copied (cp.async) while this one is summed, and the list is read
 // two batches ahead; without it the gathers' latency took 60 % of the warps'
-// time.  Slot g of U takes batches g, g + U, ..., at least kGramMin<T> points, and
-// writes hp[ccd][slot][pair][MP]; a short list uses few slots.  The x-edge
+// time.  What bounds it now are the issue slots (44 %) and shared-memory reads of
+// the patches: 96 us for a 4096 x 2048 CCD with saturated stars and two dead
+// columns.  Slot g of U takes batches g, g + U, ..., at least kGramMin<T> points,
+// and writes hp[ccd][slot][pair][MP]; a short list uses few slots.  The x-edge
 // blocks, whose lists are the longer, come first.
 constexpr int kGramP = 5;
 constexpr int kGramPts = 32;
@@ -200,8 +206,8 @@ constexpr int kGramThreads = 256;
 constexpr int kGramPatch = 125;   // L^2 <= 121 values, then 1 (single offsets) and padding to an odd pitch
 // least points of a slot: FP64 multiply-adds are 64 times slower than FP32
 // ones, so there a short list spreads over more slots (one 512 x 512 pair,
-// L = 7, D_K = 1: 1.6 ms with 256 points, 1.1 ms with 32).  FP32: a single CCD
-// with 0.3 % of its pixels masked has too few points to fill the chip at 256
+// L = 7, D_K = 1: 1.6 ms with 256 points, 1.1 ms with 32).  FP32: the
+// edges of a single CCD's stars and columns fill too few slots of 256 points
 // (4096 x 2048, L = 11, D_K = 2: 104 us with 256, 96 us with 128)
 template <typename T> constexpr int kGramMin = sizeof(T) == 4 ? 128 : kGramPts;
 
@@ -315,7 +321,7 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
     if (b + U < nb) stage(b + U, s ^ 1);
     const int m = min(kGramPts, n - b * kGramPts);
     // two points at a time: the second's reads pass the first's multiply-adds
-    // (ten CCDs 983 -> 965 us, L = 9, D_K = 1 94.7 -> 87.5 us)
+    // (ten CCDs 983 -> 965 us, five of L = 9, D_K = 1 94.7 -> 87.5 us)
 #pragma unroll 2
     for (int pt = 0; pt < m; ++pt) {
       T mv[MP];
@@ -389,6 +395,8 @@ __host__ __device__ inline int xpair_single(int L, int ix) {
 // into shared memory; a thread per power of yt then walks the x
 // chain at u_y = w, and a thread per (u_x, power of xt) the y chains, in FP64.
 // shift(h) acts within one power: new_k = sum_i binom(k, i) h^(k - i) old_i.
+// The chain's FP64 additions, one after another, bound it (23 us at L = 11,
+// D_K = 2; about the same for ten CCDs).
 template <int DEG>
 __device__ __forceinline__ void shift_poly(double (&f)[DEG + 1], int deg, double h) {
   // repeated synthetic division: f(x) coefficients' dual, highest first

@@ -64,10 +64,10 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // are the tile's 32 rows, each lane walks its row with the NT taps in a
 // sliding register window and keeps (rows of powers) x (taps) sums in
 // registers, so a shared-memory value read once feeds 2 x NT multiply-adds
-// per row of powers.  What bounds it is the FP32 FMA pipe (44 packed FMAs per
-// pixel, centre and tap row at D_K = 2); lanes as rows need no reduction
-// until the row's end, and the odd pitch keeps their reads free of bank
-// conflicts.
+// per row of powers.  What bounds it is the FP32 FMA pipe (55 multiply-adds per
+// pixel, centre and tap row at D_K = 2, packed in pairs); lanes as rows need no
+// reduction until the row's end, and the odd pitch keeps their reads free of
+// bank conflicts.
 enum { TAP_CS = 0, TAP_C = 1, TAP_S = 2, TAP_M = 3, TAP_MOM = 4 };
 enum { TAP_FIT_EDGE = 0, TAP_FIT_ALL = 1 };
 
