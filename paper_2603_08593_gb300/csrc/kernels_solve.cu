@@ -843,8 +843,8 @@ k_chol_solve(const T* __restrict__ Lf, const T* __restrict__ dinv, const double*
 // the status word's code: a wait that gave up leaves the normal matrix or the
 // factor partly unwritten, which then also looks singular or non-finite: the
 // time-out is the cause and is reported first
-__device__ __forceinline__ int32_t info_code(int s) {
-  return (s & 4) ? SFFT_ERR_TIMEOUT : ((s & 2) ? SFFT_ERR_NONFINITE : ((s & 1) ? SFFT_ERR_SINGULAR : SFFT_OK));
+__device__ __forceinline__ void set_info(int32_t* info, int c, int s) {
+  info[c] = (s & 4) ? SFFT_ERR_TIMEOUT : ((s & 2) ? SFFT_ERR_NONFINITE : ((s & 1) ? SFFT_ERR_SINGULAR : SFFT_OK));
 }
 
 // background between offset and original units: B = B' + s_S - s_R sum_j K_j
@@ -868,7 +868,7 @@ k_theta_units(const double* __restrict__ src, double* __restrict__ dst, const do
     }
     if (lane == 0) d[NKK + q] = s[NKK + q] + (q == 0 ? sg * sS : 0.0) - sg * sR * ks;
   }
-  if (info && threadIdx.x == 0) info[ccd] = info_code(status[ccd]);
+  if (info && threadIdx.x == 0) set_info(info, ccd, status[ccd]);
 }
 
 __global__ void k_kernel_at(const double* __restrict__ theta, double* __restrict__ K, int L, int DK, int NK, int NB,
