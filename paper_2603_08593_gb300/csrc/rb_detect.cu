@@ -23,6 +23,7 @@ namespace {
 
 constexpr int kMargin = 15, kHalf = 15, kNms = 2, kMaxR = 15;
 constexpr int kStatBlocks = 608, kStatPasses = 4;   // four CTAs per SM
+constexpr int kClipWords = 8;   // words of a row in flight per warp of a pass
 constexpr double kClipNsig = 3.0, kClipVarShare = 0.97334;
 
 struct Taps {
@@ -99,64 +100,64 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
   int n = 0;
   float s1 = 0.f, e1 = 0.f, s2 = 0.f, e2 = 0.f;
   double b1 = 0.0, b2 = 0.0;
-  constexpr int U = 8;   // words in flight per warp
-  for (int y = blockIdx.x; y < H; y += gridDim.x) {
+  constexpr int U = kClipWords;
+  const int ng = (nw + U - 1) / U, nit = ((H - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) * ng;
+  for (int it = warp; it < nit; it += 8) {   // the CTA's (row, word group) pairs
+    const int y = blockIdx.x + it / ng * gridDim.x, w0 = it % ng * U;
     const bool row_in = y >= kMargin && y < H - kMargin;
     if (!FIRST && !row_in) continue;
-    for (int w0 = warp * U; w0 < nw; w0 += 8 * U) {
-      float v[U];
-      unsigned m[U];
+    float v[U];
+    unsigned m[U];
 #pragma unroll
-      for (int k = 0; k < U; ++k) {
-        const int x = (w0 + k) * 32 + lane;
-        const bool in = x < W;
-        v[k] = in ? Db[(int64_t)y * W + x] : 0.f;
-        if (FIRST) m[k] = in && bb ? bb[(int64_t)y * W + x] : 0u;
-        else m[k] = w0 + k < nw ? gw[(int64_t)y * nw + w0 + k] : 0u;
-      }
-      unsigned wide = 0;   // words whose square or its error leaves the range of a float
+    for (int k = 0; k < U; ++k) {
+      const int x = (w0 + k) * 32 + lane;
+      const bool in = x < W;
+      v[k] = in ? Db[(int64_t)y * W + x] : 0.f;
+      if (FIRST) m[k] = in && bb ? bb[(int64_t)y * W + x] : 0u;
+      else m[k] = w0 + k < nw ? gw[(int64_t)y * nw + w0 + k] : 0u;
+    }
+    unsigned wide = 0;   // words whose square or its error leaves the range of a float
 #pragma unroll
-      for (int k = 0; k < U; ++k) {
-        const int x = (w0 + k) * 32 + lane;
-        bool ok;
-        if (FIRST) {
-          const bool isbad = m[k] != 0u;
-          ok = x < W && !isbad && isfinite(v[k]);
-          const unsigned g = __ballot_sync(0xffffffffu, ok), q = __ballot_sync(0xffffffffu, isbad);
-          if (lane == 0 && w0 + k < nw) {
-            gw[(int64_t)y * nw + w0 + k] = g;
-            if (bb) bw[(int64_t)y * nw + w0 + k] = q;
-          }
-        } else {
-          ok = ((m[k] >> lane) & 1u) && v[k] >= lo && v[k] <= hi;
+    for (int k = 0; k < U; ++k) {
+      const int x = (w0 + k) * 32 + lane;
+      bool ok;
+      if (FIRST) {
+        const bool isbad = m[k] != 0u;
+        ok = x < W && !isbad && isfinite(v[k]);
+        const unsigned g = __ballot_sync(0xffffffffu, ok), q = __ballot_sync(0xffffffffu, isbad);
+        if (lane == 0 && w0 + k < nw) {
+          gw[(int64_t)y * nw + w0 + k] = g;
+          if (bb) bw[(int64_t)y * nw + w0 + k] = q;
         }
-        ok = ok && row_in && x >= kMargin && x < W - kMargin;
-        n += ok;
-        // a pixel that does not count adds zeros, which change no sum
-        float dl = 0.f, t;
-        float d = FIRST ? v[k] : two_sum(v[k], -shift, dl);
-        const float ad = fabsf(d);
-        if (ok && (ad > 1e18f || (ad < 1e-12f && ad > 0.f))) wide |= 1u << k;
-        ok = ok && !(wide >> k & 1u);
-        d = ok ? d : 0.f;
-        dl = ok ? dl : 0.f;
-        s1 = two_sum(s1, d, t);
-        e1 += t + dl;
-        const float p = __fmul_rn(d, d), pe = __fmaf_rn(2.f * d, dl, __fmaf_rn(d, d, -p));
-        s2 = two_sum(s2, p, t);
-        e2 += t + pe;
+      } else {
+        ok = ((m[k] >> lane) & 1u) && v[k] >= lo && v[k] <= hi;
       }
-      if (wide) {
+      ok = ok && row_in && x >= kMargin && x < W - kMargin;
+      n += ok;
+      // a pixel that does not count adds zeros, which change no sum
+      float dl = 0.f, t;
+      float d = FIRST ? v[k] : two_sum(v[k], -shift, dl);
+      const float ad = fabsf(d);
+      if (ok && (ad > 1e18f || (ad < 1e-12f && ad > 0.f))) wide |= 1u << k;
+      ok = ok && !(wide >> k & 1u);
+      d = ok ? d : 0.f;
+      dl = ok ? dl : 0.f;
+      s1 = two_sum(s1, d, t);
+      e1 += t + dl;
+      const float p = __fmul_rn(d, d), pe = __fmaf_rn(2.f * d, dl, __fmaf_rn(d, d, -p));
+      s2 = two_sum(s2, p, t);
+      e2 += t + pe;
+    }
+    if (wide) {
 #pragma unroll
-        for (int k = 0; k < U; ++k)
-          if (wide >> k & 1u) {
-            float dl = 0.f;
-            const float d = FIRST ? v[k] : two_sum(v[k], -shift, dl);
-            const double dd = (double)d + (double)dl;
-            b1 += dd;
-            b2 += dd * dd;
-          }
-      }
+      for (int k = 0; k < U; ++k)
+        if (wide >> k & 1u) {
+          float dl = 0.f;
+          const float d = FIRST ? v[k] : two_sum(v[k], -shift, dl);
+          const double dd = (double)d + (double)dl;
+          b1 += dd;
+          b2 += dd * dd;
+        }
     }
   }
   __shared__ double red[3][8];
@@ -576,7 +577,10 @@ extern "C" sfft_status_t rb_detect(int32_t H, int32_t W, int32_t batch, const fl
   }
   cudaError_t z = cudaMemsetAsync(counter, 0, L.zero_bytes, s);
   if (z != cudaSuccess) return fail(z, "rb_detect");
-  const dim3 gs(std::min(kStatBlocks, H), batch);
+  // eight words of a row per warp at least: a narrow image's rows share CTAs
+  // (with a CTA per row, one of its eight warps had work at 200 columns)
+  const int groups = (L.words + kClipWords - 1) / kClipWords;
+  const dim3 gs((int)std::min<int64_t>(std::min(kStatBlocks, H), ((int64_t)H * groups + 7) / 8), batch);
   k_clip_pass<true><<<gs, 256, 0, s>>>(H, W, D, bad, goodw, badw, part, stats, counter, 0, taps);
   for (int p = 1; p < kStatPasses; ++p)
     k_clip_pass<false><<<gs, 256, 0, s>>>(H, W, D, bad, goodw, badw, part, stats, counter, p, taps);
