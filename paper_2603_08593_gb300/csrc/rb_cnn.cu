@@ -75,26 +75,13 @@ void abi_to_master(const float* a, std::vector<float>& m) {
   m[OB5] = b5[0];
 }
 
-// the inverse of abi_to_master as an index map
-std::vector<int> abi_map() {
-  std::vector<float> a(RB_NPARAM), m;
-  for (int i = 0; i < RB_NPARAM; ++i) a[i] = (float)(i + 1);   // exact; 0 marks padding
-  abi_to_master(a.data(), m);
-  std::vector<int> map(RB_NPARAM);
-  for (size_t i = 0; i < m.size(); ++i)
-    if (m[i] > 0.f) map[(size_t)m[i] - 1] = (int)i;
-  return map;
-}
-
-
 }  // namespace
 
 struct rb_model_s {
   int max_batch = 0;
   int64_t step = 0;
   float *params = nullptr, *grads = nullptr, *adam_m = nullptr, *adam_v = nullptr;
-  int* map = nullptr;                          // C-ABI index -> master index
-  float* abi = nullptr;                        // a vector in C-ABI order
+  ParamReader reader;                          // the vectors in C-ABI order
   bf16* wbf = nullptr;                         // bf16 copy of the master vector
   // activations / scratch for max_batch stamps
   bf16 *xn = nullptr, *a1 = nullptr, *a2 = nullptr, *a3 = nullptr, *dzb = nullptr, *dz4 = nullptr;
@@ -111,7 +98,8 @@ struct rb_model_s {
 namespace {
 
 void free_model(rb_model_s* m) {
-  void* ptrs[] = {m->map, m->abi, m->params, m->grads, m->adam_m, m->adam_v, m->wbf, m->xn,  m->a1,   m->a2,   m->a3,
+  m->reader.destroy();
+  void* ptrs[] = {m->params, m->grads, m->adam_m, m->adam_v, m->wbf, m->xn,  m->a1,   m->a2,   m->a3,
                   m->dzb,    m->dz4,   m->z1,     m->z2,     m->z3,  m->z4, m->logit, m->dz5,  m->da,
                   m->part,   m->i1,    m->i2,     m->i3,  m->img1, m->img2, m->img3, m->p2,   m->p3,
                   m->err};
@@ -237,7 +225,7 @@ extern "C" sfft_status_t rb_create(const int32_t* desc, rb_model_t* out) {
   if (!m) return SFFT_ERR_NOMEM;
   const int B = desc[0];
   m->max_batch = B;
-  bool ok = alloc(&m->map, RB_NPARAM) && alloc(&m->abi, RB_NPARAM) && alloc(&m->params, NMASTER) && alloc(&m->grads, NMASTER) && alloc(&m->adam_m, NMASTER) &&
+  bool ok = m->reader.create(RB_NPARAM, abi_to_master) && alloc(&m->params, NMASTER) && alloc(&m->grads, NMASTER) && alloc(&m->adam_m, NMASTER) &&
             alloc(&m->adam_v, NMASTER) && alloc(&m->wbf, NMASTER) && alloc(&m->xn, (size_t)B * rbtc::kXnStride) &&
             alloc(&m->a1, (size_t)B * PIX2 * C1) && alloc(&m->a2, (size_t)B * PIX3 * C2) &&
             alloc(&m->a3, (size_t)B * PIX4 * C3) &&
@@ -268,9 +256,7 @@ extern "C" sfft_status_t rb_create(const int32_t* desc, rb_model_t* out) {
   }
   std::vector<float> master;
   abi_to_master(abi.data(), master);
-  const std::vector<int> map = abi_map();
   cudaError_t e = cudaMemcpy(m->params, master.data(), sizeof(float) * NMASTER, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->map, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(m->adam_m, 0, sizeof(float) * NMASTER);
   if (e == cudaSuccess) e = cudaMemset(m->adam_v, 0, sizeof(float) * NMASTER);
   if (e == cudaSuccess) e = cudaMemset(m->grads, 0, sizeof(float) * NMASTER);
@@ -311,12 +297,7 @@ extern "C" sfft_status_t rb_set_weights(rb_model_t m, const void* host_buf, size
 
 static sfft_status_t get_vec(rb_model_s* m, const float* dev, void* host_buf, size_t bytes, const char* where) {
   if (!dev || !host_buf || bytes != sizeof(float) * RB_NPARAM) return SFFT_ERR_ARG;
-  cudaError_t e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) {
-    k_gather<<<grid1(RB_NPARAM), 256>>>(dev, m->map, RB_NPARAM, m->abi);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaMemcpy(host_buf, m->abi, sizeof(float) * RB_NPARAM, cudaMemcpyDeviceToHost);
+  const cudaError_t e = m->reader.read(dev, host_buf);
   return e == cudaSuccess ? SFFT_OK : fail(e, where);
 }
 

@@ -9,6 +9,8 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <mutex>
+#include <vector>
 
 #include "common.cuh"
 #include "rb_gemm.cuh"
@@ -412,17 +414,61 @@ __global__ void k_to_bf16(const float* __restrict__ x, int64_t n, bf16* __restri
     y[e] = __float2bfloat16(x[e]);
 }
 
-// A parameter vector in the C ABI's order, gathered on the device: converting
-// it on the host walked half a megabyte with strides after the copy (a
-// 256-stamp backward pass with its gradients: 556 us, 280 of them on the host)
-__global__ void k_gather(const float* __restrict__ x, const int* __restrict__ map, int n, float* __restrict__ y) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) y[e] = x[map[e]];
-}
-
 int grid1(int64_t n) {
   int64_t g = (n + 255) / 256;
   return (int)(g > 4096 ? 4096 : (g < 1 ? 1 : g));
 }
+
+__global__ void k_gather(const float* __restrict__ x, const int* __restrict__ map, int n, float* __restrict__ y) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) y[e] = x[map[e]];
+}
+
+// A model's parameter vectors read in the C ABI's order, gathered on the device:
+// converting them on the host walked half a megabyte with strides after the copy
+// (a 256-stamp backward pass with its gradients: 556 us, 280 of them on the
+// host).  All readers of a model share the buffer of the gathered vector, from
+// any thread, so one holds the lock from its gather to the end of its copy.
+struct ParamReader {
+  int device = 0, n = 0;
+  int* map = nullptr;     // C-ABI index -> master index
+  float* abi = nullptr;   // the gathered vector
+  std::mutex mu;
+
+  // to_master: the model's conversion from the C ABI's order, inverted here
+  bool create(int n_param, void (*to_master)(const float*, std::vector<float>&)) {
+    n = n_param;
+    std::vector<float> a(n), m;
+    for (int i = 0; i < n; ++i) a[i] = (float)(i + 1);   // exact; 0 marks padding
+    to_master(a.data(), m);
+    std::vector<int> h(n);
+    for (size_t i = 0; i < m.size(); ++i)
+      if (m[i] > 0.f) h[(size_t)m[i] - 1] = (int)i;
+    return cudaGetDevice(&device) == cudaSuccess && cudaMalloc((void**)&map, sizeof(int) * n) == cudaSuccess &&
+           cudaMalloc((void**)&abi, sizeof(float) * n) == cudaSuccess &&
+           cudaMemcpy(map, h.data(), sizeof(int) * n, cudaMemcpyHostToDevice) == cudaSuccess;
+  }
+  void destroy() {
+    if (map) cudaFree(map);
+    if (abi) cudaFree(abi);
+    map = nullptr;
+    abi = nullptr;
+  }
+  // master (on the model's device, whatever device is current) -> host_buf
+  cudaError_t read(const float* master, void* host_buf) {
+    std::lock_guard<std::mutex> lk(mu);
+    int current = 0;
+    cudaError_t e = cudaGetDevice(&current);
+    if (e == cudaSuccess && current != device) e = cudaSetDevice(device);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) {
+      k_gather<<<grid1(n), 256>>>(master, map, n, abi);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(host_buf, abi, sizeof(float) * n, cudaMemcpyDeviceToHost);
+    if (current != device) cudaSetDevice(current);
+    return e;
+  }
+};
 
 // splitmix64 -> uniform in [0, 1)
 double hash_uniform(uint64_t seed, uint64_t i) {

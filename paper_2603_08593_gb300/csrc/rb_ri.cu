@@ -141,25 +141,13 @@ void abi_to_master(const float* a, std::vector<float>& m) {
   m[QB5] = a[o + F4];
 }
 
-// the inverse of abi_to_master as an index map
-std::vector<int> abi_map() {
-  std::vector<float> a(RBRI_NPARAM), m;
-  for (int i = 0; i < RBRI_NPARAM; ++i) a[i] = (float)(i + 1);   // exact; 0 marks padding
-  abi_to_master(a.data(), m);
-  std::vector<int> map(RBRI_NPARAM);
-  for (size_t i = 0; i < m.size(); ++i)
-    if (m[i] > 0.f) map[(size_t)m[i] - 1] = (int)i;
-  return map;
-}
-
 }  // namespace
 
 struct rbri_model_s {
   int max_batch = 0;
   int64_t step = 0;
   float *params = nullptr, *grads = nullptr, *adam_m = nullptr, *adam_v = nullptr;
-  int* map = nullptr;                          // C-ABI index -> master index
-  float* abi = nullptr;                        // a vector in C-ABI order
+  ParamReader reader;                          // the vectors in C-ABI order
   bf16* wbf = nullptr;
   // activations for 4 max_batch rotated stamps (FP32 pre-activations, BF16 activations)
   bf16 *xn = nullptr, *xr = nullptr, *a1 = nullptr, *ra = nullptr, *r1 = nullptr, *a2 = nullptr, *rc = nullptr,
@@ -172,7 +160,8 @@ struct rbri_model_s {
 namespace {
 
 void free_model(rbri_model_s* m) {
-  void* ptrs[] = {m->map, m->abi, m->params, m->grads, m->adam_m, m->adam_v, m->wbf, m->xn, m->xr, m->a1, m->ra, m->r1, m->a2,
+  m->reader.destroy();
+  void* ptrs[] = {m->params, m->grads, m->adam_m, m->adam_v, m->wbf, m->xn, m->xr, m->a1, m->ra, m->r1, m->a2,
                   m->rc, m->a3, m->fb, m->dz4, m->dzA, m->dzB, m->z1, m->za, m->zb, m->z2, m->zc, m->zd, m->f,
                   m->z4, m->logit, m->dz5, m->da, m->part, m->i1, m->i2, m->i3};
   for (void* p : ptrs)
@@ -338,7 +327,7 @@ extern "C" sfft_status_t rbri_create(const int32_t* desc, rbri_model_t* out) {
   const int B = desc[0];
   const size_t B4 = (size_t)NROT * B;
   m->max_batch = B;
-  bool ok = alloc(&m->map, RBRI_NPARAM) && alloc(&m->abi, RBRI_NPARAM) && alloc(&m->params, QMASTER) && alloc(&m->grads, QMASTER) && alloc(&m->adam_m, QMASTER) &&
+  bool ok = m->reader.create(RBRI_NPARAM, abi_to_master) && alloc(&m->params, QMASTER) && alloc(&m->grads, QMASTER) && alloc(&m->adam_m, QMASTER) &&
             alloc(&m->adam_v, QMASTER) && alloc(&m->wbf, QMASTER) && alloc(&m->xn, (size_t)B * PIX1 * 3) &&
             alloc(&m->xr, B4 * PIX1 * 3) && alloc(&m->a1, B4 * PIX2 * C1) && alloc(&m->ra, B4 * PIX2 * C1) &&
             alloc(&m->r1, B4 * PIX2 * C1) && alloc(&m->a2, B4 * PIX3 * C2) && alloc(&m->rc, B4 * PIX3 * C2) &&
@@ -367,9 +356,7 @@ extern "C" sfft_status_t rbri_create(const int32_t* desc, rbri_model_t* out) {
   fill(F4, F4, 1);
   std::vector<float> master;
   abi_to_master(abi.data(), master);
-  const std::vector<int> map = abi_map();
   cudaError_t e = cudaMemcpy(m->params, master.data(), sizeof(float) * QMASTER, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(m->map, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(m->adam_m, 0, sizeof(float) * QMASTER);
   if (e == cudaSuccess) e = cudaMemset(m->adam_v, 0, sizeof(float) * QMASTER);
   if (e == cudaSuccess) e = cudaMemset(m->grads, 0, sizeof(float) * QMASTER);
@@ -406,12 +393,7 @@ extern "C" sfft_status_t rbri_set_weights(rbri_model_t m, const void* host_buf, 
 
 static sfft_status_t get_vec(rbri_model_s* m, const float* dev, void* host_buf, size_t bytes, const char* where) {
   if (!host_buf || bytes != sizeof(float) * RBRI_NPARAM) return SFFT_ERR_ARG;
-  cudaError_t e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) {
-    k_gather<<<grid1(RBRI_NPARAM), 256>>>(dev, m->map, RBRI_NPARAM, m->abi);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaMemcpy(host_buf, m->abi, sizeof(float) * RBRI_NPARAM, cudaMemcpyDeviceToHost);
+  const cudaError_t e = m->reader.read(dev, host_buf);
   return e == cudaSuccess ? SFFT_OK : fail(e, where);
 }
 
