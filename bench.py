@@ -463,7 +463,7 @@ def time_fma_engine(dev, stream, R, S, bad, Hs, args, alu_peaks, steps=3):
 
 def time_exposure(dev, stream, pairs, args, dist, steps=3, warmup=2):
     """A whole exposure (len(pairs) CCD pairs of the 60-CCD recipe) per GPU in
-    one graph-captured sfft_subtract call, plan autotuned at creation."""
+    one graph-captured sfft_subtract call (image-space assembly)."""
     import torch
     from paper_2603_08593_gb300 import Plan
     B = len(pairs)
@@ -472,7 +472,7 @@ def time_exposure(dev, stream, pairs, args, dist, steps=3, warmup=2):
     bad = torch.from_numpy(np.stack([p["bad"] for p in pairs])).to(dev).contiguous()
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
     with torch.cuda.stream(stream):
-        plan = Plan(H, W, L, DK, DB, batch=B, prec="mixed", stream=stream, device=dev, graph=True, autotune=1)
+        plan = Plan(H, W, L, DK, DB, batch=B, prec="mixed", stream=stream, device=dev, graph=True)
         out = plan.subtract(R, S, bad, None, refine=REFINE)
         for _ in range(warmup - 1):
             plan.subtract(R, S, bad, None, refine=REFINE, out=out)
@@ -488,8 +488,6 @@ def time_exposure(dev, stream, pairs, args, dist, steps=3, warmup=2):
     world = int(os.environ.get("WORLD_SIZE", "1"))
     rec = {"value": world * B * steps / sec, "unit": UNIT, "ccd_pairs_per_gpu_per_step": B, "steps": steps,
            "warmup": warmup, "ms_per_step": 1e3 * sec / steps, "ms_per_ccd": 1e3 * sec / steps / B,
-           "tiles": {"d_batch": plan.tiles[0], "rows_per_cta": plan.tiles[1], "lag_parts": plan.tiles[2],
-                     "ccd_group": plan.ccd_group},
            "kk_engine": "image_space", "clocks": clk.summary(),
            "status": [int(v) for v in out["info"].cpu()],
            "masked_fraction": [float(p["masked_fraction"]) for p in pairs],
@@ -541,15 +539,16 @@ def run_gpu(args):
     bad = torch.from_numpy(np.stack([p["bad"] for p in pairs])).to(dev).contiguous()
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
     torch.cuda.synchronize(dev)
+    # an engine flag or a tile field selects the spectral assembly; only that one has tiles to tune
+    spectral = bool(args.d_batch or args.lag_parts or (args.prec == "mixed" and (
+        args.fma_contract or args.mma_sync_contract or args.pair_lane_contract)))
+    autotune = spectral and not args.no_autotune
     with torch.cuda.stream(stream):
         plan = Plan(Hs, W, L, DK, DB, batch=B, prec=args.prec, stream=stream, device=dev, d_batch=args.d_batch,
-                    graph=batched, autotune=0 if args.no_autotune else 1, lag_parts=args.lag_parts,
+                    graph=batched, autotune=int(autotune), lag_parts=args.lag_parts,
                     fma_contract=args.fma_contract, mma_sync_contract=args.mma_sync_contract,
                     pair_lane_contract=args.pair_lane_contract)
         tiles = plan.tiles
-        # an engine flag or a tile field selects the spectral assembly
-        spectral = bool(args.d_batch or args.lag_parts or (args.prec == "mixed" and (
-            args.fma_contract or args.mma_sync_contract or args.pair_lane_contract)))
         engine = plan.engine if spectral else "image_space"
         if batched:
             # per-phase times and launch counts from an eager profiled pass of the same plan
@@ -760,8 +759,8 @@ def run_gpu(args):
             "data": "synthetic",
             "config": {"workload": workload, "H": Hs, "W": W, "L": L, "DK": DK, "DB": DB, "prec": args.prec,
                        "refine": REFINE, "ccd_pairs_per_gpu_per_step": B, "parallelism": f"replicas x{world}",
-                       "cuda_graph": batched, "autotune": not args.no_autotune,
-                       "tiles": {"d_batch": tiles[0], "rows_per_cta": tiles[1], "lag_parts": tiles[2]},
+                       "cuda_graph": batched, "autotune": autotune,
+                       "tiles": {"d_batch": tiles[0], "rows_per_cta": tiles[1], "lag_parts": tiles[2]} if spectral else None,
                        "kk_engine": engine,
                        "l2": "256 MB buffer written between timed steps (L2 flushed)"},
             "roofline": roof, "cpu_baseline": cpu_base, "e2e": e2e, "gpu_launches": launches,

@@ -98,7 +98,8 @@ typedef struct {
   int32_t DK, DB;            /* kernel / background polynomial degrees */
   int32_t batch;             /* CCD pairs per call */
   int32_t prec;              /* sfft_prec_t */
-  int32_t autotune;          /* 1: time contraction tile shapes at plan time and keep the fastest */
+  int32_t autotune;          /* 1: time the spectral assembly's tile shapes at plan time; a spectral plan keeps
+                                the fastest, an image-space plan only reports it (sfft_plan_tiles) */
   /* tile shape of the spectral assembly; a non-zero value also selects that assembly */
   int32_t d_batch;           /* kernel-offset differences per product/FFT pass (0 = auto) */
   int32_t rows_per_cta;      /* rows of one contraction partial sum (0 = auto) */
@@ -112,8 +113,10 @@ typedef struct {
 
 /* Create a plan: validates the descriptor, builds offset/monomial/lag tables,
  * allocates the plan's small constant device tables (twiddles) and, with
- * autotune=1, times contraction tile shapes on synthetic data in its own
- * temporary buffers.  `cuda_stream` is a cudaStream_t (NULL = legacy default
+ * autotune=1, times the spectral assembly's tile shapes on synthetic data in
+ * its own temporary buffers (several GB of product spectra at 2048 x 4096).
+ * Where no candidate can run, a spectral plan fails with SFFT_ERR_CUDA and an
+ * image-space plan, which needs no tiles, is made all the same.  `cuda_stream` is a cudaStream_t (NULL = legacy default
  * stream).  On success *out owns the plan; release with sfft_plan_destroy. */
 sfft_status_t sfft_plan(const sfft_desc_t* desc, void* cuda_stream, sfft_plan_t* out);
 void          sfft_plan_destroy(sfft_plan_t plan);

@@ -480,11 +480,27 @@ static sfft_status_t plan_impl(const sfft_desc_t* desc, void* cuda_stream, sfft_
   // CCD with groups of 1 / 2 / 3 / 4 CCDs, but 5.2 ms with 9 (67 GB).
   const size_t budget = size_t(64) << 30, group_budget = size_t(32) << 30;
   const int d_batch_max = (int)std::max<size_t>(1, std::min<size_t>(budget / slab, (size_t)p->n_hd));
+  // Image-space sums, unless the caller chooses a spectral engine or its tile
+  // shape: 1468 multiply-adds per pixel at L = 11, D_K = 2 in place of 221 row
+  // FFTs and a contraction of 6.4e11 flop per 2048 x 4096 CCD, 8.51 against
+  // 1.79 ms for its whole subtraction.  The line would lie at masks: their
+  // edges cost 7 ns each (y, L = 11, D_K = 2), so at 2 % to 30 % masked sky
+  // frames (10^4 - 10^5 edges) the assembly takes 0.9 ms against 6.9, and with
+  // 0.3 % isolated bad pixels 3.7; only a grid of bad pixels every 12 px
+  // (10.6 ms) passes the spectra.  The size is not known to the host, and a
+  // caller with such masks sets a tile field.  An edge's list entry holds its
+  // pixel in 31 bits.
+  const bool spectral = d.d_batch > 0 || d.rows_per_cta > 0 || d.lag_parts > 0 || d.ccd_group > 0 ||
+                        (!p->fp64 && (d.flags & (SFFT_FLAG_FMA_CONTRACT | SFFT_FLAG_MMA_SYNC_CONTRACT |
+                                                 SFFT_FLAG_PAIR_LANE_CONTRACT)));
+  p->direct = !spectral && (int64_t)d.H * d.W < (int64_t(1) << 31);
   int tuned_db = 0, tuned_rows = 0, tuned_parts = 0;
   if (d.autotune && (d.d_batch == 0 || d.rows_per_cta == 0 || d.lag_parts == 0)) {
     const sfft_status_t ts = autotune_tiles(d, (cudaStream_t)cuda_stream, d_batch_max, &tuned_db, &tuned_rows,
                                             &tuned_parts, &p->tuned_ms);
-    if (ts != SFFT_OK) {
+    // an image-space plan has no use for the tiles but to report them: where no
+    // candidate fits, it keeps the defaults
+    if (ts != SFFT_OK && !p->direct) {
       delete p;
       return ts;
     }
@@ -508,20 +524,6 @@ static sfft_status_t plan_impl(const sfft_desc_t* desc, void* cuda_stream, sfft_
   p->dl = p->umma && !(d.flags & SFFT_FLAG_PAIR_LANE_CONTRACT) && p->M % 16 == 0 && d.H >= 32 &&
           p->d_batch >= std::min(p->n_hd, 96);
   p->tc_rows = d.H;
-  // Image-space sums, unless the caller chooses a spectral engine or its tile
-  // shape: 1468 multiply-adds per pixel at L = 11, D_K = 2 in place of 221 row
-  // FFTs and a contraction of 6.4e11 flop per 2048 x 4096 CCD, 8.51 against
-  // 1.79 ms for its whole subtraction.  The line would lie at masks: their
-  // edges cost 7 ns each (y, L = 11, D_K = 2), so at 2 % to 30 % masked sky
-  // frames (10^4 - 10^5 edges) the assembly takes 0.9 ms against 6.9, and with
-  // 0.3 % isolated bad pixels 3.7; only a grid of bad pixels every 12 px
-  // (10.6 ms) passes the spectra.  The size is not known to the host, and a
-  // caller with such masks sets a tile field.  An edge's list entry holds its
-  // pixel in 31 bits.
-  const bool spectral = d.d_batch > 0 || d.rows_per_cta > 0 || d.lag_parts > 0 || d.ccd_group > 0 ||
-                        (!p->fp64 && (d.flags & (SFFT_FLAG_FMA_CONTRACT | SFFT_FLAG_MMA_SYNC_CONTRACT |
-                                                 SFFT_FLAG_PAIR_LANE_CONTRACT)));
-  p->direct = !spectral && (int64_t)d.H * d.W < (int64_t(1) << 31);
   if (p->direct) build_tap_plan(p);
   build_layout(p);
   if (!p->direct) {
