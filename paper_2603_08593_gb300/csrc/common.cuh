@@ -118,6 +118,13 @@ __device__ __forceinline__ R warp_sum(R v) {
   return v;
 }
 
+// x + y = s + e exactly (Knuth's two-sum; no contraction)
+__device__ __forceinline__ float two_sum(float x, float y, float& e) {
+  const float s = __fadd_rn(x, y), t = __fsub_rn(s, x);
+  e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, t)), __fsub_rn(y, t));
+  return s;
+}
+
 // ------------------------------------------------------------------ index helpers
 // Monomials xt^a yt^b with a + b <= D ordered by degree n, then a descending:
 // index(a, b) = n (n + 1) / 2 + (n - a).

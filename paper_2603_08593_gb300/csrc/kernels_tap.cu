@@ -199,9 +199,14 @@ k_tap_reduce(const T* __restrict__ part, const int* __restrict__ dst, TapDst d, 
 // the patches: 96 us for a 4096 x 2048 CCD with saturated stars and two dead
 // columns.  Slot g of U takes batches g, g + U, ..., at least kGramMin<T> points,
 // and writes hp[ccd][slot][pair][MP]; a short list uses few slots.  The x-edge
-// blocks, whose lists are the longer, come first.
+// blocks, whose lists are the longer, come first.  The number of slots has a
+// limit, a slot's share of a long list has none: an FP32 sum covers kGramRun
+// points, then it is added to the slot's partials as an exact pair of floats
+// (10^4 equal products one after another lose up to 1.3e-4 of their sum, 256 at
+// most 4e-6).
 constexpr int kGramP = 5;
 constexpr int kGramPts = 32;
+constexpr int kGramRun = 256;
 constexpr int kGramThreads = 256;
 constexpr int kGramPatch = 125;   // L^2 <= 121 values, then 1 (single offsets) and padding to an odd pitch
 // least points of a slot: FP64 multiply-adds are 64 times slower than FP32
@@ -217,11 +222,17 @@ struct GramArgs {
   int gy, gx;              // most slots per list
   int64_t hp_stride;       // per CCD
   int64_t hx_off;          // x partials after the y ones
+  int64_t lo_off;          // the pairs' second floats (mixed path, lists of more than kGramRun points per slot)
   double xs, ys;           // 2 / (W - 1), 2 / (H - 1)
 };
 
 template <typename T>
 __device__ __forceinline__ int gram_slots(int n, int g) { return max(1, min(g, (n + kGramMin<T> - 1) / kGramMin<T>)); }
+// whether a slot's share of n points in U slots is summed in more than one run
+template <typename T>
+__device__ __forceinline__ bool gram_runs(int n, int U) {
+  return sizeof(T) == 4 && ((n + kGramPts - 1) / kGramPts + U - 1) / U * kGramPts > kGramRun;
+}
 
 template <typename T, int DE>
 __host__ __device__ constexpr size_t gram_smem() {
@@ -312,8 +323,12 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
   }
   __syncthreads();
   if (g < nb) stage(g, 0);
-  int s = 0;
-  for (int b = g; b < nb; b += U, s ^= 1) {
+  T* out = hp + ccd * a.hp_stride + (isx ? a.hx_off : 0) + (int64_t)g * np * MP;
+  const bool runs = gram_runs<T>(n, U);
+  bool first = true;
+  int s = 0, done = 0;
+  // an empty list takes one turn without points, for the zeros
+  for (int b = g; b < max(nb, 1); b += U, s ^= 1) {
     cp_async_wait_all();
     __syncthreads();
     unsigned e2 = 0;
@@ -340,18 +355,33 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
       }
     }
     if (warp == 0) ent[s][lane] = e2;
-  }
-  T* out = hp + ccd * a.hp_stride + (isx ? a.hx_off : 0) + (int64_t)g * np * MP;
+    done += kGramPts;
+    const bool end = b + U >= nb;
+    if (!end && !(runs && done % kGramRun == 0)) continue;
 #pragma unroll
-  for (int p = 0; p < kGramP; ++p) {
-    const int id = (blk * kGramP + p) * kGramThreads + tid;
-    if (id < np)
+    for (int p = 0; p < kGramP; ++p) {
+      const int id = (blk * kGramP + p) * kGramThreads + tid;
+      if (id < np)
 #pragma unroll
-      for (int k = 0; k < MP; ++k) out[(int64_t)id * MP + k] = v2_get(acc[p][k / 2], k & 1);
+        for (int k = 0; k < MP; ++k) {
+          T* o = out + (int64_t)id * MP + k;
+          T v = v2_get(acc[p][k / 2], k & 1);
+          if constexpr (sizeof(T) == 4)
+            if (runs) {
+              float e = 0.f;
+              if (!first) v = two_sum(*o, v, e);
+              o[a.lo_off] = first ? 0.f : o[a.lo_off] + e;
+            }
+          *o = v;
+        }
+#pragma unroll
+      for (int k = 0; k < MP / 2; ++k) v2_zero(acc[p][k]);
+    }
+    first = false;
   }
 }
 
-// the slots' partial sums, FP64 (FP32 in fours first on the mixed path)
+// the slots' partial sums: FP64, on the mixed path as pairs of floats
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_edge_reduce(const T* __restrict__ hp, GramArgs a, const int* __restrict__ cnt, int64_t cnt_stride, int H, int MP,
@@ -360,17 +390,25 @@ k_edge_reduce(const T* __restrict__ hp, GramArgs a, const int* __restrict__ cnt,
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= ny + nx) return;
   const bool isx = i >= ny;
-  const int U = gram_slots<T>(cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H], isx ? a.gx : a.gy);
+  const int n = cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H], U = gram_slots<T>(n, isx ? a.gx : a.gy);
   const int64_t st = isx ? nx : ny;
   const T* p = hp + ccd * a.hp_stride + (isx ? a.hx_off + i - ny : i);
   double s = 0.0;
-  int g = 0;
-#pragma unroll 2
-  for (; g + 3 < U; g += 4) {
-    const T v0 = p[g * st], v1 = p[(g + 1) * st], v2_ = p[(g + 2) * st], v3 = p[(g + 3) * st];
-    s += (double)((v0 + v1) + (v2_ + v3));
+  if constexpr (sizeof(T) == 4) {
+    const bool runs = gram_runs<T>(n, U);
+    float h = 0.f, l = 0.f;
+#pragma unroll 4
+    for (int g = 0; g < U; ++g) {
+      float e;
+      h = two_sum(h, p[g * st], e);
+      l += e;
+      if (runs) l += p[g * st + a.lo_off];
+    }
+    s = (double)h + (double)l;
+  } else {
+#pragma unroll 4
+    for (int g = 0; g < U; ++g) s += p[g * st];
   }
-  for (; g < U; ++g) s += (double)p[g * st];
   hs[(int64_t)ccd * (ny + nx) + i] = s;
 }
 
@@ -614,7 +652,7 @@ void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs
   const size_t B = p->d.batch;
   *part = p->elem * B * std::max((size_t)t.ntile * t.nout, (size_t)t.ntile_rhs * t.nout_rhs);
   const bool edge = t.mode == TAP_FIT_EDGE;
-  *hp = edge ? p->elem * B * ((size_t)t.gy * t.npy + (size_t)t.gx * t.npx) * t.MP : 0;
+  *hp = edge ? sizeof(double) * B * ((size_t)t.gy * t.npy + (size_t)t.gx * t.npx) * t.MP : 0;   // FP32: pairs
   *hs = edge ? sizeof(double) * B * (size_t)(t.npy + t.npx) * t.MP : 0;
   *list = edge ? 2 * sizeof(unsigned) * B * (size_t)edge_cap(p) : 0;
   *cnt = edge ? 2 * sizeof(int) * B * (size_t)(p->d.H + 1) : 0;
@@ -694,7 +732,8 @@ static cudaError_t edge_sums_T(const sfft_plan_s* p, void* ws) {
   a.gy = t.gy; a.gx = t.gx;
   a.xs = step_of(W); a.ys = step_of(H);
   a.hx_off = (int64_t)t.gy * t.npy * t.MP;
-  a.hp_stride = a.hx_off + (int64_t)t.gx * t.npx * t.MP;
+  a.lo_off = a.hx_off + (int64_t)t.gx * t.npx * t.MP;
+  a.hp_stride = sizeof(T) == 4 ? 2 * a.lo_off : a.lo_off;
   const unsigned* lx = ws_at<unsigned>(ws, p->elist);
   const int* cnt = ws_at<int>(ws, p->ecnt);
   const int64_t cap = edge_cap(p), cs = 2 * (int64_t)(H + 1);

@@ -61,12 +61,7 @@ struct DetectLayout {
   }
 };
 
-// x + y = s + e exactly (Knuth's two-sum; no contraction)
-__device__ __forceinline__ float two_sum(float x, float y, float& e) {
-  const float s = __fadd_rn(x, y), t = __fsub_rn(s, x);
-  e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, t)), __fsub_rn(y, t));
-  return s;
-}
+using sfft::two_sum;
 
 // the clipping rule of a pass
 __device__ __forceinline__ bool kept(float x, double mean, double thr) { return fabs((double)x - mean) <= thr; }
