@@ -382,8 +382,8 @@ extern "C" int64_t sfft_debug_live_allocations(void) { return (int64_t)g_live_al
 static void free_plan_device(sfft_plan_s* p) {
   plan_free(p->tap.d_tasks);
   plan_free(p->tap.d_dst);
-  plan_free(p->tap.d_pairs);
-  p->tap.d_tasks = nullptr; p->tap.d_dst = nullptr; p->tap.d_pairs = nullptr;
+  plan_free(p->tap.d_tiles);
+  p->tap.d_tasks = nullptr; p->tap.d_dst = nullptr; p->tap.d_tiles = nullptr;
   plan_free(p->d_dljobs);
   plan_free(p->d_dlpairs);
   plan_free(p->d_tcjobs);
@@ -483,13 +483,12 @@ static sfft_status_t plan_impl(const sfft_desc_t* desc, void* cuda_stream, sfft_
   // Image-space sums, unless the caller chooses a spectral engine or its tile
   // shape: 1468 multiply-adds per pixel at L = 11, D_K = 2 in place of 221 row
   // FFTs and a contraction of 6.4e11 flop per 2048 x 4096 CCD, 8.51 against
-  // 1.79 ms for its whole subtraction.  The line would lie at masks: their
-  // edges cost 7 ns each (y, L = 11, D_K = 2), so at 2 % to 30 % masked sky
-  // frames (10^4 - 10^5 edges) the assembly takes 0.9 ms against 6.9, and with
-  // 0.3 % isolated bad pixels 3.7; only a grid of bad pixels every 12 px
-  // (10.6 ms) passes the spectra.  The size is not known to the host, and a
-  // caller with such masks sets a tile field.  An edge's list entry holds its
-  // pixel in 31 bits.
+  // 1.72 ms for its whole subtraction.  Its time grows with the mask's edges,
+  // which the host does not know: 0.9 ms of assembly against 6.9 at the 10^4 -
+  // 10^5 edges of sky frames with 2 % to 30 % masked, 1.5 with 0.1 % isolated bad
+  // pixels, and 6.4 with one every 12 px each way, the densest that an erosion by
+  // 11 x 11 leaves.  Spectra were slower on every mask, kernel size and degree
+  // measured.  An edge's list entry holds its pixel in 31 bits.
   const bool spectral = d.d_batch > 0 || d.rows_per_cta > 0 || d.lag_parts > 0 || d.ccd_group > 0 ||
                         (!p->fp64 && (d.flags & (SFFT_FLAG_FMA_CONTRACT | SFFT_FLAG_MMA_SYNC_CONTRACT |
                                                  SFFT_FLAG_PAIR_LANE_CONTRACT)));
@@ -545,7 +544,7 @@ static sfft_status_t plan_impl(const sfft_desc_t* desc, void* cuda_stream, sfft_
   if (p->direct) {
     st = upload((void**)&p->tap.d_tasks, p->tap.tasks);
     if (st == SFFT_OK) st = upload((void**)&p->tap.d_dst, p->tap.dst);
-    if (st == SFFT_OK) st = upload((void**)&p->tap.d_pairs, p->tap.pairs);
+    if (st == SFFT_OK) st = upload((void**)&p->tap.d_tiles, p->tap.tiles);
   } else if (p->fp64) {
     std::vector<double2> a, b, c;
     fill_twiddles<double2, double>(p, a, b, c);

@@ -191,34 +191,44 @@ k_tap_reduce(const T* __restrict__ part, const int* __restrict__ dst, TapDst d, 
 
 // ------------------------------------------------------------------ edge sums
 // H_m(u, u') over one list: a CTA stages 32 edge points at a time (the L^2
-// reference values around each, and the signed monomials) and each thread
-// keeps kGramP pairs x all monomials in registers.  The points of the next
-// batch are copied (cp.async) while this one is summed, and the list is read
-// two batches ahead; without it the gathers' latency took 60 % of the warps'
-// time.  What bounds it now are the issue slots (44 %) and shared-memory reads of
-// the patches: 96 us for a 4096 x 2048 CCD with saturated stars and two dead
-// columns.  Slot g of U takes batches g, g + U, ..., at least kGramMin<T> points,
-// and writes hp[ccd][slot][pair][MP]; a short list uses few slots.  The x-edge
-// blocks, whose lists are the longer, come first.  The number of slots has a
-// limit, a slot's share of a long list has none: an FP32 sum covers kGramRun
-// points, then it is added to the slot's partials as an exact pair of floats
+// reference values around each, signed powers of xt and powers of yt) and each
+// thread keeps a 2 x 2 tile of pairs x all monomials in registers.  The points
+// of the next batch are copied (cp.async) while this one is summed, and the list
+// is read two batches ahead; without it the gathers' latency took 60 % of the
+// warps' time.  The list is in row order: a thread sums the powers of xt over a
+// row's points and takes the result times the powers of yt at the row's end, 5
+// multiply-adds per pair and point and 15 per row at D_K = 2 in place of 15 per
+// point.  That, and two reads of neighbouring offsets for four pairs (five pairs
+// with offsets of their own took ten), is for masks with many edges, whose rows
+// are long.  Assembly of 4096 x 2048, L = 11, D_K = 2: bad pixels every 12 px
+// 11.1 -> 6.4 ms, bad rows every 16 8.2 -> 4.4 ms (6.9 and 6.8 ms from spectra);
+// four of 1024 x 2048, L = 7, bad pixels every 8 px 9.2 -> 2.0 ms (4.2 ms); one
+// with saturated stars and two dead columns: 80 us in this kernel, 96 before.
+// What bounds it are issue slots and shared-memory reads (about half of either).
+// Slot g of U takes batches g, g + U, ..., at least kGramMin<T> points, and writes
+// hp[ccd][slot][pair][NM]; a short list uses few slots.  The x-edge blocks, whose
+// lists are the longer, come first.  The number of slots has a limit, a slot's
+// share of a long list has none: an FP32 sum covers kGramRun rows (of at most 32
+// points), then it is added to the slot's partials as an exact pair of floats
 // (10^4 equal products one after another lose up to 1.3e-4 of their sum, 256 at
 // most 4e-6).
-constexpr int kGramP = 5;
 constexpr int kGramPts = 32;
 constexpr int kGramRun = 256;
 constexpr int kGramThreads = 256;
-constexpr int kGramPatch = 125;   // L^2 <= 121 values, then 1 (single offsets) and padding to an odd pitch
+constexpr int kGramOne = 122;     // L^2 <= 121 values, then (1, 0): the partner of single offsets
+constexpr int kGramPatch = 124;   // even: two neighbouring offsets in one read
+constexpr int kGramPow = 10;      // powers of a coordinate, in rows that spread over the banks
 // least points of a slot: FP64 multiply-adds are 64 times slower than FP32
-// ones, so there a short list spreads over more slots (one 512 x 512 pair,
-// L = 7, D_K = 1: 1.6 ms with 256 points, 1.1 ms with 32).  FP32: the
-// edges of a single CCD's stars and columns fill too few slots of 256 points
-// (4096 x 2048, L = 11, D_K = 2: 104 us with 256, 96 us with 128)
-template <typename T> constexpr int kGramMin = sizeof(T) == 4 ? 128 : kGramPts;
+// ones, so there a short list spreads over more slots (a 512 x 512 pair, L = 7,
+// D_K = 1: 853 us with 64 points, 819 us with 32).  FP32: more slots cost
+// k_edge_reduce more than they give here (a 4096 x 2048 pair, L = 11, D_K = 2:
+// 1742 us with 64 points, 1734 with 128, 1727 with 256)
+template <typename T> constexpr int kGramMin = sizeof(T) == 4 ? 256 : kGramPts;
 
 struct GramArgs {
-  const int* pairs;        // i | j << 8: y pairs, then x pairs
-  int npy, npx, nbx;       // pairs and x blocks
+  const int* tiles;        // i | j << 8, the tile's first offsets: y tiles, then x tiles
+  int nty, ntx, nbx;       // tiles and x blocks
+  int npy, npx;            // pairs
   int gy, gx;              // most slots per list
   int64_t hp_stride;       // per CCD
   int64_t hx_off;          // x partials after the y ones
@@ -228,105 +238,138 @@ struct GramArgs {
 
 template <typename T>
 __device__ __forceinline__ int gram_slots(int n, int g) { return max(1, min(g, (n + kGramMin<T> - 1) / kGramMin<T>)); }
-// whether a slot's share of n points in U slots is summed in more than one run
+// whether a slot's share of n points in U slots may be summed in more than one run
 template <typename T>
 __device__ __forceinline__ bool gram_runs(int n, int U) {
   return sizeof(T) == 4 && ((n + kGramPts - 1) / kGramPts + U - 1) / U * kGramPts > kGramRun;
 }
 
-template <typename T, int DE>
+// Pair numbering shared by the tiles and the chains.  y pairs: offsets
+// i, j < L (L - 1) in row-major order, j <= i; then the single offsets i.
+// x pairs: i in the row u_y = w with u_x < w, j <= i with u_x < w; then the
+// single offsets.
+__device__ __forceinline__ int ypair_id(int i, int j) { return i * (i + 1) / 2 + j; }
+__host__ __device__ inline int ypair_single(int L, int i) { const int n = L * (L - 1); return n * (n + 1) / 2 + i; }
+__device__ __forceinline__ int xpair_id(int L, int ix, int jy, int jx) {   // biased indices 0 .. L-1
+  const int q = (L - 1) * (L - 1);
+  return ix * q + ix * (ix + 1) / 2 + (jy < L - 1 ? jy * (L - 1) + jx : q + jx);
+}
+__host__ __device__ inline int xpair_single(int L, int ix) {
+  const int q = (L - 1) * (L - 1), n = L - 1;
+  return n * q + n * (n + 1) / 2 + ix;
+}
+// the pair of the offsets i and j (or kGramOne) of a tile; -1: not one of the list's pairs
+__device__ __forceinline__ int gram_pair(int L, bool isx, int i, int j) {
+  const int n = L * (L - 1);
+  if (isx) {
+    const int ix = i - n;
+    if (ix >= L - 1) return -1;
+    if (j >= kGramOne) return j == kGramOne ? xpair_single(L, ix) : -1;
+    if (j >= n) return j - n <= ix ? xpair_id(L, ix, L - 1, j - n) : -1;
+    return j % L < L - 1 ? xpair_id(L, ix, j / L, j % L) : -1;
+  }
+  if (i >= kGramOne) return i == kGramOne && j < n ? ypair_single(L, j) : -1;
+  return j <= i ? ypair_id(i, j) : -1;
+}
+
+template <typename T>
 __host__ __device__ constexpr size_t gram_smem() {
-  constexpr int MP = (n_mono(DE) + 3) / 4 * 4;
-  return 2 * sizeof(T) * kGramPts * (MP + kGramPatch) + 2 * kGramPts * sizeof(unsigned);
+  // per buffer and point: the patch, xt^a and yt^a (FP32: twice, as operand pairs), the list entry; the row ends
+  return 2 * (sizeof(T) * kGramPts * (kGramPatch + 2 * kGramPow * (sizeof(T) == 4 ? 2 : 1)) + sizeof(int4) * kGramPts +
+              sizeof(unsigned));
 }
 
 template <typename T, int DE>
 __global__ void __launch_bounds__(kGramThreads, sizeof(T) == 4 ? 2 : 1)
 k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const unsigned* __restrict__ ly, int64_t lstride,
             const int* __restrict__ cnt, int64_t cnt_stride, GramArgs a, T* __restrict__ hp, int H, int W, int L) {
-  constexpr int NM = n_mono(DE), MP = (NM + 3) / 4 * 4;
+  constexpr int NM = n_mono(DE), CD = sizeof(T) == 4 ? 2 : 1, PW = kGramPow * CD;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T(*mono)[kGramPts][MP] = reinterpret_cast<T(*)[kGramPts][MP]>(smraw);
-  T(*patch)[kGramPts][kGramPatch] =
-      reinterpret_cast<T(*)[kGramPts][kGramPatch]>(smraw + 2 * sizeof(T) * kGramPts * MP);
-  unsigned(*ent)[kGramPts] =
-      reinterpret_cast<unsigned(*)[kGramPts]>(smraw + 2 * sizeof(T) * kGramPts * (MP + kGramPatch));
+  __shared__ int2 offs[kGramPatch];   // u as a distance in the image; u_y and u_x
+  T(*px)[kGramPts][PW] = reinterpret_cast<T(*)[kGramPts][PW]>(smraw);
+  T(*py)[kGramPts][PW] = px + 2;
+  T(*patch)[kGramPts][kGramPatch] = reinterpret_cast<T(*)[kGramPts][kGramPatch]>(py + 2);
+  int4(*ent)[kGramPts] = reinterpret_cast<int4(*)[kGramPts]>(patch + 2);   // x, y, sign, patch inside the image
+  unsigned* ends = reinterpret_cast<unsigned*>(ent + 2);   // the last points of the batch's rows
   const int ccd = blockIdx.z, tid = threadIdx.x, w = (L - 1) / 2, lane = tid & 31, warp = tid >> 5;
   const bool isx = (int)blockIdx.y < a.nbx;
   const int n = cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H];
   const int U = gram_slots<T>(n, isx ? a.gx : a.gy), g = blockIdx.x;
   if (g >= U) return;
-  const int blk = isx ? blockIdx.y : blockIdx.y - a.nbx;
-  const int np = isx ? a.npx : a.npy;
-  const int* ptab = a.pairs + (isx ? a.npy : 0);
+  const int tile = (isx ? blockIdx.y : blockIdx.y - a.nbx) * kGramThreads + tid, nt = isx ? a.ntx : a.nty;
   const unsigned* list = (isx ? lx : ly) + ccd * lstride;
-  int pi[kGramP], pj[kGramP];
-#pragma unroll
-  for (int p = 0; p < kGramP; ++p) {
-    const int id = (blk * kGramP + p) * kGramThreads + tid;
-    const int v = id < np ? ptab[id] : 0;
-    pi[p] = v & 255;
-    pj[p] = v >> 8;
+  const int v = tile < nt ? a.tiles[(isx ? a.nty : 0) + tile] : 0, ti = v & 255, tj = v >> 8;
+  const bool idle = tile - lane >= nt;   // a warp without tiles only copies
+  if (tid < kGramPatch) {
+    const int uy = tid / L - w, ux = tid % L - w;
+    offs[tid] = make_int2(uy * W + ux, (uy + w) << 8 | (ux + w));
   }
-  // this lane's offsets j = lane + 32 k: u_y, u_x
-  int oy[4], ox[4];
+  // (j, j + 1) packed, for i and i + 1: sums over a row, and all rows times yt^b
+  v2<T> rs[2][DE + 1], acc[2][NM];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int j = lane + 32 * k;
-    oy[k] = j / L - w;
-    ox[k] = j % L - w;
+  for (int q = 0; q < 2; ++q) {
+#pragma unroll
+    for (int k = 0; k <= DE; ++k) v2_zero(rs[q][k]);
+#pragma unroll
+    for (int k = 0; k < NM; ++k) v2_zero(acc[q][k]);
   }
-  v2<T> acc[kGramP][MP / 2];
-#pragma unroll
-  for (int p = 0; p < kGramP; ++p)
-#pragma unroll
-    for (int m = 0; m < MP / 2; ++m) v2_zero(acc[p][m]);
-  const double xs = a.xs, ys = a.ys;
   const T* img = Rm + (int64_t)ccd * H * W;
-  if (tid < 2 * kGramPts) patch[tid / kGramPts][tid % kGramPts][L * L] = (T)1;
+  if (tid < 2 * kGramPts) {
+    patch[tid / kGramPts][tid % kGramPts][kGramOne] = (T)1;
+    patch[tid / kGramPts][tid % kGramPts][kGramOne + 1] = (T)0;
+  }
   const int nb = (n + kGramPts - 1) / kGramPts;
   // the points of batch b into buffer s
   auto stage = [&](int b, int s) {
     const int m = min(kGramPts, n - b * kGramPts);
     for (int pt = warp; pt < m; pt += kGramThreads / 32) {
-      const unsigned e = ent[s][pt] >> 1;
-      const int y = (int)(e / (unsigned)W), x = (int)(e % (unsigned)W);
+      const int4 e = ent[s][pt];
+      const T* src = img + ((int64_t)e.y * W + e.x);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int j = lane + 32 * k;
-        const int yy = y - oy[k], xx = x - ox[k];
-        const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
-        if (j < L * L) cp_async<sizeof(T)>(&patch[s][pt][j], img + (in ? (int64_t)yy * W + xx : 0), in);
+        if (j < L * L) {
+          const int2 o = offs[j];
+          bool in = true;
+          if (!e.w) {
+            const int yy = e.y + w - (o.y >> 8), xx = e.x + w - (o.y & 255);
+            in = yy >= 0 && yy < H && xx >= 0 && xx < W;
+          }
+          cp_async<sizeof(T)>(&patch[s][pt][j], in ? src - o.x : img, in);
+        }
       }
     }
     if (warp == kGramThreads / 32 - 1) {
-      const unsigned e = ent[s][lane];
-      const T sg = lane >= m ? (T)0 : ((e & 1u) ? (T)-1 : (T)1);
-      const T xt = (T)((double)((e >> 1) % (unsigned)W) * xs - 1.0), yt = (T)((double)((e >> 1) / (unsigned)W) * ys - 1.0);
-      T px[DE + 1], py[DE + 1];
-      px[0] = sg;
-      py[0] = 1;
+      const int4 e = ent[s][lane];
+      const int yn = __shfl_down_sync(0xffffffffu, e.y, 1);
+      const unsigned last = __ballot_sync(0xffffffffu, lane < m && (lane == m - 1 || yn != e.y));
+      if (lane == 0) ends[s] = last;
+      const T xt = (T)(e.x * a.xs - 1.0), yt = (T)(e.y * a.ys - 1.0);
+      T qx = (T)e.z, qy = 1;
 #pragma unroll
-      for (int k = 1; k <= DE; ++k) { px[k] = px[k - 1] * xt; py[k] = py[k - 1] * yt; }
-#pragma unroll
-      for (int q = 0; q <= DE; ++q)
-#pragma unroll
-        for (int k = 0; k <= q; ++k) mono[s][lane][mono_index(q - k, k)] = px[q - k] * py[k];
-#pragma unroll
-      for (int k = NM; k < MP; ++k) mono[s][lane][k] = 0;
+      for (int k = 0; k <= DE; ++k) {
+        st_dup(&px[s][lane][CD * k], qx);
+        st_dup(&py[s][lane][CD * k], qy);
+        qx *= xt;
+        qy *= yt;
+      }
     }
   };
   auto entry = [&](int b) { return b < nb && b * kGramPts + lane < n ? list[(int64_t)b * kGramPts + lane] : 0u; };
+  auto put = [&](unsigned e, int s) {
+    const int y = (int)((e >> 1) / (unsigned)W), x = (int)((e >> 1) - (unsigned)y * (unsigned)W);
+    ent[s][lane] = make_int4(x, y, (e & 1u) ? -1 : 1, y >= w && y < H - w && x >= w && x < W - w);
+  };
   if (warp == 0) {
-    ent[0][lane] = entry(g);
-    ent[1][lane] = entry(g + U);
+    put(entry(g), 0);
+    put(entry(g + U), 1);
   }
   __syncthreads();
   if (g < nb) stage(g, 0);
-  T* out = hp + ccd * a.hp_stride + (isx ? a.hx_off : 0) + (int64_t)g * np * MP;
+  T* out = hp + ccd * a.hp_stride + (isx ? a.hx_off : 0) + (int64_t)g * (isx ? a.npx : a.npy) * NM;
   const bool runs = gram_runs<T>(n, U);
   bool first = true;
-  int s = 0, done = 0;
+  int s = 0, rows = 0;
   // an empty list takes one turn without points, for the zeros
   for (int b = g; b < max(nb, 1); b += U, s ^= 1) {
     cp_async_wait_all();
@@ -335,37 +378,54 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
     if (warp == 0) e2 = entry(b + 2 * U);
     if (b + U < nb) stage(b + U, s ^ 1);
     const int m = min(kGramPts, n - b * kGramPts);
-    // two points at a time: the second's reads pass the first's multiply-adds
-    // (ten CCDs 983 -> 965 us, five of L = 9, D_K = 1 94.7 -> 87.5 us)
-#pragma unroll 2
-    for (int pt = 0; pt < m; ++pt) {
-      T mv[MP];
+    const unsigned last = m > 0 ? ends[s] : 0u;
+    for (int pt = 0; pt < m && !idle;) {
+      const int c = __ffs(last >> pt);   // points of the row
+      const T *pj = &patch[s][pt][tj], *pi = &patch[s][pt][ti], *pq = &px[s][pt][0];
+#pragma unroll 4
+      for (int i = 0; i < c; ++i, pj += kGramPatch, pi += kGramPatch, pq += PW) {
+        const v2<T> rj = v2_load(pj), ri = v2_load(pi);
+        const v2<T> r0 = v2_make(v2_get(ri, 0) * v2_get(rj, 0), v2_get(ri, 0) * v2_get(rj, 1));
+        const v2<T> r1 = v2_make(v2_get(ri, 1) * v2_get(rj, 0), v2_get(ri, 1) * v2_get(rj, 1));
 #pragma unroll
-      for (int k = 0; k < MP; k += 4) {
-        T q[4];
-        ld4(&mono[s][pt][k], q);
+        for (int k = 0; k <= DE; k += 2) {
+          v2<T> q[2];
+          v2_dup2(pq + CD * k, q[0], q[1]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) mv[k + i] = q[i];
+          for (int h = 0; h < 2 && k + h <= DE; ++h) {
+            v2_fmav(rs[0][k + h], q[h], r0);
+            v2_fmav(rs[1][k + h], q[h], r1);
+          }
+        }
+      }
+      pt += c;
+#pragma unroll
+      for (int q = 0; q <= DE; ++q) {
+        const v2<T> yb = v2_dup(&py[s][pt - 1][CD * q]);
+#pragma unroll
+        for (int k = 0; k <= DE - q; ++k) {
+          v2_fmav(acc[0][mono_index(k, q)], yb, rs[0][k]);
+          v2_fmav(acc[1][mono_index(k, q)], yb, rs[1][k]);
+        }
       }
 #pragma unroll
-      for (int p = 0; p < kGramP; ++p) {
-        const T r = patch[s][pt][pi[p]] * patch[s][pt][pj[p]];
-#pragma unroll
-        for (int k = 0; k < MP / 2; ++k) v2_fma(acc[p][k], mv[2 * k], mv[2 * k + 1], r);
+      for (int k = 0; k <= DE; ++k) {
+        v2_zero(rs[0][k]);
+        v2_zero(rs[1][k]);
       }
     }
-    if (warp == 0) ent[s][lane] = e2;
-    done += kGramPts;
+    if (warp == 0) put(e2, s);
+    rows += __popc(last);
     const bool end = b + U >= nb;
-    if (!end && !(runs && done % kGramRun == 0)) continue;
+    if (!end && !(runs && rows > kGramRun - kGramPts)) continue;
 #pragma unroll
-    for (int p = 0; p < kGramP; ++p) {
-      const int id = (blk * kGramP + p) * kGramThreads + tid;
-      if (id < np)
+    for (int p = 0; p < 4; ++p) {
+      const int id = tile < nt ? gram_pair(L, isx, ti + (p >> 1), tj + (p & 1)) : -1;
+      if (id >= 0)
 #pragma unroll
-        for (int k = 0; k < MP; ++k) {
-          T* o = out + (int64_t)id * MP + k;
-          T v = v2_get(acc[p][k / 2], k & 1);
+        for (int k = 0; k < NM; ++k) {
+          T* o = out + (int64_t)id * NM + k;
+          T v = v2_get(acc[p >> 1][k], p & 1);
           if constexpr (sizeof(T) == 4)
             if (runs) {
               float e = 0.f;
@@ -374,19 +434,22 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
             }
           *o = v;
         }
-#pragma unroll
-      for (int k = 0; k < MP / 2; ++k) v2_zero(acc[p][k]);
     }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int k = 0; k < NM; ++k) v2_zero(acc[q][k]);
     first = false;
+    rows = 0;
   }
 }
 
 // the slots' partial sums: FP64, on the mixed path as pairs of floats
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_edge_reduce(const T* __restrict__ hp, GramArgs a, const int* __restrict__ cnt, int64_t cnt_stride, int H, int MP,
+k_edge_reduce(const T* __restrict__ hp, GramArgs a, const int* __restrict__ cnt, int64_t cnt_stride, int H, int NM,
               double* __restrict__ hs) {
-  const int ccd = blockIdx.y, ny = a.npy * MP, nx = a.npx * MP;
+  const int ccd = blockIdx.y, ny = a.npy * NM, nx = a.npx * NM;
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= ny + nx) return;
   const bool isx = i >= ny;
@@ -397,7 +460,7 @@ k_edge_reduce(const T* __restrict__ hp, GramArgs a, const int* __restrict__ cnt,
   if constexpr (sizeof(T) == 4) {
     const bool runs = gram_runs<T>(n, U);
     float h = 0.f, l = 0.f;
-#pragma unroll 4
+#pragma unroll 8
     for (int g = 0; g < U; ++g) {
       float e;
       h = two_sum(h, p[g * st], e);
@@ -406,25 +469,10 @@ k_edge_reduce(const T* __restrict__ hp, GramArgs a, const int* __restrict__ cnt,
     }
     s = (double)h + (double)l;
   } else {
-#pragma unroll 4
+#pragma unroll 8
     for (int g = 0; g < U; ++g) s += p[g * st];
   }
   hs[(int64_t)ccd * (ny + nx) + i] = s;
-}
-
-// Pair numbering shared by the table (host) and the chains.  y pairs: offsets
-// i, j < L (L - 1) in row-major order, j <= i; then the single offsets i.
-// x pairs: i in the row u_y = w with u_x < w, j <= i with u_x < w; then the
-// single offsets.
-__host__ __device__ inline int ypair_id(int i, int j) { return i * (i + 1) / 2 + j; }
-__host__ __device__ inline int ypair_single(int L, int i) { const int n = L * (L - 1); return n * (n + 1) / 2 + i; }
-__host__ __device__ inline int xpair_id(int L, int ix, int jy, int jx) {   // biased indices 0 .. L-1
-  const int q = (L - 1) * (L - 1);
-  return ix * q + ix * (ix + 1) / 2 + (jy < L - 1 ? jy * (L - 1) + jx : q + jx);
-}
-__host__ __device__ inline int xpair_single(int L, int ix) {
-  const int q = (L - 1) * (L - 1), n = L - 1;
-  return n * q + n * (n + 1) / 2 + ix;
 }
 
 // ------------------------------------------------------------------ chains
@@ -615,32 +663,29 @@ void build_tap_plan(sfft_plan_s* p) {
   // the refinement's half tiles (kernels_apply.cu)
   t.ntile_rhs = 2 * conv_tiles(p->d.H, p->d.W, conv_half_width(p->d.H, p->d.W, B));
   // edge sums
-  t.pairs.clear();
-  t.npy = t.npx = 0;
+  t.tiles.clear();
+  t.npy = t.npx = t.nty = t.ntx = 0;
   if (t.mode == TAP_FIT_EDGE) {
-    const int one = L * L, n = L * (L - 1);
-    for (int i = 0; i < n; ++i)
-      for (int j = 0; j <= i; ++j) t.pairs.push_back(i | j << 8);
-    for (int i = 0; i < n; ++i) t.pairs.push_back(i | one << 8);
-    t.npy = (int)t.pairs.size();
-    for (int ix = 0; ix < L - 1; ++ix) {
-      const int i = (L - 1) * L + ix;
-      for (int jy = 0; jy < L - 1; ++jy)
-        for (int jx = 0; jx < L - 1; ++jx) t.pairs.push_back(i | (jy * L + jx) << 8);
-      for (int jx = 0; jx <= ix; ++jx) t.pairs.push_back(i | ((L - 1) * L + jx) << 8);
+    const int n = L * (L - 1);   // offsets below the row u_y = w, an even number
+    t.npy = ypair_single(L, n);
+    t.npx = xpair_single(L, L - 1);
+    for (int i = 0; i < n; i += 2)
+      for (int j = 0; j <= i; j += 2) t.tiles.push_back(i | j << 8);
+    for (int j = 0; j < n; j += 2) t.tiles.push_back(kGramOne | j << 8);
+    t.nty = (int)t.tiles.size();
+    for (int ix = 0; ix < L - 1; ix += 2) {
+      for (int j = 0; j <= n + ix; j += 2) t.tiles.push_back((n + ix) | j << 8);
+      t.tiles.push_back((n + ix) | kGramOne << 8);
     }
-    for (int ix = 0; ix < L - 1; ++ix) t.pairs.push_back(((L - 1) * L + ix) | one << 8);
-    t.npx = (int)t.pairs.size() - t.npy;
-    // two CTAs per SM when both lists fill their slots: the x pairs take one
-    // block at L = 11, the y pairs five
-    t.gx = std::max(64, 304 / B);
-    t.gy = std::max(16, 64 / B);
-    const int per = kGramP * kGramThreads;
-    t.nby = (t.npy + per - 1) / per;
-    t.nbx = (t.npx + per - 1) / per;
+    t.ntx = (int)t.tiles.size() - t.nty;
+    t.nby = (t.nty + kGramThreads - 1) / kGramThreads;
+    t.nbx = (t.ntx + kGramThreads - 1) / kGramThreads;
+    // a list that fills its slots gives every SM two rounds of two CTAs
+    t.gy = std::max(16, 608 / (t.nby * B));
+    t.gx = std::max(64, 304 / (t.nbx * B));
   }
   t.DE = std::max(dKK, dKB);
-  t.MP = (n_mono(t.DE) + 3) / 4 * 4;
+  t.MP = n_mono(t.DE);
   // M is an erosion by L x L: its zero runs are at least L wide between the borders
   t.row_cap = L == 1 ? p->d.W : std::min(p->d.W, 2 * (p->d.W / (L + 1) + 2));
   t.col_cap = L == 1 ? p->d.H : std::min(p->d.H, 2 * (p->d.H / (L + 1) + 2));
@@ -727,8 +772,9 @@ static cudaError_t edge_sums_T(const sfft_plan_s* p, void* ws) {
   const TapPlan& t = p->tap;
   const int H = p->d.H, W = p->d.W, L = p->d.L, B = p->d.batch;
   GramArgs a;
-  a.pairs = t.d_pairs;
-  a.npy = t.npy; a.npx = t.npx; a.nbx = t.nbx;
+  a.tiles = t.d_tiles;
+  a.nty = t.nty; a.ntx = t.ntx; a.nbx = t.nbx;
+  a.npy = t.npy; a.npx = t.npx;
   a.gy = t.gy; a.gx = t.gx;
   a.xs = step_of(W); a.ys = step_of(H);
   a.hx_off = (int64_t)t.gy * t.npy * t.MP;
@@ -743,9 +789,9 @@ static cudaError_t edge_sums_T(const sfft_plan_s* p, void* ws) {
   cudaError_t e = cudaSuccess;
 #define SFFT_GRAM(D)                                                                                                  \
   case D:                                                                                                             \
-    e = cudaFuncSetAttribute(k_edge_gram<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem<T, D>()); \
+    e = cudaFuncSetAttribute(k_edge_gram<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem<T>()); \
     if (e != cudaSuccess) return e;                                                                                   \
-    k_edge_gram<T, D><<<grid, kGramThreads, gram_smem<T, D>(), p->stream>>>(rm, lx, lx + cap, 2 * cap, cnt, cs, a, hp, \
+    k_edge_gram<T, D><<<grid, kGramThreads, gram_smem<T>(), p->stream>>>(rm, lx, lx + cap, 2 * cap, cnt, cs, a, hp, \
                                                                             H, W, L);                                 \
     break
   switch (t.DE) {

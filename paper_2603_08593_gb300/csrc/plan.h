@@ -57,19 +57,19 @@ constexpr int kDlChunk = 16;
 constexpr int kDlMaxU = 6;
 
 // Image-space assembly (kernels_tap.cu): tap-sum tasks (the fit's, then the
-// right-hand side's), the destinations of their outputs, the pair table of the
-// mask-edge sums, and the tile and slot counts.
+// right-hand side's), the destinations of their outputs, the tiles of pairs of
+// the mask-edge sums, and the tile and slot counts.
 struct TapPlan {
   int mode = 0, nt = 0, tw = 0, ntile = 0;
   int ntask = 0, nout = 0, nsplit = 1, ntask_rhs = 0, nout_rhs = 0, ntile_rhs = 0;
-  int npy = 0, npx = 0, nby = 0, nbx = 0, gy = 0, gx = 0;
-  int DE = 0, MP = 0;           // degree and padded monomial count of the edge sums
+  int npy = 0, npx = 0, nty = 0, ntx = 0, nby = 0, nbx = 0, gy = 0, gx = 0;
+  int DE = 0, MP = 0;           // degree and monomial count of the edge sums
   int row_cap = 0, col_cap = 0; // most x edges of a row, y edges of a column
   std::vector<int4> tasks;
-  std::vector<int> dst, pairs;
+  std::vector<int> dst, tiles;
   int4* d_tasks = nullptr;
   int* d_dst = nullptr;
-  int* d_pairs = nullptr;
+  int* d_tiles = nullptr;
 };
 
 }  // namespace sfft

@@ -37,6 +37,27 @@ __device__ __forceinline__ v2<float> v2_dup(const float* p) {
   return r;
 }
 __device__ __forceinline__ v2<double> v2_dup(const double* p) { return v2_make(*p, *p); }
+// the dups of two neighbouring values, 16-byte aligned
+__device__ __forceinline__ void v2_dup2(const float* p, v2<float>& a, v2<float>& b) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  a.p = make_float2(q.x, q.y);
+  b.p = make_float2(q.z, q.w);
+}
+__device__ __forceinline__ void v2_dup2(const double* p, v2<double>& a, v2<double>& b) {
+  const double2 q = *reinterpret_cast<const double2*>(p);
+  a = v2_make(q.x, q.x);
+  b = v2_make(q.y, q.y);
+}
+// (p[0], p[1]) of an even element of an aligned row
+__device__ __forceinline__ v2<float> v2_load(const float* p) {
+  v2<float> r;
+  r.p = *reinterpret_cast<const float2*>(p);
+  return r;
+}
+__device__ __forceinline__ v2<double> v2_load(const double* p) {
+  const double2 q = *reinterpret_cast<const double2*>(p);
+  return v2_make(q.x, q.y);
+}
 __device__ __forceinline__ void st_dup(float* p, float v) { *reinterpret_cast<float2*>(p) = make_float2(v, v); }
 __device__ __forceinline__ void st_dup(double* p, double v) { *p = v; }
 __device__ __forceinline__ float v2_get(const v2<float>& a, int i) { return i ? a.p.y : a.p.x; }

@@ -63,3 +63,35 @@ def test_dense_edges_in_a_batch(L, DK, DB, period, kind):
         bad[:, :, L // 2::period] = 1
     sky = torch.tensor([[1000.0, 1001.0]] * B, dtype=torch.float64, device=DEV)
     _compare(R, S, bad, sky, L, DK, DB)
+
+
+@pytest.mark.parametrize("shape,L,DK,period,kind", [((2048, 2048), 11, 2, 12, "specks"), ((2048, 2048), 11, 2, 12, "rows"),
+                                                    ((2048, 2048), 7, 2, 8, "specks")])
+def test_densest_masks_cost_no_more_than_spectra(shape, L, DK, period, kind):
+    """The masks with the most edges: the default assembly against the spectral
+    one, whose time does not depend on the mask (a set d_batch of every
+    difference).  A tenth is allowed for the clock."""
+    from paper_2603_08593_gb300 import Plan
+    H, W = shape
+    g = torch.Generator(device=DEV)
+    g.manual_seed(period)
+    R, S = (1000.0 + 32.0 * torch.randn(1, H, W, generator=g, device=DEV) for _ in range(2))
+    bad = torch.zeros(1, H, W, dtype=torch.uint8, device=DEV)
+    if kind == "specks":
+        bad[:, L // 2::period, L // 2::period] = 1
+    else:
+        bad[:, L // 2::period, :] = 1
+    ms = []
+    for d_batch in (0, 4 * L * L):
+        p = Plan(H, W, L, DK, DK, batch=1, prec="mixed", d_batch=d_batch)
+        A, b = p.build_normal(R, S, bad)
+        ev = []
+        for _ in range(7):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            p.build_normal(R, S, bad, A=A, b=b)
+            e[1].record()
+            ev.append(e)
+        torch.cuda.synchronize()
+        ms.append(sorted(x.elapsed_time(y) for x, y in ev)[3])
+    assert ms[0] <= 1.1 * ms[1], ms
