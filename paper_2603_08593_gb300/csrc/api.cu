@@ -131,9 +131,10 @@ static void build_layout(sfft_plan_s* p) {
   add_region(p->uspec, cur, spectra * slab * (p->d.DK + 1) * B);
   add_region(p->rhat, cur, spectra * slab * B);
   add_region(p->phat, cur, spectra * slab * p->d_batch * p->ccd_group);
-  size_t part = 0, hp = 0, hs = 0, list = 0, cnt = 0;
-  if (p->direct) tap_region_bytes(p, &part, &hp, &hs, &list, &cnt);
+  size_t part = 0, mpart = 0, hp = 0, hs = 0, list = 0, cnt = 0;
+  if (p->direct) tap_region_bytes(p, &part, &mpart, &hp, &hs, &list, &cnt);
   add_region(p->tappart, cur, part);
+  add_region(p->mompart, cur, mpart);
   add_region(p->hpart, cur, hp);
   add_region(p->hsum, cur, hs);
   add_region(p->elist, cur, list);

@@ -80,6 +80,8 @@ struct ConvArgs {
   T* E;
   const int4* tasks;
   T* part;
+  double* mpart;
+  char3 need;              // moments taken
   int ntask, nout_tot;
   int H, W, L, DB, hw;
   double xsc, ysc;         // 2 / (W - 1), 2 / (H - 1): an FP64 division per thread cost a tenth of the kernel
@@ -95,6 +97,7 @@ k_conv(const ConvArgs<T> a) {
   constexpr int wt = (NT - 1) / 2, NA = DK + 1, NK = n_mono(DK);
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned char ot[2][kTapMaxOut][2];
+  __shared__ double ypd[MODE == CV_SUMS ? 5 : 1][32];
   __shared__ int next;
   const int H = a.H, W = a.W, hw = a.hw, L = a.L, w = (L - 1) / 2;
   constexpr int CD = kCvDup<T>;
@@ -344,7 +347,7 @@ k_conv(const ConvArgs<T> a) {
     if (warp == 0) {
       const double y = (y0 + row) * ysc - 1.0;
       double v = 1.0;
-      for (int b = 0; b < 5; ++b) { yp[b * kTapScrPitch + lane] = (T)v; v *= y; }
+      for (int b = 0; b < 5; ++b) { yp[b * kTapScrPitch + lane] = (T)v; ypd[b][lane] = v; v *= y; }
     }
     __syncthreads();
     // a task takes half of the lanes' columns: 22 taps tasks and 2 of moments at
@@ -367,9 +370,9 @@ k_conv(const ConvArgs<T> a) {
       t.yp = yp;
       t.scr = scr + warp * kTapScr * kTapScrPitch;
       t.ot = ot[type == TAP_S ? 0 : 1];
-      T* out = a.part + (((int64_t)ccd * gridDim.x + tile) * 2 + (k & 1)) * a.nout_tot + q.w;
-      if (type == TAP_S) tap_task<T, NT, NT, 0, NA, false, CD>(t, 0, 0, q.z, nout, out);
-      else tap_moments<T, false>(t, wt, w, nout, out);
+      const int64_t half_tile = ((int64_t)ccd * gridDim.x + tile) * 2 + (k & 1);
+      if (type == TAP_S) tap_task<T, NT, NT, 0, NA, false, CD>(t, 0, 0, q.z, nout, a.part + half_tile * a.nout_tot + q.w);
+      else tap_moments<T, false>(t, wt, w, ypd, a.need, a.mpart + half_tile * kTapMom);
     }
   }
 }
@@ -475,6 +478,8 @@ static cudaError_t residual_sums_T(const sfft_plan_s* p, const float* S, const d
   a.ntask = p->tap.ntask_rhs;
   a.nout_tot = p->tap.nout_rhs;
   a.part = ws_at<T>(ws, p->tappart);
+  a.mpart = ws_at<double>(ws, p->mompart);
+  a.need = tap_moment_need(p, false);
   p->nlaunch += 1;
   return conv<T, CV_SUMS>(p->stream, a, p->d.DK, p->d.batch);
 }

@@ -50,10 +50,11 @@ template <typename T, int NT, int DK, int MODE>
 __global__ void __launch_bounds__(kTapWarps * 32, sizeof(T) == 4 ? 3 : 2)
 k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const unsigned* __restrict__ mfitw,
            const double* __restrict__ sky, const int4* __restrict__ tasks, int ntask,
-           T* __restrict__ part, int nout_tot, int H, int W, int w, int tw, double xs, double ys) {
+           T* __restrict__ part, int nout_tot, double* __restrict__ mpart, char3 need, int H, int W, int w, int tw, double xs, double ys) {
   constexpr int wt = (NT - 1) / 2, RC = 2 * DK + 1, RS = DK + 1, RM = DK + 3;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ unsigned char ot[5][kTapMaxOut][2];
+  __shared__ double ypd[5][32];
   __shared__ int next;
   const int pitch = (tw + 2 * wt) | 1, spitch = tw | 1, nw = tw / 32;
   T* yp = reinterpret_cast<T*>(smraw);
@@ -76,7 +77,7 @@ k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const unsigned
   if (tid < kTapRows) {
     const double y = (y0 + tid) * ys - 1.0;
     double v = 1.0;
-    for (int b = 0; b < 5; ++b) { yp[b * kTapScrPitch + tid] = (T)v; v *= y; }
+    for (int b = 0; b < 5; ++b) { yp[b * kTapScrPitch + tid] = (T)v; ypd[b][tid] = v; v *= y; }
   }
   // R with its halo, zero outside the image: copied asynchronously, every
   // element in flight at once (plain loads kept 29 % of the warps' time
@@ -138,12 +139,13 @@ k_tap_sums(const T* __restrict__ Rm, const float* __restrict__ S, const unsigned
     if (type == TAP_CS) tap_task<T, NT, NT, RC, RS, false, 1>(t, u0x, u0y, q.z, nout, out);
     else if (type == TAP_C) tap_task<T, NT, KC, RC, 0, false, 1>(t, u0x, u0y, q.z, nout, out);
     else if (MODE == TAP_FIT_ALL && type == TAP_M) tap_task<T, NT, NT, RM, 0, true, 1>(t, 0, 0, q.z, nout, out);
-    else tap_moments<T, true>(t, wt, w, nout, out);
+    else tap_moments<T, true>(t, wt, w, ypd, need, mpart + ((int64_t)ccd * gridDim.x + tile) * kTapMom);
   }
 }
 
 // Sums of the tiles' partial sums, FP32 in fours and FP64 over them (FP64
-// throughout on the FP64 path), to the G and moment arrays: dst = region << 28
+// throughout on the FP64 path and for the moments, which follow the tap sums'
+// nout outputs), to the G and moment arrays: dst = region << 28
 // | offset, -1 = not needed.
 struct TapDst {
   double* base[5];
@@ -157,12 +159,24 @@ constexpr int kRedOut = 8, kRedGroups = 64;
 
 template <typename T>
 __global__ void __launch_bounds__(kRedOut * kRedGroups)
-k_tap_reduce(const T* __restrict__ part, const int* __restrict__ dst, TapDst d, int ntile, int nout) {
-  __shared__ double red[kRedGroups][kRedOut + 1];
-  const int ccd = blockIdx.y, lane = threadIdx.x % kRedOut, g = threadIdx.x / kRedOut;
-  const int o = blockIdx.x * kRedOut + lane;
+k_tap_reduce(const T* __restrict__ part, const double* __restrict__ mpart, const int* __restrict__ dst, TapDst d,
+             int ntile, int nout) {
+  constexpr int NTH = kRedOut * kRedGroups;
+  __shared__ double red[kRedGroups * (kRedOut + 1)];
+  const int ccd = blockIdx.y, ntap = (nout + kRedOut - 1) / kRedOut;
+  const bool mom = (int)blockIdx.x >= ntap;
+  // lanes: the outputs of the CTA; groups of tiles
+  const int nl = mom ? 1 : kRedOut, lane = threadIdx.x % nl, g = threadIdx.x / nl;
+  const int o = mom ? nout + (int)blockIdx.x - ntap : (int)blockIdx.x * kRedOut + lane;
+  const int q = o < nout || mom ? dst[o] : -1;
+  if (mom && q < 0) return;
   double s = 0.0;
-  if (o < nout) {
+  if (mom) {
+    // one output per CTA: FP64 additions of a CTA run one warp after another
+    const double* p = mpart + (int64_t)ccd * ntile * kTapMom + o - nout;
+#pragma unroll 4
+    for (int t = g; t < ntile; t += NTH) s += p[(int64_t)t * kTapMom];
+  } else if (o < nout) {
     const T* p = part + (int64_t)ccd * ntile * nout + o;
     int t = g * 4;
 #pragma unroll 2
@@ -173,19 +187,16 @@ k_tap_reduce(const T* __restrict__ part, const int* __restrict__ dst, TapDst d, 
     }
     for (int k = t; k < min(t + 4, ntile); ++k) s += (double)p[(int64_t)k * nout];
   }
-  red[g][lane] = s;
+  const int pitch = mom ? 1 : kRedOut + 1;
+  red[g * pitch + lane] = s;
   __syncthreads();
-#pragma unroll
-  for (int k = kRedGroups / 2; k > 0; k >>= 1) {
-    if (g < k) red[g][lane] += red[g + k][lane];
+  for (int k = NTH / nl / 2; k > 0; k >>= 1) {
+    if (g < k) red[g * pitch + lane] += red[(g + k) * pitch + lane];
     __syncthreads();
   }
-  if (g == 0 && o < nout) {
-    const int q = dst[o];
-    if (q >= 0) {
-      const int r = q >> 28;
-      d.base[r][ccd * d.stride[r] + (q & 0xfffffff)] = red[0][lane];
-    }
+  if (g == 0 && q >= 0) {
+    const int r = q >> 28;
+    d.base[r][ccd * d.stride[r] + (q & 0xfffffff)] = red[lane];
   }
 }
 
@@ -618,7 +629,9 @@ void build_tap_plan(sfft_plan_s* p) {
     }
   };
   auto moments = [&](std::vector<int4>& tasks, std::vector<int>& dst, bool fit) {
-    tasks.push_back(int4{TAP_MOM | 36 << 8, 0, 0, (int)dst.size()});
+    // partial sums of their own; first, since its chain of FP64 sums is the longest of a small image's tasks
+    // (160 x 192, L = 5: 13.4 us, 15.9 with the task last)
+    tasks.insert(tasks.begin(), int4{TAP_MOM | kTapMom << 8, 0, 0, 0});
     const int64_t corner = (int64_t)(L * L - 1) * nkb;   // the single offset (w, w)
     for (int m = 0; m < 15; ++m) dst.push_back(fit && m < n_mono(2 * DB) ? q(3, m) : -1);
     for (int m = 0; m < 6; ++m) dst.push_back(m < n_mono(DB) ? q(4, m) : -1);
@@ -642,9 +655,9 @@ void build_tap_plan(sfft_plan_s* p) {
   for (int uy = -w; uy <= w; ++uy) add(rhs_tasks, rhs_dst, TAP_S, 0, 0, uy);
   moments(rhs_tasks, rhs_dst, false);
   t.ntask = (int)t.tasks.size();
-  t.nout = (int)t.dst.size();
+  t.nout = (int)t.dst.size() - kTapMom;
   t.ntask_rhs = (int)rhs_tasks.size();
-  t.nout_rhs = (int)rhs_dst.size();
+  t.nout_rhs = (int)rhs_dst.size() - kTapMom;
   t.tasks.insert(t.tasks.end(), rhs_tasks.begin(), rhs_tasks.end());
   t.dst.insert(t.dst.end(), rhs_dst.begin(), rhs_dst.end());
   // wide tiles amortise the halo and the fold of yt^b; a small image takes
@@ -692,15 +705,23 @@ void build_tap_plan(sfft_plan_s* p) {
 }
 
 // ------------------------------------------------------------------ launchers
-void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs, size_t* list, size_t* cnt) {
+void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* mpart, size_t* hp, size_t* hs, size_t* list, size_t* cnt) {
   const TapPlan& t = p->tap;
   const size_t B = p->d.batch;
   *part = p->elem * B * std::max((size_t)t.ntile * t.nout, (size_t)t.ntile_rhs * t.nout_rhs);
+  *mpart = sizeof(double) * B * std::max(t.ntile, t.ntile_rhs) * kTapMom;
   const bool edge = t.mode == TAP_FIT_EDGE;
   *hp = edge ? sizeof(double) * B * ((size_t)t.gy * t.npy + (size_t)t.gx * t.npx) * t.MP : 0;   // FP32: pairs
   *hs = edge ? sizeof(double) * B * (size_t)(t.npy + t.npx) * t.MP : 0;
   *list = edge ? 2 * sizeof(unsigned) * B * (size_t)edge_cap(p) : 0;
   *cnt = edge ? 2 * sizeof(int) * B * (size_t)(p->d.H + 1) : 0;
+}
+
+// how many moments of M, of s and of c a fit (or its right-hand side) takes
+char3 tap_moment_need(const sfft_plan_s* p, bool fit) {
+  const bool edge = p->tap.mode == TAP_FIT_EDGE;
+  return char3{(signed char)(fit ? n_mono(p->DM_BB) : 0), (signed char)n_mono(p->d.DB),
+               (signed char)(fit && edge ? n_mono(p->DM_KB) : 0)};
 }
 
 // one pixel in xt or yt
@@ -716,7 +737,7 @@ static cudaError_t tap_sums(const sfft_plan_s* p, const float* S, void* ws) {
   dim3 grid(t.ntile, t.nsplit, p->d.batch);
   kern<<<grid, kTapWarps * 32, smem, p->stream>>>(ws_at<T>(ws, p->rm), S, ws_at<unsigned>(ws, p->mfitw),
                                                   ws_at<double>(ws, p->sky), t.d_tasks, t.ntask,
-                                                  ws_at<T>(ws, p->tappart), t.nout, p->d.H, p->d.W, p->w, t.tw,
+                                                  ws_at<T>(ws, p->tappart), t.nout, ws_at<double>(ws, p->mompart), tap_moment_need(p, true), p->d.H, p->d.W, p->w, t.tw,
                                                   step_of(p->d.W), step_of(p->d.H));
   p->nlaunch += 1;
   return cudaGetLastError();
@@ -740,8 +761,8 @@ static cudaError_t tap_reduce(const sfft_plan_s* p, bool rhs, void* ws) {
   const int64_t stride[5] = {(int64_t)p->n_hd * LL * n_mono(p->DM_KK), (int64_t)LL * n_mono(p->DM_KB),
                              (int64_t)LL * n_mono(p->DM_bK), n_mono(p->DM_BB), n_mono(p->d.DB)};
   for (int i = 0; i < 5; ++i) { d.base[i] = ws_at<double>(ws, *reg[i]); d.stride[i] = stride[i]; }
-  k_tap_reduce<T><<<dim3((nout + kRedOut - 1) / kRedOut, p->d.batch), kRedOut * kRedGroups, 0, p->stream>>>(
-      ws_at<T>(ws, p->tappart), t.d_dst + (rhs ? t.nout : 0), d, rhs ? t.ntile_rhs : t.ntile, nout);
+  k_tap_reduce<T><<<dim3((nout + kRedOut - 1) / kRedOut + kTapMom, p->d.batch), kRedOut * kRedGroups, 0, p->stream>>>(
+      ws_at<T>(ws, p->tappart), ws_at<double>(ws, p->mompart), t.d_dst + (rhs ? t.nout + kTapMom : 0), d, rhs ? t.ntile_rhs : t.ntile, nout);
   p->nlaunch += 1;
   return cudaGetLastError();
 }

@@ -128,7 +128,7 @@ struct sfft_plan_s {
   // workspace regions (per-CCD strides where noted)
   sfft::Region sky, skyacc, good, gh, mfit, rowflag, rm, wspec, uspec, rhat, phat, gkk, gkb, gbk,
       mom_bb, mom_b, eimg, lfac, scale, dinv, gbar, swave, vec, theta_off, status, cbuf,
-      tappart, hpart, hsum, elist, ecnt, goodw, mfitw;
+      tappart, mompart, hpart, hsum, elist, ecnt, goodw, mfitw;
   size_t ws_bytes = 0;
   // graph cache for sfft_subtract
   std::map<std::vector<uintptr_t>, cudaGraphExec_t> graphs;
@@ -166,7 +166,8 @@ cudaError_t launch_lag_dft(const sfft_plan_s* p, int batch_index, int c0, int nc
 cudaError_t launch_contract_slot0(const sfft_plan_s* p, int DM, int job0, int njobs, void* ws);
 // image-space assembly
 void build_tap_plan(sfft_plan_s* p);
-void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* hp, size_t* hs, size_t* list, size_t* cnt);
+void tap_region_bytes(const sfft_plan_s* p, size_t* part, size_t* mpart, size_t* hp, size_t* hs, size_t* list, size_t* cnt);
+char3 tap_moment_need(const sfft_plan_s* p, bool fit);
 cudaError_t launch_tap_fit(const sfft_plan_s* p, const float* S, void* ws);
 cudaError_t launch_tap_rhs_reduce(const sfft_plan_s* p, void* ws);
 int conv_half_width(int H, int W, int batch);

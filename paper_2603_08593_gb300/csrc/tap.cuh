@@ -98,6 +98,7 @@ constexpr int kTapU = 8;          // pixels per unrolled step
 constexpr int kTapScr = 16;       // staged rows of the y fold per warp
 constexpr int kTapScrPitch = 36;
 constexpr int kTapMaxOut = 40;
+constexpr int kTapMomS = 15, kTapMomC = 21, kTapMom = 36;   // moments: of M, of s from kTapMomS, of c from kTapMomC
 
 // outputs of each task type: (row of powers, power of yt), in monomial order
 __device__ __forceinline__ void tap_outputs(int type, int DK, unsigned char (*ot)[2]) {
@@ -237,9 +238,13 @@ __device__ __forceinline__ void tap_task(const TapTile<T>& t, int u0x, int u0y, 
   }
 }
 
-// Moments without taps (FIT; else those of s alone): M xt^a (a <= 4), s xt^a (a <= 2), c xt^a (a <= 4), c = M R(. - (w, w))
+// Moments without taps (FIT; else those of s alone): M xt^a (a <= 4), s xt^a (a <= 2), c xt^a (a <= 4),
+// c = M R(. - (w, w)).  The background block of A, b_B and the corner of the kernel-background block come from
+// these alone, so only a row's sums over the run are in T, in groups of kTapU; yt^b and the sums over rows are
+// FP64 (ypd: [5][32]; with FP32 powers and sums over the rows A's block was off by 1.2e-7, now by 2e-8).
 template <typename T, bool FIT>
-__device__ __forceinline__ void tap_moments(const TapTile<T>& t, int wt, int w, int nout, T* __restrict__ out) {
+__device__ __forceinline__ void tap_moments(const TapTile<T>& t, int wt, int w, const double (*ypd)[32], char3 need,
+                                            double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const T* cr = t.r + (wt - w) * t.pitch + (wt - w);
   const T* sr = t.s;
@@ -247,28 +252,52 @@ __device__ __forceinline__ void tap_moments(const TapTile<T>& t, int wt, int w, 
   T acc[13];
 #pragma unroll
   for (int a = 0; a < 13; ++a) acc[a] = 0;
-  for (int x = 0; x < t.n; ++x) {
-    const bool on = FIT && ((mr[x >> 5] >> (x & 31)) & 1u);
-    const T m = on ? (T)1 : (T)0, c = on ? cr[x] : (T)0, s = sr[x];
-    const T* xp = t.xp + 4 * x;
-    acc[5] += s;
-    acc[6] += s * xp[0];
-    acc[7] += s * xp[1];
-    if (FIT) {
-      acc[0] += m;
-      acc[8] += c;
+  for (int x0 = 0; x0 < t.n; x0 += kTapU) {
+    T g[13];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        acc[1 + a] += m * xp[a];
-        acc[9 + a] += c * xp[a];
+    for (int a = 0; a < 13; ++a) g[a] = 0;
+#pragma unroll
+    for (int x = x0; x < x0 + kTapU; ++x) {
+      const bool on = FIT && ((mr[x >> 5] >> (x & 31)) & 1u);
+      const T m = on ? (T)1 : (T)0, c = on ? cr[x] : (T)0, s = sr[x];
+      const T* xp = t.xp + 4 * x;
+      g[5] += s;
+      g[6] += s * xp[0];
+      g[7] += s * xp[1];
+      if (FIT) {
+        g[0] += m;
+        g[8] += c;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          g[1 + a] += m * xp[a];
+          g[9 + a] += c * xp[a];
+        }
       }
     }
+#pragma unroll
+    for (int a = 0; a < 13; ++a) acc[a] += g[a];
   }
   __syncwarp();
 #pragma unroll
   for (int a = 0; a < 13; ++a) t.scr[a * kTapScrPitch + lane] = acc[a];
   __syncwarp();
-  for (int o = lane; o < nout; o += 32) out[o] = fold_row(t, t.ot[o][0], t.ot[o][1]);
+  // the first need.x outputs of M, need.y of s and need.z of c; a quarter of the rows per lane: an FP64
+  // instruction occupies its pipe for 16 cycles whatever its lanes do
+  const int n = need.x + need.y + need.z;
+#pragma unroll 1
+  for (int k0 = 0; k0 < 4 * n; k0 += 32) {
+    int o = min((k0 + lane) / 4, n - 1);
+    const int r0 = 8 * (lane & 3);
+    o = o < need.x ? o : (o - need.x < need.y ? o - need.x + kTapMomS : o - need.x - need.y + kTapMomC);
+    const T* v = t.scr + t.ot[o][0] * kTapScrPitch + r0;
+    const double* y = ypd[t.ot[o][1]] + r0;
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s = fma((double)v[i], y[i], s);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if ((lane & 3) == 0) out[o] = s;
+  }
 }
 
 }  // namespace sfft
