@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 
 #include "common.cuh"
 #include "plan.h"
@@ -36,6 +37,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // What one statistics pass hands to the next, and the last one to the filter
 struct PassStats {
   float shift, lo, hi;   // the next pass sums about shift the pixels in [lo, hi]
+  int about0;            // ... with the loop's sums about zero, and no value that float arithmetic could lose
   float scale;           // 1 / (sigma_D ||G||)
 };
 
@@ -63,6 +65,24 @@ struct DetectLayout {
 
 using sfft::two_sum;
 
+// (s, e, f) += x, and e and f alone for an x below s's last place
+__device__ __forceinline__ void add_low(float& e, float& f, float x) {
+  float u;
+  e = two_sum(e, x, u);
+  f += u;
+}
+__device__ __forceinline__ void add_triple(float& s, float& e, float& f, float x) {
+  float r;
+  s = two_sum(s, x, r);
+  add_low(e, f, r);
+}
+// two_sum of both halves, in packed instructions
+__device__ __forceinline__ float2 two_sum2(float2 x, float2 y, float2& e) {
+  const float2 m1 = make_float2(-1.f, -1.f), s = __fadd2_rn(x, y), t = __ffma2_rn(x, m1, s);   // products by -1 are exact
+  e = __fadd2_rn(__ffma2_rn(__ffma2_rn(t, m1, s), m1, x), __ffma2_rn(t, m1, y));
+  return s;
+}
+
 // the clipping rule of a pass
 __device__ __forceinline__ bool kept(float x, double mean, double thr) { return fabs((double)x - mean) <= thr; }
 
@@ -74,15 +94,23 @@ __device__ __forceinline__ unsigned float_key(float x) {
 __device__ __forceinline__ float key_float(unsigned k) { return __uint_as_float(k ^ (k >> 31 ? 0x80000000u : 0xffffffffu)); }
 
 // One statistics pass over the rows blockIdx.x, blockIdx.x + gridDim.x, ...
-// Sums n, sum d, sum d^2 of d = x - shift in pairs of floats (two-sums and an
-// exact product, about 2^-46 relative: FP64 additions run at 1/64 of the FP32
-// rate and took 70 us per pass of 2048 x 4096), FP64 from the thread's end on.
+// Sums n, sum d, sum d^2 of d = x - shift in triples of floats: d as an exact
+// pair, its square with every term down to 2^-48, and both sums with their
+// rounding errors summed exactly once more, so that what is left is below an
+// FP64 sum's error (1e-16 of a thread's sum; FP64 additions, at 1/64 of the FP32
+// rate, left 7e-16 and took 70 us per pass of 2048 x 4096, pairs of floats 5e-15
+// and 25 us, these 28 us).  FP64 from the thread's end on.  Where the mean lies
+// within three times the scatter, as it does in a difference image, the loop sums
+// about zero, where d is one float (9 us for the four passes), and the thread's
+// triples are moved to the shift at its end: they hold some 70 bits, of which
+// that takes a few.
 // The loop is without branches but for values whose square leaves the range of a
-// float, which wait for the word group's end (4096 x 2048: 30.7 us a pass with
-// the branches, 28.6 us without).  What bounds a pass are its issue slots and, of
-// a small image, the last CTA's chain of FP64 operations: warp 0 tests the
-// candidates of both interval ends at once, and a pass forms only what the next
-// kernel reads (128 x 128: 11.4 -> 9.4 us a pass; 4096 x 2048: 28.6 -> 25.5 us).
+// float, which wait for the word group's end.  What bounds a pass is the wait for
+// its pixels between the arithmetic of two word groups (more of them in flight
+// cost a CTA per SM: 207 against 204 us for the detector) and, of a small image,
+// the last CTA's chain of FP64 operations: warp 0 tests the candidates of both
+// interval ends at once, and a pass forms only what the next kernel reads
+// (128 x 128: 11.4 -> 9.4 us a pass).
 // The last CTA to finish adds the partials in index order and prepares the next
 // pass: its clipping rule |x - mean| <= 3 sqrt(var), evaluated in FP64, becomes
 // the float interval of the pixels that satisfy it (the rule is monotone on
@@ -100,9 +128,11 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
   unsigned* bw = badw + (int64_t)b * H * nw;
   double* pb = part + (int64_t)b * kStatBlocks * 3;
   float shift = 0.f, lo = 0.f, hi = 0.f;
-  if (!FIRST) { shift = stats[b].shift; lo = stats[b].lo; hi = stats[b].hi; }
-  int n = 0;
-  float s1 = 0.f, e1 = 0.f, s2 = 0.f, e2 = 0.f;
+  bool about0 = true;
+  if (!FIRST) { shift = stats[b].shift; lo = stats[b].lo; hi = stats[b].hi; about0 = stats[b].about0 != 0; }
+  int n = 0, n_wide = 0;   // pixels, and those among them in b1 and b2
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 s = zero, e = zero, f = zero;   // sum d in .x, sum d^2 in .y
   double b1 = 0.0, b2 = 0.0;
   constexpr int U = kClipWords;
   const int ng = (nw + U - 1) / U, nit = ((H - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) * ng;
@@ -121,52 +151,84 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
       else m[k] = w0 + k < nw ? gw[(int64_t)y * nw + w0 + k] : 0u;
     }
     unsigned wide = 0;   // words whose square or its error leaves the range of a float
+    auto group = [&](auto about0) {   // about0: the shift is zero, and d the pixel's value
+      constexpr bool ABOUT0 = decltype(about0)::value;
 #pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int x = (w0 + k) * 32 + lane;
-      bool ok;
-      if (FIRST) {
-        const bool isbad = m[k] != 0u;
-        ok = x < W && !isbad && isfinite(v[k]);
-        const unsigned g = __ballot_sync(0xffffffffu, ok), q = __ballot_sync(0xffffffffu, isbad);
-        if (lane == 0 && w0 + k < nw) {
-          gw[(int64_t)y * nw + w0 + k] = g;
-          if (bb) bw[(int64_t)y * nw + w0 + k] = q;
+      for (int k = 0; k < U; ++k) {
+        const int x = (w0 + k) * 32 + lane;
+        bool ok;
+        if (FIRST) {
+          const bool isbad = m[k] != 0u;
+          ok = x < W && !isbad && isfinite(v[k]);
+          const unsigned g = __ballot_sync(0xffffffffu, ok), q = __ballot_sync(0xffffffffu, isbad);
+          if (lane == 0 && w0 + k < nw) {
+            gw[(int64_t)y * nw + w0 + k] = g;
+            if (bb) bw[(int64_t)y * nw + w0 + k] = q;
+          }
+        } else {
+          ok = ((m[k] >> lane) & 1u) && v[k] >= lo && v[k] <= hi;
         }
-      } else {
-        ok = ((m[k] >> lane) & 1u) && v[k] >= lo && v[k] <= hi;
+        ok = ok && row_in && x >= kMargin && x < W - kMargin;
+        n += ok;
+        // a pixel that does not count adds zeros, which change no sum
+        float dl = 0.f;
+        float d = ABOUT0 ? v[k] : two_sum(v[k], -shift, dl);
+        if (FIRST || !ABOUT0) {
+          const float ad = fabsf(d);
+          if (ok && (ad > 1e17f || (ad < 1e-12f && ad > 0.f))) wide |= 1u << k;
+          ok = ok && !(wide >> k & 1u);
+        }
+        d = ok ? d : 0.f;
+        dl = ok ? dl : 0.f;
+        const float p = __fmul_rn(d, d), pe = __fmaf_rn(d, d, -p);
+        float2 r, u;
+        s = two_sum2(s, make_float2(d, p), r);
+        e = two_sum2(e, r, u);
+        f = __fadd2_rn(f, u);
+        add_low(e.y, f.y, pe);
+        if (!ABOUT0) {   // d's second float, and the square's terms in it
+          add_low(e.x, f.x, dl);
+          const float q = __fmul_rn(2.f * d, dl);
+          add_low(e.y, f.y, q);
+          f.y += __fmaf_rn(dl, dl, __fmaf_rn(2.f * d, dl, -q));
+        }
       }
-      ok = ok && row_in && x >= kMargin && x < W - kMargin;
-      n += ok;
-      // a pixel that does not count adds zeros, which change no sum
-      float dl = 0.f, t;
-      float d = FIRST ? v[k] : two_sum(v[k], -shift, dl);
-      const float ad = fabsf(d);
-      if (ok && (ad > 1e18f || (ad < 1e-12f && ad > 0.f))) wide |= 1u << k;
-      ok = ok && !(wide >> k & 1u);
-      d = ok ? d : 0.f;
-      dl = ok ? dl : 0.f;
-      s1 = two_sum(s1, d, t);
-      e1 += t + dl;
-      const float p = __fmul_rn(d, d), pe = __fmaf_rn(2.f * d, dl, __fmaf_rn(d, d, -p));
-      s2 = two_sum(s2, p, t);
-      e2 += t + pe;
-    }
+    };
+    if (about0) group(std::true_type{});
+    else group(std::false_type{});
     if (wide) {
 #pragma unroll
       for (int k = 0; k < U; ++k)
         if (wide >> k & 1u) {
+          ++n_wide;
           float dl = 0.f;
-          const float d = FIRST ? v[k] : two_sum(v[k], -shift, dl);
+          const float d = two_sum(v[k], -shift, dl);
           const double dd = (double)d + (double)dl;
           b1 += dd;
           b2 += dd * dd;
         }
     }
   }
+  if (!FIRST && about0) {
+    // sum (x - c) = S1 - n c and sum (x - c)^2 = S2 - c (S1 + (S1 - n c)), c the shift
+    const float c = shift, nf = (float)(n - n_wide), p = __fmul_rn(nf, c);
+    float3 o = make_float3(s.x, e.x, f.x);
+    add_triple(s.x, e.x, f.x, -p);
+    add_low(e.x, f.x, -__fmaf_rn(nf, c, -p));
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float q = __fmul_rn(c, o.x), ql = __fmul_rn(c, o.y);
+      add_triple(s.y, e.y, f.y, -q);
+      add_low(e.y, f.y, -__fmaf_rn(c, o.x, -q));
+      add_low(e.y, f.y, -ql);
+      f.y -= __fmaf_rn(c, o.y, -ql) + c * o.z;
+      o = make_float3(s.x, e.x, f.x);
+    }
+  }
   __shared__ double red[3][8];
   __shared__ bool last;
-  double v[3] = {(double)__reduce_add_sync(0xffffffffu, n), (double)s1 + (double)e1 + b1, (double)s2 + (double)e2 + b2};
+  double v[3] = {(double)__reduce_add_sync(0xffffffffu, n), (double)s.x + ((double)e.x + (double)f.x) + b1,
+                 (double)s.y + ((double)e.y + (double)f.y) + b2};
   for (int q = 1; q < 3; ++q) v[q] = sfft::warp_sum(v[q]);
   if (lane == 0)
     for (int q = 0; q < 3; ++q) red[q][warp] = v[q];
@@ -216,6 +278,7 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
   const bool any = inl != 0u && inh != 0u;
   if (lane == 0) {
     stats[b].shift = (float)mean;
+    stats[b].about0 = fabs(mean) <= thr && thr <= 1e16 && thr >= 1e-9;
     stats[b].lo = any ? lo_x : INFINITY;
     stats[b].hi = any ? hi_x : -INFINITY;
   }
