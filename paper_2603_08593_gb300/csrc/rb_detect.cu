@@ -227,8 +227,12 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
   }
   __shared__ double red[3][8];
   __shared__ bool last;
-  double v[3] = {(double)__reduce_add_sync(0xffffffffu, n), (double)s.x + ((double)e.x + (double)f.x) + b1,
-                 (double)s.y + ((double)e.y + (double)f.y) + b2};
+  double v[3] = {(double)__reduce_add_sync(0xffffffffu, n), (double)s.x + ((double)e.x + (double)f.x),
+                 (double)s.y + ((double)e.y + (double)f.y)};
+  if (n_wide) {
+    v[1] += b1;
+    v[2] += b2;
+  }
   for (int q = 1; q < 3; ++q) v[q] = sfft::warp_sum(v[q]);
   if (lane == 0)
     for (int q = 0; q < 3; ++q) red[q][warp] = v[q];
@@ -245,18 +249,17 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
   __syncthreads();
   if (!last) return;
   __threadfence();
-  double t[3] = {0.0, 0.0, 0.0};
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x)
-    for (int q = 0; q < 3; ++q) t[q] += __ldcg(pb + i * 3 + q);
-  for (int q = 0; q < 3; ++q) t[q] = sfft::warp_sum(t[q]);
-  if (lane == 0)
-    for (int q = 0; q < 3; ++q) red[q][warp] = t[q];
+  // a warp per sum: an FP64 addition occupies its pipe for 16 cycles whatever the lanes hold
+  if (warp < 3) {
+    double a = 0.0;
+#pragma unroll 4
+    for (int i = lane; i < (int)gridDim.x; i += 32) a += __ldcg(pb + i * 3 + warp);
+    a = sfft::warp_sum(a);
+    if (lane == 0) red[warp][0] = a;
+  }
   __syncthreads();
   if (warp != 0) return;
-  for (int q = 0; q < 3; ++q) {
-    t[q] = 0.0;
-    for (int w = 0; w < 8; ++w) t[q] += red[q][w];
-  }
+  const double t[3] = {red[0][0], red[1][0], red[2][0]};
   const double m1 = t[1] / t[0];
   const double mean = (double)shift + m1, var = t[2] / t[0] - m1 * m1;
   if (pass == kStatPasses - 1) {   // only the matched filter's scale is left to form
