@@ -1,4 +1,7 @@
-"""A plan-time tuning of which every candidate fails (the only candidate's first
+"""Plan-time tuning: the tiles that it reports reach a plan of the spectral
+assembly that is given them, and give the same normal equations.
+
+A plan-time tuning of which every candidate fails (the only candidate's first
 device allocation is made to fail): an image-space plan, which runs without
 the tuned tiles, is made and gives the fit; a plan of the spectral assembly is
 refused and leaves nothing behind."""
@@ -41,3 +44,23 @@ def test_spectral_plan_still_reports_failed_tuning(monkeypatch):
     monkeypatch.setenv("SFFT_FAIL_ALLOC", "1")
     assert lib.sfft_plan(ctypes.byref(desc), None, ctypes.byref(h)) == binding.SFFT_ERR_CUDA
     assert h.value is None and lib.sfft_debug_live_allocations() == before
+
+
+def test_tuned_tiles_run_in_a_spectral_plan():
+    """The two assemblies of one pair, each within the stated 2e-5 of max|A|."""
+    from paper_2603_08593_gb300 import Plan
+    L, DK, DB = 5, 1, 1
+    d = small_pair(300, 210, seed=6301, mask_fraction=0.02)
+    dev = [torch.from_numpy(d[k])[None].cuda() for k in ("R", "S", "bad")]
+    sky = torch.tensor([[1000.0, 1001.0]], dtype=torch.float64, device="cuda")
+    pt = Plan(300, 210, L, DK, DB, batch=1, prec="mixed", autotune=1)
+    ps = Plan(300, 210, L, DK, DB, batch=1, prec="mixed", d_batch=pt.tiles[0], rows_per_cta=pt.tiles[1],
+              lag_parts=pt.tiles[2])
+    assert ps.tiles == pt.tiles
+    ps.profile()
+    (A, b), (As, bs) = pt.build_normal(*dev, sky), ps.build_normal(*dev, sky)
+    torch.cuda.synchronize()
+    prof = ps.profile_read()
+    assert prof["fft_prod"][1] > 0 and prof["fft_weights"][1] > 0      # it did form spectra
+    assert float((A - As).abs().max()) <= 4e-5 * float(As.abs().max())
+    assert float((b - bs).abs().max()) <= 4e-5 * float(bs.abs().max())

@@ -69,3 +69,28 @@ def test_exposure_batch_matches_oracle(exposure, mode):
         o = p.subtract(R, S, bad, None, refine=1, out=o)    # graph replay
     s.synchronize()
     _check(o, pairs, refs)
+
+
+def test_default_plan_batch_matches_oracle(exposure):
+    """The call as users make it, no tile field set: four CCDs (the first one
+    twice, whose outputs are then the same bits) through the image-space
+    assembly, graph capture and replay."""
+    from paper_2603_08593_gb300 import Plan
+    pairs, refs = exposure
+    pairs, refs = pairs + pairs[:1], refs + refs[:1]
+    dev = torch.device("cuda", torch.cuda.current_device())
+    R, S, bad = (torch.from_numpy(np.stack([d[k] for d in pairs])).to(dev) for k in ("R", "S", "bad"))
+    s = torch.cuda.Stream(device=dev)
+    with torch.cuda.stream(s):
+        p = Plan(4096, 2048, L, DK, DB, batch=len(pairs), prec="mixed", graph=True, stream=s, device=dev)
+        o = p.subtract(R, S, bad, None, refine=1)
+        s.synchronize()
+        _check(o, pairs, refs)
+        for k in ("theta", "D", "info"):
+            o[k].zero_()
+        o = p.subtract(R, S, bad, None, refine=1, out=o)    # graph replay
+    s.synchronize()
+    _check(o, pairs, refs)
+    for k in ("A", "b", "theta"):
+        assert torch.equal(o[k][0], o[k][3])
+    assert torch.equal(o["D"][0].nan_to_num(), o["D"][3].nan_to_num())
