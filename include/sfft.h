@@ -137,9 +137,9 @@ sfft_status_t sfft_plan_tiles(sfft_plan_t plan, int32_t* out3);
 int32_t       sfft_plan_ccd_group(sfft_plan_t plan);
 /* Failure detection (no counterpart in the paper).  The FP64 factorisation
  * separates its block steps by a grid-wide barrier whose wait is bounded:
- * after `tries` polls (each at least 64 ns) a CTA gives up, every CCD of the
+ * after `tries` polls (0.3 to 0.5 us each) a CTA gives up, every CCD of the
  * call gets SFFT_ERR_TIMEOUT in `info` and the kernel returns with the
- * context intact.  The default (about a second) applies after plan creation
+ * context intact.  The default (2^24: some six seconds) applies after plan creation
  * and again for tries < 0; small values let a test make the wait run out.
  * The barrier is a software flag wait with no asynchronous copies or
  * tensor-core work in flight, so giving up leaves nothing pending. */

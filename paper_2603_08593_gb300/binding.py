@@ -229,7 +229,7 @@ class Plan:
             pass
 
     def set_wait_limit(self, tries):
-        """Polls before the factorisation's grid-barrier wait gives up (< 0: the default, about a second)."""
+        """Polls before the factorisation's grid-barrier wait gives up (< 0: the default, some six seconds)."""
         _check(self.lib.sfft_plan_set_wait_limit(self.h, int(tries)), "sfft_plan_set_wait_limit")
 
     def set_stream(self, stream):

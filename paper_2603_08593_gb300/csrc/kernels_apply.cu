@@ -89,8 +89,10 @@ struct ConvArgs {
   unsigned magic;          // ceil(2^20 / groups per staged row)
 };
 
-// Two CTAs per SM; FP64 only where window and sums fit 128 registers without
-// spills (L = 7, D_K = 1, one 512 x 512 pair: 64.8 us, 121.5 us at one CTA)
+// Two CTAs per SM; FP64 only where window and sums fit 128 registers (L = 7,
+// D_K = 1, one 512 x 512 pair: 64.8 us, 121.5 us at one CTA) or miss them by a few
+// spilled values (L = 3, D_K = 2: 44 bytes, 102 us per 1024 x 1024 against 105 at one
+// CTA; the residual image at L = 11, D_K = 0: 16 bytes)
 template <typename T, int NT, int DK, int MODE>
 __global__ void __launch_bounds__(kCvWarps * 32, sizeof(T) == 4 || NT * (DK + 1) <= 14 ? 2 : 1)
 k_conv(const ConvArgs<T> a) {

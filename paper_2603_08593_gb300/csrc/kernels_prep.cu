@@ -276,8 +276,8 @@ k_moments(const uint8_t* __restrict__ mfit, const float* __restrict__ S, const d
 }
 
 // ------------------------------------------------------------------ masks as bits, mask edges
-// R_m and the good pixels as bits: a warp per run of words, eight in flight.
-// 17 bytes in and 4 (8) out per pixel; the byte masks it replaces cost two
+// R_m and the good pixels as bits: a warp per run of words, four in flight.
+// 9 bytes in (R, S, bad) and 4 (FP64: 8) out per pixel; the byte masks it replaces cost two
 // more passes over the image (k_prep, k_erode_rows and k_erode_cols: 94 us per
 // 2048 x 4096 CCD).
 template <typename T>

@@ -42,7 +42,7 @@ __host__ __device__ constexpr size_t tap_smem(int wt, int tw) {
 // One CTA: a tile of 32 rows x tw columns and every nsplit-th task of the
 // table, taken in order by its warps.  Partial sums go to
 // part[ccd][tile][nout_tot]; k_tap_reduce adds the tiles in FP64.
-// One 4096 x 2048 CCD, L = 11, D_K = 2: 497 us = 50 TFLOP/s, 0.65 of the FP32
+// One 4096 x 2048 CCD, L = 11, D_K = 2: 502 us = 49 TFLOP/s, 0.65 of the FP32
 // FMA peak (the row FFTs of the 221 products and their contraction took 6.0 ms);
 // copies of the tile through registers took 638 us, R stored as
 // operand pairs (two CTAs of six warps instead of three of four) 572 us.
@@ -215,7 +215,9 @@ k_tap_reduce(const T* __restrict__ part, const double* __restrict__ mpart, const
 // 11.1 -> 6.4 ms, bad rows every 16 8.2 -> 4.4 ms (6.9 and 6.8 ms from spectra);
 // four of 1024 x 2048, L = 7, bad pixels every 8 px 9.2 -> 2.0 ms (4.2 ms); one
 // with saturated stars and two dead columns: 80 us in this kernel, 96 before.
-// What bounds it are issue slots and shared-memory reads (about half of either).
+// What bounds it are issue slots and shared-memory reads (about half of either);
+// at D_K = 2 the 80 registers of sums leave spills of 68 bytes (FP64: 24), not in the
+// loop over points.
 // Slot g of U takes batches g, g + U, ..., at least kGramMin<T> points, and writes
 // hp[ccd][slot][pair][NM]; a short list uses few slots.  The x-edge blocks, whose
 // lists are the longer, come first.  The number of slots has a limit, a slot's
@@ -594,6 +596,12 @@ void build_tap_plan(sfft_plan_s* p) {
   const int nkk = n_mono(dKK), nkb = n_mono(dKB), nbk = n_mono(DK);
   TapPlan& t = p->tap;
   t.nt = std::max(L, 3);
+  // The line is right for the small images of small kernels and lies at L alone:
+  // assembly by every pair against edge sums, in us, L = 5, D_K = 2 (L = 3) on
+  // the mixed path: 160 x 192 59 / 106 (50 / 102), 512 x 512 92 / 118 (57 / 110),
+  // 1024 x 1024 189 / 133 (78 / 119), 4096 x 2048 894 / 306 (259 / 235); FP64
+  // 1024 x 1024 5331 / 976 (1059 / 506).  Row spectra took 2545 us where every
+  // pair takes 894, and 9990 where it takes 5331.
   t.mode = L <= 5 ? TAP_FIT_ALL : TAP_FIT_EDGE;
   const int wt = (t.nt - 1) / 2;
   auto half_id = [&](int dy, int dx) {

@@ -96,7 +96,7 @@ struct sfft_plan_s {
   sfft::TapPlan tap;
   int tc_rows = 0;                    // weight rows per CTA of the tensor-core contraction
   double tuned_ms = 0.0;              // autotuned build_normal time per CCD (0: not tuned)
-  int bar_spin_limit = 1 << 24;       // tries of the factorisation's grid-barrier wait (about a second)
+  int bar_spin_limit = 1 << 24;       // tries of the factorisation's grid-barrier wait (some six seconds)
   size_t elem = 4;                    // sizeof(T)
   // plan-owned constant device tables
   void* twM = nullptr;                // c_t [M]       exp(-2 pi i j / M)
