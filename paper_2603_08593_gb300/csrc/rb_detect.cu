@@ -225,24 +225,50 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
       o = make_float3(s.x, e.x, f.x);
     }
   }
-  __shared__ double red[3][8];
+  // The threads' triples are joined as triples, four at a time in shared memory,
+  // and the CTA's goes to FP64: an FP64 instruction occupies its pipe for 16
+  // cycles, and conversions and shuffled additions in every warp took 5 us of a pass.
+  __shared__ float tr[6][256];
+  __shared__ double rb[2][8], red[3];
+  __shared__ int rn[8], any_wide;
   __shared__ bool last;
-  double v[3] = {(double)__reduce_add_sync(0xffffffffu, n), (double)s.x + ((double)e.x + (double)f.x),
-                 (double)s.y + ((double)e.y + (double)f.y)};
-  if (n_wide) {
-    v[1] += b1;
-    v[2] += b2;
-  }
-  for (int q = 1; q < 3; ++q) v[q] = sfft::warp_sum(v[q]);
-  if (lane == 0)
-    for (int q = 0; q < 3; ++q) red[q][warp] = v[q];
+  const int tid = threadIdx.x;
+  n = __reduce_add_sync(0xffffffffu, n);
+  if (lane == 0) rn[warp] = n;
+  if (tid == 0) any_wide = 0;
+  tr[0][tid] = s.x; tr[1][tid] = s.y; tr[2][tid] = e.x; tr[3][tid] = e.y; tr[4][tid] = f.x; tr[5][tid] = f.y;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int q = 0; q < 3; ++q) {
-      double s = 0.0;
-      for (int w = 0; w < 8; ++w) s += red[q][w];
-      pb[blockIdx.x * 3 + q] = s;
+  if (n_wide) any_wide = 1;
+  for (int m = 64; m > 0; m >>= 2) {
+    if (tid < m) {
+#pragma unroll
+      for (int k = m; k < 4 * m; k += m) {
+        float2 r, u;
+        s = two_sum2(s, make_float2(tr[0][tid + k], tr[1][tid + k]), r);
+        e = two_sum2(e, r, u);
+        f = __fadd2_rn(f, u);
+        e = two_sum2(e, make_float2(tr[2][tid + k], tr[3][tid + k]), u);
+        f = __fadd2_rn(__fadd2_rn(f, u), make_float2(tr[4][tid + k], tr[5][tid + k]));
+      }
+      tr[0][tid] = s.x; tr[1][tid] = s.y; tr[2][tid] = e.x; tr[3][tid] = e.y; tr[4][tid] = f.x; tr[5][tid] = f.y;
     }
+    __syncthreads();
+  }
+  if (any_wide) {
+    b1 = sfft::warp_sum(b1);
+    b2 = sfft::warp_sum(b2);
+    if (lane == 0) { rb[0][warp] = b1; rb[1][warp] = b2; }
+    __syncthreads();
+  }
+  if (tid == 0) {
+    double v1 = (double)s.x + ((double)e.x + (double)f.x), v2 = (double)s.y + ((double)e.y + (double)f.y);
+    int c = 0;
+    for (int w = 0; w < 8; ++w) c += rn[w];
+    if (any_wide)
+      for (int w = 0; w < 8; ++w) { v1 += rb[0][w]; v2 += rb[1][w]; }
+    pb[blockIdx.x * 3] = (double)c;
+    pb[blockIdx.x * 3 + 1] = v1;
+    pb[blockIdx.x * 3 + 2] = v2;
     __threadfence();
     last = atomicAdd(&counter[b * kStatPasses + pass], 1) == (int)gridDim.x - 1;
   }
@@ -255,11 +281,11 @@ k_clip_pass(int H, int W, const float* __restrict__ D, const uint8_t* __restrict
 #pragma unroll 4
     for (int i = lane; i < (int)gridDim.x; i += 32) a += __ldcg(pb + i * 3 + warp);
     a = sfft::warp_sum(a);
-    if (lane == 0) red[warp][0] = a;
+    if (lane == 0) red[warp] = a;
   }
   __syncthreads();
   if (warp != 0) return;
-  const double t[3] = {red[0][0], red[1][0], red[2][0]};
+  const double t[3] = {red[0], red[1], red[2]};
   const double m1 = t[1] / t[0];
   const double mean = (double)shift + m1, var = t[2] / t[0] - m1 * m1;
   if (pass == kStatPasses - 1) {   // only the matched filter's scale is left to form
