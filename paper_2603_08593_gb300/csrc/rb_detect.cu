@@ -101,16 +101,18 @@ __device__ __forceinline__ float key_float(unsigned k) { return __uint_as_float(
 // rate, left 7e-16 and took 70 us per pass of 2048 x 4096, pairs of floats 5e-15
 // and 25 us, these 28 us).  FP64 from the thread's end on.  Where the mean lies
 // within three times the scatter, as it does in a difference image, the loop sums
-// about zero, where d is one float (9 us for the four passes), and the thread's
+// about zero, where d is one float (11 us for the four passes), and the thread's
 // triples are moved to the shift at its end: they hold some 70 bits, of which
 // that takes a few.
 // The loop is without branches but for values whose square leaves the range of a
 // float, which wait for the word group's end.  What bounds a pass is the wait for
 // its pixels between the arithmetic of two word groups (more of them in flight
 // cost a CTA per SM: 207 against 204 us for the detector) and, of a small image,
-// the last CTA's chain of FP64 operations: warp 0 tests the candidates of both
-// interval ends at once, and a pass forms only what the next kernel reads
-// (128 x 128: 11.4 -> 9.4 us a pass).
+// the chain of FP64 operations at the end: a CTA converts its sums once, the last
+// one takes a warp per sum, warp 0 tests the candidates of both interval ends at
+// once, and a pass forms only what the next kernel reads (the whole detector,
+// conversions and FP64 additions in every warp -> one per CTA: 128 x 128
+// 66 -> 59 us, 1024 x 1024 95 -> 78 us, 4096 x 2048 197 -> 191 us).
 // The last CTA to finish adds the partials in index order and prepares the next
 // pass: its clipping rule |x - mean| <= 3 sqrt(var), evaluated in FP64, becomes
 // the float interval of the pixels that satisfy it (the rule is monotone on
