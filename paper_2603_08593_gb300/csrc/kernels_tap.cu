@@ -203,7 +203,7 @@ k_tap_reduce(const T* __restrict__ part, const double* __restrict__ mpart, const
 // ------------------------------------------------------------------ edge sums
 // H_m(u, u') over one list: a CTA stages 32 edge points at a time (the L^2
 // reference values around each, signed powers of xt and powers of yt) and each
-// thread keeps a 2 x 2 tile of pairs x all monomials in registers.  The points
+// thread keeps a tile of 2 x 2 (or 4) pairs x all monomials in registers.  The points
 // of the next batch are copied (cp.async) while this one is summed, and the list
 // is read two batches ahead; without it the gathers' latency took 60 % of the
 // warps' time.  The list is in row order: a thread sums the powers of xt over a
@@ -229,20 +229,30 @@ constexpr int kGramPts = 32;
 constexpr int kGramRun = 256;
 constexpr int kGramThreads = 256;
 constexpr int kGramOne = 122;     // L^2 <= 121 values, then (1, 0): the partner of single offsets
+// offsets j of a tile: with few monomials a point's sums are few, and the copies
+// of its patch in every block of tiles weigh more (assembly of four CCDs of
+// 1000 x 300, L = 11, D_K = 0: 167 us with two, 160 us with four; at D_K = 1 and
+// 512 x 512, L = 9, 115 with two and 121 with four)
+constexpr int gram_tj(int DE) { return DE <= 1 ? 4 : 2; }
 constexpr int kGramPatch = 124;   // even: two neighbouring offsets in one read
 constexpr int kGramPow = 10;      // powers of a coordinate, in rows that spread over the banks
 // least points of a slot: FP64 multiply-adds are 64 times slower than FP32
 // ones, so there a short list spreads over more slots (a 512 x 512 pair, L = 7,
 // D_K = 1: 853 us with 64 points, 819 us with 32).  FP32: more slots cost
 // k_edge_reduce more than they give here (a 4096 x 2048 pair, L = 11, D_K = 2:
-// 1742 us with 64 points, 1734 with 128, 1727 with 256)
+// 1742 us with 64 points, 1734 with 128, 1727 with 256) ...
 template <typename T> constexpr int kGramMin = sizeof(T) == 4 ? 256 : kGramPts;
+// ... but for the slots that give every SM a CTA: the lists of a small image are
+// a few hundred points, one after another in a few CTAs (assembly of 512 x 512,
+// L = 9, D_K = 1: 138 us without, 115 with; L = 11, D_K = 2: 195 and 167)
+constexpr int kGramFew = 32;
 
 struct GramArgs {
   const int* tiles;        // i | j << 8, the tile's first offsets: y tiles, then x tiles
   int nty, ntx, nbx;       // tiles and x blocks
   int npy, npx;            // pairs
   int gy, gx;              // most slots per list
+  int fy, fx;              // slots that give every SM a CTA
   int64_t hp_stride;       // per CCD
   int64_t hx_off;          // x partials after the y ones
   int64_t lo_off;          // the pairs' second floats (mixed path, lists of more than kGramRun points per slot)
@@ -250,7 +260,9 @@ struct GramArgs {
 };
 
 template <typename T>
-__device__ __forceinline__ int gram_slots(int n, int g) { return max(1, min(g, (n + kGramMin<T> - 1) / kGramMin<T>)); }
+__device__ __forceinline__ int gram_slots(int n, int g, int fill) {
+  return max(1, min(g, max((n + kGramMin<T> - 1) / kGramMin<T>, min((n + kGramFew - 1) / kGramFew, fill))));
+}
 // whether a slot's share of n points in U slots may be summed in more than one run
 template <typename T>
 __device__ __forceinline__ bool gram_runs(int n, int U) {
@@ -296,7 +308,7 @@ template <typename T, int DE>
 __global__ void __launch_bounds__(kGramThreads, sizeof(T) == 4 ? 2 : 1)
 k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const unsigned* __restrict__ ly, int64_t lstride,
             const int* __restrict__ cnt, int64_t cnt_stride, GramArgs a, T* __restrict__ hp, int H, int W, int L) {
-  constexpr int NM = n_mono(DE), CD = sizeof(T) == 4 ? 2 : 1, PW = kGramPow * CD;
+  constexpr int NM = n_mono(DE), CD = sizeof(T) == 4 ? 2 : 1, PW = kGramPow * CD, NJ = gram_tj(DE) / 2;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int2 offs[kGramPatch];   // u as a distance in the image; u_y and u_x
   T(*px)[kGramPts][PW] = reinterpret_cast<T(*)[kGramPts][PW]>(smraw);
@@ -307,7 +319,7 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
   const int ccd = blockIdx.z, tid = threadIdx.x, w = (L - 1) / 2, lane = tid & 31, warp = tid >> 5;
   const bool isx = (int)blockIdx.y < a.nbx;
   const int n = cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H];
-  const int U = gram_slots<T>(n, isx ? a.gx : a.gy), g = blockIdx.x;
+  const int U = gram_slots<T>(n, isx ? a.gx : a.gy, isx ? a.fx : a.fy), g = blockIdx.x;
   if (g >= U) return;
   const int tile = (isx ? blockIdx.y : blockIdx.y - a.nbx) * kGramThreads + tid, nt = isx ? a.ntx : a.nty;
   const unsigned* list = (isx ? lx : ly) + ccd * lstride;
@@ -317,10 +329,10 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
     const int uy = tid / L - w, ux = tid % L - w;
     offs[tid] = make_int2(uy * W + ux, (uy + w) << 8 | (ux + w));
   }
-  // (j, j + 1) packed, for i and i + 1: sums over a row, and all rows times yt^b
-  v2<T> rs[2][DE + 1], acc[2][NM];
+  // (j, j + 1) packed, for i and i + 1 (and the same for j + 2): sums over a row, and all rows times yt^b
+  v2<T> rs[2 * NJ][DE + 1], acc[2 * NJ][NM];
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
+  for (int q = 0; q < 2 * NJ; ++q) {
 #pragma unroll
     for (int k = 0; k <= DE; ++k) v2_zero(rs[q][k]);
 #pragma unroll
@@ -397,18 +409,23 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
       const T *pj = &patch[s][pt][tj], *pi = &patch[s][pt][ti], *pq = &px[s][pt][0];
 #pragma unroll 4
       for (int i = 0; i < c; ++i, pj += kGramPatch, pi += kGramPatch, pq += PW) {
-        const v2<T> rj = v2_load(pj), ri = v2_load(pi);
-        const v2<T> r0 = v2_make(v2_get(ri, 0) * v2_get(rj, 0), v2_get(ri, 0) * v2_get(rj, 1));
-        const v2<T> r1 = v2_make(v2_get(ri, 1) * v2_get(rj, 0), v2_get(ri, 1) * v2_get(rj, 1));
+        const v2<T> ri = v2_load(pi);
+        v2<T> r[2 * NJ];
+#pragma unroll
+        for (int h = 0; h < NJ; ++h) {
+          const v2<T> rj = v2_load(pj + 2 * h);
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            r[2 * h + q] = v2_make(v2_get(ri, q) * v2_get(rj, 0), v2_get(ri, q) * v2_get(rj, 1));
+        }
 #pragma unroll
         for (int k = 0; k <= DE; k += 2) {
-          v2<T> q[2];
-          v2_dup2(pq + CD * k, q[0], q[1]);
+          v2<T> x[2];
+          v2_dup2(pq + CD * k, x[0], x[1]);
 #pragma unroll
-          for (int h = 0; h < 2 && k + h <= DE; ++h) {
-            v2_fmav(rs[0][k + h], q[h], r0);
-            v2_fmav(rs[1][k + h], q[h], r1);
-          }
+          for (int h = 0; h < 2 && k + h <= DE; ++h)
+#pragma unroll
+            for (int q = 0; q < 2 * NJ; ++q) v2_fmav(rs[q][k + h], x[h], r[q]);
         }
       }
       pt += c;
@@ -416,24 +433,22 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
       for (int q = 0; q <= DE; ++q) {
         const v2<T> yb = v2_dup(&py[s][pt - 1][CD * q]);
 #pragma unroll
-        for (int k = 0; k <= DE - q; ++k) {
-          v2_fmav(acc[0][mono_index(k, q)], yb, rs[0][k]);
-          v2_fmav(acc[1][mono_index(k, q)], yb, rs[1][k]);
-        }
+        for (int k = 0; k <= DE - q; ++k)
+#pragma unroll
+          for (int h = 0; h < 2 * NJ; ++h) v2_fmav(acc[h][mono_index(k, q)], yb, rs[h][k]);
       }
 #pragma unroll
-      for (int k = 0; k <= DE; ++k) {
-        v2_zero(rs[0][k]);
-        v2_zero(rs[1][k]);
-      }
+      for (int k = 0; k <= DE; ++k)
+#pragma unroll
+        for (int h = 0; h < 2 * NJ; ++h) v2_zero(rs[h][k]);
     }
     if (warp == 0) put(e2, s);
     rows += __popc(last);
     const bool end = b + U >= nb;
     if (!end && !(runs && rows > kGramRun - kGramPts)) continue;
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int id = tile < nt ? gram_pair(L, isx, ti + (p >> 1), tj + (p & 1)) : -1;
+    for (int p = 0; p < 4 * NJ; ++p) {
+      const int id = tile < nt ? gram_pair(L, isx, ti + ((p >> 1) & 1), tj + 2 * (p >> 2) + (p & 1)) : -1;
       if (id >= 0)
 #pragma unroll
         for (int k = 0; k < NM; ++k) {
@@ -449,7 +464,7 @@ k_edge_gram(const T* __restrict__ Rm, const unsigned* __restrict__ lx, const uns
         }
     }
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
+    for (int q = 0; q < 2 * NJ; ++q)
 #pragma unroll
       for (int k = 0; k < NM; ++k) v2_zero(acc[q][k]);
     first = false;
@@ -466,7 +481,7 @@ k_edge_reduce(const T* __restrict__ hp, GramArgs a, const int* __restrict__ cnt,
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= ny + nx) return;
   const bool isx = i >= ny;
-  const int n = cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H], U = gram_slots<T>(n, isx ? a.gx : a.gy);
+  const int n = cnt[ccd * cnt_stride + (isx ? 0 : H + 1) + H], U = gram_slots<T>(n, isx ? a.gx : a.gy, isx ? a.fx : a.fy);
   const int64_t st = isx ? nx : ny;
   const T* p = hp + ccd * a.hp_stride + (isx ? a.hx_off + i - ny : i);
   double s = 0.0;
@@ -684,19 +699,22 @@ void build_tap_plan(sfft_plan_s* p) {
   // the refinement's half tiles (kernels_apply.cu)
   t.ntile_rhs = 2 * conv_tiles(p->d.H, p->d.W, conv_half_width(p->d.H, p->d.W, B));
   // edge sums
+  t.DE = std::max(dKK, dKB);
+  t.MP = n_mono(t.DE);
   t.tiles.clear();
   t.npy = t.npx = t.nty = t.ntx = 0;
   if (t.mode == TAP_FIT_EDGE) {
     const int n = L * (L - 1);   // offsets below the row u_y = w, an even number
     t.npy = ypair_single(L, n);
     t.npx = xpair_single(L, L - 1);
+    const int tj = gram_tj(t.DE), one = kGramOne / tj * tj;   // the tile that holds the ones
     for (int i = 0; i < n; i += 2)
-      for (int j = 0; j <= i; j += 2) t.tiles.push_back(i | j << 8);
-    for (int j = 0; j < n; j += 2) t.tiles.push_back(kGramOne | j << 8);
+      for (int j = 0; j <= i + 1; j += tj) t.tiles.push_back(i | j << 8);
+    for (int j = 0; j < n; j += tj) t.tiles.push_back(kGramOne | j << 8);
     t.nty = (int)t.tiles.size();
     for (int ix = 0; ix < L - 1; ix += 2) {
-      for (int j = 0; j <= n + ix; j += 2) t.tiles.push_back((n + ix) | j << 8);
-      t.tiles.push_back((n + ix) | kGramOne << 8);
+      for (int j = 0; j <= n + ix + 1; j += tj) t.tiles.push_back((n + ix) | j << 8);
+      t.tiles.push_back((n + ix) | one << 8);
     }
     t.ntx = (int)t.tiles.size() - t.nty;
     t.nby = (t.nty + kGramThreads - 1) / kGramThreads;
@@ -705,8 +723,6 @@ void build_tap_plan(sfft_plan_s* p) {
     t.gy = std::max(16, 608 / (t.nby * B));
     t.gx = std::max(64, 304 / (t.nbx * B));
   }
-  t.DE = std::max(dKK, dKB);
-  t.MP = n_mono(t.DE);
   // M is an erosion by L x L: its zero runs are at least L wide between the borders
   t.row_cap = L == 1 ? p->d.W : std::min(p->d.W, 2 * (p->d.W / (L + 1) + 2));
   t.col_cap = L == 1 ? p->d.H : std::min(p->d.H, 2 * (p->d.H / (L + 1) + 2));
@@ -805,6 +821,7 @@ static cudaError_t edge_sums_T(const sfft_plan_s* p, void* ws) {
   a.nty = t.nty; a.ntx = t.ntx; a.nbx = t.nbx;
   a.npy = t.npy; a.npx = t.npx;
   a.gy = t.gy; a.gx = t.gx;
+  a.fy = 152 / (t.nby * B); a.fx = 152 / (t.nbx * B);
   a.xs = step_of(W); a.ys = step_of(H);
   a.hx_off = (int64_t)t.gy * t.npy * t.MP;
   a.lo_off = a.hx_off + (int64_t)t.gx * t.npx * t.MP;
